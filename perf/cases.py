@@ -213,7 +213,7 @@ def draw(rng):
         precision, flavour = rng.choice([("mixed", "precond"), ("mixed", "precond"), ("mixed", "cholesky"),
                                          ("fp64", "precond"), ("fp64", "cholesky")])
         norb = rng.choice([4, 8, 13, 16, 23])
-        top = 900 if precision == "fp64" else 2944 if flavour == "cholesky" else {4: 2500, 23: 3000}.get(norb, 6000)
+        top = 900 if precision == "fp64" else 2944 if flavour == "cholesky" else {4: 2500, 8: 5000, 23: 3000}.get(norb, 6000)
         return {"kind": kind, "units": max(4, log_int(rng, 100, top) // norb), "norb": norb, "precision": precision,
                 "flavour": flavour}
     if kind == "scf":
