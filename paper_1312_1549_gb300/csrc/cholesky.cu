@@ -37,77 +37,181 @@ constexpr int NB = 64;
 
 // Factor the b x b diagonal block at A (ld lda) in place (lower) and write
 // its inverse to Linv (NB x NB, row-major, zero above the diagonal); with Pblk
-// (ld ldp) also the block Linv^T Linv (both triangles). Every division is a
-// multiplication by one reciprocal per pivot: float64 division is a long
-// instruction sequence on this GPU's narrow float64 pipe. R is the arithmetic
-// type: double, or float for a preconditioner, which needs far less than float64
-// accuracy and which the float64 pipe (about 2 instructions per SM and clock)
-// would make the serial bottleneck of the recursive inverse.
-template <typename R>
-__global__ void __launch_bounds__(256)
-potf2_inv_kernel(double* A, long lda, int b, double* Linv, int* info, int col_offset, double* Pblk, long ldp) {
-  __shared__ R L[NB][NB + 1];
-  __shared__ R X[NB][NB + 1];
-  __shared__ R rdiag[NB];
-  const int tid = threadIdx.x;
-  for (int idx = tid; idx < NB * NB; idx += blockDim.x) {
+// (ld ldp) also the block Linv^T Linv (both triangles), in float64 on one CTA.
+// The factor, the inverse and the Gram block take 44 thousand FMAs each, 11 us
+// each at the two per clock of one SM, so the work is laid out for that pipe:
+// no FMA on zeros beyond 8-wide blocks, all eight warps busy, short dependent
+// chains. Right-looking in panels of eight columns: warp 0 factors a panel
+// with its rows in registers (pivots and column entries by shuffles, one
+// rsqrt per pivot), then all warps apply its rank-8 update on 8 x 8 blocks.
+// The inverse joins inverted diagonal blocks of edge 8, 16 and 32:
+// X21 = -X22 (L21 X11), the contraction cut at the triangles.
+// (One column at a time with three barriers each, one thread per column of the
+// inverse and two divisions per pivot it took 150-215 us per block; the float64-class inverse at
+// m = 3328, 52 blocks one after another, went from 30.1 to 25.9 ms.)
+constexpr int kLeaf64Threads = 256;
+
+__global__ void __launch_bounds__(kLeaf64Threads)
+leaf_f64_kernel(double* A, long lda, int b, double* Linv, int* info, int col_offset, double* Pblk, long ldp) {
+  __shared__ double L[NB][NB + 1];
+  __shared__ double X[NB][NB + 1];
+  __shared__ double rdiag[NB];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  constexpr int kWarps = kLeaf64Threads / 32;
+  for (int idx = tid; idx < NB * NB; idx += kLeaf64Threads) {
     const int i = idx / NB, j = idx % NB;
-    L[i][j] = (i < b && j < b && j <= i) ? (R)A[(long)i * lda + j] : (R)0;
+    L[i][j] = (i < b && j <= i) ? A[(long)i * lda + j] : 0.0;
+    X[i][j] = 0.0;
   }
   __syncthreads();
-  for (int j = 0; j < b; ++j) {
-    if (tid == 0) {
-      R d = L[j][j];
-      if (!(d > (R)0)) {
-        atomicCAS(info, 0, col_offset + j + 1);
-        d = (R)1;
+  for (int p0 = 0; p0 < b; p0 += 8) {
+    const int pw = min(8, b - p0);
+    if (warp == 0) {  // lane l holds rows p0 + l and p0 + l + 32
+      double r[2][8];
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        const int i = p0 + lane + 32 * t;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) r[t][c] = (i < b && c < pw && p0 + c <= i) ? L[i][p0 + c] : 0.0;
       }
-      const R r = sqrt(d);
-      L[j][j] = r;
-      rdiag[j] = (R)1 / r;
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        if (c < pw) {
+          double d = __shfl_sync(0xffffffffu, r[0][c], c);  // the pivot, row p0 + c
+          if (!(d > 0.0)) {
+            if (lane == 0) atomicCAS(info, 0, col_offset + p0 + c + 1);
+            d = 1.0;
+          }
+          // 1 / sqrt(d) and sqrt(d) to the last place: one Newton step each on rsqrt's value
+          double rs = rsqrt(d), sq = sqrt(d);
+          if (rs > 0.0) rs = fma(0.5 * rs, fma(-(d * rs), rs, 1.0), rs);  // (0 only for an infinite pivot)
+#pragma unroll
+          for (int t = 0; t < 2; ++t) {
+            const int i = p0 + lane + 32 * t;
+            if (i > p0 + c) r[t][c] *= rs;
+            else if (i == p0 + c) r[t][c] = sq;
+          }
+          if (lane == 0) rdiag[p0 + c] = rs;
+#pragma unroll
+          for (int l = 0; l < 8; ++l) {
+            if (l > c) {
+              const double lc = __shfl_sync(0xffffffffu, r[0][c], l);  // L[p0 + l][p0 + c]
+              if (lane >= l) r[0][l] = fma(-r[0][c], lc, r[0][l]);
+              if (p0 + 32 < b) r[1][l] = fma(-r[1][c], lc, r[1][l]);
+            }
+          }
+        }
+      }
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        const int i = p0 + lane + 32 * t;
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+          if (i < b && c < pw && p0 + c <= i) L[i][p0 + c] = r[t][c];
+      }
     }
     __syncthreads();
-    const R rj = rdiag[j];
-    for (int i = j + 1 + tid; i < b; i += blockDim.x) L[i][j] *= rj;
-    __syncthreads();
-    const int r = b - j - 1;
-    for (int idx = tid; idx < r * r; idx += blockDim.x) {
-      const int i = j + 1 + idx / r, l = j + 1 + idx % r;
-      if (l <= i) L[i][l] = fma(-L[i][j], L[l][j], L[i][l]);
+    // trailing lower triangle in 8 x 8 blocks (I, J <= I), a warp per block, two rows per lane
+    const int q0 = p0 + 8, nb8 = (b - q0 + 7) / 8;
+    for (int q = warp, I = 0, base = 0; I < nb8; ) {
+      if (q >= base + I + 1) { base += I + 1; ++I; continue; }
+      const int J = q - base;
+      const int i = q0 + 8 * I + (lane >> 3), j = q0 + 8 * J + (lane & 7);
+      double a0 = L[i][j], a1 = L[i + 4][j];  // (rows and columns past b hold zeros)
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const double lj = L[j][p0 + k];
+        a0 = fma(-L[i][p0 + k], lj, a0);
+        a1 = fma(-L[i + 4][p0 + k], lj, a1);
+      }
+      if (j <= i) L[i][j] = a0;
+      if (j <= i + 4) L[i + 4][j] = a1;
+      q += kWarps;
     }
     __syncthreads();
   }
-  for (int idx = tid; idx < b * b; idx += blockDim.x) {
-    const int i = idx / b, j = idx % b;
-    A[(long)i * lda + j] = (j <= i) ? (double)L[i][j] : 0.0;
-  }
-  // inverse of the lower-triangular block: column c solves L x = e_c
-  if (tid < NB) {
-    const int c = tid;
-    for (int i = 0; i < NB; ++i) X[i][c] = (R)0;
-    if (c < b) {
-      X[c][c] = rdiag[c];
-      for (int i = c + 1; i < b; ++i) {
-        R acc = (R)0;
-        for (int k = c; k < i; ++k) acc = fma(L[i][k], X[k][c], acc);
-        X[i][c] = -acc * rdiag[i];
+  // inverses of the 8 x 8 diagonal blocks: warp w's lane c solves column c of block w
+  if (8 * warp < b && lane < 8 && 8 * warp + lane < b) {
+    const int o = 8 * warp, c = lane, e = min(8, b - o);
+    double x[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      x[i] = 0.0;
+      if (i == c) x[i] = rdiag[o + i];
+      if (i > c && i < e) {
+        double acc = 0.0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          if (k >= c && k < i) acc = fma(L[o + i][o + k], x[k], acc);
+        x[i] = -acc * rdiag[o + i];
       }
     }
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (i >= c && i < e) X[o + i][o + c] = x[i];
   }
   __syncthreads();
-  for (int idx = tid; idx < NB * NB; idx += blockDim.x) {
+  // Join blocks of edge s: T = L21 X11 (kept transposed in the unused upper triangle of L: T[i][j] of
+  // the pair at o in L[o + j][o + s + i]), X21 = -X22 T. For T a warp takes four rows and walks the
+  // column groups of eight, contracting from the group's first column; for X21 four columns and the row
+  // groups, contracting to the group's last row. (Rows past b are zero in L and X.)
+  for (int s = 8; s < b; s *= 2) {
+    const int wpp = s / 4;  // warps per pair
+    const int pairs = (b + 2 * s - 1) / (2 * s);
+    for (int u = warp; u < pairs * wpp; u += kWarps) {
+      const int o = 2 * s * (u / wpp), i = 4 * (u % wpp) + (lane >> 3);
+      for (int g = 0; g < s; g += 8) {
+        const int j = g + (lane & 7);
+        double acc0 = 0.0, acc1 = 0.0;
+        for (int k = g; k < s; k += 2) {
+          acc0 = fma(L[o + s + i][o + k], X[o + k][o + j], acc0);
+          acc1 = fma(L[o + s + i][o + k + 1], X[o + k + 1][o + j], acc1);
+        }
+        L[o + j][o + s + i] = acc0 + acc1;
+      }
+    }
+    __syncthreads();
+    for (int u = warp; u < pairs * wpp; u += kWarps) {
+      const int o = 2 * s * (u / wpp), j = 4 * (u % wpp) + (lane >> 3);
+      for (int g = 0; g < s; g += 8) {
+        const int i = g + (lane & 7);
+        double acc0 = 0.0, acc1 = 0.0;
+        for (int k = 0; k < g + 8; k += 2) {
+          acc0 = fma(X[o + s + i][o + s + k], L[o + j][o + s + k], acc0);
+          acc1 = fma(X[o + s + i][o + s + k + 1], L[o + j][o + s + k + 1], acc1);
+        }
+        if (o + s + i < b) X[o + s + i][o + j] = -(acc0 + acc1);
+      }
+    }
+    __syncthreads();
+  }
+  for (int idx = tid; idx < NB * NB; idx += kLeaf64Threads) {
     const int i = idx / NB, j = idx % NB;
-    Linv[idx] = (double)X[i][j];
+    if (i < b && j < b) A[(long)i * lda + j] = (j <= i) ? L[i][j] : 0.0;
+    Linv[idx] = X[i][j];
   }
   if (Pblk != nullptr) {
-    // (X^T X)_ij = sum_{k >= i} X_ki X_kj for j <= i, mirrored
-    for (int idx = tid; idx < b * b; idx += blockDim.x) {
-      const int i = idx / b, j = idx % b;
-      if (j > i) continue;
-      R acc = (R)0;
-      for (int k = i; k < b; ++k) acc = fma(X[k][i], X[k][j], acc);
-      Pblk[(long)i * ldp + j] = (double)acc;
-      Pblk[(long)j * ldp + i] = (double)acc;
+    // (X^T X)_ij = sum_{k >= i} X_ki X_kj for j <= i, mirrored: 8 x 8 blocks (I, J <= I), two rows per lane
+    const int nb8 = (b + 7) / 8;
+    for (int q = warp, I = 0, base = 0; I < nb8; ) {
+      if (q >= base + I + 1) { base += I + 1; ++I; continue; }
+      const int J = q - base;
+      const int i = 8 * I + (lane >> 3), j = 8 * J + (lane & 7);
+      double a0 = 0.0, a1 = 0.0;
+      for (int k = 8 * I; k < b; ++k) {  // (X is zero above its diagonal)
+        const double xj = X[k][j];
+        a0 = fma(X[k][i], xj, a0);
+        a1 = fma(X[k][i + 4], xj, a1);
+      }
+      if (i < b && j <= i) {
+        Pblk[(long)i * ldp + j] = a0;
+        Pblk[(long)j * ldp + i] = a0;
+      }
+      if (i + 4 < b && j <= i + 4) {
+        Pblk[(long)(i + 4) * ldp + j] = a1;
+        Pblk[(long)j * ldp + i + 4] = a1;
+      }
+      q += kWarps;
     }
   }
 }
@@ -143,7 +247,7 @@ __device__ __forceinline__ double to_f64(float v) {
 // One CTA: Cholesky factor of the b x b diagonal block at A (b <= 128, read only: the caller
 // does not need L itself), its inverse X = L^-1 into Linv (NL x NL, row-major, zero above the
 // diagonal) and, with Pblk, the block X^T X (both triangles) -- all in float32, for the
-// preconditioner (see potf2_inv_kernel). The triangular inverse is blocked so that all threads
+// preconditioner, which needs far less than float64 accuracy. The triangular inverse is blocked so that all threads
 // work: 16 x 16 diagonal blocks are inverted by one warp each, then pairs of inverted blocks are
 // joined level by level, X21 = -X22 (L21 X11).
 __global__ void __launch_bounds__(kLeafThreads)
@@ -394,7 +498,7 @@ void factor_blocked(cudaStream_t st, int m, double* A, const Work& w, int* info_
     const int k = kb * NB;
     const int b = (m - k < NB) ? (m - k) : NB;
     double* Akk = A + (long)k * m + k;
-    potf2_inv_kernel<double><<<1, 256, 0, st>>>(Akk, m, b, w.Dinv + (long)kb * NB * NB, info_dev, k, nullptr, 0);
+    leaf_f64_kernel<<<1, kLeaf64Threads, 0, st>>>(Akk, m, b, w.Dinv + (long)kb * NB * NB, info_dev, k, nullptr, 0);
     OMM_LAUNCH_CHECK();
     const int r = m - k - b;
     if (r > 0) {
@@ -504,7 +608,7 @@ void leaf(SlicedWork& w, int r0, int b) {
   if (w.nb == NL)  // a preconditioner: 128-wide float32 leaves (see leaf_f32_kernel)
     leaf_f32_kernel<<<1, kLeafThreads, kLeafSmem, w.main.st>>>(w.A + r0 * m + r0, m, b, w.leaf, w.info, r0, pb, m);
   else
-    potf2_inv_kernel<double><<<1, 256, 0, w.main.st>>>(w.A + r0 * m + r0, m, b, w.leaf, w.info, r0, pb, m);
+    leaf_f64_kernel<<<1, kLeaf64Threads, 0, w.main.st>>>(w.A + r0 * m + r0, m, b, w.leaf, w.info, r0, pb, m);
   OMM_LAUNCH_CHECK();
   copy_block_kernel<<<16, 256, 0, w.main.st>>>(b, w.leaf, w.nb, w.Y + r0 * m + r0, m);
   OMM_LAUNCH_CHECK();
