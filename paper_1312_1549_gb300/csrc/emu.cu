@@ -31,43 +31,124 @@ constexpr int kSliceBits = 5;
 
 __device__ __forceinline__ bool stopped(const Scalars* sc) { return sc != nullptr && (sc->done | sc->halt); }
 
-// One warp per row. The row scale sigma = 2^esig comes from the largest
-// magnitude (compared as integer bit patterns). Each element becomes the
-// integer N = rint(x 2^(5s - esig)) (|N| < 2^(5s-1); one float64 multiply by
-// a power of two and one conversion), whose balanced base-32 digits
-// a_{s-1}, ..., a_0 in [-16, 16] are peeled off on the integer pipe:
-// x = sigma sum_i a_i 2^-5(i+1) + r, |r| <= sigma 2^-(5s+1). Slice i holds
-// a_i 2^(esig - 5(i+1)), exact in bf16 (at most 5 significant bits).
-__global__ void slice_rows_kernel(const double* __restrict__ src, long rows, long cols, long ld_src, int s,
-                                  __nv_bfloat16* __restrict__ dst, long ld_dst, long slice_stride,
-                                  const Scalars* sc) {
+// TPR threads per row, four neighbouring columns per thread and step. The row scale sigma = 2^esig
+// comes from the largest magnitude (compared as integer bit patterns). Each element becomes the
+// integer N = rint(x 2^(5s - esig)) (|N| < 2^(5s-1)), whose balanced base-32 digits
+// a_{s-1}, ..., a_0 in [-16, 16] give x = sigma sum_i a_i 2^-5(i+1) + r, |r| <= sigma 2^-(5s+1).
+// Slice i holds a_i 2^(esig - 5(i+1)), exact in bf16 (at most 5 significant bits).
+// Bound by memory (8 bytes in, 2s out per element) once nothing runs on the float64 pipe (two
+// lanes per SM and clock) and the stores are wide: N is the significand shifted and rounded to
+// nearest even as an integer; with 16 added to every lower digit, the balanced digits are plain
+// 5-bit fields of N; a digit becomes its slice value by one float32 FMA on 2^23 + digit. Rows of up
+// to 4 CH TPR columns stay in registers between the maximum and the digits; longer ones are read
+// twice. (With one warp per row, a 2-byte store per slice and float64 conversions the 51 million
+// elements of a 1024 x 6656 x 6656 product took 1.3 ms, 1.1 TB/s.)
+template <int TPR, int CH>
+__global__ void __launch_bounds__(TPR < 256 ? 256 : TPR)
+slice_rows_kernel(const double* __restrict__ src, long rows, long cols, long ld_src, int s,
+                  __nv_bfloat16* __restrict__ dst, long ld_dst, long slice_stride, const Scalars* sc) {
+  constexpr int THREADS = TPR < 256 ? 256 : TPR, RPB = THREADS / TPR, WPR = TPR / 32;
   if (stopped(sc)) return;
-  const long row = (long)blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (row >= rows) return;
-  const double* x = src + row * ld_src;
+  const int sub = threadIdx.x / TPR, t = threadIdx.x % TPR;
+  const long row = (long)blockIdx.x * RPB + sub;
+  const bool active = row < rows;
+  const double* x = src + (active ? row : 0) * ld_src;
+  const bool vec = (reinterpret_cast<uintptr_t>(x) & 15) == 0;
+  auto load4 = [&](long c, unsigned long long (&u)[4]) {
+    if (vec && c + 3 < cols) {
+      const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(x + c), b = *reinterpret_cast<const ulonglong2*>(x + c + 2);
+      u[0] = a.x; u[1] = a.y; u[2] = b.x; u[3] = b.y;
+    } else {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) u[k] = c + k < cols ? (unsigned long long)__double_as_longlong(x[c + k]) : 0ull;
+    }
+  };
+  constexpr unsigned long long kAbs = 0x7FFFFFFFFFFFFFFFull;
+  unsigned long long v[CH][4];
   unsigned long long mx = 0;  // |x| as bits: ordered like the magnitudes (finite values)
-  for (long c = lane; c < cols; c += 32)
-    mx = max(mx, (unsigned long long)__double_as_longlong(x[c]) & 0x7FFFFFFFFFFFFFFFull);
+  if (active) {
+#pragma unroll
+    for (int h = 0; h < CH; ++h) {
+      const long c = 4L * (t + h * TPR);
+      if (c < cols) {
+        load4(c, v[h]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) mx = max(mx, v[h][k] & kAbs);
+      }
+    }
+    for (long c = 4L * (t + CH * TPR); c < cols; c += 4L * TPR) {
+      unsigned long long u[4];
+      load4(c, u);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) mx = max(mx, u[k] & kAbs);
+    }
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (WPR > 1) {
+    __shared__ unsigned long long sh[THREADS / 32];
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = mx;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < WPR; ++w) mx = max(mx, sh[sub * WPR + w]);
+  }
+  if (!active) return;
   int e = 0;  // max|x| < 2^e (frexp convention; 0 for an all-zero row)
   const int ebits = (int)(mx >> 52);
   if (ebits > 0) e = ebits - 1022;
   else if (mx != 0) frexp(__longlong_as_double((long long)mx), &e);  // subnormal maximum
   const int esig = e + 1;  // sigma = 2^esig > 2 max|x|
   __nv_bfloat16* out = dst + row * ld_dst;
-  const double to_int = ldexp(1.0, kSliceBits * s - esig);
-  for (long c = lane; c < cols; c += 32) {
-    long long N = __double2ll_rn(x[c] * to_int);  // |x| 2^-esig < 1/2, so |N| < 2^(5s-1)
-    for (int i = s - 1; i >= 0; --i) {
-      long long a = N;
-      if (i > 0) {
-        a = ((N + 16) & 31) - 16;  // balanced digit in [-16, 15]
-        N = (N - a) >> kSliceBits;
-      }
-      out[i * slice_stride + c] = __float2bfloat16_rn(ldexpf((float)a, esig - kSliceBits * (i + 1)));
+  const bool plain = esig <= 100 && esig - kSliceBits * s >= -125;  // every slice unit times 2^24 is a normal float32
+  // 16 for every digit below the top one, in its place
+  const unsigned long long bias = s > 1 ? 16ull * (((1ull << (kSliceBits * (s - 1))) - 1) / 31) : 0ull;
+  auto emit = [&](long c, const unsigned long long (&u)[4]) {
+    long long N[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const unsigned long long mag = u[k] & kAbs;
+      const int eb = (int)(mag >> 52);
+      const unsigned long long M = (mag & 0x000FFFFFFFFFFFFFull) | (eb ? 1ull << 52 : 0ull);
+      const int shift = esig + 1075 - kSliceBits * s - (eb ? eb : 1);  // x 2^(5s - esig) = M 2^-shift
+      unsigned long long q = 0;
+      if (shift <= 0) q = M << -shift;  // (rows whose maximum is subnormal)
+      else if (shift < 64) q = (M + ((1ull << (shift - 1)) - 1) + ((M >> shift) & 1ull)) >> shift;
+      N[k] = (long long)((u[k] >> 63) ? 0ull - q : q) + (long long)bias;
     }
+    for (int i = 0; i < s; ++i) {
+      const int at = kSliceBits * (s - 1 - i);
+      unsigned short h[4];
+      if (plain) {
+        const float unit = __uint_as_float((unsigned)(esig - kSliceBits * (i + 1) + 127) << 23);
+        const int off = i > 0 ? 16 : 0;
+        const float base = -(12582912.f + (float)off) * unit;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int field = i > 0 ? (int)((unsigned long long)N[k] >> at) & 31 : (int)(N[k] >> at);
+          const float f = fmaf(__uint_as_float(0x4B400000u + (unsigned)field), unit, base);  // exact
+          h[k] = (unsigned short)(__float_as_uint(f) >> 16);
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int a = i > 0 ? ((int)((unsigned long long)N[k] >> at) & 31) - 16 : (int)(N[k] >> at);
+          h[k] = __bfloat16_as_ushort(__float2bfloat16_rn(ldexpf((float)a, esig - kSliceBits * (i + 1))));
+        }
+      }
+      __nv_bfloat16* o = out + i * slice_stride + c;
+      // (ld_dst is a multiple of 8; columns past cols up to the next multiple of 4 are zeros)
+      *reinterpret_cast<uint2*>(o) = make_uint2(h[0] | ((unsigned)h[1] << 16), h[2] | ((unsigned)h[3] << 16));
+    }
+  };
+#pragma unroll
+  for (int h = 0; h < CH; ++h) {
+    const long c = 4L * (t + h * TPR);
+    if (c < cols) emit(c, v[h]);
+  }
+  for (long c = 4L * (t + CH * TPR); c < cols; c += 4L * TPR) {
+    unsigned long long u[4];
+    load4(c, u);
+    emit(c, u);
   }
 }
 
@@ -103,11 +184,16 @@ namespace emu {
 void slice_rows(cudaStream_t st, const double* src, long rows, long cols, long ld_src, int s,
                 __nv_bfloat16* dst, long ld_dst, const Scalars* sc) {
   if (rows <= 0) return;
-  const int warps = 8;
-  const long blocks = (rows + warps - 1) / warps;
-  slice_rows_kernel<<<(unsigned)blocks, warps * 32, 0, st>>>(src, rows, cols, ld_src, s, dst, ld_dst,
-                                                               rows * ld_dst, sc);
-  OMM_LAUNCH_CHECK();
+  auto go = [&](auto kernel, int threads, int rows_per_block) {
+    kernel<<<(unsigned)((rows + rows_per_block - 1) / rows_per_block), threads, 0, st>>>(
+        src, rows, cols, ld_src, s, dst, ld_dst, rows * ld_dst, sc);
+    OMM_LAUNCH_CHECK();
+  };
+  // a row's threads: as few as hold it in registers (4 CH TPR columns), so that short rows fill whole warps
+  if (cols <= 128) go(slice_rows_kernel<32, 1>, 256, 8);
+  else if (cols <= 512) go(slice_rows_kernel<32, 4>, 256, 8);
+  else if (cols <= 2048) go(slice_rows_kernel<128, 4>, 256, 2);
+  else go(slice_rows_kernel<256, 8>, 256, 1);
 }
 
 void transpose(cudaStream_t st, const double* src, long rows, long cols, long ld_src, double* dst, long ld_dst) {
