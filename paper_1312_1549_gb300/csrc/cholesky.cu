@@ -25,6 +25,7 @@
 // of the blocks that follow.
 #include "emu.cuh"
 #include "omm_internal.cuh"
+#include "split_device.cuh"
 #include "tc_gemm.cuh"
 
 #include <algorithm>
@@ -221,28 +222,9 @@ constexpr int NL = 128;
 constexpr int kLeafThreads = 512;
 constexpr int kLeafSmem = (3 * NL * (NL + 1) + NL) * (int)sizeof(float);
 
-// float64 <-> float32 on the integer pipe (normal numbers; magnitudes outside the float32 normal
-// range become zero or infinity), so that the leaf's conversions stay off the narrow float64 units
-__device__ __forceinline__ float to_f32(double x) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
-  const unsigned int sign = (unsigned int)(u >> 32) & 0x80000000u;
-  const int e = (int)((u >> 52) & 0x7FFu);
-  if (e < 1023 - 126) return __uint_as_float(sign);
-  if (e > 1023 + 127) return __uint_as_float(sign | 0x7F800000u);
-  // round the 52-bit fraction to 23 bits, ties to even (a carry moves into the exponent)
-  const unsigned long long f = u & 0x000FFFFFFFFFFFFFull;
-  const unsigned long long r = f + 0x0FFFFFFFull + ((f >> 29) & 1ull);
-  return __uint_as_float(sign + ((unsigned int)(e - 1023 + 127) << 23) + (unsigned int)(r >> 29));
-}
-__device__ __forceinline__ double to_f64(float v) {
-  const unsigned int u = __float_as_uint(v);
-  const unsigned int e = (u >> 23) & 0xFFu;
-  const unsigned long long sign = (unsigned long long)(u & 0x80000000u) << 32;
-  if (e == 0) return __longlong_as_double((long long)sign);  // zero (subnormals flushed)
-  if (e == 0xFFu) return __longlong_as_double((long long)(sign | (0x7FFull << 52) | ((unsigned long long)(u & 0x7FFFFFu) << 29)));
-  return __longlong_as_double(
-      (long long)(sign | ((unsigned long long)(e + 1023u - 127u) << 52) | ((unsigned long long)(u & 0x7FFFFFu) << 29)));
-}
+// float64 <-> float32 on the integer pipe, so that the leaf's conversions stay off the narrow float64 units
+__device__ __forceinline__ float to_f32(double x) { return dev::f32_rne_bits(x); }
+__device__ __forceinline__ double to_f64(float v) { return dev::f64_of_f32(v); }
 
 // One CTA: Cholesky factor of the b x b diagonal block at A (b <= 128, read only: the caller
 // does not need L itself), its inverse X = L^-1 into Linv (NL x NL, row-major, zero above the
@@ -552,8 +534,7 @@ struct Lane {
   double* tr1 = nullptr;
   __nv_bfloat16* sl0 = nullptr;  // slices of two operands
   __nv_bfloat16* sl1 = nullptr;
-  double* partial = nullptr;  // per-chunk sums of the products with few output tiles
-  long partial_cap = 0;
+  double* slab = nullptr;     // float64 sums of the sliced products
 };
 
 struct SlicedWork {
@@ -597,8 +578,7 @@ void sliced_nt(Lane& L, int* err, int M, int N, int K, double alpha, const doubl
     emu::slice_rows(L.st, B, N, K, ldb, s, L.sl1, ld, nullptr);
     ob = tc::make_operand(L.sl1, N, K, ld, s, false);
   }
-  emu::gemm(L.st, oa, ob, K, s, tc::Epilogue{C, ldc, N, 0, alpha, beta, M, N, nullptr, err}, L.partial,
-            L.partial_cap);
+  emu::gemm(L.st, oa, ob, K, s, tc::Epilogue{C, ldc, N, 0, alpha, beta, M, N, nullptr, err}, L.slab);
 }
 
 // leaf: factor A[r0:r0+b, r0:r0+b] in place, write its inverse into Y and Y_leaf^T Y_leaf into P
@@ -674,17 +654,11 @@ void chol_inv(SlicedWork& w, int r0, int b) {
 
 }  // namespace
 
-// chunk sums of the GEMMs with fewer than ~76 output tiles of 128 x 256 (at most 11 chunks)
-long partial_capacity(int m) {
-  const long h = (m + 1) / 2 + NL;
-  return std::min(11L * h * h, 11L * 76 * 128 * 256);
-}
-
 size_t spd_inverse_sliced_workspace_bytes(int m) {
   const long h = (m + 1) / 2 + NL;  // the largest off-diagonal block edge (either leaf size)
-  // Y, prod, leaf; per lane: tr0, tr1, partial
+  // Y, prod, leaf; per lane: tr0, tr1, slab
   const size_t f64 = (size_t)m * m + (size_t)h * h + (size_t)NL * NL +
-                     2 * (2 * (size_t)h * h + (size_t)partial_capacity(m));
+                     2 * (2 * (size_t)h * h + (size_t)tc::sliced_workspace_doubles());
   const size_t bf = 2 * 2 * (size_t)kInvSlices * (size_t)h * round8(h);  // per lane: sl0, sl1
   return f64 * sizeof(double) + bf * sizeof(__nv_bfloat16) + 4 * 256;
 }
@@ -714,9 +688,8 @@ void sliced_impl(cudaStream_t st, int m, double* A, double* P, double* Y_out, vo
     f += h * h;
     L->tr1 = f;
     f += h * h;
-    L->partial = f;
-    L->partial_cap = partial_capacity(m);
-    f += L->partial_cap;
+    L->slab = f;
+    f += tc::sliced_workspace_doubles();
   }
   uintptr_t p = (reinterpret_cast<uintptr_t>(f) + 255) & ~uintptr_t(255);
   const size_t sl = (size_t)kInvSlices * h * round8(h);

@@ -203,24 +203,37 @@ void transpose(cudaStream_t st, const double* src, long rows, long cols, long ld
 }
 
 tc::PairList level_chunks(int K, int s) {
-  // Every chunk holds at most g slice pairs of one level, so that its FP32 sum
-  // of integer units stays below 2^24 and is exact; the float64 epilogue adds
-  // the chunks, smallest level first.
-  const long g_max = (1L << 24) / (256L * (K > 0 ? K : 1));
-  const int g = (int)(g_max < 1 ? 1 : (g_max > tc::kMaxPairs ? tc::kMaxPairs : g_max));
+  // A chunk's FP32 sum is exact while its magnitudes, in units of its smallest level, stay within
+  // 2^24: a product of the level d adds 256 K units of its own level, 32 times as many for every
+  // level below it that the chunk holds. The pairs are taken level by level, smallest first, into as
+  // few chunks as that allows (5 for K = 64, 11 for K = 6656); the float64 epilogue adds the chunks.
+  const long budget = std::max(1L, (1L << 24) / (256L * (K > 0 ? K : 1)));
   tc::PairList pl{};
+  long used = 0;
+  int bottom = -1;  // the smallest level of the open chunk
+  auto close = [&]() {
+    if (bottom < 0) return;
+    if (pl.nchunk == tc::kMaxChunks) throw CudaError{cudaErrorInvalidValue, "emu: too many chunks"};
+    pl.chunk_end[pl.nchunk++] = (unsigned char)pl.n;
+    bottom = -1;
+    used = 0;
+  };
   for (int d = s - 1; d >= 0; --d) {
-    for (int i0 = 0; i0 <= d; i0 += g) {
-      for (int i = i0; i <= d && i < i0 + g; ++i) {
-        if (pl.n == tc::kMaxPairs) throw CudaError{cudaErrorInvalidValue, "emu: too many slice pairs"};
-        pl.a[pl.n] = (unsigned char)i;
-        pl.b[pl.n] = (unsigned char)(d - i);
-        ++pl.n;
+    for (int i = 0; i <= d; ++i) {
+      long cost = bottom < 0 ? 1 : (bottom - d > 6 ? budget + 1 : 1L << (kSliceBits * (bottom - d)));
+      if (bottom >= 0 && used + cost > budget) {
+        close();
+        cost = 1;
       }
-      if (pl.nchunk == tc::kMaxChunks) throw CudaError{cudaErrorInvalidValue, "emu: too many chunks"};
-      pl.chunk_end[pl.nchunk++] = (unsigned char)pl.n;
+      if (bottom < 0) bottom = d;
+      if (pl.n == tc::kMaxPairs) throw CudaError{cudaErrorInvalidValue, "emu: too many slice pairs"};
+      pl.a[pl.n] = (unsigned char)i;
+      pl.b[pl.n] = (unsigned char)(d - i);
+      ++pl.n;
+      used += cost;
     }
   }
+  close();
   return pl;
 }
 
@@ -231,19 +244,17 @@ thread_local Profiler* t_prof = nullptr;
 void set_profiler(Profiler* p) { t_prof = p; }
 
 void gemm(cudaStream_t st, const tc::Operand& A, const tc::Operand& B, int K, int s, const tc::Epilogue& ep,
-          double* partial, long partial_capacity, const tc::BlockLists* sparse) {
-  // one persistent launch: every output tile runs its chunks in order on one CTA (or, for a
-  // product of few tiles with scratch given, every chunk on its own CTA, then one reduction)
+          double* slab, const tc::BlockLists* sparse) {
   const tc::PairList pl = level_chunks(K, s);
   if (t_prof) t_prof->begin(st);
-  tc::gemm_persistent(st, A, B, K, pl, ep, partial, partial_capacity, sparse);
+  tc::gemm_sliced(st, A, B, K, pl, ep, slab, sparse);
   // issued tensor flops (only the visited K blocks of a block-sparse product)
   if (t_prof) t_prof->end(st, 2.0 * ep.M * (double)ep.N * K * pl.n * tc::block_density(sparse));
 }
 
 void gemm_split(cudaStream_t st, const tc::Operand& A, const tc::Operand& B, int K, const tc::Epilogue& ep) {
   if (t_prof) t_prof->begin(st);
-  tc::gemm_persistent(st, A, B, K, tc::pairs_split3(), ep);
+  tc::gemm_split(st, A, B, K, ep);
   if (t_prof) t_prof->end(st, 2.0 * ep.M * (double)ep.N * K * 3.0);
 }
 
@@ -264,8 +275,7 @@ struct EmuState {
   long ldn = 0;
   tc::Operand opHS, opC, opY, opW, opYT, opCT, opXT, opSW, opCTb;  // opCTb: C^T as a B operand
   int* err = nullptr;
-  double* partial = nullptr;  // per-chunk sums of the products with few output tiles
-  long partial_cap = 0;
+  double* slab = nullptr;     // float64 sums of the sliced products (tc::sliced_workspace_doubles)
   tc::BlockLists hs_blocks;   // block sparsity of [H~; S] (256-row blocks)
 };
 
@@ -294,9 +304,7 @@ EmuState* emu_create(cudaStream_t st, int m, int n, int slices, const double* HS
     alloc(&es->XTs, (size_t)kDensitySlices * m * es->ldn, st);
     alloc(&es->SWs, (size_t)kDensitySlices * n * es->ldn, st);
     alloc(&es->err, 1, st);
-    // the [S_W | H_W] product (n x 2n) is the one with few tiles; 11 chunks at most for K <= 16384
-    es->partial_cap = std::min(11L * n * 2L * n, 1L << 25);
-    alloc(&es->partial, (size_t)es->partial_cap, st);
+    alloc(&es->slab, (size_t)tc::sliced_workspace_doubles(), st);
     OMM_CUDA_TRY(cudaMemsetAsync(es->err, 0, sizeof(int), st));
     emu::slice_rows(st, HS, 2L * m, m, m, slices, es->HSs, ldm, nullptr);
     tc::block_lists(st, HS, 2L * m, m, m, 256, es->hs_blocks);
@@ -323,7 +331,7 @@ void emu_update_H(EmuState* es, cudaStream_t st, const double* HS) {
 
 void emu_destroy(EmuState* es, cudaStream_t st) {
   if (!es) return;
-  void* bufs[] = {es->HSs, es->Cs, es->Ys, es->Ws, es->YTs, es->T64, es->CTs, es->XTs, es->SWs, es->err, es->partial};
+  void* bufs[] = {es->HSs, es->Cs, es->Ys, es->Ws, es->YTs, es->T64, es->CTs, es->XTs, es->SWs, es->err, es->slab};
   for (void* b : bufs) mem::release(b, st);
   tc::free_block_lists(es->hs_blocks, st);
   delete es;
@@ -344,12 +352,11 @@ void emu_recompute_state(EmuState* es, cudaStream_t st, Scalars* sc, const doubl
   emu::slice_rows(st, C, n, m, m, s, es->Cs, es->ldm, nullptr);
   // [HC; SC] (n x m layout) = C [H~; S]^T
   emu::gemm(st, es->opC, es->opHS, m, s, tc::Epilogue{Y4, m, m, nm, 1.0, 0.0, n, 2 * m, nullptr, es->err},
-            es->partial, es->partial_cap, &es->hs_blocks);
+            es->slab, &es->hs_blocks);
   emu::slice_rows(st, Y4, 2L * n, m, m, s, es->Ys, es->ldm, nullptr);
   // [S_W | H_W] = C [SC; HC]^T
   emu::gemm(st, es->opC, es->opY, m, s,
-            tc::Epilogue{SWHW + n, 2L * n, n, -(long)n, 1.0, 0.0, n, 2 * n, nullptr, es->err}, es->partial,
-            es->partial_cap);
+            tc::Epilogue{SWHW + n, 2L * n, n, -(long)n, 1.0, 0.0, n, 2 * n, nullptr, es->err}, es->slab);
   launch_functional(st, n, SWHW, part2);
   launch_finish_functional(st, sc, part2, traces_blocks(n));
   // G = 8 HC - 4 [S_W | H_W] [HC; SC]
@@ -358,7 +365,7 @@ void emu_recompute_state(EmuState* es, cudaStream_t st, Scalars* sc, const doubl
   emu::slice_rows(st, es->T64, m, 2L * n, 2L * n, s, es->YTs, es->ld2n, nullptr);
   launch_scale_copy(st, nm, Y4, 8.0, G, nullptr);
   emu::gemm(st, es->opW, es->opYT, 2 * n, s, tc::Epilogue{G, m, m, 0, -4.0, 1.0, n, m, nullptr, es->err},
-            es->partial, es->partial_cap);
+            es->slab);
   launch_gmax(st, nm, G, part);
   launch_finish_gmax(st, sc, part);
 }
@@ -387,11 +394,11 @@ void emu_density(EmuState* es, cudaStream_t st, const double* C, const double* S
   emu::transpose(st, C, n, m, m, CT, n);
   emu::slice_rows(st, CT, m, n, n, s, es->CTs, es->ldn, nullptr);
   emu::slice_rows(st, SWHW, n, n, 2L * n, s, es->SWs, es->ldn, nullptr);   // S_W is symmetric
-  emu::gemm(st, es->opCT, es->opSW, n, s, tc::Epilogue{XT, n, n, 0, 1.0, 0.0, m, n, nullptr, es->err});
+  emu::gemm(st, es->opCT, es->opSW, n, s, tc::Epilogue{XT, n, n, 0, 1.0, 0.0, m, n, nullptr, es->err}, es->slab);
   combine_kernel<<<(unsigned)std::min<long>((mn + 255) / 256, 4096), 256, 0, st>>>(mn, 4.0, CT, -2.0, XT, XT);
   OMM_LAUNCH_CHECK();
   emu::slice_rows(st, XT, m, n, n, s, es->XTs, es->ldn, nullptr);
-  emu::gemm(st, es->opXT, es->opCTb, n, s, tc::Epilogue{D, m, m, 0, 1.0, 0.0, m, m, nullptr, es->err});
+  emu::gemm(st, es->opXT, es->opCTb, n, s, tc::Epilogue{D, m, m, 0, 1.0, 0.0, m, m, nullptr, es->err}, es->slab);
 }
 
 // out = -(2 C^T H~_W C + eta D) given out = D (dE/dS at the minimum), float64-class:
@@ -401,9 +408,9 @@ void emu_minus_edm(EmuState* es, cudaStream_t st, const double* SWHW, double eta
   const int m = es->m, n = es->n, s = kDensitySlices;
   double* VT = es->T64 + (long)m * n;  // m x n
   emu::slice_rows(st, SWHW + n, n, n, 2L * n, s, es->SWs, es->ldn, nullptr);  // H_W is symmetric
-  emu::gemm(st, es->opCT, es->opSW, n, s, tc::Epilogue{VT, n, n, 0, 1.0, 0.0, m, n, nullptr, es->err});
+  emu::gemm(st, es->opCT, es->opSW, n, s, tc::Epilogue{VT, n, n, 0, 1.0, 0.0, m, n, nullptr, es->err}, es->slab);
   emu::slice_rows(st, VT, m, n, n, s, es->XTs, es->ldn, nullptr);
-  emu::gemm(st, es->opXT, es->opCTb, n, s, tc::Epilogue{out, m, m, 0, -2.0, -eta, m, m, nullptr, es->err});
+  emu::gemm(st, es->opXT, es->opCTb, n, s, tc::Epilogue{out, m, m, 0, -2.0, -eta, m, m, nullptr, es->err}, es->slab);
 }
 
 }  // namespace omm

@@ -15,9 +15,10 @@ void transpose(cudaStream_t st, const double* src, long rows, long cols, long ld
 tc::PairList level_chunks(int K, int s);
 // CUDA-event timing of every sliced product issued by this host thread (nullptr: off)
 void set_profiler(Profiler* p);
-// C = alpha A B^T + beta C from s-slice operands (A, B made by slice_rows)
+// C = alpha A B^T + beta C from s-slice operands (A, B made by slice_rows); slab: tc::sliced_workspace_doubles()
+// doubles of scratch
 void gemm(cudaStream_t st, const tc::Operand& A, const tc::Operand& B, int K, int s, const tc::Epilogue& ep,
-          double* partial = nullptr, long partial_capacity = 0, const tc::BlockLists* sparse = nullptr);
+          double* slab, const tc::BlockLists* sparse = nullptr);
 // C = alpha A B^T + beta C from bf16 hi/lo operands (the 3-term split form), timed like the sliced products
 void gemm_split(cudaStream_t st, const tc::Operand& A, const tc::Operand& B, int K, const tc::Epilogue& ep);
 }  // namespace emu

@@ -238,12 +238,13 @@ __device__ __forceinline__ void direction_body(long count, const double* __restr
 // normal range become zero (the float64 units of this GPU retire about two lanes per SM and clock,
 // so even conversions are kept off them where 2^-23 relative accuracy is enough)
 __device__ __forceinline__ float f32_trunc(double x) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
-  const unsigned int sign = (unsigned int)(u >> 32) & 0x80000000u;
-  const int e = (int)((u >> 52) & 0x7FFu);
-  if (e < 1023 - 126) return __uint_as_float(sign);
-  if (e > 1023 + 127) return __uint_as_float(sign | 0x7F800000u);
-  return __uint_as_float(sign | ((unsigned int)(e - 1023 + 127) << 23) | (unsigned int)((u >> 29) & 0x7FFFFFu));
+  // (selects instead of branches, as in f32_rne_bits)
+  const unsigned int hi = (unsigned int)__double2hiint(x), lo = (unsigned int)__double2loint(x);
+  const unsigned int e = (hi >> 20) & 0x7FFu;
+  unsigned int mag = (__funnelshift_l(lo, hi, 3) + 0x40000000u) & 0x7FFFFFFFu;
+  mag = e < 1023u - 126u ? 0u : mag;
+  mag = e > 1023u + 127u ? 0x7F800000u : mag;
+  return __uint_as_float(mag | (hi & 0x80000000u));
 }
 
 // The trace products of Eq. 13, Tr(XY) = sum_ij X_ij Y_ji, on 32x32 tiles

@@ -299,14 +299,13 @@ omm_status omm_kernel_gemm_emu(int M, int N, int K, const double* A, const doubl
   const long ld = (K + 7) / 8 * 8;
   __nv_bfloat16* buf = nullptr;
   int* err = nullptr;
-  double* partial = nullptr;  // chunk sums, for products of few tiles (as the solver runs them)
-  const long partial_cap = std::min(11L * M * N, 1L << 24);
+  double* slab = nullptr;  // float64 sums of the sliced product
   omm_status rc = OMM_OK;
   try {
     const size_t na = (size_t)slices * M * ld, nb = (size_t)slices * N * ld;
     if (cudaMalloc((void**)&buf, (na + nb) * sizeof(__nv_bfloat16)) != cudaSuccess ||
         cudaMalloc((void**)&err, sizeof(int)) != cudaSuccess ||
-        cudaMalloc((void**)&partial, partial_cap * sizeof(double)) != cudaSuccess) {
+        cudaMalloc((void**)&slab, tc::sliced_workspace_doubles() * sizeof(double)) != cudaSuccess) {
       cudaGetLastError();
       if (buf) cudaFree(buf);
       if (err) cudaFree(err);
@@ -318,8 +317,7 @@ omm_status omm_kernel_gemm_emu(int M, int N, int K, const double* A, const doubl
     emu::slice_rows(st, B, N, K, K, slices, buf + na, ld, nullptr);
     tc::Operand oa = tc::make_operand(buf, M, K, ld, slices, true);
     tc::Operand ob = tc::make_operand(buf + na, N, K, ld, slices, false);
-    emu::gemm(st, oa, ob, K, slices, tc::Epilogue{C, N, N, 0, alpha, beta, M, N, nullptr, err}, partial,
-              partial_cap);
+    emu::gemm(st, oa, ob, K, slices, tc::Epilogue{C, N, N, 0, alpha, beta, M, N, nullptr, err}, slab);
     int h = 0;
     OMM_CUDA_TRY(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, st));
     OMM_CUDA_TRY(cudaStreamSynchronize(st));
@@ -332,7 +330,7 @@ omm_status omm_kernel_gemm_emu(int M, int N, int K, const double* A, const doubl
   }
   if (buf) cudaFree(buf);
   if (err) cudaFree(err);
-  if (partial) cudaFree(partial);
+  if (slab) cudaFree(slab);
   return rc;
 }
 

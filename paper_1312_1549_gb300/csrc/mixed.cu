@@ -307,7 +307,7 @@ void mixed_recompute_state(MixedState* ms, cudaStream_t st, Scalars* sc, const d
   eg.x1f = ms->dY32;
   eg.ldf = ldm;
   eg.xs = 8.0;
-  tc::gemm_persistent(st, ms->opW, ms->opYgrad, 4 * n, tc::pairs_split3(), eg);
+  tc::gemm_split(st, ms->opW, ms->opYgrad, 4 * n, eg);
   launch_gmax(st, nm, G, part);
   launch_finish_gmax(st, sc, part);
 }

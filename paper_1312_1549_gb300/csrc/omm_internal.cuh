@@ -140,7 +140,6 @@ void spd_inverse(cudaStream_t st, int m, double* A, double* P, double* work, int
 // 2..10; 10 is float64-class); A is overwritten. err_dev receives a nonzero code if a bounded
 // wait of a tensor-core GEMM expired.
 size_t spd_inverse_sliced_workspace_bytes(int m);
-long partial_capacity(int m);  // chunk-sum scratch (doubles) of the sliced products of an m x m inverse
 void spd_inverse_sliced(cudaStream_t st, int m, double* A, double* P, void* work, int* info_dev, int* err_dev,
                         int slices = 10);
 // The factor alone, for the reduction to standard form: A = L L^T with L left in A (lower

@@ -90,41 +90,36 @@ __device__ __forceinline__ void split_bits(double x, unsigned short& h, unsigned
   l = bf16_bits_rne(__longlong_as_double((long long)bits));
 }
 
-// float64 -> float32 rounded to nearest even on the integer pipe (the float64 units retire about
-// one lane per SM and clock); magnitudes below the float32 normal range become zero, above it
-// infinity
+// Conversions between float64 and float32 on the integer pipe, without branches: the float64 units
+// of this GPU retire about two lanes per SM and clock (a hardware conversion takes a warp some 60
+// clocks in a GEMM epilogue), and a version that branches on the special cases took 100 clocks per
+// element, most of an epilogue's time (128 columns: 13 thousand clocks), for its divergence
+// bookkeeping. Here the special cases are selects on about ten 32-bit instructions.
+
+// float64 -> float32 rounded to nearest even; magnitudes below the float32 normal range become
+// zero, above it infinity
 __device__ __forceinline__ float f32_rne_bits(double x) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
-  const unsigned int hi32 = (unsigned int)(u >> 32);
-  const unsigned int sign = hi32 & 0x80000000u;
-  const int e = (int)((hi32 >> 20) & 0x7FFu);
-  if (e < 1023 - 126) return __uint_as_float(sign);
-  if (e > 1023 + 127) return __uint_as_float(sign | 0x7F800000u);
-  // fraction f (52 bits) -> 23 bits: add half an ulp minus one plus the lsb (ties to even); a
-  // carry out of the fraction moves into the exponent
-  const unsigned long long f = u & 0x000FFFFFFFFFFFFFull;
-  const unsigned long long r = f + 0x000000000FFFFFFFull + ((f >> 29) & 1ull);
-  return __uint_as_float(sign + ((unsigned int)(e - 1023 + 127) << 23) + (unsigned int)(r >> 29));
+  const unsigned int hi = (unsigned int)__double2hiint(x), lo = (unsigned int)__double2loint(x);
+  // exponent and top 23 fraction bits, the exponent rebiased by -896 (modulo 2^32: 896 << 23)
+  const unsigned int t = __funnelshift_l(lo, hi, 3) + 0x40000000u;
+  // one unit more if the 29 bits below round up (ties to even); a carry moves into the exponent
+  const unsigned int up = ((lo & 0x1FFFFFFFu) + 0x0FFFFFFFu + (t & 1u)) >> 29;
+  const unsigned int e = (hi >> 20) & 0x7FFu;
+  unsigned int mag = (t & 0x7FFFFFFFu) + up;
+  mag = e < 1023u - 126u ? 0u : mag;
+  mag = e > 1023u + 127u ? 0x7F800000u : mag;
+  return __uint_as_float(mag | (hi & 0x80000000u));
 }
 
-// float32 -> float64 on the integer pipe (exact; zeros keep their sign, subnormals are
-// normalised, infinities and NaNs keep their class)
+// float32 -> float64 (exact; zeros keep their sign, infinities and NaNs their class)
 __device__ __forceinline__ double f64_of_f32(float f) {
-  const unsigned int u = __float_as_uint(f);
-  const unsigned int e = (u >> 23) & 0xFFu, m = u & 0x7FFFFFu;
-  const unsigned long long sign = (unsigned long long)(u & 0x80000000u) << 32;
-  unsigned long long bits;
-  if (e != 0 && e != 0xFFu) {
-    bits = sign | ((unsigned long long)(e + (1023u - 127u)) << 52) | ((unsigned long long)m << 29);
-  } else if (e == 0xFFu) {
-    bits = sign | (0x7FFull << 52) | ((unsigned long long)m << 29);
-  } else if (m == 0) {
-    bits = sign;
-  } else {  // subnormal: m 2^-149 with its top bit at position p
-    const int p = 31 - __clz(m);
-    bits = sign | ((unsigned long long)(p - 149 + 1023) << 52) | (((unsigned long long)m << (52 - p)) & 0x000FFFFFFFFFFFFFull);
-  }
-  return __longlong_as_double((long long)bits);
+  const bool tiny = (__float_as_uint(f) & 0x7F800000u) == 0u;  // zero or subnormal: scaled by 2^64 (exact)
+  const unsigned int u = __float_as_uint(tiny ? f * 18446744073709551616.0f : f);
+  const unsigned int mag = u & 0x7FFFFFFFu;
+  // exponent + 896 (832 after the scaling; 1792 takes 255 to 2047)
+  const unsigned int bias = tiny ? 832u << 20 : (mag >= 0x7F800000u ? 1792u << 20 : 896u << 20);
+  const unsigned int hi = mag == 0u ? 0u : (mag >> 3) + bias;
+  return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(mag << 29));
 }
 
 // hi/lo of a float32 value (the float32 side quantities of the mixed line search): two hardware

@@ -173,29 +173,8 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// float -> float64 on the integer pipe (exact): the float64 units of this GPU
-// retire about two instructions per SM and clock, so the epilogue widens the
-// FP32 accumulator by rebiasing the exponent (127 -> 1023) and shifting the
-// mantissa; zeros keep their sign, subnormals are normalised, infinities and
-// NaNs keep their class.
-__device__ __forceinline__ double widen(float f) {
-  const unsigned int u = __float_as_uint(f);
-  const unsigned int e = (u >> 23) & 0xFFu, m = u & 0x7FFFFFu;
-  const unsigned long long sign = (unsigned long long)(u & 0x80000000u) << 32;
-  unsigned long long bits;
-  if (e != 0 && e != 0xFFu) {
-    bits = sign | ((unsigned long long)(e + (1023u - 127u)) << 52) | ((unsigned long long)m << 29);
-  } else if (e == 0xFFu) {
-    bits = sign | (0x7FFull << 52) | ((unsigned long long)m << 29);
-  } else if (m == 0) {
-    bits = sign;
-  } else {  // subnormal: m 2^-149 with its top bit at position p
-    const int p = 31 - __clz(m);
-    bits = sign | ((unsigned long long)(p - 149 + 1023) << 52) |
-           (((unsigned long long)m << (52 - p)) & 0x000FFFFFFFFFFFFFull);
-  }
-  return __longlong_as_double((long long)bits);
-}
+// float -> float64 on the integer pipe (exact)
+__device__ __forceinline__ double widen(float f) { return dev::f64_of_f32(f); }
 
 // alpha a + beta c in float64 (the same operations on every path)
 __device__ __forceinline__ double combine(const Epilogue& ep, double a, const double* c) {
@@ -732,12 +711,9 @@ __device__ __forceinline__ KBlocks tile_kblocks(const GroupDesc* g, int local, i
   return kb;
 }
 
-// With a chunked pair list (emulation levels) every chunk of a tile is one
-// accumulator round: the MMA thread fills a TMEM buffer with the chunk's pairs,
-// the epilogue adds it to C, and the chunks of a tile stay on one CTA, in order.
 template <bool FUSED, int TBN>
 __device__ __forceinline__ void persistent_body(const GroupDesc* __restrict__ groups, int ngroups, int total_tiles,
-                                                const PairList& pl, int* err, double* partial) {
+                                                const PairList& pl, int* err) {
   // TBN: output tile width (256 or 128); the stage ring keeps the same shared memory
   constexpr int TB_BYTES = TBN * BK * 2;
   constexpr int TSTAGE = A_BYTES + TB_BYTES;
@@ -753,17 +729,6 @@ __device__ __forceinline__ void persistent_body(const GroupDesc* __restrict__ gr
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * NS + 5);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nchunk = (FUSED || pl.nchunk <= 0) ? 1 : pl.nchunk;
-  auto chunk_begin = [&](int c) { return (c == 0 || pl.nchunk <= 0) ? 0 : (int)pl.chunk_end[c - 1]; };
-  auto chunk_end = [&](int c) { return pl.nchunk <= 0 ? pl.n : (int)pl.chunk_end[c]; };
-  // Work units: a tile with all its chunks, or (with a partial buffer, for GEMMs of few
-  // tiles) a single chunk of a tile, whose FP32 sum goes to its own float64 slice of
-  // `partial` for chunk_reduce_kernel to add in chunk order
-  const int upt = (partial != nullptr && !FUSED) ? nchunk : 1;  // units per tile
-  const int total_units = total_tiles * upt;
-  auto unit_tile = [&](int u) { return u / upt; };
-  auto unit_c0 = [&](int u) { return upt == 1 ? 0 : u % upt; };
-  auto unit_c1 = [&](int u) { return upt == 1 ? nchunk : u % upt + 1; };
 
   if (threadIdx.x == 0) {
     for (int q = 0; q < NS; ++q) {
@@ -802,8 +767,7 @@ __device__ __forceinline__ void persistent_body(const GroupDesc* __restrict__ gr
   if (warp == 0 && lane == 0) {
     // ---------------- TMA producer
     uint32_t it = 0;
-    for (int u = blockIdx.x; u < total_units && !*abort_flag; u += gridDim.x) {
-      const int tile = unit_tile(u);
+    for (int tile = blockIdx.x; tile < total_tiles && !*abort_flag; tile += gridDim.x) {
       const GroupDesc* g = groups + find_group(groups, ngroups, tile);
       const int* skip = g->ep.skip;
       if (skip != nullptr && (skip[0] | skip[1])) continue;
@@ -813,8 +777,7 @@ __device__ __forceinline__ void persistent_body(const GroupDesc* __restrict__ gr
       const int m0 = (local % tiles_m) * BM, n0 = (local / tiles_m) * TBN;
       const KBlocks kbs = tile_kblocks(g, local, tiles_m);
       const int nkb = kbs.count;
-      const int p0 = chunk_begin(unit_c0(u));
-      const int total = FUSED ? nkb : (chunk_end(unit_c1(u) - 1) - p0) * nkb;
+      const int total = FUSED ? nkb : pl.n * nkb;
       for (int t = 0; t < total; ++t, ++it) {
         const int q = it % NS;
         const uint32_t r = it / NS;
@@ -844,7 +807,7 @@ __device__ __forceinline__ void persistent_body(const GroupDesc* __restrict__ gr
             tma_load_2d(sa + 2 * A_BYTES + TB_BYTES, mB, full, kb * BK, g->rowsB + g->offB + n0);
           }
         } else {
-          const int p = p0 + t / nkb, kb = kbs.at(t % nkb);
+          const int p = t / nkb, kb = kbs.at(t % nkb);
           tma_load_2d(sa, mA, full, kb * BK, (int)pl.a[p] * g->rowsA + g->offA + m0);
           if (g->b_mn) {
 #pragma unroll
@@ -865,8 +828,7 @@ __device__ __forceinline__ void persistent_body(const GroupDesc* __restrict__ gr
     // ---------------- MMA issuer
     constexpr uint32_t idesc_k = idesc_bf16(BM, TBN);
     uint32_t it = 0, lt = 0;
-    for (int u = blockIdx.x; u < total_units && !*abort_flag; u += gridDim.x) {
-      const int tile = unit_tile(u);
+    for (int tile = blockIdx.x; tile < total_tiles && !*abort_flag; tile += gridDim.x) {
       const GroupDesc* g = groups + find_group(groups, ngroups, tile);
       const int* skip = g->ep.skip;
       if (skip != nullptr && (skip[0] | skip[1])) continue;
@@ -877,45 +839,43 @@ __device__ __forceinline__ void persistent_body(const GroupDesc* __restrict__ gr
       auto bdesc = [bmn](uint32_t addr, int k) {
         return bmn ? smem_desc_mn(addr + (uint32_t)k * 2048u) : smem_desc(addr + (uint32_t)k * 32u);
       };
-      for (int c = unit_c0(u); c < unit_c1(u) && !*abort_flag; ++c) {
-        const uint32_t buf = lt & 1, use = lt >> 1;
-        if (!mbar_wait(smem_u32(&bars[2 * NS + 2 + buf]), (use & 1) ^ 1)) {
+      const uint32_t buf = lt & 1, use = lt >> 1;
+      if (!mbar_wait(smem_u32(&bars[2 * NS + 2 + buf]), (use & 1) ^ 1)) {
+        *abort_flag = 1;
+        atomicCAS(err, 0, 4);
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t d = tmem + buf * ACC_COLS;
+      const int total = FUSED ? nkb : pl.n * nkb;
+      for (int t = 0; t < total; ++t, ++it) {
+        const int q = it % NS;
+        const uint32_t r = it / NS;
+        if (!mbar_wait(smem_u32(&bars[q]), r & 1)) {
           *abort_flag = 1;
-          atomicCAS(err, 0, 4);
+          atomicCAS(err, 0, 2);
           break;
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t d = tmem + buf * ACC_COLS;
-        const int total = FUSED ? nkb : (chunk_end(c) - chunk_begin(c)) * nkb;
-        for (int t = 0; t < total; ++t, ++it) {
-          const int q = it % NS;
-          const uint32_t r = it / NS;
-          if (!mbar_wait(smem_u32(&bars[q]), r & 1)) {
-            *abort_flag = 1;
-            atomicCAS(err, 0, 2);
-            break;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t sa = smem_u32(smem + q * SB);
-          if (FUSED) {
-            const uint32_t alo = sa + A_BYTES, bhi = sa + 2 * A_BYTES, blo = bhi + TB_BYTES;
+        const uint32_t sa = smem_u32(smem + q * SB);
+        if (FUSED) {
+          const uint32_t alo = sa + A_BYTES, bhi = sa + 2 * A_BYTES, blo = bhi + TB_BYTES;
 #pragma unroll
-            for (int k = 0; k < BK / 16; ++k) {
-              umma_bf16(d, smem_desc(sa + k * 32), bdesc(bhi, k), idesc, (t > 0 || k > 0) ? 1u : 0u);
-              umma_bf16(d, smem_desc(sa + k * 32), bdesc(blo, k), idesc, 1u);
-              umma_bf16(d, smem_desc(alo + k * 32), bdesc(bhi, k), idesc, 1u);
-            }
-          } else {
-            const uint32_t sb = sa + A_BYTES;
-#pragma unroll
-            for (int k = 0; k < BK / 16; ++k)
-              umma_bf16(d, smem_desc(sa + k * 32), bdesc(sb, k), idesc, (t > 0 || k > 0) ? 1u : 0u);
+          for (int k = 0; k < BK / 16; ++k) {
+            umma_bf16(d, smem_desc(sa + k * 32), bdesc(bhi, k), idesc, (t > 0 || k > 0) ? 1u : 0u);
+            umma_bf16(d, smem_desc(sa + k * 32), bdesc(blo, k), idesc, 1u);
+            umma_bf16(d, smem_desc(alo + k * 32), bdesc(bhi, k), idesc, 1u);
           }
-          umma_commit(smem_u32(&bars[NS + q]));
+        } else {
+          const uint32_t sb = sa + A_BYTES;
+#pragma unroll
+          for (int k = 0; k < BK / 16; ++k)
+            umma_bf16(d, smem_desc(sa + k * 32), bdesc(sb, k), idesc, (t > 0 || k > 0) ? 1u : 0u);
         }
-        umma_commit(smem_u32(&bars[2 * NS + buf]));  // this chunk's accumulator is complete
-        ++lt;
+        umma_commit(smem_u32(&bars[NS + q]));
       }
+      umma_commit(smem_u32(&bars[2 * NS + buf]));  // this tile's accumulator is complete
+      ++lt;
     }
     if (*abort_flag) {  // every MMA issued so far is complete before the tensor memory is freed
       umma_commit(smem_u32(&bars[2 * NS + 4]));
@@ -926,51 +886,35 @@ __device__ __forceinline__ void persistent_body(const GroupDesc* __restrict__ gr
     const int lane_base = (warp & 3) * 32;
     uint32_t lt = 0;
     bool failed = false;
-    for (int u = blockIdx.x; u < total_units && !failed; u += gridDim.x) {
-      const int tile = unit_tile(u);
+    for (int tile = blockIdx.x; tile < total_tiles && !failed; tile += gridDim.x) {
       const GroupDesc* g = groups + find_group(groups, ngroups, tile);
       const int* skip = g->ep.skip;
       if (skip != nullptr && (skip[0] | skip[1])) continue;
-      for (int c = unit_c0(u); c < unit_c1(u); ++c) {
-        const uint32_t buf = lt & 1, use = lt >> 1;
-        const bool ok = !*abort_flag && mbar_wait(smem_u32(&bars[2 * NS + buf]), use & 1);
-        if (!ok) {
-          atomicCAS(err, 0, 3);
-          failed = true;
-          break;
-        }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        Epilogue ep = g->ep;
-        if (upt > 1) {  // this chunk's FP32 sum, widened, into its slice of the partial buffer
-          ep.C = partial + (long)c * ep.M * ep.N;
-          ep.ldc = ep.N;
-          ep.split_cols = ep.N;
-          ep.split_stride = 0;
-          ep.alpha = 1.0;
-          ep.beta = 0.0;
-          ep.mode = kEpPlain;
-          ep.c_f32 = 0;
-          ep.bf_hi = nullptr;
-        } else if (c > 0) {
-          ep.beta = 1.0;
-        }
-        const int local = tile - g->tile_begin, tiles_m = (ep.M + BM - 1) / BM;
-        const int m0 = (local % tiles_m) * BM, n0 = (local / tiles_m) * TBN;
-        const int row = m0 + lane_base + lane;
-        EpiRed red;
-        red.have_dir = ep.mode == kEpReduce && ep.sc != nullptr && ep.sc->have_dir;
-#pragma unroll 1
-        for (int j = 0; j < TBN / 32; ++j) {
-          float v[32];
-          tmem_ld32(tmem + buf * ACC_COLS + ((uint32_t)lane_base << 16) + (uint32_t)(j * 32), v);
-          store_chunk(ep, row, n0 + j * 32, v, red);
-        }
-        flush_reduce(ep, local, warp & 3, red);
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&bars[2 * NS + 2 + buf]));
-        ++lt;
+      const uint32_t buf = lt & 1, use = lt >> 1;
+      const bool ok = !*abort_flag && mbar_wait(smem_u32(&bars[2 * NS + buf]), use & 1);
+      if (!ok) {
+        atomicCAS(err, 0, 3);
+        failed = true;
+        break;
       }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const Epilogue ep = g->ep;
+      const int local = tile - g->tile_begin, tiles_m = (ep.M + BM - 1) / BM;
+      const int m0 = (local % tiles_m) * BM, n0 = (local / tiles_m) * TBN;
+      const int row = m0 + lane_base + lane;
+      EpiRed red;
+      red.have_dir = ep.mode == kEpReduce && ep.sc != nullptr && ep.sc->have_dir;
+#pragma unroll 1
+      for (int j = 0; j < TBN / 32; ++j) {
+        float v[32];
+        tmem_ld32(tmem + buf * ACC_COLS + ((uint32_t)lane_base << 16) + (uint32_t)(j * 32), v);
+        store_chunk(ep, row, n0 + j * 32, v, red);
+      }
+      flush_reduce(ep, local, warp & 3, red);
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&bars[2 * NS + 2 + buf]));
+      ++lt;
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1055,9 +999,7 @@ constexpr uint32_t PAIR_TMEM_COLS = 512;  // two accumulator buffers, 256 column
 constexpr uint64_t PAIR_ABORT_SETTLE_NS = 200000ull;
 
 // SPLIT: the 3-term split form (stages hold A_hi, A_lo, B_hi, B_lo); otherwise the pair list pl
-// (stages hold one slice of A and one of B), chunk by chunk: every chunk of a tile is one
-// accumulator round whose FP32 sum the epilogue adds to C in chunk order (the first with the
-// Epilogue's beta, the later ones with beta = 1), as in the single-SM kernel.
+// (stages hold one slice of A and one of B).
 // NP = 2: a cluster of two pairs side by side along N (a work unit is 256 x 2 TBN) that share A:
 // CTA r of pair p loads rows [64 p, 64 p + 64) of the 128 A rows its CTA position needs and
 // multicasts them to CTA r of both pairs, so every A byte leaves L2 once per two column tiles.
@@ -1093,9 +1035,6 @@ __device__ __forceinline__ void pair_body(const GroupDesc* __restrict__ groups, 
   const uint16_t mask_all = (uint16_t)((1u << (2 * NP)) - 1u);      // every CTA of the cluster
   const uint16_t mask_pair = (uint16_t)(3u << (2 * pp));            // the CTAs of this pair
   const uint16_t mask_a = (uint16_t)((1u << rr) | (1u << (2 + rr)));  // CTA rr of both pairs (NP = 2)
-  const int nchunk = (SPLIT || pl.nchunk <= 0) ? 1 : pl.nchunk;
-  auto chunk_begin = [&](int c) { return (c == 0 || pl.nchunk <= 0) ? 0 : (int)pl.chunk_end[c - 1]; };
-  auto chunk_end = [&](int c) { return pl.nchunk <= 0 ? pl.n : (int)pl.chunk_end[c]; };
 
   if (threadIdx.x == 0) {
     for (int q = 0; q < NS; ++q) {
@@ -1144,7 +1083,7 @@ __device__ __forceinline__ void pair_body(const GroupDesc* __restrict__ groups, 
       const int n0 = ((local / tiles_m) * NP + pp) * TBN + rr * TBH;        // this CTA's half of B
       const KBlocks kbs = tile_kblocks(g, local, tiles_m);
       const int nkb = kbs.count;
-      const int total = SPLIT ? nkb : pl.n * nkb;  // every pair of every chunk of the tile
+      const int total = SPLIT ? nkb : pl.n * nkb;
       for (int t = 0; t < total; ++t, ++it) {
         const int q = it % NS;
         const uint32_t r = it / NS;
@@ -1206,40 +1145,38 @@ __device__ __forceinline__ void pair_body(const GroupDesc* __restrict__ groups, 
       auto bdesc = [bmn](uint32_t addr, int k) {
         return bmn ? smem_desc_mn(addr + (uint32_t)k * 2048u) : smem_desc(addr + (uint32_t)k * 32u);
       };
-      for (int c = 0; c < nchunk && !*abort_flag; ++c) {
-        const uint32_t buf = lt & 1, use = lt >> 1;
-        if (!mbar_wait(smem_u32(&bars[2 * NS + 2 + buf]), (use & 1) ^ 1)) {
+      const uint32_t buf = lt & 1, use = lt >> 1;
+      if (!mbar_wait(smem_u32(&bars[2 * NS + 2 + buf]), (use & 1) ^ 1)) {
+        *abort_flag = 1;
+        atomicCAS(err, 0, 4);
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t d = tmem + buf * ACC_STRIDE;
+      const int total = SPLIT ? nkb : pl.n * nkb;
+      for (int t = 0; t < total; ++t, ++it) {
+        const int q = it % NS;
+        const uint32_t r = it / NS;
+        if (!mbar_wait(smem_u32(&bars[q]), r & 1)) {
           *abort_flag = 1;
-          atomicCAS(err, 0, 4);
+          atomicCAS(err, 0, 2);
           break;
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t d = tmem + buf * ACC_STRIDE;
-        const int total = SPLIT ? nkb : (chunk_end(c) - chunk_begin(c)) * nkb;
-        for (int t = 0; t < total; ++t, ++it) {
-          const int q = it % NS;
-          const uint32_t r = it / NS;
-          if (!mbar_wait(smem_u32(&bars[q]), r & 1)) {
-            *abort_flag = 1;
-            atomicCAS(err, 0, 2);
-            break;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t sa = smem_u32(smem + q * SB);
-          const uint32_t alo = sa + A_BYTES, bhi = sa + B_OFF, blo = bhi + BH_BYTES;
+        const uint32_t sa = smem_u32(smem + q * SB);
+        const uint32_t alo = sa + A_BYTES, bhi = sa + B_OFF, blo = bhi + BH_BYTES;
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k) {
-            umma_bf16_pair(d, smem_desc(sa + k * 32), bdesc(bhi, k), idesc, (t > 0 || k > 0) ? 1u : 0u);
-            if (SPLIT) {
-              umma_bf16_pair(d, smem_desc(sa + k * 32), bdesc(blo, k), idesc, 1u);
-              umma_bf16_pair(d, smem_desc(alo + k * 32), bdesc(bhi, k), idesc, 1u);
-            }
+        for (int k = 0; k < BK / 16; ++k) {
+          umma_bf16_pair(d, smem_desc(sa + k * 32), bdesc(bhi, k), idesc, (t > 0 || k > 0) ? 1u : 0u);
+          if (SPLIT) {
+            umma_bf16_pair(d, smem_desc(sa + k * 32), bdesc(blo, k), idesc, 1u);
+            umma_bf16_pair(d, smem_desc(alo + k * 32), bdesc(bhi, k), idesc, 1u);
           }
-          umma_commit_pair(smem_u32(&bars[NS + q]), mask_all);  // this pair is done with stage q
         }
-        umma_commit_pair(smem_u32(&bars[2 * NS + buf]), mask_pair);  // both halves of the accumulator are complete
-        ++lt;
+        umma_commit_pair(smem_u32(&bars[NS + q]), mask_all);  // this pair is done with stage q
       }
+      umma_commit_pair(smem_u32(&bars[2 * NS + buf]), mask_pair);  // both halves of the accumulator are complete
+      ++lt;
     }
     if (*abort_flag) {  // every MMA issued so far is complete before the tensor memory is freed
       umma_commit_pair_local(smem_u32(&bars[2 * NS + 4]));
@@ -1255,36 +1192,30 @@ __device__ __forceinline__ void pair_body(const GroupDesc* __restrict__ groups, 
       const GroupDesc* g = groups + find_group(groups, ngroups, u);
       const int* skip = g->ep.skip;
       if (skip != nullptr && (skip[0] | skip[1])) continue;
-      bool failed = false;
-      for (int c = 0; c < nchunk; ++c) {
-        const uint32_t buf = lt & 1, use = lt >> 1;
-        const bool ok = !*abort_flag && mbar_wait(smem_u32(&bars[2 * NS + buf]), use & 1);
-        if (!ok) {
-          atomicCAS(err, 0, 3);
-          failed = true;
-          break;
-        }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        Epilogue ep = g->ep;
-        if (c > 0) ep.beta = 1.0;
-        const int local = u - g->tile_begin, tiles_m = (ep.M + 2 * BM - 1) / (2 * BM);
-        const int m0 = (local % tiles_m) * 2 * BM + rr * BM, n0 = ((local / tiles_m) * NP + pp) * TBN;
-        const int row = m0 + lane_base + lane;
-        EpiRed red;
-        red.have_dir = ep.mode == kEpReduce && ep.sc != nullptr && ep.sc->have_dir;
-#pragma unroll 1
-        for (int j = 0; j < TBN / 32; ++j) {
-          float v[32];
-          tmem_ld32(tmem + buf * ACC_STRIDE + ((uint32_t)lane_base << 16) + (uint32_t)(j * 32), v);
-          store_chunk(ep, row, n0 + j * 32, v, red);
-        }
-        flush_reduce(ep, (local * NP + pp) * 2 + rr, warp & 3, red);  // slots of 128 x TBN quarters
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(buf ? acc_empty1 : acc_empty0);
-        ++lt;
+      const uint32_t buf = lt & 1, use = lt >> 1;
+      const bool ok = !*abort_flag && mbar_wait(smem_u32(&bars[2 * NS + buf]), use & 1);
+      if (!ok) {
+        atomicCAS(err, 0, 3);
+        break;
       }
-      if (failed) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const Epilogue ep = g->ep;
+      const int local = u - g->tile_begin, tiles_m = (ep.M + 2 * BM - 1) / (2 * BM);
+      const int m0 = (local % tiles_m) * 2 * BM + rr * BM, n0 = ((local / tiles_m) * NP + pp) * TBN;
+      const int row = m0 + lane_base + lane;
+      EpiRed red;
+      red.have_dir = ep.mode == kEpReduce && ep.sc != nullptr && ep.sc->have_dir;
+#pragma unroll 1
+      for (int j = 0; j < TBN / 32; ++j) {
+        float v[32];
+        tmem_ld32(tmem + buf * ACC_STRIDE + ((uint32_t)lane_base << 16) + (uint32_t)(j * 32), v);
+        store_chunk(ep, row, n0 + j * 32, v, red);
+      }
+      flush_reduce(ep, (local * NP + pp) * 2 + rr, warp & 3, red);  // slots of 128 x TBN quarters
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster(buf ? acc_empty1 : acc_empty0);
+      ++lt;
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1314,46 +1245,28 @@ gemm_quad_kernel(const GroupDesc* __restrict__ groups, int ngroups, int total_un
   pair_body<TBN, SPLIT, 2>(groups, ngroups, total_units, pl, err);
 }
 
-// one GEMM, its descriptor (tensor maps included) in the kernel's parameter space
-template <int TBN, bool SPLIT>
+// one split-form GEMM, its descriptor (tensor maps included) in the kernel's parameter space
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
 gemm_pair_one_kernel(const __grid_constant__ GroupDesc g, int total_units, const __grid_constant__ PairList pl,
                      int* err) {
-  pair_body<TBN, SPLIT, 1>(&g, 1, total_units, pl, err);
+  pair_body<256, true, 1>(&g, 1, total_units, pl, err);
 }
 
 template <bool FUSED, int TBN>
 __global__ void __launch_bounds__(NTHREADS, 1)
 gemm_persistent_kernel(const GroupDesc* __restrict__ groups, int ngroups, int total_tiles,
                        const __grid_constant__ PairList pl, int* err) {
-  persistent_body<FUSED, TBN>(groups, ngroups, total_tiles, pl, err, nullptr);
+  persistent_body<FUSED, TBN>(groups, ngroups, total_tiles, pl, err);
 }
 
-// one GEMM, its descriptor (tensor maps included) in the kernel's parameter space
-template <bool FUSED>
+// one split-form GEMM, its descriptor (tensor maps included) in the kernel's parameter space
 __global__ void __launch_bounds__(NTHREADS, 1)
 gemm_persistent_one_kernel(const __grid_constant__ GroupDesc g, int total_tiles, const __grid_constant__ PairList pl,
-                           int* err, double* partial) {
-  persistent_body<FUSED, BN>(&g, 1, total_tiles, pl, err, partial);
+                           int* err) {
+  persistent_body<true, BN>(&g, 1, total_tiles, pl, err);
 }
 
-// C = beta C + alpha sum_c partial[c] (chunk order; the same float64 operations, in the same
-// order, as the in-kernel chunk epilogues)
-__global__ void chunk_reduce_kernel(const double* __restrict__ partial, int nchunk, Epilogue ep) {
-  const long count = (long)ep.M * ep.N;
-  for (long idx = blockIdx.x * (long)blockDim.x + threadIdx.x; idx < count; idx += (long)gridDim.x * blockDim.x) {
-    const long row = idx / ep.N, col = idx % ep.N;
-    const long blk = col / ep.split_cols;
-    double* p = ep.C + blk * ep.split_stride + row * ep.ldc + (col - blk * ep.split_cols);
-    const double a0 = partial[idx];
-    double acc;
-    if (ep.beta == 0.0) acc = (ep.alpha == 1.0) ? a0 : ep.alpha * a0;
-    else if (ep.beta == 1.0) acc = fma(ep.alpha, a0, *p);
-    else acc = fma(ep.beta, *p, ep.alpha * a0);
-    for (int c = 1; c < nchunk; ++c) acc = fma(ep.alpha, partial[(long)c * count + idx], acc);
-    *p = acc;
-  }
-}
+#include "sliced_body.cuh"
 
 int sm_count() {
   static const int n = [] {
@@ -1579,14 +1492,13 @@ void prepare_persistent() {
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
     OMM_CUDA_TRY(cudaFuncSetAttribute(gemm_persistent_kernel<true, 128>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
-    OMM_CUDA_TRY(cudaFuncSetAttribute(gemm_persistent_one_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      SMEM_BYTES));
-    OMM_CUDA_TRY(cudaFuncSetAttribute(gemm_persistent_one_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    OMM_CUDA_TRY(cudaFuncSetAttribute(gemm_persistent_one_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       SMEM_BYTES));
     for (const void* f : {(const void*)gemm_pair_kernel<128, true>, (const void*)gemm_pair_kernel<192, true>,
                           (const void*)gemm_pair_kernel<256, true>, (const void*)gemm_pair_kernel<128, false>,
                           (const void*)gemm_pair_kernel<192, false>, (const void*)gemm_pair_kernel<256, false>,
-                          (const void*)gemm_pair_one_kernel<256, true>, (const void*)gemm_pair_one_kernel<256, false>,
+                          (const void*)gemm_pair_one_kernel, (const void*)sliced_pair_kernel,
+                          (const void*)sliced_kernel<256>, (const void*)sliced_kernel<128>,
                           (const void*)gemm_quad_kernel<128, true>, (const void*)gemm_quad_kernel<192, true>,
                           (const void*)gemm_quad_kernel<256, true>, (const void*)gemm_quad_kernel<128, false>,
                           (const void*)gemm_quad_kernel<192, false>, (const void*)gemm_quad_kernel<256, false>})
@@ -1643,42 +1555,87 @@ void gemm_persistent(cudaStream_t st, const GroupDesc* groups_dev, int ngroups, 
   OMM_LAUNCH_CHECK();
 }
 
-void gemm_persistent(cudaStream_t st, const Operand& A, const Operand& B, int K, const PairList& pl,
-                     const Epilogue& ep, double* partial, long partial_capacity, const BlockLists* sparse) {
+void gemm_split(cudaStream_t st, const Operand& A, const Operand& B, int K, const Epilogue& ep) {
   prepare_persistent();
+  const PairList pl = pairs_split3();
   check_pairs(pl, A.slices, B.slices);
   const int tiles = tiles_of(ep);
   if (tiles <= 0 || K <= 0) return;
-  const GroupDesc g = make_group(A, B, K, ep, 0, BN, sparse);
-  const bool fused = is_split3(pl) && pl.nchunk <= 1 && A.slices >= 2 && B.slices >= 2;
-  // a GEMM of few tiles spreads its chunks over the SMs when scratch for them was given
-  const int nchunk = pl.nchunk > 0 ? pl.nchunk : 1;
-  const bool split = !fused && partial != nullptr && nchunk > 1 && 2 * tiles < sm_count() &&
-                     (long)nchunk * ep.M * ep.N <= partial_capacity && ep.skip == nullptr;
   // a product with at least a wave of 256-row tiles runs on SM pairs (half the B bytes per SM)
   const int pair_units = tiles_of(ep, BN, true);
-  if (!split && ep.M >= 2 * BM && pair_units >= pair_clusters()) {
-    const GroupDesc gp = make_group(A, B, K, ep, 0, BN, sparse, true);
+  if (ep.M >= 2 * BM && pair_units >= pair_clusters()) {
+    const GroupDesc gp = make_group(A, B, K, ep, 0, BN, nullptr, true);
     const unsigned pgrid = 2u * (unsigned)std::min(pair_units, pair_clusters());
-    if (fused)
-      gemm_pair_one_kernel<BN, true><<<pgrid, NTHREADS, SMEM_BYTES, st>>>(gp, pair_units, pl, ep.err);
-    else
-      gemm_pair_one_kernel<BN, false><<<pgrid, NTHREADS, SMEM_BYTES, st>>>(gp, pair_units, pl, ep.err);
-    OMM_LAUNCH_CHECK();
-    return;
+    gemm_pair_one_kernel<<<pgrid, NTHREADS, SMEM_BYTES, st>>>(gp, pair_units, pl, ep.err);
+  } else {
+    const GroupDesc g = make_group(A, B, K, ep, 0, BN);
+    gemm_persistent_one_kernel<<<(unsigned)std::min(tiles, sm_count()), NTHREADS, SMEM_BYTES, st>>>(g, tiles, pl, ep.err);
   }
-  const int units = split ? tiles * nchunk : tiles;
-  const unsigned grid = (unsigned)std::min(units, sm_count());
-  if (fused)
-    gemm_persistent_one_kernel<true><<<grid, NTHREADS, SMEM_BYTES, st>>>(g, tiles, pl, ep.err, nullptr);
-  else
-    gemm_persistent_one_kernel<false><<<grid, NTHREADS, SMEM_BYTES, st>>>(g, tiles, pl, ep.err,
-                                                                          split ? partial : nullptr);
   OMM_LAUNCH_CHECK();
-  if (split) {
-    const long count = (long)ep.M * ep.N;
-    const unsigned rb = (unsigned)std::min<long>((count + 255) / 256, 4L * sm_count());
-    chunk_reduce_kernel<<<rb, 256, 0, st>>>(partial, nchunk, ep);
+}
+
+long sliced_workspace_doubles() { return 2L * BM * BN * sm_count(); }
+
+void gemm_sliced(cudaStream_t st, const Operand& A, const Operand& B, int K, const PairList& pl, const Epilogue& ep,
+                 double* slab, const BlockLists* sparse) {
+  prepare_persistent();
+  check_pairs(pl, A.slices, B.slices);
+  if (ep.skip != nullptr || ep.mode != kEpPlain || ep.c_f32 || ep.bf_hi != nullptr || slab == nullptr)
+    throw CudaError{cudaErrorInvalidValue, "tc::gemm_sliced: plain float64 epilogue and a workspace"};
+  if (ep.M <= 0 || ep.N <= 0 || K <= 0) return;
+  const long nkb = (K + BK - 1) / BK;
+  const int nchunk = pl.nchunk > 0 ? pl.nchunk : 1;
+  // Tile shape and number of workers with the shortest estimated time, in SM clocks. A stage takes as
+  // long as its copies: about 55 bytes per clock land in an SM's shared memory, 32 KB for a pair's 256 x
+  // 256 or one SM's 128 x 128 tile, 48 KB for 128 x 256. Adding a piece to a running sum costs a float64
+  // add per element, about one per clock and SM, beside the stages that follow; the last piece's add and
+  // about 5000 clocks of start-up are exposed, and where shares do not end with tiles the slab pass too.
+  struct Shape { int bn; bool pair; double cycles; };
+  const Shape shapes[3] = {{256, true, 600.0}, {256, false, 900.0}, {128, false, 600.0}};
+  // shares at arbitrary places only while the slices stay in L2 (see sliced_body.cuh)
+  int slices = 0;
+  for (int p = 0; p < pl.n; ++p) slices = std::max(slices, std::max((int)pl.a[p], (int)pl.b[p]) + 1);
+  const bool resident = 2.0 * slices * ((double)ep.M + ep.N) * K <= 100e6;
+  SlicedWork best{};
+  Shape best_shape = shapes[1];
+  double best_t = 0.0;
+  bool best_whole = false;
+  for (const Shape& sh : shapes) {
+    if (sparse != nullptr && sh.bn != 256) continue;  // block lists are made for 256 rows
+    const int bmt = sh.pair ? 2 * BM : BM, workers = sh.pair ? pair_clusters() : sm_count();
+    const int tm = (ep.M + bmt - 1) / bmt, tn = (ep.N + sh.bn - 1) / sh.bn, tiles = tm * tn;
+    const double per_tile = sparse ? (double)pl.n * sparse->nnz / tn : (double)pl.n * nkb;
+    const int full = tiles / workers, left = tiles - full * workers;
+    const int most = std::min<int>(workers, std::max<int>(left, (int)(left * per_tile / 8)));  // 8 stages each or more
+    const double add = (double)std::min(ep.M, BM) * std::min(ep.N, sh.bn);  // elements of one CTA's piece
+    for (int k = 0; k < 2; ++k) {
+      // left-over tiles in equal parts (one or more workers each), or evenly over all workers
+      const int nr = left == 0 ? 0 : (k == 0 ? left * (most / left) : most);
+      if (k == 1 && (left == 0 || !resident)) continue;
+      const bool whole = nr == 0 || (sparse == nullptr && nr == left);
+      const double stages = full * per_tile + (nr ? left * per_tile / nr : 0.0);
+      const double t = std::max(stages * sh.cycles, nchunk * stages / per_tile * add) + add + 5000.0 +
+                       (whole ? 0.0 : 9000.0 + add / 8.0);
+      if (best_t == 0.0 || t < best_t) {
+        best = SlicedWork{slab, full > 0 ? workers : nr, full, nr, tm, tiles};
+        best_shape = sh;
+        best_whole = whole;
+        best_t = t;
+      }
+    }
+  }
+  const GroupDesc g = make_group(A, B, K, ep, 0, best_shape.bn, sparse, best_shape.pair);
+  if (best_shape.pair)
+    sliced_pair_kernel<<<2u * (unsigned)best.nw, NTHREADS, SMEM_BYTES, st>>>(g, pl, best, ep.err);
+  else if (best_shape.bn == 256)
+    sliced_kernel<256><<<(unsigned)best.nw, NTHREADS, SMEM_BYTES, st>>>(g, pl, best, ep.err);
+  else
+    sliced_kernel<128><<<(unsigned)best.nw, NTHREADS, SMEM_BYTES, st>>>(g, pl, best, ep.err);
+  OMM_LAUNCH_CHECK();
+  if (!best_whole) {  // some share starts inside a tile
+    const int bmt = best_shape.pair ? 2 * BM : BM;
+    const int left = best.tiles - best.full * best.nw;
+    slab_reduce_kernel<<<(unsigned)(left * (bmt / 32) * (best_shape.bn / 32)), 256, 0, st>>>(g, pl.n, best, bmt);
     OMM_LAUNCH_CHECK();
   }
 }

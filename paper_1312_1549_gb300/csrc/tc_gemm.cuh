@@ -37,10 +37,9 @@ struct Operand {
 
 // Which slice products one GEMM accumulates. With nchunk > 0 the pairs are cut
 // into consecutive chunks: chunk c holds pairs [chunk_end[c-1], chunk_end[c]),
-// is summed in an FP32 accumulator of its own and added to the float64 output
-// by its own epilogue pass, in chunk order (the first pass with the Epilogue's
-// beta, the later ones with beta = 1). nchunk = 0: all pairs form one chunk.
-// Chunks are honoured by the persistent launch only.
+// whose products are summed in FP32 accumulators of their own (one, or several
+// over parts of the contraction) and added in float64. nchunk = 0: all pairs
+// form one chunk. Chunks are honoured by gemm_sliced only.
 constexpr int kMaxPairs = 64;
 constexpr int kMaxChunks = 32;
 struct PairList {
@@ -180,12 +179,13 @@ void prepare_persistent();  // kernel attributes (call before a stream capture)
 // nonzero code if a bounded wait expired
 void gemm_persistent(cudaStream_t st, const GroupDesc* groups_dev, int ngroups, int total_tiles, const PairList& pl,
                      int* err, int bn = 256, bool pair = false, bool quad = false);
-// the same persistent kernel for one GEMM whose descriptor travels as a kernel parameter.
-// partial (optional, partial_capacity doubles): scratch that lets a GEMM of few output tiles run
-// each chunk of its pair list on its own CTA and add the chunks afterwards, in chunk order.
-void gemm_persistent(cudaStream_t st, const Operand& A, const Operand& B, int K, const PairList& pl,
-                     const Epilogue& ep, double* partial = nullptr, long partial_capacity = 0,
-                     const BlockLists* sparse = nullptr);
+// one split-form GEMM (pairs_split3) whose descriptor travels as a kernel parameter
+void gemm_split(cudaStream_t st, const Operand& A, const Operand& B, int K, const Epilogue& ep);
+// one chunked product C = alpha sum A_i B_j^T + beta C (a plain float64 epilogue, no skip flags), its
+// stages shared evenly among the SMs. slab: sliced_workspace_doubles() doubles, used on st only.
+void gemm_sliced(cudaStream_t st, const Operand& A, const Operand& B, int K, const PairList& pl, const Epilogue& ep,
+                 double* slab, const BlockLists* sparse = nullptr);
+long sliced_workspace_doubles();
 
 // Tile-shape autotuner: times one persistent launch over these GEMMs (the operands as given,
 // the outputs redirected to scratch) with each candidate shape -- 128 x 256 and 128 x 128 on one
