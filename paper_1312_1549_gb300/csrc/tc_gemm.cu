@@ -47,7 +47,8 @@ constexpr int RING_BYTES = 192 * 1024;
 constexpr int MAX_STAGES = 10;          // barrier room: 2 * stages + 5 barriers in 256 bytes
 constexpr int TMEM_COLS = 256;
 constexpr int NTHREADS = 192;
-constexpr int SMEM_BYTES = RING_BYTES + 1024 /*align*/ + 256 /*barriers*/;
+constexpr int EPI_BYTES = 4 * 32 * 33 * 4;  // the epilogue warps' transposition blocks
+constexpr int SMEM_BYTES = RING_BYTES + 1024 /*align*/ + 256 /*barriers*/ + EPI_BYTES;
 constexpr int ring_stages(int stage_bytes) {
   return RING_BYTES / stage_bytes < MAX_STAGES ? RING_BYTES / stage_bytes : MAX_STAGES;
 }
@@ -190,319 +191,166 @@ struct EpiRed {
   bool have_dir = false;
 };
 
-// One output element of a fused form (see Epilogue): accumulator value a (FP32) at row, column
-// col of block blk (cb = col within the block); stores C (and its split) and returns nothing.
-__device__ __forceinline__ void fused_element(const Epilogue& ep, float a, int row, long blk, long cb, EpiRed& red) {
-  const long offc = blk * ep.split_stride + (long)row * ep.ldc + cb;
-  double out;
-  if (ep.mode == kEpGrad) {
-    const long ox = (long)row * ep.ldx + cb, of = (long)row * ep.ldf + cb;
-    out = ep.x0[ox] + widen(fmaf((float)ep.xs, ep.x1f[of], (float)ep.alpha * a));
-  } else if (ep.mode == kEpReduce) {
-    const long ox = (long)row * ep.ldx + cb, of = (long)row * ep.ldf + cb;
-    const double pg = widen(a), g = ep.x0[ox];
-    red.v0 = fma(g, pg, red.v0);
-    if (red.have_dir) {
-      red.v1 = fma(ep.x1[ox], pg, red.v1);
-      red.v2 = fma(g, dev::f64_of_f32(ep.x2f[of]), red.v2);
-    }
-    red.mb = max(red.mb, (unsigned long long)__double_as_longlong(g) & 0x7FFFFFFFFFFFFFFFull);
-    ep.xout[ox] = g;
-    reinterpret_cast<float*>(ep.C)[offc] = a;
-    if (ep.bf_hi != nullptr) {
-      __nv_bfloat16* hp = ep.bf_hi + blk * ep.bf_blk + (long)row * ep.bf_ld;
-      dev::split_store_f32(a, hp, hp + ep.bf_lo, cb);
-    }
-    return;
-  } else if (ep.c_f32) {
-    const float o = ep.alpha == 1.0 ? a : (float)ep.alpha * a;
-    reinterpret_cast<float*>(ep.C)[offc] = o;
-    if (ep.bf_hi != nullptr) {
-      __nv_bfloat16* hp = ep.bf_hi + blk * ep.bf_blk + (long)row * ep.bf_ld;
-      dev::split_store_f32(o, hp, hp + ep.bf_lo, cb);
-    }
-    return;
-  } else {
-    out = combine(ep, widen(a), ep.C + offc);
-  }
-  ep.C[offc] = out;
-  if (ep.bf_hi != nullptr) {
-    __nv_bfloat16* hp = ep.bf_hi + blk * ep.bf_blk + (long)row * ep.bf_ld;
-    dev::split_store_fast(out, hp, hp + ep.bf_lo, cb);
-  }
+// C = alpha acc + beta C, or a fused form (see Epilogue), for the 32 x 32 block at (row0, col0) of an
+// epilogue warp: lane l holds row row0 + l of the accumulator in v. The block goes through shared memory
+// (st, 33 floats per row: conflict-free both ways) so that afterwards the lanes stand on 32 neighbouring
+// columns of one row: every global access is a contiguous run of 32 elements whatever the alignment of
+// the rows or the place where a stacked output's blocks meet, and rows and columns past the edge are
+// just masked. Sixteen rows at a time, all their loads before their stores, so that one memory latency
+// covers them. (With a row per lane, each access touched 32 rows; an odd leading dimension took 8-byte
+// accesses, and the ragged last columns or a block border inside the 32 columns element by element with
+// a load-to-store dependence each: 75 to 97 us for the products of an m = 1495, n = 260 line search.)
+constexpr int kEpiPitch = 33;
+static_assert(EPI_BYTES == 4 * 32 * kEpiPitch * 4, "one block per epilogue warp");
+
+__device__ __forceinline__ float lds_f32(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
+  return v;
+}
+__device__ __forceinline__ void sts_f32(uint32_t addr, float v) {
+  asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(v));
 }
 
-// eight bf16 values into one 16-byte store
-__device__ __forceinline__ void store_bf8(__nv_bfloat16* p, const unsigned short (&h)[8]) {
-  *reinterpret_cast<uint4*>(p) = make_uint4(h[0] | ((uint32_t)h[1] << 16), h[2] | ((uint32_t)h[3] << 16),
-                                            h[4] | ((uint32_t)h[5] << 16), h[6] | ((uint32_t)h[7] << 16));
-}
-
-// The fused forms, float32 outputs and split outputs for the 32 accumulator columns of a row whose
-// float64 data (C unless c_f32, x0, x1, xout) starts on an 8-byte but not a 16-byte boundary (a
-// row of an odd leading dimension): eight columns at a time, 8-byte accesses to those arrays and
-// the usual vector accesses to the float32 and split arrays. offc, offx, offf, bf0: the row's first
-// element in C, in x0/x1/xout, in x1f/x2f and in the split outputs.
-__device__ __forceinline__ float f4_at(const float4& q, int i) { return i == 0 ? q.x : (i == 1 ? q.y : (i == 2 ? q.z : q.w)); }
-
-__device__ __forceinline__ void store_chunk_odd(const Epilogue& ep, long offc, long offx, long offf, long bf0,
-                                                const float (&v)[32], EpiRed& red) {
-  const bool unit = ep.alpha == 1.0 && ep.beta == 0.0;
+// the block's rows, sixteen at a time: their accumulator values (at st in shared memory, this lane's
+// column) and their inputs are all read before the first store, which might alias them for all the
+// compiler knows (a read behind a store waited for it, 115 clocks per row)
+template <bool FULL>
+__device__ __forceinline__ void store_block(const Epilogue& ep, uint32_t st, int row0, int col0, EpiRed& red) {
+  const int nrow = FULL ? 32 : min(32, ep.M - row0), col = col0 + (int)(threadIdx.x & 31);
+  const bool ok = FULL || col < ep.N;
+  const int sc = (int)ep.split_cols;
+  const int blk = ok && sc < ep.N ? col / sc : 0, cb = ok ? col - blk * sc : 0;
+  const long ldc = ep.ldc, bf_ld = ep.bf_ld, bf_lo = ep.bf_lo;
+  __nv_bfloat16* hp = nullptr;  // the element of row row0 in the split output
+  if (ep.bf_hi != nullptr) hp = ep.bf_hi + blk * ep.bf_blk + row0 * bf_ld + cb;
+#pragma unroll 1
+  for (int r0 = 0; r0 < nrow; r0 += 16) {
+    auto in = [&](int k) { return FULL || (ok && r0 + k < nrow); };
+    const int row = row0 + r0;
+    float a[16];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int c8 = 8 * q;
-    if (ep.c_f32) {
-      float o[8];
-      const float al = (float)ep.alpha;
+    for (int k = 0; k < 16; ++k) a[k] = lds_f32(st + (uint32_t)((r0 + k) * kEpiPitch * 4));
+    if (ep.mode == kEpReduce) {
+      const long ldx = ep.ldx;
+      const long ox = row * ldx + cb;
+      double g[16], go[16];
+      float d[16];
+      const double* q = ep.x0 + ox;
 #pragma unroll
-      for (int k = 0; k < 8; ++k) o[k] = (ep.mode == kEpReduce || unit) ? v[c8 + k] : al * v[c8 + k];
-      if (ep.mode == kEpReduce) {
-        double g[8], go[8];
-        float4 d[2];
+      for (int k = 0; k < 16; ++k, q += ldx) g[k] = in(k) ? __ldg(q) : 0.0;
+      if (red.have_dir) {
+        q = ep.x1 + ox;  // may alias xout
 #pragma unroll
-        for (int k = 0; k < 8; ++k) g[k] = __ldg(ep.x0 + offx + c8 + k);
-        if (red.have_dir) {
+        for (int k = 0; k < 16; ++k, q += ldx) go[k] = in(k) ? *q : 0.0;
+        const long ldf = ep.ldf;
+        const float* f = ep.x2f + row * ldf + cb;
 #pragma unroll
-          for (int k = 0; k < 8; ++k) go[k] = ep.x1[offx + c8 + k];  // x1 may alias xout
+        for (int k = 0; k < 16; ++k, f += ldf) d[k] = in(k) ? __ldg(f) : 0.f;
+      } else {
 #pragma unroll
-          for (int k = 0; k < 2; ++k) d[k] = __ldg(reinterpret_cast<const float4*>(ep.x2f + offf + c8) + k);
+        for (int k = 0; k < 16; ++k) {
+          go[k] = 0.0;
+          d[k] = 0.f;
         }
-        // float32 sums of these 8 products, widened into the float64 running sums (as in the
-        // 16-column form)
-        float s0 = 0.f, s1 = 0.f, s2 = 0.f;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const float gk = dev::f32_rne_bits(g[k]);
-          s0 = fmaf(gk, o[k], s0);
-          red.mb = max(red.mb, (unsigned long long)__double_as_longlong(g[k]) & 0x7FFFFFFFFFFFFFFFull);
-          if (red.have_dir) {
-            s1 = fmaf(dev::f32_rne_bits(go[k]), o[k], s1);
-            s2 = fmaf(gk, f4_at(d[k >> 2], k & 3), s2);
-          }
-        }
-        red.v0 += widen(s0);
-        if (red.have_dir) {
-          red.v1 += widen(s1);
-          red.v2 += widen(s2);
-        }
-#pragma unroll
-        for (int k = 0; k < 8; ++k) ep.xout[offx + c8 + k] = g[k];
       }
-      float4* c4 = reinterpret_cast<float4*>(reinterpret_cast<float*>(ep.C) + offc + c8);
-      c4[0] = make_float4(o[0], o[1], o[2], o[3]);
-      c4[1] = make_float4(o[4], o[5], o[6], o[7]);
-      if (ep.bf_hi != nullptr) {
-        unsigned short h[8], l[8];
+      float* c = reinterpret_cast<float*>(ep.C) + row * ldc + cb;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) dev::split_bits_f32(o[k], h[k], l[k]);
-        __nv_bfloat16* hp = ep.bf_hi + bf0 + c8;
-        store_bf8(hp, h);
-        store_bf8(hp + ep.bf_lo, l);
+      for (int k = 0; k < 16; ++k, c += ldc)
+        if (in(k)) *c = a[k];
+      // the sums of these 16 products in float32 (g rounded to float32 on the integer pipe),
+      // then widened into the float64 running sums: 3 float64 adds per 16 elements instead of
+      // 3 float64 FMAs per element on this GPU's narrow float64 pipe. The sums steer the
+      // direction (Polak-Ribiere) and give the slope <G, Delta>; 16-term float32 sums carry
+      // about 2^-20 of their absolute terms, far below what either needs.
+      float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+      double* xo = ep.xout + ox;
+#pragma unroll
+      for (int k = 0; k < 16; ++k, xo += ldx) {
+        const float gf = dev::f32_rne_bits(g[k]), ak = in(k) ? a[k] : 0.f;
+        s0 = fmaf(gf, ak, s0);
+        s1 = fmaf(dev::f32_rne_bits(go[k]), ak, s1);
+        s2 = fmaf(gf, d[k], s2);
+        red.mb = max(red.mb, (unsigned long long)__double_as_longlong(g[k]) & 0x7FFFFFFFFFFFFFFFull);
+        if (in(k)) *xo = g[k];
+      }
+      red.v0 += widen(s0);
+      if (red.have_dir) {
+        red.v1 += widen(s1);
+        red.v2 += widen(s2);
       }
       continue;
     }
-    double out[8];
+    if (ep.c_f32) {  // float32 output: the accumulator itself, or alpha times it
+      const float al = (float)ep.alpha;
+      float* c = reinterpret_cast<float*>(ep.C) + blk * ep.split_stride + row * ldc + cb;
+#pragma unroll
+      for (int k = 0; k < 16; ++k, c += ldc) {
+        a[k] *= al;
+        if (in(k)) *c = a[k];
+      }
+      if (hp != nullptr) {
+        __nv_bfloat16* h = hp + r0 * bf_ld;
+#pragma unroll
+        for (int k = 0; k < 16; ++k, h += bf_ld)
+          if (in(k)) dev::split_store_f32(a[k], h, h + bf_lo, 0);
+      }
+      continue;
+    }
+    double o[16];
+    double* const c0 = ep.C + blk * ep.split_stride + row * ldc + cb;
     if (ep.mode == kEpGrad) {
-      double a0[8];
-      float4 a1[2];
+      const long ldx = ep.ldx, ldf = ep.ldf;
+      const double* q = ep.x0 + row * ldx + cb;
+      const float* f = ep.x1f + row * ldf + cb;
+      float x1[16];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) a0[k] = __ldg(ep.x0 + offx + c8 + k);
+      for (int k = 0; k < 16; ++k, q += ldx) o[k] = in(k) ? __ldg(q) : 0.0;
 #pragma unroll
-      for (int k = 0; k < 2; ++k) a1[k] = __ldg(reinterpret_cast<const float4*>(ep.x1f + offf + c8) + k);
+      for (int k = 0; k < 16; ++k, f += ldf) x1[k] = in(k) ? __ldg(f) : 0.f;
+      // the increment xs x1f + alpha acc in float32 (one rounding, 2^-24 of it, far below the
+      // split product's own 2^-17), then one float64 add onto x0
       const float alf = (float)ep.alpha, xsf = (float)ep.xs;
 #pragma unroll
-      for (int k = 0; k < 8; ++k) out[k] = a0[k] + widen(fmaf(xsf, f4_at(a1[k >> 2], k & 3), alf * v[c8 + k]));
-    } else if (unit) {
+      for (int k = 0; k < 16; ++k) o[k] += widen(fmaf(xsf, x1[k], alf * a[k]));
+    } else if (ep.beta == 0.0) {
 #pragma unroll
-      for (int k = 0; k < 8; ++k) out[k] = widen(v[c8 + k]);
+      for (int k = 0; k < 16; ++k) o[k] = widen(a[k]);
+      if (ep.alpha != 1.0) {
+#pragma unroll
+        for (int k = 0; k < 16; ++k) o[k] *= ep.alpha;
+      }
     } else {
+      const double* q = c0;
 #pragma unroll
-      for (int k = 0; k < 8; ++k) out[k] = combine(ep, widen(v[c8 + k]), ep.C + offc + c8 + k);
+      for (int k = 0; k < 16; ++k, q += ldc) o[k] = in(k) ? *q : 0.0;
+#pragma unroll
+      for (int k = 0; k < 16; ++k) o[k] = combine(ep, widen(a[k]), &o[k]);
     }
+    double* c = c0;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) ep.C[offc + c8 + k] = out[k];
-    if (ep.bf_hi != nullptr) {
-      unsigned short h[8], l[8];
+    for (int k = 0; k < 16; ++k, c += ldc)
+      if (in(k)) *c = o[k];
+    if (hp != nullptr) {
+      __nv_bfloat16* h = hp + r0 * bf_ld;
 #pragma unroll
-      for (int k = 0; k < 8; ++k) dev::split_bits_fast(out[k], h[k], l[k]);
-      __nv_bfloat16* hp = ep.bf_hi + bf0 + c8;
-      store_bf8(hp, h);
-      store_bf8(hp + ep.bf_lo, l);
+      for (int k = 0; k < 16; ++k, h += bf_ld)
+        if (in(k)) dev::split_store_fast(o[k], h, h + bf_lo, 0);
     }
   }
 }
 
-// C = alpha * v + beta * C (or a fused form) for the 32 accumulator columns [col0, col0 + 32) of one row.
-__device__ __forceinline__ void store_chunk(const Epilogue& ep, int row, int col0, const float (&v)[32], EpiRed& red) {
-  if (row >= ep.M || col0 >= ep.N) return;
-  const int nvalid = min(32, ep.N - col0);
-  const long blk0 = col0 / ep.split_cols;
-  const long blk1 = (col0 + nvalid - 1) / ep.split_cols;
-  if (ep.mode == kEpPlain && ep.bf_hi == nullptr && !ep.c_f32) {
-    if (blk0 == blk1) {  // specialised loops, no per-element branching
-      double* base = ep.C + blk0 * ep.split_stride + (long)row * ep.ldc + (col0 - blk0 * ep.split_cols);
-      if (ep.beta == 0.0) {
-        if (ep.alpha == 1.0) {
+__device__ __forceinline__ void store_chunk(const Epilogue& ep, uint32_t st, int row0, int col0, const float (&v)[32],
+                                            EpiRed& red) {
+  if (row0 >= ep.M || col0 >= ep.N) return;  // warp-uniform
+  const uint32_t lane = threadIdx.x & 31;
+  __syncwarp();  // the previous block has been read
 #pragma unroll
-          for (int j = 0; j < 32; ++j)
-            if (j < nvalid) base[j] = widen(v[j]);
-        } else {
-#pragma unroll
-          for (int j = 0; j < 32; ++j)
-            if (j < nvalid) base[j] = ep.alpha * widen(v[j]);
-        }
-      } else if (ep.beta == 1.0) {
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          if (j < nvalid) base[j] = fma(ep.alpha, widen(v[j]), base[j]);
-      } else {
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          if (j < nvalid) base[j] = fma(ep.beta, base[j], ep.alpha * widen(v[j]));
-      }
-      return;
-    }
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      if (j >= nvalid) break;
-      const int col = col0 + j;
-      const long blk = col / ep.split_cols;
-      double* p = ep.C + blk * ep.split_stride + (long)row * ep.ldc + (col - blk * ep.split_cols);
-      *p = combine(ep, widen(v[j]), p);
-    }
-    return;
-  }
-  // fused forms, float32 outputs and split outputs. Every index into v is a compile-time constant
-  // (the accumulator values stay in registers); sixteen columns at a time, their inputs loaded
-  // first (read-only path, 16-byte vectors) so that one memory latency covers them all.
-  const long cb0 = col0 - blk0 * ep.split_cols;
-  const long offc = blk0 * ep.split_stride + (long)row * ep.ldc + cb0;
-  const long offx = (long)row * ep.ldx + cb0, offf = (long)row * ep.ldf + cb0;
-  const long bf0 = blk0 * ep.bf_blk + (long)row * ep.bf_ld + cb0;
-  const bool fused = ep.mode != kEpPlain;
-  const bool vec8 = blk0 == blk1 && nvalid == 32 && (!ep.c_f32 || (offc & 3) == 0) && (!fused || (offf & 3) == 0) &&
-                    (ep.bf_hi == nullptr || ((bf0 & 7) == 0 && (ep.bf_lo & 7) == 0));
-  // the float64 rows on 16-byte boundaries too (an even leading dimension)
-  const bool vec = vec8 && (ep.c_f32 || (offc & 1) == 0) && (!fused || (offx & 1) == 0);
-  if (vec8 && !vec) {
-    store_chunk_odd(ep, offc, offx, offf, bf0, v, red);
-    return;
-  }
-  if (vec) {
-    const bool unit = ep.alpha == 1.0 && ep.beta == 0.0;  // plain store of the accumulator
-#pragma unroll
-    for (int h16 = 0; h16 < 2; ++h16) {
-      const int c16 = 16 * h16;
-      if (ep.c_f32) {  // float32 output: the accumulator itself (kEpReduce, or kEpPlain with alpha 1)
-        float o[16];
-        const float al = (float)ep.alpha;
-#pragma unroll
-        for (int k = 0; k < 16; ++k) o[k] = (ep.mode == kEpReduce || unit) ? v[c16 + k] : al * v[c16 + k];
-        if (ep.mode == kEpReduce) {
-          double2 g[8], go[8];
-          float4 d[4];
-#pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            g[k] = __ldg(reinterpret_cast<const double2*>(ep.x0 + offx + c16) + k);
-            if (red.have_dir) go[k] = *(reinterpret_cast<const double2*>(ep.x1 + offx + c16) + k);
-          }
-          if (red.have_dir) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) d[k] = __ldg(reinterpret_cast<const float4*>(ep.x2f + offf + c16) + k);
-          }
-          // the sums of these 16 products in float32 (g rounded to float32 on the integer pipe),
-          // then widened into the float64 running sums: 3 float64 adds per 16 elements instead of
-          // 3 float64 FMAs per element on this GPU's narrow float64 pipe. The sums steer the
-          // direction (Polak-Ribiere) and give the slope <G, Delta>; 16-term float32 sums carry
-          // about 2^-20 of their absolute terms, far below what either needs.
-          float s0 = 0.f, s1 = 0.f, s2 = 0.f;
-#pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            const float gx = dev::f32_rne_bits(g[k].x), gy = dev::f32_rne_bits(g[k].y);
-            s0 = fmaf(gx, o[2 * k], s0);
-            s0 = fmaf(gy, o[2 * k + 1], s0);
-            red.mb = max(red.mb, (unsigned long long)__double_as_longlong(g[k].x) & 0x7FFFFFFFFFFFFFFFull);
-            red.mb = max(red.mb, (unsigned long long)__double_as_longlong(g[k].y) & 0x7FFFFFFFFFFFFFFFull);
-            if (red.have_dir) {
-              s1 = fmaf(dev::f32_rne_bits(go[k].x), o[2 * k], s1);
-              s1 = fmaf(dev::f32_rne_bits(go[k].y), o[2 * k + 1], s1);
-              const float dx = (k & 1) ? d[k >> 1].z : d[k >> 1].x, dy = (k & 1) ? d[k >> 1].w : d[k >> 1].y;
-              s2 = fmaf(gx, dx, s2);
-              s2 = fmaf(gy, dy, s2);
-            }
-          }
-          red.v0 += widen(s0);
-          if (red.have_dir) {
-            red.v1 += widen(s1);
-            red.v2 += widen(s2);
-          }
-#pragma unroll
-          for (int k = 0; k < 8; ++k) *(reinterpret_cast<double2*>(ep.xout + offx + c16) + k) = g[k];
-        }
-        float4* c4 = reinterpret_cast<float4*>(reinterpret_cast<float*>(ep.C) + offc + c16);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) c4[k] = make_float4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
-        if (ep.bf_hi != nullptr) {
-#pragma unroll
-          for (int g8 = 0; g8 < 2; ++g8) {
-            unsigned short h[8], l[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) dev::split_bits_f32(o[8 * g8 + k], h[k], l[k]);
-            __nv_bfloat16* hp = ep.bf_hi + bf0 + c16 + 8 * g8;
-            store_bf8(hp, h);
-            store_bf8(hp + ep.bf_lo, l);
-          }
-        }
-        continue;
-      }
-      double out[16];
-      if (ep.mode == kEpGrad) {
-        double2 a0[8];
-        float4 a1[4];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) a0[k] = __ldg(reinterpret_cast<const double2*>(ep.x0 + offx + c16) + k);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) a1[k] = __ldg(reinterpret_cast<const float4*>(ep.x1f + offf + c16) + k);
-        // the increment xs x1f + alpha acc in float32 (one rounding, 2^-24 of it, far below the
-        // split product's own 2^-17), then one float64 add onto x0
-        const float alf = (float)ep.alpha, xsf = (float)ep.xs;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const float fx = (k & 1) ? a1[k >> 1].z : a1[k >> 1].x, fy = (k & 1) ? a1[k >> 1].w : a1[k >> 1].y;
-          out[2 * k] = a0[k].x + widen(fmaf(xsf, fx, alf * v[c16 + 2 * k]));
-          out[2 * k + 1] = a0[k].y + widen(fmaf(xsf, fy, alf * v[c16 + 2 * k + 1]));
-        }
-      } else if (unit) {
-#pragma unroll
-        for (int k = 0; k < 16; ++k) out[k] = widen(v[c16 + k]);
-      } else {
-#pragma unroll
-        for (int k = 0; k < 16; ++k) out[k] = combine(ep, widen(v[c16 + k]), ep.C + offc + c16 + k);
-      }
-      double2* c2 = reinterpret_cast<double2*>(ep.C + offc + c16);
-#pragma unroll
-      for (int k = 0; k < 8; ++k) c2[k] = make_double2(out[2 * k], out[2 * k + 1]);
-      if (ep.bf_hi != nullptr) {
-#pragma unroll
-        for (int g8 = 0; g8 < 2; ++g8) {
-          unsigned short h[8], l[8];
-#pragma unroll
-          for (int k = 0; k < 8; ++k) dev::split_bits_fast(out[8 * g8 + k], h[k], l[k]);
-          __nv_bfloat16* hp = ep.bf_hi + bf0 + c16 + 8 * g8;
-          store_bf8(hp, h);
-          store_bf8(hp + ep.bf_lo, l);
-        }
-      }
-    }
-    return;
-  }
-#pragma unroll
-  for (int j = 0; j < 32; ++j) {
-    if (j >= nvalid) break;
-    const int col = col0 + j;
-    const long blk = col / ep.split_cols;
-    fused_element(ep, v[j], row, blk, col - blk * ep.split_cols, red);
-  }
+  for (int j = 0; j < 32; ++j) sts_f32(st + (lane * kEpiPitch + j) * 4, v[j]);
+  __syncwarp();
+  // a whole block runs without a mask: a masked access is a branch around it
+  if (row0 + 32 <= ep.M && col0 + 32 <= ep.N) store_block<true>(ep, st + lane * 4, row0, col0, red);
+  else store_block<false>(ep, st + lane * 4, row0, col0, red);
 }
 
 // kEpReduce: the epilogue warp's sums of this tile into its partial slot (fixed order)
@@ -645,15 +493,15 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap* mA, const CUtensorM
     if (!ok) atomicCAS(ep.err, 0, 3);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const int lane_base = (warp & 3) * 32;
-    const int row = m0 + lane_base + lane;
     const bool write = ok && !*abort_flag;
+    const uint32_t st = smem_u32(smem + RING_BYTES + 256) + (uint32_t)(warp & 3) * 32 * kEpiPitch * 4;
     EpiRed red;
     red.have_dir = ep.mode == kEpReduce && ep.sc != nullptr && ep.sc->have_dir;
 #pragma unroll 1
     for (int c = 0; c < BN / 32; ++c) {
       float v[32];
       tmem_ld32(tmem + ((uint32_t)lane_base << 16) + (uint32_t)(c * 32), v);
-      if (write) store_chunk(ep, row, n0 + c * 32, v, red);
+      if (write) store_chunk(ep, st, m0 + lane_base, n0 + c * 32, v, red);
     }
     if (write) flush_reduce(ep, tile, warp & 3, red);
   }
@@ -884,6 +732,7 @@ __device__ __forceinline__ void persistent_body(const GroupDesc* __restrict__ gr
   } else if (warp >= 2) {
     // ---------------- epilogue
     const int lane_base = (warp & 3) * 32;
+    const uint32_t st = smem_u32(smem + RING_BYTES + 256) + (uint32_t)(warp & 3) * 32 * kEpiPitch * 4;
     uint32_t lt = 0;
     bool failed = false;
     for (int tile = blockIdx.x; tile < total_tiles && !failed; tile += gridDim.x) {
@@ -901,14 +750,13 @@ __device__ __forceinline__ void persistent_body(const GroupDesc* __restrict__ gr
       const Epilogue ep = g->ep;
       const int local = tile - g->tile_begin, tiles_m = (ep.M + BM - 1) / BM;
       const int m0 = (local % tiles_m) * BM, n0 = (local / tiles_m) * TBN;
-      const int row = m0 + lane_base + lane;
       EpiRed red;
       red.have_dir = ep.mode == kEpReduce && ep.sc != nullptr && ep.sc->have_dir;
 #pragma unroll 1
       for (int j = 0; j < TBN / 32; ++j) {
         float v[32];
         tmem_ld32(tmem + buf * ACC_COLS + ((uint32_t)lane_base << 16) + (uint32_t)(j * 32), v);
-        store_chunk(ep, row, n0 + j * 32, v, red);
+        store_chunk(ep, st, m0 + lane_base, n0 + j * 32, v, red);
       }
       flush_reduce(ep, local, warp & 3, red);
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1187,6 +1035,7 @@ __device__ __forceinline__ void pair_body(const GroupDesc* __restrict__ groups, 
     const int lane_base = (warp & 3) * 32;
     const uint32_t acc_empty0 = mapa_shared(smem_u32(&bars[2 * NS + 2]), lead_rank);
     const uint32_t acc_empty1 = mapa_shared(smem_u32(&bars[2 * NS + 3]), lead_rank);
+    const uint32_t st = smem_u32(smem + RING_BYTES + 256) + (uint32_t)(warp & 3) * 32 * kEpiPitch * 4;
     uint32_t lt = 0;
     for (int u = cluster; u < total_units; u += nclusters) {
       const GroupDesc* g = groups + find_group(groups, ngroups, u);
@@ -1202,14 +1051,13 @@ __device__ __forceinline__ void pair_body(const GroupDesc* __restrict__ groups, 
       const Epilogue ep = g->ep;
       const int local = u - g->tile_begin, tiles_m = (ep.M + 2 * BM - 1) / (2 * BM);
       const int m0 = (local % tiles_m) * 2 * BM + rr * BM, n0 = ((local / tiles_m) * NP + pp) * TBN;
-      const int row = m0 + lane_base + lane;
       EpiRed red;
       red.have_dir = ep.mode == kEpReduce && ep.sc != nullptr && ep.sc->have_dir;
 #pragma unroll 1
       for (int j = 0; j < TBN / 32; ++j) {
         float v[32];
         tmem_ld32(tmem + buf * ACC_STRIDE + ((uint32_t)lane_base << 16) + (uint32_t)(j * 32), v);
-        store_chunk(ep, row, n0 + j * 32, v, red);
+        store_chunk(ep, st, m0 + lane_base, n0 + j * 32, v, red);
       }
       flush_reduce(ep, (local * NP + pp) * 2 + rr, warp & 3, red);  // slots of 128 x TBN quarters
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
