@@ -341,13 +341,10 @@ __device__ __forceinline__ void traces_body(int n, const double* __restrict__ SW
       }
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-#pragma unroll
-      for (int q = 0; q < kNumTraces; ++q) {
-        double acc = 0.0;
-        for (int k = 0; k < TB / 32; ++k) acc += sh[q][k];
-        part[(long)bx_ * kNumTraces + q] = acc;
-      }
+    if (threadIdx.x < kNumTraces) {  // one lane per trace
+      double acc = 0.0;
+      for (int k = 0; k < TB / 32; ++k) acc += sh[threadIdx.x][k];
+      part[(long)bx_ * kNumTraces + threadIdx.x] = acc;
     }
     return;
   }
@@ -359,16 +356,34 @@ __device__ __forceinline__ void traces_body(int n, const double* __restrict__ SW
 }
 __device__ __forceinline__ void control_linesearch_body(Scalars* sc, const double* part, int nblocks, int bx_, int nbx_) {
   if (stopped(sc)) return;
+  // Sums over the blocks: thread (seg, q) adds every kSegs-th block's q-th sum, then thread q its kSegs
+  // partial sums, in fixed order. A float64 add takes its warp about 30 clocks of the SM's float64 unit
+  // however many lanes are active, so the eleven sums lie side by side in the lanes (a tree of shuffles
+  // for each of them in each warp cost 600 adds, 9 us; this is about 40).
+  constexpr int kSegs = TB / 16;
+  static_assert(kNumTraces <= 16, "one lane per trace in a group of 16");
+  __shared__ double seg_sum[kSegs][kNumTraces];
+  __shared__ double total[kNumTraces];
+  {
+    const int q = threadIdx.x % 16, seg = threadIdx.x / 16;
+    if (q < kNumTraces) {
+      double v = 0.0;
+      for (int b = seg; b < nblocks; b += kSegs) v += part[(long)b * kNumTraces + q];
+      seg_sum[seg][q] = v;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < kNumTraces) {
+    double v = 0.0;
+#pragma unroll
+    for (int k = 0; k < kSegs; ++k) v += seg_sum[k][threadIdx.x];
+    total[threadIdx.x] = v;
+  }
+  __syncwarp();
+  if (threadIdx.x != 0) return;
   double t[kNumTraces];
 #pragma unroll
-  for (int q = 0; q < kNumTraces; ++q) t[q] = 0.0;
-  for (int b = threadIdx.x; b < nblocks; b += TB) {
-#pragma unroll
-    for (int q = 0; q < kNumTraces; ++q) t[q] += part[(long)b * kNumTraces + q];
-  }
-  __shared__ double sh[kNumTraces][TB / 32];
-  block_sum<kNumTraces>(t, sh);
-  if (threadIdx.x != 0) return;
+  for (int q = 0; q < kNumTraces; ++q) t[q] = total[q];
   double a[5];
   a[0] = sc->E;
   a[1] = 8.0 * t[0] - 4.0 * t[1] - 4.0 * t[2];

@@ -265,7 +265,12 @@ int traces_blocks(int n) {
   const int t = (n + 31) / 32;
   return t * t;
 }
-int traces_partials(int n) { return (traces_blocks(n) + 3) / 4; }
+// a tile per CTA while two waves of CTAs hold them all (n <= 544: with four tiles per CTA an n = 128 solve
+// ran them on 4 SMs, 23 us); above, four tiles per CTA, so that fewer partial sums are left
+int traces_partials(int n) {
+  const int tiles = traces_blocks(n);
+  return tiles <= 2 * 152 ? tiles : (tiles + 3) / 4;
+}
 void launch_traces(cudaStream_t st, int n, const double* SWHW, const double* Proj, double* part,
                    const Scalars* sc, bool fp32_products) {
   if (fp32_products) traces_kernel<true><<<traces_partials(n), TB, 0, st>>>(n, SWHW, Proj, part, sc);
