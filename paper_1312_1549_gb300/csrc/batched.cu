@@ -322,7 +322,7 @@ omm_status omm_create_batched(int count, const int* m, const int* n, const doubl
       mixed_epilogues(c->mixed, c->sc, c->G, c->Gold, c->Y4, c->Proj, ep);
       if (b->precond) spg.push_back(tc::GemmSpec{v.opG, v.opP, mi, ep[0]});
       tc::GemmSpec hd{v.opD, v.opHS, mi, ep[1]};
-      for (int q = 0; q < 3; ++q) hd.sparse[q] = &v.hs_blocks[q];
+      for (int q = 0; q < 4; ++q) hd.sparse[q] = &v.hs_blocks[q];
       shd.push_back(hd);
       spr.push_back(tc::GemmSpec{v.opD, v.opYproj, mi, ep[2]});
       sg.push_back(tc::GemmSpec{v.opW, v.opYgrad, 4 * ni, ep[3]});

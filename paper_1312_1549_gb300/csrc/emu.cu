@@ -276,7 +276,7 @@ struct EmuState {
   tc::Operand opHS, opC, opY, opW, opYT, opCT, opXT, opSW, opCTb;  // opCTb: C^T as a B operand
   int* err = nullptr;
   double* slab = nullptr;     // float64 sums of the sliced products (tc::sliced_workspace_doubles)
-  tc::BlockLists hs_blocks;   // block sparsity of [H~; S] (256-row blocks)
+  const tc::BlockLists* hs_blocks = nullptr;  // block sparsity of [H~; S] (256-row blocks), the mixed state's
 };
 
 namespace {
@@ -284,7 +284,7 @@ namespace {
 constexpr int kDensitySlices = 8;
 }
 
-EmuState* emu_create(cudaStream_t st, int m, int n, int slices, const double* HS) {
+EmuState* emu_create(cudaStream_t st, int m, int n, int slices, const double* HS, const tc::BlockLists* hs_blocks) {
   EmuState* es = new EmuState();
   try {
     es->m = m;
@@ -307,7 +307,7 @@ EmuState* emu_create(cudaStream_t st, int m, int n, int slices, const double* HS
     alloc(&es->slab, (size_t)tc::sliced_workspace_doubles(), st);
     OMM_CUDA_TRY(cudaMemsetAsync(es->err, 0, sizeof(int), st));
     emu::slice_rows(st, HS, 2L * m, m, m, slices, es->HSs, ldm, nullptr);
-    tc::block_lists(st, HS, 2L * m, m, m, 256, es->hs_blocks);
+    es->hs_blocks = hs_blocks;
     es->opHS = tc::make_operand(es->HSs, 2L * m, m, ldm, slices, false);
     es->opC = tc::make_operand(es->Cs, n, m, ldm, slices, true);
     es->opY = tc::make_operand(es->Ys, 2L * n, m, ldm, slices, false);
@@ -326,14 +326,12 @@ EmuState* emu_create(cudaStream_t st, int m, int n, int slices, const double* HS
 
 void emu_update_H(EmuState* es, cudaStream_t st, const double* HS) {
   emu::slice_rows(st, HS, 2L * es->m, es->m, es->m, es->s, es->HSs, es->ldm, nullptr);
-  tc::block_lists(st, HS, 2L * es->m, es->m, es->m, 256, es->hs_blocks);
 }
 
 void emu_destroy(EmuState* es, cudaStream_t st) {
   if (!es) return;
   void* bufs[] = {es->HSs, es->Cs, es->Ys, es->Ws, es->YTs, es->T64, es->CTs, es->XTs, es->SWs, es->err, es->slab};
   for (void* b : bufs) mem::release(b, st);
-  tc::free_block_lists(es->hs_blocks, st);
   delete es;
 }
 
@@ -352,7 +350,7 @@ void emu_recompute_state(EmuState* es, cudaStream_t st, Scalars* sc, const doubl
   emu::slice_rows(st, C, n, m, m, s, es->Cs, es->ldm, nullptr);
   // [HC; SC] (n x m layout) = C [H~; S]^T
   emu::gemm(st, es->opC, es->opHS, m, s, tc::Epilogue{Y4, m, m, nm, 1.0, 0.0, n, 2 * m, nullptr, es->err},
-            es->slab, &es->hs_blocks);
+            es->slab, es->hs_blocks);
   emu::slice_rows(st, Y4, 2L * n, m, m, s, es->Ys, es->ldm, nullptr);
   // [S_W | H_W] = C [SC; HC]^T
   emu::gemm(st, es->opC, es->opY, m, s,

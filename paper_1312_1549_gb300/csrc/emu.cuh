@@ -24,7 +24,8 @@ void gemm_split(cudaStream_t st, const tc::Operand& A, const tc::Operand& B, int
 }  // namespace emu
 
 struct EmuState;
-EmuState* emu_create(cudaStream_t st, int m, int n, int slices, const double* HS);
+// hs_blocks: the 256-row block lists of HS, kept by the caller (and brought up to date before emu_update_H)
+EmuState* emu_create(cudaStream_t st, int m, int n, int slices, const double* HS, const tc::BlockLists* hs_blocks);
 void emu_update_H(EmuState* es, cudaStream_t st, const double* HS);
 void emu_destroy(EmuState* es, cudaStream_t st);  // st: the owner's current stream
 int emu_error(EmuState* es, cudaStream_t st);

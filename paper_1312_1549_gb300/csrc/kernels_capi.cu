@@ -229,7 +229,7 @@ omm_status gemm_tc_impl(const char* name, int M, int N, int K, const double* A, 
       tc::split(st, B, N, K, K, b_hi, b_lo, ldb, nullptr);
       ob = tc::make_operand(b_hi, N, K, ldb, 2, false);
     }
-    if (block_sparse) tc::block_lists(st, B, N, K, K, tile_n, lists);
+    if (block_sparse) tc::block_lists(st, B, N, K, K, 1, &tile_n, &lists);
     const tc::Epilogue ep{C, N, N, 0, alpha, beta, M, N, nullptr, err};
     const tc::GroupDesc g = tc::make_group(oa, ob, K, ep, 0, tile_n, block_sparse ? &lists : nullptr, pair, quad);
     OMM_CUDA_TRY(cudaMemcpyAsync(desc, &g, sizeof(g), cudaMemcpyHostToDevice, st));

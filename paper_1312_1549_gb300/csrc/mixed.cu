@@ -45,7 +45,7 @@ struct MixedState {
   float* HD32 = nullptr;                               // 2n x m
   float* dY32 = nullptr;                               // 2n x m
   tc::Operand opHS, opP, opG, opD, opYproj, opYgrad, opYhc, opW;
-  tc::BlockLists hs_blocks[3];  // block sparsity of [H~; S] for 256-, 128- and 192-row blocks (Sec. 2.6)
+  tc::BlockLists hs_blocks[4];  // block sparsity of [H~; S] by row blocks of tc::kSparseWidths (Sec. 2.6)
   int* err = nullptr;
   int expire = 0;  // tests: the first line-search GEMM of every line search waits on nothing and expires
   // the four line-search GEMMs as persistent-launch descriptors (device), built on first use
@@ -64,9 +64,10 @@ struct MixedState {
 namespace {
 
 long round8(long x) { return (x + 7) / 8 * 8; }
-// output tiles of the P G product (n x m) counted as 128 x 128 tiles, rounded so that 256-row tiles
-// (two slots of four warps each) and the odd column tile of a two-pair cluster fit too
-long red_tiles(long n, long m) { return 2 * ((n + 255) / 256) * ((m + 127) / 128 + 1); }
+// partial-sum slots of the P G product's epilogue (n x m): one per epilogue warp and tile, four warps on
+// 128 rows, at the narrowest tile (32 columns); 256-row tiles and the odd column tile of a two-pair
+// cluster are rounded up into it
+long red_slots(long n, long m) { return 4 * 2 * ((n + 255) / 256) * ((m + 31) / 32 + 8); }
 
 template <typename T>
 void alloc(T** p, size_t count, cudaStream_t st) {
@@ -102,12 +103,10 @@ MixedState* mixed_create(cudaStream_t st, int m, int n, const double* HS, const 
     alloc(&ms->HD32, 2L * n * ldm, st);
     alloc(&ms->dY32, 2L * n * ldm, st);
     OMM_CUDA_TRY(cudaMemsetAsync(ms->Dir32, 0, (size_t)n * ldm * sizeof(float), st));
-    // 4 sums per epilogue warp (4 per 128-row tile, 8 per 256-row tile) and output tile, at the
-    // narrowest tile (128 columns)
-    alloc(&ms->red, (size_t)16 * red_tiles(n, m), st);
+    alloc(&ms->red, (size_t)4 * red_slots(n, m), st);  // 4 sums per slot
     alloc(&ms->err, 1, st);
     OMM_CUDA_TRY(cudaMemsetAsync(ms->err, 0, sizeof(int), st));
-    OMM_CUDA_TRY(cudaMemsetAsync(ms->red, 0, (size_t)16 * red_tiles(n, m) * sizeof(double), st));
+    OMM_CUDA_TRY(cudaMemsetAsync(ms->red, 0, (size_t)4 * red_slots(n, m) * sizeof(double), st));
     // padding columns stay zero (the tensor maps never read them, but keep them defined)
     OMM_CUDA_TRY(cudaMemsetAsync(ms->Y_hi, 0, 2 * (size_t)6 * n * ldm * 2, st));
     OMM_CUDA_TRY(cudaMemsetAsync(ms->W_hi, 0, 2 * (size_t)n * ld4n * 2, st));
@@ -125,7 +124,7 @@ MixedState* mixed_create(cudaStream_t st, int m, int n, const double* HS, const 
     ms->opYhc = tc::make_operand_view(ms->Y_hi, 6L * n, m, ldm, 2, false, 2 * n, 2L * n);
     ms->opW = tc::make_operand(ms->W_hi, n, 4L * n, ld4n, 2, true);
     // finite-range H and S: the operator product skips the K blocks where [H~; S] is zero
-    for (int bn : {256, 128, 192}) tc::block_lists(st, HS, 2L * m, m, m, bn, ms->hs_blocks[tc::sparse_slot(bn)]);
+    tc::block_lists(st, HS, 2L * m, m, m, 4, tc::kSparseWidths, ms->hs_blocks);
   } catch (...) {
     mixed_destroy(ms, st);
     throw;
@@ -186,8 +185,7 @@ MixedView mixed_view(MixedState* ms) {
 
 void mixed_update_H(MixedState* ms, cudaStream_t st, const double* HS) {
   tc::split(st, HS, ms->m, ms->m, ms->m, ms->HS_hi, ms->HS_lo, ms->ldm, nullptr);
-  for (int bn : {256, 128, 192})  // the pattern may change
-    tc::block_lists(st, HS, 2L * ms->m, ms->m, ms->m, bn, ms->hs_blocks[tc::sparse_slot(bn)]);
+  tc::block_lists(st, HS, 2L * ms->m, ms->m, ms->m, 4, tc::kSparseWidths, ms->hs_blocks);  // the pattern may change
 }
 
 void mixed_destroy(MixedState* ms, cudaStream_t st) {
@@ -335,7 +333,7 @@ void build_plans(MixedState* ms, cudaStream_t st, Scalars* sc, double* G, double
     // product runs block-sparse over [H~; S]
     tc::GemmSpec spec{opA[k], opB[k], K[k], ep[k]};
     if (k == kPlanHD)
-      for (int q = 0; q < 3; ++q) spec.sparse[q] = &ms->hs_blocks[q];
+      for (int q = 0; q < 4; ++q) spec.sparse[q] = &ms->hs_blocks[q];
     double ms_tune = 0.0;
     const tc::TileShape ts = tc::choose_tile_shape(st, {spec}, plan_pairs(k), &ms_tune);
     ms->plan_shape[k] = ts;

@@ -263,8 +263,8 @@ void destroy(omm_ctx* c) {
   if (c->sc_host) cudaFreeHost(c->sc_host);
   for (auto& e : c->ev)
     if (e) cudaEventDestroy(e);
-  if (c->mixed) mixed_destroy(c->mixed, c->st);
   if (c->emu) emu_destroy(c->emu, c->st);
+  if (c->mixed) mixed_destroy(c->mixed, c->st);
   if (c->red) reduction_destroy(c->red, c->st);
   delete c;
 }
@@ -390,7 +390,7 @@ omm_status omm_create(int m, int n, const double* H, const double* S, const doub
       c->mixed = mixed_create(c->st, m, n, c->HS, c->P);
       if (o.debug_expire_wait) mixed_set_expire(c->mixed, 1);
       if (4.0 * m * (double)m * n + 8.0 * m * (double)n * n >= kSlicedStateMinFlop)
-        c->emu = emu_create(c->st, m, n, kEmuSlices, c->HS);
+        c->emu = emu_create(c->st, m, n, kEmuSlices, c->HS, &mixed_view(c->mixed).hs_blocks[tc::sparse_slot(256)]);
     }
     OMM_CUDA_TRY(cudaEventRecord(c->ev[1], c->st));
     int info = 0, ierr = 0;

@@ -16,7 +16,7 @@ struct MixedView {
   double *Gref, *Wref, *red;
   float *Dir32, *PG32, *HD32, *dY32;  // float32 side quantities, leading dimension ldm
   const tc::Operand *opHS, *opP, *opG, *opD, *opYproj, *opYgrad, *opW;
-  const tc::BlockLists* hs_blocks;  // [0]: 256-row blocks, [1]: 128-row blocks, [2]: 192-row blocks
+  const tc::BlockLists* hs_blocks;  // by tc::sparse_slot(width)
   int* err;
   int npass;
   bool precond;

@@ -90,9 +90,10 @@ Reduction* reduction_create(cudaStream_t st, int m, bool sliced, double* S, int*
       spd_factor_inverse_sliced(st, m, S, r->Y, work, info_dev, r->err);
       emu::transpose(st, S, m, m, m, r->L, m);     // L^T
       emu::transpose(st, r->Y, m, m, m, r->YT, m);  // L^-T
-      tc::block_lists(st, r->Y, m, m, m, 256, r->blY);
-      tc::block_lists(st, r->YT, m, m, m, 256, r->blYT);
-      tc::block_lists(st, r->L, m, m, m, 256, r->blLT);
+      const int width = 256;
+      tc::block_lists(st, r->Y, m, m, m, 1, &width, &r->blY);
+      tc::block_lists(st, r->YT, m, m, m, 1, &width, &r->blYT);
+      tc::block_lists(st, r->L, m, m, m, 1, &width, &r->blLT);
     } else {
       alloc(reinterpret_cast<double**>(&work), spd_inverse_workspace(m), st);
       spd_factor_inverse(st, m, S, r->Y, static_cast<double*>(work), info_dev);

@@ -26,6 +26,8 @@
 #include "tc_gemm.cuh"
 
 #include <algorithm>
+#include <cstdlib>
+#include <cstring>
 #include <map>
 #include <mutex>
 #include <string>
@@ -562,7 +564,9 @@ __device__ __forceinline__ KBlocks tile_kblocks(const GroupDesc* g, int local, i
 template <bool FUSED, int TBN>
 __device__ __forceinline__ void persistent_body(const GroupDesc* __restrict__ groups, int ngroups, int total_tiles,
                                                 const PairList& pl, int* err) {
-  // TBN: output tile width (256 or 128); the stage ring keeps the same shared memory
+  // TBN: output tile width (32 to 256); the stage ring keeps the same shared memory. The narrow tiles
+  // serve small products: an epilogue takes 2 to 8 thousand clocks per 32 columns (float64 adds, memory
+  // round trips), so a 128 x 256 output is finished sooner by eight SMs than by two
   constexpr int TB_BYTES = TBN * BK * 2;
   constexpr int TSTAGE = A_BYTES + TB_BYTES;
   constexpr int SB = FUSED ? 2 * TSTAGE : TSTAGE;
@@ -1294,12 +1298,12 @@ GroupDesc make_group(const Operand& A, const Operand& B, int K, const Epilogue& 
   if (quad) pair = true;
   if (quad && sparse != nullptr)
     throw CudaError{cudaErrorInvalidValue, "tc::make_group: clusters of two pairs need a dense B"};
-  if (pair ? (bn != 256 && bn != 192 && bn != 128) : (bn != 256 && bn != 128))
+  if (pair ? (bn != 256 && bn != 192 && bn != 128) : (bn != 256 && bn != 128 && bn != 64 && bn != 32))
     throw CudaError{cudaErrorInvalidValue, "tc::make_group: tile width"};
   // the TMA boxes must match the tile: A in 128-row boxes, B in boxes of the tile width (of half of
   // it on an SM pair), or, MN-major, in 64 x 64 boxes (then the width an SM stages is a multiple of 64)
   if (A.mn_major || A.box_rows != BM || (!B.mn_major && !pair && bn == 256 && B.box_rows != 256) ||
-      (B.mn_major && pair && (bn / 2) % 64 != 0))
+      (B.mn_major && (pair ? bn / 2 : bn) % 64 != 0))
     throw CudaError{cudaErrorInvalidValue, "tc::make_group: operand boxes do not match the tile"};
   if (B.mn_major && (sparse != nullptr || K > B.rows))
     throw CudaError{cudaErrorInvalidValue, "tc::make_group: MN-major B: no block lists, K <= its rows"};
@@ -1311,7 +1315,7 @@ GroupDesc make_group(const Operand& A, const Operand& B, int K, const Epilogue& 
   else if (pair)
     g.b = bn == 256 ? B.map_n128 : make_map(B.base, B.map_rows, B.cols, B.ld, bn / 2);
   else
-    g.b = bn == 128 ? B.map_n128 : B.map;
+    g.b = bn == 128 ? B.map_n128 : (bn == 256 ? B.map : make_map(B.base, B.map_rows, B.cols, B.ld, bn));
   g.pair = pair ? 1 : 0;
   g.ep = ep;
   g.K = K;
@@ -1332,17 +1336,13 @@ GroupDesc make_group(const Operand& A, const Operand& B, int K, const Epilogue& 
 void prepare_persistent() {
   static bool attr_set = false;
   if (!attr_set) {
-    OMM_CUDA_TRY(cudaFuncSetAttribute(gemm_persistent_kernel<false, 256>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
-    OMM_CUDA_TRY(cudaFuncSetAttribute(gemm_persistent_kernel<true, 256>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
-    OMM_CUDA_TRY(cudaFuncSetAttribute(gemm_persistent_kernel<false, 128>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
-    OMM_CUDA_TRY(cudaFuncSetAttribute(gemm_persistent_kernel<true, 128>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
     OMM_CUDA_TRY(cudaFuncSetAttribute(gemm_persistent_one_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       SMEM_BYTES));
-    for (const void* f : {(const void*)gemm_pair_kernel<128, true>, (const void*)gemm_pair_kernel<192, true>,
+    for (const void* f : {(const void*)gemm_persistent_kernel<false, 256>, (const void*)gemm_persistent_kernel<true, 256>,
+                          (const void*)gemm_persistent_kernel<false, 128>, (const void*)gemm_persistent_kernel<true, 128>,
+                          (const void*)gemm_persistent_kernel<false, 64>, (const void*)gemm_persistent_kernel<true, 64>,
+                          (const void*)gemm_persistent_kernel<false, 32>, (const void*)gemm_persistent_kernel<true, 32>,
+                          (const void*)gemm_pair_kernel<128, true>, (const void*)gemm_pair_kernel<192, true>,
                           (const void*)gemm_pair_kernel<256, true>, (const void*)gemm_pair_kernel<128, false>,
                           (const void*)gemm_pair_kernel<192, false>, (const void*)gemm_pair_kernel<256, false>,
                           (const void*)gemm_pair_one_kernel, (const void*)sliced_pair_kernel,
@@ -1390,16 +1390,15 @@ void gemm_persistent(cudaStream_t st, const GroupDesc* groups_dev, int ngroups, 
     OMM_LAUNCH_CHECK();
     return;
   }
-  if (bn != 256 && bn != 128) throw CudaError{cudaErrorInvalidValue, "tc::gemm_persistent: tile width"};
   const unsigned grid = (unsigned)std::min(total_tiles, sm_count());
-  if (bn == 256 && fused)
-    gemm_persistent_kernel<true, 256><<<grid, NTHREADS, SMEM_BYTES, st>>>(groups_dev, ngroups, total_tiles, pl, err);
-  else if (bn == 256)
-    gemm_persistent_kernel<false, 256><<<grid, NTHREADS, SMEM_BYTES, st>>>(groups_dev, ngroups, total_tiles, pl, err);
-  else if (fused)
-    gemm_persistent_kernel<true, 128><<<grid, NTHREADS, SMEM_BYTES, st>>>(groups_dev, ngroups, total_tiles, pl, err);
-  else
-    gemm_persistent_kernel<false, 128><<<grid, NTHREADS, SMEM_BYTES, st>>>(groups_dev, ngroups, total_tiles, pl, err);
+  auto go = [&](auto kernel) {
+    kernel<<<grid, NTHREADS, SMEM_BYTES, st>>>(groups_dev, ngroups, total_tiles, pl, err);
+  };
+  if (bn == 256) fused ? go(gemm_persistent_kernel<true, 256>) : go(gemm_persistent_kernel<false, 256>);
+  else if (bn == 128) fused ? go(gemm_persistent_kernel<true, 128>) : go(gemm_persistent_kernel<false, 128>);
+  else if (bn == 64) fused ? go(gemm_persistent_kernel<true, 64>) : go(gemm_persistent_kernel<false, 64>);
+  else if (bn == 32) fused ? go(gemm_persistent_kernel<true, 32>) : go(gemm_persistent_kernel<false, 32>);
+  else throw CudaError{cudaErrorInvalidValue, "tc::gemm_persistent: tile width"};
   OMM_LAUNCH_CHECK();
 }
 
@@ -1507,57 +1506,64 @@ occupancy_kernel(const double* __restrict__ B, long rows, long cols, long ld, in
 }
 }  // namespace
 
-void block_lists(cudaStream_t st, const double* B, long rows, long cols, long ld, int bn, BlockLists& bl) {
-  if (bn != 128 && bn != 192 && bn != 256) throw CudaError{cudaErrorInvalidValue, "tc::block_lists: tile width"};
+void block_lists(cudaStream_t st, const double* B, long rows, long cols, long ld, int count, const int* widths,
+                 BlockLists* lists) {
   const int nkb = (int)((cols + BK - 1) / BK);
   const long nrb64 = (rows + OCC_ROWS - 1) / OCC_ROWS;
   unsigned char* occ = nullptr;
   std::vector<unsigned char> h(nrb64 * nkb);
-  OMM_CUDA_TRY(cudaMallocAsync((void**)&occ, h.size(), st));
+  mem::alloc(&occ, h.size(), st);
   try {
     occupancy_kernel<<<(unsigned)(nrb64 * nkb), 256, 0, st>>>(B, rows, cols, ld, nkb, occ);
     OMM_LAUNCH_CHECK();
     OMM_CUDA_TRY(cudaMemcpyAsync(h.data(), occ, h.size(), cudaMemcpyDeviceToHost, st));
     OMM_CUDA_TRY(cudaStreamSynchronize(st));
   } catch (...) {
-    cudaFreeAsync(occ, st);
+    mem::release(occ, st);
     throw;
   }
-  cudaFreeAsync(occ, st);
-  const int per = bn / OCC_ROWS;  // 64-row blocks per row block of bn
-  const int nblocks = (int)((rows + bn - 1) / bn);
-  std::vector<int> off(nblocks + 1, 0), idx;
-  for (int r = 0; r < nblocks; ++r) {
-    const size_t before = idx.size();
-    for (int kb = 0; kb < nkb; ++kb) {
-      bool any = false;
-      for (int q = 0; q < per; ++q) {
-        const long r64 = (long)r * per + q;
-        if (r64 < nrb64 && h[r64 * nkb + kb]) any = true;
+  mem::release(occ, st);
+  std::vector<std::vector<int>> off(count), idx(count);
+  for (int w = 0; w < count; ++w) {
+    const int bn = widths[w];
+    BlockLists& bl = lists[w];
+    if (bn != 64 && bn != 128 && bn != 192 && bn != 256)
+      throw CudaError{cudaErrorInvalidValue, "tc::block_lists: tile width"};
+    const int per = bn / OCC_ROWS;  // 64-row blocks per row block of bn
+    const int nblocks = (int)((rows + bn - 1) / bn);
+    off[w].assign(nblocks + 1, 0);
+    for (int r = 0; r < nblocks; ++r) {
+      const size_t before = idx[w].size();
+      for (int kb = 0; kb < nkb; ++kb) {
+        bool any = false;
+        for (int q = 0; q < per; ++q) {
+          const long r64 = (long)r * per + q;
+          if (r64 < nrb64 && h[r64 * nkb + kb]) any = true;
+        }
+        if (any) idx[w].push_back(kb);
       }
-      if (any) idx.push_back(kb);
+      if (idx[w].size() == before) idx[w].push_back(0);  // an all-zero block row still writes its zeros
+      off[w][r + 1] = (int)idx[w].size();
     }
-    if (idx.size() == before) idx.push_back(0);  // an all-zero block row still writes its zeros
-    off[r + 1] = (int)idx.size();
-  }
-  if (bl.off != nullptr && (bl.nblocks != nblocks || bl.dense != (long)nblocks * nkb))
-    throw CudaError{cudaErrorInvalidValue, "tc::block_lists: shape changed"};
-  if (bl.off == nullptr) {  // capacity for a dense pattern: later updates rewrite in place
-    bl.nblocks = nblocks;
-    bl.dense = (long)nblocks * nkb;
-    try {
-      mem::alloc(&bl.off, off.size(), st);
-      mem::alloc(&bl.idx, (size_t)bl.dense, st);
-    } catch (...) {
-      free_block_lists(bl, st);
-      throw;
+    if (bl.off != nullptr && (bl.nblocks != nblocks || bl.dense != (long)nblocks * nkb))
+      throw CudaError{cudaErrorInvalidValue, "tc::block_lists: shape changed"};
+    if (bl.off == nullptr) {  // capacity for a dense pattern: later updates rewrite in place
+      bl.nblocks = nblocks;
+      bl.dense = (long)nblocks * nkb;
+      try {
+        mem::alloc(&bl.off, off[w].size(), st);
+        mem::alloc(&bl.idx, (size_t)bl.dense, st);
+      } catch (...) {
+        free_block_lists(bl, st);
+        throw;
+      }
     }
+    bl.nnz = (long)idx[w].size();
+    // the stream was synchronised above, so no earlier launch still reads the old lists; the host
+    // vectors live until the copies are done
+    OMM_CUDA_TRY(cudaMemcpyAsync(bl.off, off[w].data(), off[w].size() * sizeof(int), cudaMemcpyHostToDevice, st));
+    OMM_CUDA_TRY(cudaMemcpyAsync(bl.idx, idx[w].data(), idx[w].size() * sizeof(int), cudaMemcpyHostToDevice, st));
   }
-  bl.nnz = (long)idx.size();
-  // the stream was synchronised above, so no earlier launch still reads the old lists; the host
-  // vectors live until the copies are done
-  OMM_CUDA_TRY(cudaMemcpyAsync(bl.off, off.data(), off.size() * sizeof(int), cudaMemcpyHostToDevice, st));
-  OMM_CUDA_TRY(cudaMemcpyAsync(bl.idx, idx.data(), idx.size() * sizeof(int), cudaMemcpyHostToDevice, st));
   OMM_CUDA_TRY(cudaStreamSynchronize(st));
 }
 
@@ -1585,16 +1591,18 @@ TileShape choose_tile_shape(cudaStream_t st, const std::vector<GemmSpec>& specs,
   if (specs.empty()) return TileShape{};
   // candidates: one SM per 128-row tile, and (split form or single pass) SM pairs; 192-wide pair
   // tiles need K-major B (an SM stages 96 rows) and, for a block-sparse B, lists for that width
-  std::vector<TileShape> cands = {{256, false}, {128, false}};
+  std::vector<TileShape> cands = {{256, false}, {128, false}, {64, false}};
   const bool split = is_split3(pl);
-  bool pair_ok = allow_pair && (split || is_single(pl)), w192 = true, dense = true;
+  bool pair_ok = allow_pair && (split || is_single(pl)), w192 = true, dense = true, w32 = true;
   for (const GemmSpec& g : specs) {
     // (a GEMM of fewer than 256 rows runs on pairs too, its second CTA's rows past M; the timing
     // decides whether that pays)
     if (split && (g.A->slices < 2 || g.B->slices < 2)) pair_ok = false;
     if (g.B->mn_major || (g.sparse[0] != nullptr && g.sparse[2] == nullptr)) w192 = false;
     if (g.sparse[0] != nullptr) dense = false;
+    if (g.B->mn_major || g.sparse[0] != nullptr) w32 = false;
   }
+  if (w32) cands.push_back({32, false});
   if (pair_ok) {
     cands.push_back({256, true});
     cands.push_back({128, true});
@@ -1606,51 +1614,86 @@ TileShape choose_tile_shape(cudaStream_t st, const std::vector<GemmSpec>& specs,
     }
   }
   std::string key = std::to_string(pl.n) + (is_split3(pl) ? "s" : "g") + (pair_ok ? "p" : "");
-  long out_elems = 0;
+  // scratch of each GEMM's redirected outputs: C, xout, the bf16 split, the partial sums
+  auto round16 = [](long b) { return (b + 15) / 16 * 16; };
+  struct Out { long c, x, bf, part; };
+  std::vector<Out> out;
+  long out_bytes = 0;
+  for (const GemmSpec& g : specs) {
+    const Epilogue& e = g.ep;
+    const long blocks = (e.N + e.split_cols - 1) / e.split_cols;
+    // (a negative block stride -- [S_W | H_W] written back to front -- only turns the blocks round)
+    const long c = ((blocks - 1) * std::labs(e.split_stride) + (long)e.M * e.ldc) * (e.c_f32 ? 4 : 8);
+    const long x = e.xout != nullptr ? (long)e.M * e.ldx * 8 : 0;
+    const long bf = e.bf_hi != nullptr ? ((blocks - 1) * e.bf_blk + (long)e.M * e.bf_ld + e.bf_lo) * 2 : 0;
+    const long part = e.mode == kEpReduce ? 4L * 8 * (2 * ((e.M + 255) / 256)) * 2 * ((e.N + 31) / 32 + 8) * 4 : 0;
+    out.push_back(Out{out_bytes, out_bytes + round16(c), out_bytes + round16(c) + round16(x),
+                      out_bytes + round16(c) + round16(x) + round16(bf)});
+    out_bytes = out.back().part + round16(part);
+  }
   for (const GemmSpec& g : specs) {
     key += ":" + std::to_string(g.ep.M) + "x" + std::to_string(g.ep.N) + "x" + std::to_string(g.K);
     if (g.B->mn_major) key += "t";
     if (g.sparse[0]) key += "s" + std::to_string(g.sparse[0]->nnz) + "/" + std::to_string(g.sparse[1]->nnz);
-    out_elems += (long)g.ep.M * g.ep.N;
+    key += "e" + std::to_string(g.ep.mode);
   }
   {
     std::lock_guard<std::mutex> lock(tune_mutex());
     auto it = tune_cache().find(key);
     if (it != tune_cache().end()) return it->second;
   }
-  // time every candidate on the real operands; outputs go to scratch (beta = 0, no skip flags)
-  double* scratch = nullptr;
+  // time every candidate on the real operands and with the real epilogues, which decide between the
+  // shapes of a small product; outputs go to scratch, and no skip flags
+  char* scratch = nullptr;
+  Scalars* sc = nullptr;  // a previous direction exists, as in every line search but a round's first
   int* err = nullptr;
   GroupDesc* dev = nullptr;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   TileShape best{};
   float best_ms = 0.f;
   auto release = [&]() {
-    if (scratch) cudaFree(scratch);
-    if (err) cudaFree(err);
-    if (dev) cudaFree(dev);
+    mem::release(scratch, st);
+    mem::release(sc, st);
+    mem::release(err, st);
+    mem::release(dev, st);
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
   };
   try {
-    OMM_CUDA_TRY(cudaMalloc((void**)&scratch, out_elems * sizeof(double)));
-    OMM_CUDA_TRY(cudaMalloc((void**)&err, sizeof(int)));
-    OMM_CUDA_TRY(cudaMalloc((void**)&dev, specs.size() * sizeof(GroupDesc)));
+    mem::alloc(&scratch, (size_t)out_bytes, st);
+    mem::alloc(&sc, 1, st);
+    mem::alloc(&err, 1, st);
+    mem::alloc(&dev, specs.size(), st);
     OMM_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int), st));
+    Scalars hs;
+    std::memset(&hs, 0, sizeof(hs));
+    hs.have_dir = 1;
+    OMM_CUDA_TRY(cudaMemcpyAsync(sc, &hs, sizeof(hs), cudaMemcpyHostToDevice, st));
     OMM_CUDA_TRY(cudaEventCreate(&e0));
     OMM_CUDA_TRY(cudaEventCreate(&e1));
     float total_ms = 0.f;
     bool first = true;
     for (const TileShape& ts : cands) {
       std::vector<GroupDesc> h;
-      long off = 0;
       int tiles = 0;
-      for (const GemmSpec& g : specs) {
-        Epilogue ep{scratch + off, g.ep.N, g.ep.N, 0, 1.0, 0.0, g.ep.M, g.ep.N, nullptr, err};
+      for (size_t i = 0; i < specs.size(); ++i) {
+        const GemmSpec& g = specs[i];
+        Epilogue ep = g.ep;
+        ep.skip = nullptr;
+        ep.err = err;
+        ep.expire = 0;
+        ep.C = reinterpret_cast<double*>(scratch + out[i].c);
+        if (ep.split_stride < 0)
+          ep.C -= ((ep.N + ep.split_cols - 1) / ep.split_cols - 1) * ep.split_stride;
+        if (ep.xout != nullptr) ep.xout = reinterpret_cast<double*>(scratch + out[i].x);
+        if (ep.bf_hi != nullptr) ep.bf_hi = reinterpret_cast<__nv_bfloat16*>(scratch + out[i].bf);
+        if (ep.mode == kEpReduce) {
+          ep.part = reinterpret_cast<double*>(scratch + out[i].part);
+          ep.sc = sc;
+        }
         h.push_back(make_group(*g.A, *g.B, g.K, ep, tiles, ts.bn, ts.quad ? nullptr : g.sparse[sparse_slot(ts.bn)],
                                ts.pair, ts.quad));
         tiles += tiles_of(ep, ts.bn, ts.pair, ts.quad);
-        off += (long)g.ep.M * g.ep.N;
       }
       OMM_CUDA_TRY(cudaMemcpyAsync(dev, h.data(), h.size() * sizeof(GroupDesc), cudaMemcpyHostToDevice, st));
       gemm_persistent(st, dev, (int)h.size(), tiles, pl, err, ts.bn, ts.pair, ts.quad);  // warm-up

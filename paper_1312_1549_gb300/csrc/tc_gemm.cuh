@@ -117,7 +117,8 @@ void gemm(cudaStream_t st, const Operand& A, const Operand& B, int K, const Pair
 inline void gemm(cudaStream_t st, const Operand& A, const Operand& B, int K, int npass, const Epilogue& ep) {
   gemm(st, A, B, K, npass == 3 ? pairs_split3() : pairs_single(), ep);
 }
-// Output tiles of a persistent launch: 128 x bn on one SM (bn = 128 or 256), or, with pair,
+// Output tiles of a persistent launch: 128 x bn on one SM (bn = 32, 64, 128 or 256; 32 for a K-major B
+// only), or, with pair,
 // 256 x bn on a cluster of two SMs that share the MMA (tcgen05 cta_group::2; bn = 128, 192 or 256;
 // the split form or a single pass).
 // With quad (pair set too), a cluster of two SM pairs side by side along N shares the A operand
@@ -146,12 +147,12 @@ struct BlockLists {
   long nnz = 0;
   long dense = 0;  // nblocks x K blocks
 };
-// (re)computes bl for B (rows x cols float64, leading dimension ld, device) and row blocks of bn;
-// (bn = 128, 192 or 256); the first call allocates room for a dense pattern (from the library's
-// pool, on st), later calls
-// (same shape) rewrite in place so that descriptors holding the pointers stay valid. Synchronises
-// the stream.
-void block_lists(cudaStream_t st, const double* B, long rows, long cols, long ld, int bn, BlockLists& bl);
+// (re)computes lists[k] for B (rows x cols float64, leading dimension ld, device) and row blocks of
+// widths[k] (64, 128, 192 or 256), k < count, from one pass over B; the first call allocates room for a
+// dense pattern (from the library's pool, on st), later calls (same shape) rewrite in place so that
+// descriptors holding the pointers stay valid. Synchronises the stream.
+void block_lists(cudaStream_t st, const double* B, long rows, long cols, long ld, int count, const int* widths,
+                 BlockLists* lists);
 void free_block_lists(BlockLists& bl, cudaStream_t st);  // st: the owner's current stream
 // fraction of the K blocks a product over these lists visits (1 for a dense product)
 inline double block_density(const BlockLists* bl) {
@@ -188,19 +189,20 @@ void gemm_sliced(cudaStream_t st, const Operand& A, const Operand& B, int K, con
 long sliced_workspace_doubles();
 
 // Tile-shape autotuner: times one persistent launch over these GEMMs (the operands as given,
-// the outputs redirected to scratch) with each candidate shape -- 128 x 256 and 128 x 128 on one
-// SM, and (split form or single pass, allow_pair) 256 x 128, 256 x 192 and 256 x 256 on SM pairs,
-// and (dense B) the same on clusters of two pairs sharing A
+// their epilogues with the outputs redirected to scratch) with each candidate shape -- 128 x 256, 128
+// x 128, 128 x 64 and (dense K-major B) 128 x 32 on one SM, and (split form or single pass, allow_pair)
+// 256 x 128, 256 x 192 and 256 x 256 on SM pairs, and (dense B) the same on clusters of two pairs sharing A
 // -- returns the fastest, and remembers it per shape signature for the life of the process.
 // ms_spent receives the time spent timing (0 when the answer came from the cache).
 struct GemmSpec {
   const Operand* A;
   const Operand* B;
   int K;
-  Epilogue ep;                                            // only M and N are used
-  const BlockLists* sparse[3] = {nullptr, nullptr, nullptr};  // block lists of B for bn = 256, 128, 192
+  Epilogue ep;
+  const BlockLists* sparse[4] = {nullptr, nullptr, nullptr, nullptr};  // block lists of B, by sparse_slot(bn)
 };
-inline int sparse_slot(int bn) { return bn == 256 ? 0 : (bn == 128 ? 1 : 2); }
+constexpr int kSparseWidths[4] = {256, 128, 192, 64};
+inline int sparse_slot(int bn) { return bn == 256 ? 0 : (bn == 128 ? 1 : (bn == 192 ? 2 : 3)); }
 TileShape choose_tile_shape(cudaStream_t st, const std::vector<GemmSpec>& specs, const PairList& pl,
                             double* ms_spent = nullptr, bool allow_pair = true);
 
