@@ -228,12 +228,13 @@ __device__ __forceinline__ double to_f64(float v) { return dev::f64_of_f32(v); }
 
 // One CTA: Cholesky factor of the b x b diagonal block at A (b <= 128, read only: the caller
 // does not need L itself), its inverse X = L^-1 into Linv (NL x NL, row-major, zero above the
-// diagonal) and, with Pblk, the block X^T X (both triangles) -- all in float32, for the
+// diagonal) or, with Xhi, as the bf16 pair (Xhi, Xlo) of its b x b elements, and, with Pblk, the block X^T X (both triangles) -- all in float32, for the
 // preconditioner, which needs far less than float64 accuracy. The triangular inverse is blocked so that all threads
 // work: 16 x 16 diagonal blocks are inverted by one warp each, then pairs of inverted blocks are
 // joined level by level, X21 = -X22 (L21 X11).
 __global__ void __launch_bounds__(kLeafThreads)
-leaf_f32_kernel(const double* A, long lda, int b, double* Linv, int* info, int col_offset, double* Pblk, long ldp) {
+leaf_f32_kernel(const double* A, long lda, int b, double* Linv, __nv_bfloat16* Xhi, __nv_bfloat16* Xlo, long ldx,
+                int* info, int col_offset, double* Pblk, long ldp) {
   extern __shared__ float smf[];
   float (*L)[NL + 1] = reinterpret_cast<float (*)[NL + 1]>(smf);
   float (*X)[NL + 1] = reinterpret_cast<float (*)[NL + 1]>(smf + NL * (NL + 1));
@@ -370,7 +371,8 @@ leaf_f32_kernel(const double* A, long lda, int b, double* Linv, int* info, int c
   }
   for (int idx = tid; idx < NL * NL; idx += nt) {
     const int i = idx / NL, j = idx % NL;
-    Linv[idx] = to_f64(X[i][j]);
+    if (Xhi == nullptr) Linv[idx] = to_f64(X[i][j]);
+    else if (i < b && j < b) dev::split_store_f32(X[i][j], Xhi, Xlo, (long)i * ldx + j);
   }
   if (Pblk != nullptr) {
     // (X^T X)_ij = sum_{k >= i} X_ki X_kj for j <= i, mirrored (X is zero above its diagonal, so
@@ -529,7 +531,7 @@ long round8(long x) { return (x + 7) / 8 * 8; }
 // scratch of one stream's products
 struct Lane {
   cudaStream_t st = nullptr;
-  int slices = kInvSlices;   // fixed-point slices of every product on this lane (1: the 3-term bf16 split)
+  int slices = kInvSlices;   // fixed-point slices of every product on this lane
   double* tr0 = nullptr;     // float64 transposes
   double* tr1 = nullptr;
   __nv_bfloat16* sl0 = nullptr;  // slices of two operands
@@ -557,18 +559,6 @@ void sliced_nt(Lane& L, int* err, int M, int N, int K, double alpha, const doubl
                long ldb, double beta, double* C, long ldc) {
   const long ld = round8(K);
   const int s = L.slices;
-  if (s == 1) {  // preconditioner grade from bf16 hi/lo splits: three products, about 2^-16 of |A||B|
-    const tc::Epilogue ep{C, ldc, N, 0, alpha, beta, M, N, nullptr, err};
-    tc::split(L.st, A, M, K, lda, L.sl0, L.sl0 + (long)M * ld, ld, nullptr);
-    const tc::Operand oa = tc::make_operand(L.sl0, M, K, ld, 2, true);
-    if (B == A && ldb == lda && N == M) {
-      emu::gemm_split(L.st, oa, tc::make_operand(L.sl0, N, K, ld, 2, false), K, ep);
-    } else {
-      tc::split(L.st, B, N, K, ldb, L.sl1, L.sl1 + (long)N * ld, ld, nullptr);
-      emu::gemm_split(L.st, oa, tc::make_operand(L.sl1, N, K, ld, 2, false), K, ep);
-    }
-    return;
-  }
   emu::slice_rows(L.st, A, M, K, lda, s, L.sl0, ld, nullptr);
   const tc::Operand oa = tc::make_operand(L.sl0, M, K, ld, s, true);
   tc::Operand ob;
@@ -586,7 +576,8 @@ void leaf(SlicedWork& w, int r0, int b) {
   const long m = w.m;
   double* pb = w.P ? w.P + r0 * m + r0 : nullptr;
   if (w.nb == NL)  // a preconditioner: 128-wide float32 leaves (see leaf_f32_kernel)
-    leaf_f32_kernel<<<1, kLeafThreads, kLeafSmem, w.main.st>>>(w.A + r0 * m + r0, m, b, w.leaf, w.info, r0, pb, m);
+    leaf_f32_kernel<<<1, kLeafThreads, kLeafSmem, w.main.st>>>(w.A + r0 * m + r0, m, b, w.leaf, nullptr, nullptr, 0,
+                                                               w.info, r0, pb, m);
   else
     leaf_f64_kernel<<<1, kLeaf64Threads, 0, w.main.st>>>(w.A + r0 * m + r0, m, b, w.leaf, w.info, r0, pb, m);
   OMM_LAUNCH_CHECK();
@@ -652,6 +643,82 @@ void chol_inv(SlicedWork& w, int r0, int b) {
   p_update(w, r0, b1, b2);
 }
 
+// ------------------------------------------------------------------ preconditioner grade (3-term bf16 split)
+// The same recursion with every operand kept as a bf16 pair in an m x m matrix of its own: A (the part still
+// to be factored), L and Y = L^-1. The products read blocks of these matrices where they stand -- transposed
+// factors as MN-major operands -- and their epilogues write the split of the result beside or instead of
+// the float64 one, so a node of the recursion is four products on the main stream and two on the side
+// stream, with no operand to split, transpose or copy (that was fourteen launches on the main stream, on a
+// chain that runs node after node). Only A and P exist in float64: the leaves and the updates of A read A,
+// P is the result.
+struct SplitInverse {
+  int m = 0;
+  long ld = 0;
+  double* A = nullptr;
+  double* P = nullptr;
+  __nv_bfloat16 *As = nullptr, *Ls = nullptr, *Ys = nullptr;  // [hi; lo], 2m x ld each
+  int* info = nullptr;
+  int* err = nullptr;
+  cudaStream_t st = nullptr, side = nullptr;
+  std::vector<cudaEvent_t> events;
+
+  enum Role { kA, kB };
+  // block (r0, c0) as an operand: rows x cols with cols contracted, or (mn) rows contracted
+  tc::Operand view(const __nv_bfloat16* x, int r0, int c0, int rows, int cols, Role role, bool mn) const {
+    return tc::make_operand_view(x + r0 * ld + c0, m, cols, ld, 2, role == kA, 0, rows, mn, 2L * m - r0);
+  }
+  // the split of an M x N product into block (r0, c0) of x, alpha times it
+  tc::Epilogue into(__nv_bfloat16* x, int r0, int c0, int M, int N, double alpha) const {
+    tc::Epilogue ep{nullptr, 0, N, 0, alpha, 0.0, M, N, nullptr, err};
+    ep.c_f32 = 1;
+    ep.bf_hi = x + r0 * ld + c0;
+    ep.bf_ld = ld;
+    ep.bf_lo = m * ld;
+    return ep;
+  }
+
+  void node(int r0, int b) {
+    if (b <= NL) {
+      __nv_bfloat16* y = Ys + r0 * ld + r0;
+      const long at = (long)r0 * m + r0;
+      leaf_f32_kernel<<<1, kLeafThreads, kLeafSmem, st>>>(A + at, m, b, nullptr, y, y + m * ld, ld, info, r0, P + at, m);
+      OMM_LAUNCH_CHECK();
+      return;
+    }
+    const int b1 = half_of(b, NL), b2 = b - b1, r1 = r0 + b1;
+    node(r0, b1);
+    // L21 = A21 Y11^T
+    emu::gemm_split(st, view(As, r1, r0, b2, b1, kA, false), view(Ys, r0, r0, b1, b1, kB, false), b1,
+                    into(Ls, r1, r0, b2, b1, 1.0));
+    // A22 -= L21 L21^T
+    tc::Epilogue ea = into(As, r1, r1, b2, b2, -1.0);
+    ea.C = A + (long)r1 * m + r1;
+    ea.ldc = m;
+    ea.c_f32 = 0;
+    ea.beta = 1.0;
+    emu::gemm_split(st, view(Ls, r1, r0, b2, b1, kA, false), view(Ls, r1, r0, b2, b1, kB, false), b1, ea);
+    node(r1, b2);
+    // Z = Y22 L21, in the place of A21
+    emu::gemm_split(st, view(Ys, r1, r1, b2, b2, kA, false), view(Ls, r1, r0, b2, b1, kB, true), b2,
+                    into(As, r1, r0, b2, b1, 1.0));
+    // Y21 = -Z Y11
+    emu::gemm_split(st, view(As, r1, r0, b2, b1, kA, false), view(Ys, r0, r0, b1, b1, kB, true), b1,
+                    into(Ys, r1, r0, b2, b1, -1.0));
+    // this node's Y is final: its part of P = Y^T Y, beside the factorisation of the blocks that follow
+    cudaEvent_t ev = nullptr;
+    OMM_CUDA_TRY(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+    events.push_back(ev);
+    OMM_CUDA_TRY(cudaEventRecord(ev, st));
+    OMM_CUDA_TRY(cudaStreamWaitEvent(side, ev, 0));
+    const tc::Operand y21 = view(Ys, r1, r0, b2, b1, kB, true);
+    // P21 = Y22^T Y21; P11 += Y21^T Y21
+    emu::gemm_split(side, view(Ys, r1, r1, b2, b2, kA, true), y21, b2,
+                    tc::Epilogue{P + (long)r1 * m + r0, m, b1, 0, 1.0, 0.0, b2, b1, nullptr, err});
+    emu::gemm_split(side, view(Ys, r1, r0, b2, b1, kA, true), y21, b2,
+                    tc::Epilogue{P + (long)r0 * m + r0, m, b1, 0, 1.0, 1.0, b1, b1, nullptr, err});
+  }
+};
+
 }  // namespace
 
 size_t spd_inverse_sliced_workspace_bytes(int m) {
@@ -660,10 +727,64 @@ size_t spd_inverse_sliced_workspace_bytes(int m) {
   const size_t f64 = (size_t)m * m + (size_t)h * h + (size_t)NL * NL +
                      2 * (2 * (size_t)h * h + (size_t)tc::sliced_workspace_doubles());
   const size_t bf = 2 * 2 * (size_t)kInvSlices * (size_t)h * round8(h);  // per lane: sl0, sl1
+  // (the split form's three pairs of m x m need less: 12 m round8(m) bytes of these 38 m^2 and more)
   return f64 * sizeof(double) + bf * sizeof(__nv_bfloat16) + 4 * 256;
 }
 
 namespace {
+void prepare_leaf() {
+  static const cudaError_t e =  // thread-safe, once
+      cudaFuncSetAttribute(leaf_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kLeafSmem);
+  OMM_CUDA_TRY(e);
+}
+
+// P = A^-1 in the 3-term split form
+void split_impl(cudaStream_t st, int m, double* A, double* P, void* work, int* info_dev, int* err_dev) {
+  SplitInverse w;
+  w.m = m;
+  w.ld = round8(m);
+  w.A = A;
+  w.P = P;
+  w.info = info_dev;
+  w.err = err_dev;
+  w.st = st;
+  const size_t pair = 2 * (size_t)m * w.ld;
+  w.Ys = reinterpret_cast<__nv_bfloat16*>((reinterpret_cast<uintptr_t>(work) + 255) & ~uintptr_t(255));
+  w.Ls = w.Ys + pair;
+  w.As = w.Ls + pair;
+  prepare_leaf();
+  OMM_CUDA_TRY(cudaStreamCreateWithFlags(&w.side, cudaStreamNonBlocking));
+  // streams and events may be released with work pending: the driver frees them once it is done
+  auto cleanup = [&]() {
+    cudaStreamDestroy(w.side);
+    for (cudaEvent_t e : w.events) cudaEventDestroy(e);
+  };
+  try {
+    OMM_CUDA_TRY(cudaMemsetAsync(info_dev, 0, sizeof(int), st));
+    // zeros above the diagonal of Y; and every element a copy may touch past the end of a block (it meets
+    // zeros of the other operand) has to be a number
+    OMM_CUDA_TRY(cudaMemsetAsync(w.Ys, 0, 2 * pair * sizeof(__nv_bfloat16), st));
+    OMM_CUDA_TRY(cudaMemsetAsync(P, 0, sizeof(double) * m * (size_t)m, st));
+    tc::split(st, A, m, m, m, w.As, w.As + m * w.ld, w.ld, nullptr);
+    cudaEvent_t ready = nullptr;  // the side stream starts after the memsets
+    OMM_CUDA_TRY(cudaEventCreateWithFlags(&ready, cudaEventDisableTiming));
+    w.events.push_back(ready);
+    OMM_CUDA_TRY(cudaEventRecord(ready, st));
+    OMM_CUDA_TRY(cudaStreamWaitEvent(w.side, ready, 0));
+    w.node(0, m);
+    cudaEvent_t done = nullptr;  // join: the main stream waits for the last P update
+    OMM_CUDA_TRY(cudaEventCreateWithFlags(&done, cudaEventDisableTiming));
+    w.events.push_back(done);
+    OMM_CUDA_TRY(cudaEventRecord(done, w.side));
+    OMM_CUDA_TRY(cudaStreamWaitEvent(st, done, 0));
+    launch_symmetrize_lower(st, m, P);
+  } catch (...) {
+    cleanup();
+    throw;
+  }
+  cleanup();
+}
+
 // P = A^-1 (P != nullptr) and/or L, Y = L^-1 (Y_out != nullptr: A keeps L, zero above the diagonal)
 void sliced_impl(cudaStream_t st, int m, double* A, double* P, double* Y_out, void* work, int* info_dev,
                  int* err_dev, int slices) {
@@ -698,14 +819,8 @@ void sliced_impl(cudaStream_t st, int m, double* A, double* P, double* Y_out, vo
   w.side.sl0 = w.main.sl1 + sl;
   w.side.sl1 = w.side.sl0 + sl;
   w.main.st = st;
-  w.main.slices = w.side.slices = slices == 1 ? 1 : std::min(std::max(slices, 2), kInvSlices);
-  if (w.nb == NL) {
-    static bool attr = false;
-    if (!attr) {
-      OMM_CUDA_TRY(cudaFuncSetAttribute(leaf_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kLeafSmem));
-      attr = true;
-    }
-  }
+  w.main.slices = w.side.slices = std::min(std::max(slices, 2), kInvSlices);
+  if (w.nb == NL) prepare_leaf();
   if (P) OMM_CUDA_TRY(cudaStreamCreateWithFlags(&w.side.st, cudaStreamNonBlocking));
   // streams and events may be released with work pending: the driver frees them once it is done
   auto cleanup = [&]() {
@@ -747,7 +862,8 @@ void sliced_impl(cudaStream_t st, int m, double* A, double* P, double* Y_out, vo
 
 void spd_inverse_sliced(cudaStream_t st, int m, double* A, double* P, void* work, int* info_dev, int* err_dev,
                         int slices) {
-  sliced_impl(st, m, A, P, nullptr, work, info_dev, err_dev, slices);
+  if (slices == 1) split_impl(st, m, A, P, work, info_dev, err_dev);
+  else sliced_impl(st, m, A, P, nullptr, work, info_dev, err_dev, slices);
 }
 
 void spd_factor_inverse_sliced(cudaStream_t st, int m, double* A, double* Y, void* work, int* info_dev,

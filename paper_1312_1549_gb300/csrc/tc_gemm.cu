@@ -26,6 +26,7 @@
 #include "tc_gemm.cuh"
 
 #include <algorithm>
+#include <cmath>
 #include <cstdlib>
 #include <cstring>
 #include <map>
@@ -144,6 +145,7 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
 }
 // the same with B MN-major (the transpose bit of B)
 constexpr uint32_t kIdescBMN = 1u << 16;
+constexpr uint32_t kIdescAMN = 1u << 15;  // A MN-major
 
 __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
   asm volatile(
@@ -287,9 +289,11 @@ __device__ __forceinline__ void store_block(const Epilogue& ep, uint32_t st, int
       const float al = (float)ep.alpha;
       float* c = reinterpret_cast<float*>(ep.C) + blk * ep.split_stride + row * ldc + cb;
 #pragma unroll
-      for (int k = 0; k < 16; ++k, c += ldc) {
-        a[k] *= al;
-        if (in(k)) *c = a[k];
+      for (int k = 0; k < 16; ++k) a[k] *= al;
+      if (ep.C != nullptr) {
+#pragma unroll
+        for (int k = 0; k < 16; ++k, c += ldc)
+          if (in(k)) *c = a[k];
       }
       if (hp != nullptr) {
         __nv_bfloat16* h = hp + r0 * bf_ld;
@@ -645,8 +649,16 @@ __device__ __forceinline__ void persistent_body(const GroupDesc* __restrict__ gr
         // MN_BOX_BYTES apart
         if (FUSED) {
           const int kb = kbs.at(t);
-          tma_load_2d(sa, mA, full, kb * BK, g->offA + m0);
-          tma_load_2d(sa + A_BYTES, mA, full, kb * BK, g->rowsA + g->offA + m0);
+          if (g->a_mn) {
+#pragma unroll
+            for (int q = 0; q < BM / 64; ++q) {
+              tma_load_2d(sa + q * MN_BOX_BYTES, mA, full, m0 + 64 * q, g->offA + kb * BK);
+              tma_load_2d(sa + A_BYTES + q * MN_BOX_BYTES, mA, full, m0 + 64 * q, g->rowsA + g->offA + kb * BK);
+            }
+          } else {
+            tma_load_2d(sa, mA, full, kb * BK, g->offA + m0);
+            tma_load_2d(sa + A_BYTES, mA, full, kb * BK, g->rowsA + g->offA + m0);
+          }
           if (g->b_mn) {
 #pragma unroll
             for (int q = 0; q < TBN / 64; ++q) {
@@ -685,8 +697,11 @@ __device__ __forceinline__ void persistent_body(const GroupDesc* __restrict__ gr
       const int* skip = g->ep.skip;
       if (skip != nullptr && (skip[0] | skip[1])) continue;
       const int nkb = tile_kblocks(g, tile - g->tile_begin, (g->ep.M + BM - 1) / BM).count;
-      const bool bmn = g->b_mn != 0;
-      const uint32_t idesc = idesc_k | (bmn ? kIdescBMN : 0u);
+      const bool bmn = g->b_mn != 0, amn = FUSED && g->a_mn != 0;
+      const uint32_t idesc = idesc_k | (bmn ? kIdescBMN : 0u) | (amn ? kIdescAMN : 0u);
+      auto adesc = [amn](uint32_t addr, int k) {
+        return amn ? smem_desc_mn(addr + (uint32_t)k * 2048u) : smem_desc(addr + (uint32_t)k * 32u);
+      };
       // the B descriptor of k step k (16 contracted indices) of a stage whose B starts at addr
       auto bdesc = [bmn](uint32_t addr, int k) {
         return bmn ? smem_desc_mn(addr + (uint32_t)k * 2048u) : smem_desc(addr + (uint32_t)k * 32u);
@@ -714,9 +729,9 @@ __device__ __forceinline__ void persistent_body(const GroupDesc* __restrict__ gr
           const uint32_t alo = sa + A_BYTES, bhi = sa + 2 * A_BYTES, blo = bhi + TB_BYTES;
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k) {
-            umma_bf16(d, smem_desc(sa + k * 32), bdesc(bhi, k), idesc, (t > 0 || k > 0) ? 1u : 0u);
-            umma_bf16(d, smem_desc(sa + k * 32), bdesc(blo, k), idesc, 1u);
-            umma_bf16(d, smem_desc(alo + k * 32), bdesc(bhi, k), idesc, 1u);
+            umma_bf16(d, adesc(sa, k), bdesc(bhi, k), idesc, (t > 0 || k > 0) ? 1u : 0u);
+            umma_bf16(d, adesc(sa, k), bdesc(blo, k), idesc, 1u);
+            umma_bf16(d, adesc(alo, k), bdesc(bhi, k), idesc, 1u);
           }
         } else {
           const uint32_t sb = sa + A_BYTES;
@@ -949,7 +964,13 @@ __device__ __forceinline__ void pair_body(const GroupDesc* __restrict__ groups, 
         const uint32_t sa = smem_u32(smem + q * SB);
         const int p = SPLIT ? 0 : t / nkb, kb = kbs.at(SPLIT ? t : t % nkb);
         const int ra = SPLIT ? 0 : (int)pl.a[p] * g->rowsA, rb = SPLIT ? 0 : (int)pl.b[p] * g->rowsB;
-        if (NP == 1) {
+        if (SPLIT && NP == 1 && g->a_mn) {
+#pragma unroll
+          for (int h = 0; h < BM / 64; ++h) {
+            tma_load_2d_pair(sa + h * MN_BOX_BYTES, mA, full, m0 + 64 * h, g->offA + kb * BK);
+            tma_load_2d_pair(sa + A_BYTES + h * MN_BOX_BYTES, mA, full, m0 + 64 * h, g->rowsA + g->offA + kb * BK);
+          }
+        } else if (NP == 1) {
           tma_load_2d_pair(sa, mA, full, kb * BK, ra + g->offA + m0);
           if (SPLIT) tma_load_2d_pair(sa + A_BYTES, mA, full, kb * BK, g->rowsA + g->offA + m0);
         } else {  // this pair's 64-row half of the A tile, to CTA rr of both pairs (64-row boxes)
@@ -992,8 +1013,11 @@ __device__ __forceinline__ void pair_body(const GroupDesc* __restrict__ groups, 
       const int* skip = g->ep.skip;
       if (skip != nullptr && (skip[0] | skip[1])) continue;
       const int nkb = tile_kblocks(g, u - g->tile_begin, (g->ep.M + 2 * BM - 1) / (2 * BM)).count;  // NP > 1: dense
-      const bool bmn = g->b_mn != 0;
-      const uint32_t idesc = idesc_k | (bmn ? kIdescBMN : 0u);
+      const bool bmn = g->b_mn != 0, amn = SPLIT && NP == 1 && g->a_mn != 0;
+      const uint32_t idesc = idesc_k | (bmn ? kIdescBMN : 0u) | (amn ? kIdescAMN : 0u);
+      auto adesc = [amn](uint32_t addr, int k) {
+        return amn ? smem_desc_mn(addr + (uint32_t)k * 2048u) : smem_desc(addr + (uint32_t)k * 32u);
+      };
       auto bdesc = [bmn](uint32_t addr, int k) {
         return bmn ? smem_desc_mn(addr + (uint32_t)k * 2048u) : smem_desc(addr + (uint32_t)k * 32u);
       };
@@ -1019,10 +1043,10 @@ __device__ __forceinline__ void pair_body(const GroupDesc* __restrict__ groups, 
         const uint32_t alo = sa + A_BYTES, bhi = sa + B_OFF, blo = bhi + BH_BYTES;
 #pragma unroll
         for (int k = 0; k < BK / 16; ++k) {
-          umma_bf16_pair(d, smem_desc(sa + k * 32), bdesc(bhi, k), idesc, (t > 0 || k > 0) ? 1u : 0u);
+          umma_bf16_pair(d, adesc(sa, k), bdesc(bhi, k), idesc, (t > 0 || k > 0) ? 1u : 0u);
           if (SPLIT) {
-            umma_bf16_pair(d, smem_desc(sa + k * 32), bdesc(blo, k), idesc, 1u);
-            umma_bf16_pair(d, smem_desc(alo + k * 32), bdesc(bhi, k), idesc, 1u);
+            umma_bf16_pair(d, adesc(sa, k), bdesc(blo, k), idesc, 1u);
+            umma_bf16_pair(d, adesc(alo, k), bdesc(bhi, k), idesc, 1u);
           }
         }
         umma_commit_pair(smem_u32(&bars[NS + q]), mask_all);  // this pair is done with stage q
@@ -1112,10 +1136,11 @@ gemm_persistent_kernel(const GroupDesc* __restrict__ groups, int ngroups, int to
 }
 
 // one split-form GEMM, its descriptor (tensor maps included) in the kernel's parameter space
+template <int TBN>
 __global__ void __launch_bounds__(NTHREADS, 1)
 gemm_persistent_one_kernel(const __grid_constant__ GroupDesc g, int total_tiles, const __grid_constant__ PairList pl,
                            int* err) {
-  persistent_body<true, BN>(&g, 1, total_tiles, pl, err);
+  persistent_body<true, TBN>(&g, 1, total_tiles, pl, err);
 }
 
 #include "sliced_body.cuh"
@@ -1200,23 +1225,25 @@ TensorMap make_map(const __nv_bfloat16* base, long rows, long cols, long ld, int
 }
 
 Operand make_operand_view(const __nv_bfloat16* base, long slice_rows, long cols, long ld, int slices, bool is_a,
-                          int row_off, long rows, bool mn_major) {
-  if (row_off < 0 || rows <= 0 || row_off + rows > slice_rows || (mn_major && is_a))
+                          int row_off, long rows, bool mn_major, long map_rows) {
+  if (map_rows == 0) map_rows = slice_rows * slices;
+  if (row_off < 0 || rows <= 0 || row_off + rows > slice_rows ||
+      (slices - 1) * slice_rows + row_off + rows > map_rows)
     throw CudaError{cudaErrorInvalidValue, "make_operand_view: rows outside the stack"};
   Operand o;
-  // the map covers the whole stack, so every slice and row offset stays inside it
+  // the map covers the stack to its end, so every slice and row offset stays inside it
   if (mn_major) {
     o.box_rows = BK;  // BK contracted rows x 64 output columns per box
-    o.map = make_map(base, slice_rows * slices, cols, ld, BK, 64);
+    o.map = make_map(base, map_rows, cols, ld, BK, 64);
     o.map_n128 = o.map;
   } else {
     o.box_rows = is_a ? BM : BN;
-    o.map = make_map(base, slice_rows * slices, cols, ld, o.box_rows);
-    o.map_n128 = is_a ? o.map : make_map(base, slice_rows * slices, cols, ld, 128);  // 128-wide output tiles
+    o.map = make_map(base, map_rows, cols, ld, o.box_rows);
+    o.map_n128 = is_a ? o.map : make_map(base, map_rows, cols, ld, 128);  // 128-wide output tiles
   }
   o.base = base;
   o.ld = ld;
-  o.map_rows = slice_rows * slices;
+  o.map_rows = map_rows;
   o.rows = rows;
   o.cols = cols;
   o.slices = slices;
@@ -1302,11 +1329,11 @@ GroupDesc make_group(const Operand& A, const Operand& B, int K, const Epilogue& 
     throw CudaError{cudaErrorInvalidValue, "tc::make_group: tile width"};
   // the TMA boxes must match the tile: A in 128-row boxes, B in boxes of the tile width (of half of
   // it on an SM pair), or, MN-major, in 64 x 64 boxes (then the width an SM stages is a multiple of 64)
-  if (A.mn_major || A.box_rows != BM || (!B.mn_major && !pair && bn == 256 && B.box_rows != 256) ||
+  if ((A.mn_major ? quad : A.box_rows != BM) || (!B.mn_major && !pair && bn == 256 && B.box_rows != 256) ||
       (B.mn_major && (pair ? bn / 2 : bn) % 64 != 0))
     throw CudaError{cudaErrorInvalidValue, "tc::make_group: operand boxes do not match the tile"};
-  if (B.mn_major && (sparse != nullptr || K > B.rows))
-    throw CudaError{cudaErrorInvalidValue, "tc::make_group: MN-major B: no block lists, K <= its rows"};
+  if ((B.mn_major && (sparse != nullptr || K > B.rows)) || (A.mn_major && K > A.rows))
+    throw CudaError{cudaErrorInvalidValue, "tc::make_group: MN-major: no block lists, K <= its rows"};
   GroupDesc g{};
   g.a = quad ? make_map(A.base, A.map_rows, A.cols, A.ld, BM / 2) : A.map;  // quad: 64-row halves
   g.quad = quad ? 1 : 0;
@@ -1323,6 +1350,7 @@ GroupDesc make_group(const Operand& A, const Operand& B, int K, const Epilogue& 
   g.rowsB = (int)B.slice_rows;
   g.offA = A.row_off;
   g.offB = B.row_off;
+  g.a_mn = A.mn_major ? 1 : 0;
   g.b_mn = B.mn_major ? 1 : 0;
   g.tile_begin = tile_begin;
   g.bn = bn;
@@ -1336,8 +1364,6 @@ GroupDesc make_group(const Operand& A, const Operand& B, int K, const Epilogue& 
 void prepare_persistent() {
   static bool attr_set = false;
   if (!attr_set) {
-    OMM_CUDA_TRY(cudaFuncSetAttribute(gemm_persistent_one_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      SMEM_BYTES));
     for (const void* f : {(const void*)gemm_persistent_kernel<false, 256>, (const void*)gemm_persistent_kernel<true, 256>,
                           (const void*)gemm_persistent_kernel<false, 128>, (const void*)gemm_persistent_kernel<true, 128>,
                           (const void*)gemm_persistent_kernel<false, 64>, (const void*)gemm_persistent_kernel<true, 64>,
@@ -1345,7 +1371,8 @@ void prepare_persistent() {
                           (const void*)gemm_pair_kernel<128, true>, (const void*)gemm_pair_kernel<192, true>,
                           (const void*)gemm_pair_kernel<256, true>, (const void*)gemm_pair_kernel<128, false>,
                           (const void*)gemm_pair_kernel<192, false>, (const void*)gemm_pair_kernel<256, false>,
-                          (const void*)gemm_pair_one_kernel, (const void*)sliced_pair_kernel,
+                          (const void*)gemm_persistent_one_kernel<256>, (const void*)gemm_persistent_one_kernel<128>,
+                          (const void*)gemm_persistent_one_kernel<64>, (const void*)gemm_pair_one_kernel, (const void*)sliced_pair_kernel,
                           (const void*)sliced_kernel<256>, (const void*)sliced_kernel<128>,
                           (const void*)gemm_quad_kernel<128, true>, (const void*)gemm_quad_kernel<192, true>,
                           (const void*)gemm_quad_kernel<256, true>, (const void*)gemm_quad_kernel<128, false>,
@@ -1406,18 +1433,38 @@ void gemm_split(cudaStream_t st, const Operand& A, const Operand& B, int K, cons
   prepare_persistent();
   const PairList pl = pairs_split3();
   check_pairs(pl, A.slices, B.slices);
-  const int tiles = tiles_of(ep);
-  if (tiles <= 0 || K <= 0) return;
+  if (ep.M <= 0 || ep.N <= 0 || K <= 0) return;
   // a product with at least a wave of 256-row tiles runs on SM pairs (half the B bytes per SM)
   const int pair_units = tiles_of(ep, BN, true);
   if (ep.M >= 2 * BM && pair_units >= pair_clusters()) {
     const GroupDesc gp = make_group(A, B, K, ep, 0, BN, nullptr, true);
     const unsigned pgrid = 2u * (unsigned)std::min(pair_units, pair_clusters());
     gemm_pair_one_kernel<<<pgrid, NTHREADS, SMEM_BYTES, st>>>(gp, pair_units, pl, ep.err);
-  } else {
-    const GroupDesc g = make_group(A, B, K, ep, 0, BN);
-    gemm_persistent_one_kernel<<<(unsigned)std::min(tiles, sm_count()), NTHREADS, SMEM_BYTES, st>>>(g, tiles, pl, ep.err);
+    OMM_LAUNCH_CHECK();
+    return;
   }
+  // else the tile width with the shortest estimated time in SM clocks: rounds of tiles, each a stage per
+  // K block (6 clocks of MMA per column, or 55 bytes of copies per clock) and about 2500 clocks of
+  // epilogue per 32 columns
+  int bn = 256;
+  double best = 0.0;
+  for (int w : {256, 128, 64}) {
+    const double rounds = std::ceil((double)tiles_of(ep, w) / sm_count());
+    const double stage = std::max(6.0 * w, 2.0 * (A_BYTES + w * BK * 2.0) / 55.0);
+    const double t = rounds * (((K + BK - 1) / BK) * stage + std::min(w, (ep.N + 31) / 32 * 32) / 32 * 2500.0);
+    if (best == 0.0 || t < best) {
+      best = t;
+      bn = w;
+    }
+  }
+  const GroupDesc g = make_group(A, B, K, ep, 0, bn);
+  const int tiles = tiles_of(ep, bn);
+  auto go = [&](auto kernel) {
+    kernel<<<(unsigned)std::min(tiles, sm_count()), NTHREADS, SMEM_BYTES, st>>>(g, tiles, pl, ep.err);
+  };
+  if (bn == 256) go(gemm_persistent_one_kernel<256>);
+  else if (bn == 128) go(gemm_persistent_one_kernel<128>);
+  else go(gemm_persistent_one_kernel<64>);
   OMM_LAUNCH_CHECK();
 }
 

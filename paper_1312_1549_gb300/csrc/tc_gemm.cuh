@@ -18,9 +18,10 @@ struct alignas(64) TensorMap {
 // unless the operand is a view of a taller stack) and the operand's own rows
 // start at row_off inside each slice. A split pair x = hi + lo is the 2-slice
 // stack [hi; lo].
-// An MN-major operand (B role only) is stored the other way round: its rows are
-// the contracted index and its columns the output columns (K x N, row-major);
-// it is loaded in 64 x 64 boxes and handed to the MMA as an MN-major matrix.
+// An MN-major operand is stored the other way round: its rows are the contracted
+// index and its columns the output columns (B role, K x N row-major) or the output
+// rows (A role, K x M row-major; split-form products of gemm_split only); it is
+// loaded in 64 x 64 boxes and handed to the MMA as an MN-major matrix.
 struct Operand {
   TensorMap map;       // boxes of 128 rows (A role), 256 rows (B role) or 64 x 64 (MN-major)
   TensorMap map_n128;  // boxes of 128 rows (as a B operand of 128-wide output tiles)
@@ -60,7 +61,8 @@ PairList pairs_single();   // A_0 B_0
 //
 // Fused forms (mode), all with split_cols = N unless stated:
 //   kEpPlain   the above; with c_f32 C is float32 and receives alpha * acc (beta is not used;
-//              split_cols and split_stride apply, in float elements).
+//              split_cols and split_stride apply, in float elements; C may be null, then only the
+//              split is written).
 //   kEpGrad    C = x0 + (xs * x1f + alpha * acc)   (the incremental gradient about a refresh
 //              point: x0 = G_ref (float64), x1f = dHC (float32), xs = 8, alpha = -4; the
 //              increment is formed in float32 with one rounding, then added in float64)
@@ -107,10 +109,11 @@ struct Epilogue {
 // base: 16-byte aligned; ld * 2 bytes a multiple of 16.
 Operand make_operand(const __nv_bfloat16* base, long rows, long cols, long ld, int slices, bool is_a);
 // A view of rows [row_off, row_off + rows) of every slice of a stack whose slices are slice_rows
-// rows apart (a K-major A or B operand, or, with mn_major, an MN-major B operand whose rows are
-// the contracted index).
+// rows apart (K-major, or, with mn_major, an MN-major operand whose rows are the contracted index).
+// map_rows: rows from base to the end of the stack where base is not its first row (a block of a
+// larger matrix); 0: slice_rows * slices.
 Operand make_operand_view(const __nv_bfloat16* base, long slice_rows, long cols, long ld, int slices, bool is_a,
-                          int row_off, long rows, bool mn_major = false);
+                          int row_off, long rows, bool mn_major = false, long map_rows = 0);
 // C = alpha * sum_p A_{pl.a[p]} B_{pl.b[p]}^T + beta * C (FP32 accumulation, float64 epilogue)
 void gemm(cudaStream_t st, const Operand& A, const Operand& B, int K, const PairList& pl, const Epilogue& ep);
 // the npass convention of the split form: 3 -> pairs_split3(), 1 -> pairs_single()
@@ -165,7 +168,7 @@ struct alignas(64) GroupDesc {
   Epilogue ep;
   int K, rowsA, rowsB, tile_begin;  // rowsA, rowsB: rows between the slices of A and B
   int offA, offB;                   // first row of A and B inside each slice
-  int b_mn;                         // B is MN-major (its rows are the contracted index)
+  int a_mn, b_mn;                   // A, B is MN-major (its rows are the contracted index)
   int bn;    // output tile width (all groups of one launch share it, pair and quad)
   int pair;  // 256-row tiles on a cluster of two SMs
   int quad;  // two such pairs per cluster, sharing A
@@ -180,7 +183,8 @@ void prepare_persistent();  // kernel attributes (call before a stream capture)
 // nonzero code if a bounded wait expired
 void gemm_persistent(cudaStream_t st, const GroupDesc* groups_dev, int ngroups, int total_tiles, const PairList& pl,
                      int* err, int bn = 256, bool pair = false, bool quad = false);
-// one split-form GEMM (pairs_split3) whose descriptor travels as a kernel parameter
+// one split-form GEMM (pairs_split3) whose descriptor travels as a kernel parameter; either operand may
+// be MN-major
 void gemm_split(cudaStream_t st, const Operand& A, const Operand& B, int K, const Epilogue& ep);
 // one chunked product C = alpha sum A_i B_j^T + beta C (a plain float64 epilogue, no skip flags), its
 // stages shared evenly among the SMs. slab: sliced_workspace_doubles() doubles, used on st only.
