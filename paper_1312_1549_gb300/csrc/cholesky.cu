@@ -220,7 +220,7 @@ leaf_f64_kernel(double* A, long lda, int b, double* Linv, int* info, int col_off
 // ---- float32 leaves of edge up to 128 for the preconditioner-grade inverse
 constexpr int NL = 128;
 constexpr int kLeafThreads = 512;
-constexpr int kLeafSmem = (3 * NL * (NL + 1) + NL) * (int)sizeof(float);
+constexpr int kLeafSmem = (2 * NL * (NL + 1) + NL) * (int)sizeof(float);
 
 // float64 <-> float32 on the integer pipe, so that the leaf's conversions stay off the narrow float64 units
 __device__ __forceinline__ float to_f32(double x) { return dev::f32_rne_bits(x); }
@@ -228,52 +228,49 @@ __device__ __forceinline__ double to_f64(float v) { return dev::f64_of_f32(v); }
 
 // One CTA: Cholesky factor of the b x b diagonal block at A (b <= 128, read only: the caller
 // does not need L itself), its inverse X = L^-1 into Linv (NL x NL, row-major, zero above the
-// diagonal) or, with Xhi, as the bf16 pair (Xhi, Xlo) of its b x b elements, and, with Pblk, the block X^T X (both triangles) -- all in float32, for the
-// preconditioner, which needs far less than float64 accuracy. The triangular inverse is blocked so that all threads
-// work: 16 x 16 diagonal blocks are inverted by one warp each, then pairs of inverted blocks are
-// joined level by level, X21 = -X22 (L21 X11).
+// diagonal) or, with Xhi, as the bf16 pair (Xhi, Xlo) of its b x b elements, and, with Pblk,
+// the block X^T X (both triangles) -- all in float32, for the preconditioner, which needs far less
+// than float64 accuracy. The layout is leaf_f64_kernel's: panels of eight columns factored in warp
+// 0's registers, rank-8 updates on 8 x 8 blocks, the inverse by joining blocks of edge 8 to 64 with
+// the contraction cut at the triangles. Bound by shared-memory loads and the panels' dependent chain.
+// (With 16-column panels, dense joins and a third shared-memory matrix a leaf took 101 us, now 84.)
 __global__ void __launch_bounds__(kLeafThreads)
 leaf_f32_kernel(const double* A, long lda, int b, double* Linv, __nv_bfloat16* Xhi, __nv_bfloat16* Xlo, long ldx,
                 int* info, int col_offset, double* Pblk, long ldp) {
   extern __shared__ float smf[];
   float (*L)[NL + 1] = reinterpret_cast<float (*)[NL + 1]>(smf);
   float (*X)[NL + 1] = reinterpret_cast<float (*)[NL + 1]>(smf + NL * (NL + 1));
-  float (*T)[NL + 1] = reinterpret_cast<float (*)[NL + 1]>(smf + 2 * NL * (NL + 1));
-  float* rdiag = smf + 3 * NL * (NL + 1);
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int warp = tid >> 5, lane = tid & 31, nwarps = nt >> 5;
-  for (int i = warp; i < NL; i += nwarps)
+  float* rdiag = smf + 2 * NL * (NL + 1);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  constexpr int kWarps = kLeafThreads / 32;
+  static_assert(kWarps == NL / 8, "a warp per diagonal block");
+  for (int i = warp; i < NL; i += kWarps)
     for (int j = lane; j < NL; j += 32) {
       L[i][j] = (i < b && j <= i) ? to_f32(A[(long)i * lda + j]) : 0.f;
       X[i][j] = 0.f;
-      T[i][j] = 0.f;
     }
   __syncthreads();
-  // Right-looking in panels of 16 columns. Warp 0 factors a panel with its rows in registers
-  // (lane l holds rows p0 + l + 32 t), pivots and column entries passed by shuffles, no block
-  // barrier; then all warps apply the panel's rank-16 update to the trailing lower triangle
-  // (warp w on rows q0 + w, q0 + w + 16, ..., lanes on columns), each element's 16 products
-  // from independent shared-memory loads. Two barriers per panel instead of one per column: a
-  // column at a time left every warp waiting on a chain of dependent shared-memory loads.
-  for (int p0 = 0; p0 < b; p0 += 16) {
-    const int pw = min(16, b - p0);
-    if (warp == 0) {
-      float r[4][16];
+  for (int p0 = 0; p0 < b; p0 += 8) {
+    const int pw = min(8, b - p0);
+    if (warp == 0) {  // lane l holds rows p0 + l + 32 t
+      float r[4][8];
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
         const int i = p0 + lane + 32 * t;
 #pragma unroll
-        for (int c = 0; c < 16; ++c) r[t][c] = (i < b && c < pw && p0 + c <= i) ? L[i][p0 + c] : 0.f;
+        for (int c = 0; c < 8; ++c) r[t][c] = (i < b && c < pw && p0 + c <= i) ? L[i][p0 + c] : 0.f;
       }
 #pragma unroll
-      for (int c = 0; c < 16; ++c) {
+      for (int c = 0; c < 8; ++c) {
         if (c < pw) {
           float d = __shfl_sync(0xffffffffu, r[0][c], c);  // the pivot, row p0 + c
           if (!(d > 0.f)) {
             if (lane == 0) atomicCAS(info, 0, col_offset + p0 + c + 1);
             d = 1.f;
           }
-          const float sq = sqrtf(d), rs = 1.f / sq;
+          float rs = rsqrtf(d);
+          if (rs > 0.f) rs = fmaf(0.5f * rs, fmaf(-(d * rs), rs, 1.f), rs);  // (0 only for an infinite pivot)
+          const float sq = sqrtf(d);
 #pragma unroll
           for (int t = 0; t < 4; ++t) {
             const int i = p0 + lane + 32 * t;
@@ -282,12 +279,12 @@ leaf_f32_kernel(const double* A, long lda, int b, double* Linv, __nv_bfloat16* X
           }
           if (lane == 0) rdiag[p0 + c] = rs;
 #pragma unroll
-          for (int l = 0; l < 16; ++l) {
+          for (int l = 0; l < 8; ++l) {
             if (l > c) {
-              const float lc = __shfl_sync(0xffffffffu, r[0][c], l);  // L[p0 + l][p0 + c], scaled
+              const float lc = __shfl_sync(0xffffffffu, r[0][c], l);  // L[p0 + l][p0 + c]
+              if (lane >= l) r[0][l] = fmaf(-r[0][c], lc, r[0][l]);
 #pragma unroll
-              for (int t = 0; t < 4; ++t)
-                if (lane + 32 * t >= l) r[t][l] = fmaf(-r[t][c], lc, r[t][l]);
+              for (int t = 1; t < 4; ++t) r[t][l] = fmaf(-r[t][c], lc, r[t][l]);
             }
           }
         }
@@ -296,127 +293,121 @@ leaf_f32_kernel(const double* A, long lda, int b, double* Linv, __nv_bfloat16* X
       for (int t = 0; t < 4; ++t) {
         const int i = p0 + lane + 32 * t;
 #pragma unroll
-        for (int c = 0; c < 16; ++c)
+        for (int c = 0; c < 8; ++c)
           if (i < b && c < pw && p0 + c <= i) L[i][p0 + c] = r[t][c];
       }
     }
     __syncthreads();
-    const int q0 = p0 + pw;  // trailing block: rows and columns q0 .. b - 1 (empty after the last panel)
-    for (int i = q0 + warp; i < b; i += nwarps) {
-      float li[16];
+    // trailing lower triangle in 8 x 8 blocks (I, J <= I), a warp per block, two rows per lane
+    const int q0 = p0 + 8, nb8 = (b - q0 + 7) / 8;
+    for (int q = warp, I = 0, base = 0; I < nb8;) {
+      if (q >= base + I + 1) {
+        base += I + 1;
+        ++I;
+        continue;
+      }
+      const int i = q0 + 8 * I + (lane >> 3), j = q0 + 8 * (q - base) + (lane & 7);
+      float a0 = L[i][j], a1 = L[i + 4][j];  // (rows and columns past b hold zeros)
 #pragma unroll
-      for (int k = 0; k < 16; ++k) li[k] = L[i][p0 + k];
-      for (int l = q0 + lane; l <= i; l += 32) {
-        float acc = L[i][l];
+      for (int k = 0; k < 8; ++k) {
+        const float lj = L[j][p0 + k];
+        a0 = fmaf(-L[i][p0 + k], lj, a0);
+        a1 = fmaf(-L[i + 4][p0 + k], lj, a1);
+      }
+      if (j <= i) L[i][j] = a0;
+      if (j <= i + 4) L[i + 4][j] = a1;
+      q += kWarps;
+    }
+    __syncthreads();
+  }
+  // inverses of the 8 x 8 diagonal blocks: warp w's lane c solves column c of block w
+  if (8 * warp < b && lane < 8 && 8 * warp + lane < b) {
+    const int o = 8 * warp, c = lane, e = min(8, b - o);
+    float x[8];
 #pragma unroll
-        for (int k = 0; k < 16; ++k) acc = fmaf(-li[k], L[l][p0 + k], acc);
-        L[i][l] = acc;
+    for (int i = 0; i < 8; ++i) {
+      x[i] = 0.f;
+      if (i == c) x[i] = rdiag[o + i];
+      if (i > c && i < e) {
+        float acc = 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          if (k >= c && k < i) acc = fmaf(L[o + i][o + k], x[k], acc);
+        x[i] = -acc * rdiag[o + i];
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (i >= c && i < e) X[o + i][o + c] = x[i];
+  }
+  __syncthreads();
+  // Join blocks of edge s (see leaf_f64_kernel): T = L21 X11, kept transposed in the upper triangle of L,
+  // then X21 = -X22 T; every warp has one unit of four rows (columns) of one pair
+  for (int s = 8; s < b; s *= 2) {
+    const int wpp = s / 4;  // warps per pair
+    const int o = 2 * s * (warp / wpp), f = 4 * (warp % wpp) + (lane >> 3);
+    if (o < b) {
+      const int i = f;
+      for (int g = 0; g < s; g += 8) {
+        const int j = g + (lane & 7);
+        float acc0 = 0.f, acc1 = 0.f;
+#pragma unroll 4
+        for (int k = g; k < s; k += 2) {
+          acc0 = fmaf(L[o + s + i][o + k], X[o + k][o + j], acc0);
+          acc1 = fmaf(L[o + s + i][o + k + 1], X[o + k + 1][o + j], acc1);
+        }
+        L[o + j][o + s + i] = acc0 + acc1;
+      }
+    }
+    __syncthreads();
+    if (o < b) {
+      const int j = f;
+      for (int g = 0; g < s; g += 8) {
+        const int i = g + (lane & 7);
+        float acc0 = 0.f, acc1 = 0.f;
+#pragma unroll 4
+        for (int k = 0; k < g + 8; k += 2) {
+          acc0 = fmaf(X[o + s + i][o + s + k], L[o + j][o + s + k], acc0);
+          acc1 = fmaf(X[o + s + i][o + s + k + 1], L[o + j][o + s + k + 1], acc1);
+        }
+        if (o + s + i < b) X[o + s + i][o + j] = -(acc0 + acc1);
       }
     }
     __syncthreads();
   }
-  // 16 x 16 diagonal blocks: lane c of warp w solves column c of block w
-  const int nb16 = (b + 15) / 16;
-  if (warp < nb16 && lane < 16) {
-    const int o = warp * 16, e = min(16, b - o), c = lane;
-    if (c < e) {
-      X[o + c][o + c] = rdiag[o + c];
-      for (int i = c + 1; i < e; ++i) {
-        float acc = 0.f;
-        for (int k = c; k < i; ++k) acc = fmaf(L[o + i][o + k], X[o + k][o + c], acc);
-        X[o + i][o + c] = -acc * rdiag[o + i];
-      }
-    }
-  }
-  __syncthreads();
-  // Join blocks of edge s into blocks of edge 2s: T = L21 X11, then X21 = -X22 T, each a dense
-  // s x s x s product over the pair's blocks (the zeros above the diagonals of X11 and X22, and the
-  // zero rows of L, X and T at and beyond b, make the full sums exact). Warp w takes a group of four
-  // rows, its lanes the columns j = lane + 32 q, four products per loaded column entry.
-  for (int s = 16; s < b; s *= 2) {
-    const int pairs = (b + 2 * s - 1) / (2 * s);
-    const int gps = s / 4, ngroups = pairs * gps, nq = (s + 31) / 32;
-    for (int pass = 0; pass < 2; ++pass) {  // 0: T = L21 X11; 1: X21 = -X22 T
-      for (int g = warp; g < ngroups; g += nwarps) {
-        const int o = 2 * s * (g / gps), r0 = o + s + (g % gps) * 4;
-        float acc[4][2] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-        for (int k = 0; k < s; ++k) {
-          float a[4];
-#pragma unroll
-          for (int r = 0; r < 4; ++r) a[r] = pass == 0 ? L[r0 + r][o + k] : X[r0 + r][o + s + k];
-#pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            const int j = lane + 32 * q;
-            if (q < nq && j < s) {
-              const float bv = pass == 0 ? X[o + k][o + j] : T[o + s + k][o + j];
-#pragma unroll
-              for (int r = 0; r < 4; ++r) acc[r][q] = fmaf(a[r], bv, acc[r][q]);
-            }
-          }
-        }
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-#pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            const int j = lane + 32 * q;
-            if (q < nq && j < s && r0 + r < b) {
-              if (pass == 0) T[r0 + r][o + j] = acc[r][q];
-              else X[r0 + r][o + j] = -acc[r][q];
-            }
-          }
-        }
-      }
-      __syncthreads();
-    }
-  }
-  for (int idx = tid; idx < NL * NL; idx += nt) {
+  for (int idx = tid; idx < NL * NL; idx += kLeafThreads) {
     const int i = idx / NL, j = idx % NL;
     if (Xhi == nullptr) Linv[idx] = to_f64(X[i][j]);
     else if (i < b && j < b) dev::split_store_f32(X[i][j], Xhi, Xlo, (long)i * ldx + j);
   }
   if (Pblk != nullptr) {
-    // (X^T X)_ij = sum_{k >= i} X_ki X_kj for j <= i, mirrored (X is zero above its diagonal, so
-    // a sum may start below i). Warp w takes the row groups 4g .. 4g + 3 for g = w and g = 31 - w
-    // (long and short k ranges paired), its lanes the columns j = lane + 32 q; per k it loads the
-    // group's four entries of row k (broadcast) and its own columns, for up to 16 products: a
-    // quarter of the shared-memory loads per product of one row at a time.
-    static_assert(kLeafThreads == 512 && NL == 128, "32 row groups over 16 warps");
-#pragma unroll 1
-    for (int h = 0; h < 2; ++h) {
-      const int i0 = 4 * (h == 0 ? warp : NL / 4 - 1 - warp);
-      if (i0 >= b) continue;
-      const int nq = min(i0 + 3, b - 1) / 32 + 1;
-      float acc[4][NL / 32];
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int q = 0; q < NL / 32; ++q) acc[r][q] = 0.f;
-      for (int k = i0; k < b; ++k) {
-        float xi[4];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) xi[r] = X[k][i0 + r];
-#pragma unroll
-        for (int q = 0; q < NL / 32; ++q) {
-          if (q < nq) {
-            const float xj = X[k][lane + 32 * q];
-#pragma unroll
-            for (int r = 0; r < 4; ++r) acc[r][q] = fmaf(xi[r], xj, acc[r][q]);
-          }
-        }
+    // (X^T X)_ij = sum_{k >= i} X_ki X_kj for j <= i, mirrored: 8 x 8 blocks (I, J <= I), two rows per lane
+    const int nb8 = (b + 7) / 8;
+    for (int q = warp, I = 0, base = 0; I < nb8;) {
+      if (q >= base + I + 1) {
+        base += I + 1;
+        ++I;
+        continue;
       }
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int i = i0 + r;
-#pragma unroll
-        for (int q = 0; q < NL / 32; ++q) {
-          const int jj = lane + 32 * q;
-          if (i < b && q < nq && jj <= i) {
-            const double v = to_f64(acc[r][q]);
-            Pblk[(long)i * ldp + jj] = v;
-            Pblk[(long)jj * ldp + i] = v;
-          }
-        }
+      const int i = 8 * I + (lane >> 3), j = 8 * (q - base) + (lane & 7);
+      float a0 = 0.f, a1 = 0.f;
+#pragma unroll 4
+      for (int k = 8 * I; k < b; ++k) {  // (X is zero above its diagonal)
+        const float xj = X[k][j];
+        a0 = fmaf(X[k][i], xj, a0);
+        a1 = fmaf(X[k][i + 4], xj, a1);
       }
+      if (i < b && j <= i) {
+        const double v = to_f64(a0);
+        Pblk[(long)i * ldp + j] = v;
+        Pblk[(long)j * ldp + i] = v;
+      }
+      if (i + 4 < b && j <= i + 4) {
+        const double v = to_f64(a1);
+        Pblk[(long)(i + 4) * ldp + j] = v;
+        Pblk[(long)j * ldp + i + 4] = v;
+      }
+      q += kWarps;
     }
   }
 }
