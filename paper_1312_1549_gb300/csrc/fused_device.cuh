@@ -263,7 +263,7 @@ __device__ __forceinline__ void reduce_unpreconditioned_body(long n, long m, con
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, o));
-  __shared__ double sh[3][TB / 32];
+  __shared__ SumScratch<3> sh;
   __shared__ double shm[TB / 32];
   if ((threadIdx.x & 31) == 0) shm[threadIdx.x >> 5] = __longlong_as_double((long long)mb);
   block_sum<3>(v, sh);
@@ -284,11 +284,12 @@ __device__ __forceinline__ void update_subspace_split_body(int n, double* SWHW, 
                                                            const double* __restrict__ Wref,
                                                            __nv_bfloat16* __restrict__ Whi,
                                                            __nv_bfloat16* __restrict__ Wlo, long ldw,
-                                                           const Scalars* sc, int bx_, int nbx_) {
+                                                           const Scalars* sc, int bx_, int nbx_, int quarters = 1) {
   if (stopped(sc)) return;
   const double x = sc->x, x2 = x * x;
   const int tiles = (n + 31) / 32;
-  const int I = bx_ / tiles, J = bx_ % tiles;
+  const int tile = bx_ / quarters, r_first = (bx_ % quarters) * 8, r_last = quarters == 1 ? 32 : r_first + 8;
+  const int I = tile / tiles, J = tile % tiles;
   __shared__ double tH1[32][33], tS1[32][33];
   const long l2 = 2L * n, l4 = 4L * n;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -299,7 +300,7 @@ __device__ __forceinline__ void update_subspace_split_body(int n, double* SWHW, 
     tS1[r][tx] = ok ? Proj[(long)gi * l4 + n + gj] : 0.0;
   }
   __syncthreads();
-  for (int r = ty; r < 32; r += 8) {
+  for (int r = r_first + ty; r < r_last; r += 8) {
     const int gi = I * 32 + r, gj = J * 32 + tx;
     if (gi >= n || gj >= n) continue;
     const double* pr = Proj + (long)gi * l4;

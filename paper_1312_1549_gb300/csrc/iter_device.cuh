@@ -25,22 +25,41 @@ __device__ __forceinline__ double warp_max(double v) {
   }
   return v;
 }
+// Sums of N values over the TB threads; the results are in thread 0 (in v). A float64 add takes its warp
+// about 30 clocks of the SM's float64 unit however many lanes are active, so the N sums lie side by side in
+// the lanes: thread (seg, q) adds the q-th values of TB / kSegs threads, then thread q the kSegs partial sums
+// (N (TB / 32 + 2) / 2 adds or so; a shuffle tree per value and warp took 5 N per warp, 13 thousand clocks
+// for the eleven traces). sh: N x (TB + 1) doubles. Fixed order.
 template <int N>
-__device__ __forceinline__ void block_sum(double (&v)[N], double (*sh)[TB / 32]) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+struct SumScratch {
+  double v[N][TB + 1];
+  double seg[16][N];
+};
+template <int N>
+__device__ __forceinline__ void block_sum(double (&v)[N], SumScratch<N>& sh) {
+  static_assert(N <= 16 && TB == 256, "sixteen segments of sixteen threads' values");
 #pragma unroll
-  for (int q = 0; q < N; ++q) {
-    const double w = warp_sum(v[q]);
-    if (lane == 0) sh[q][wid] = w;
+  for (int q = 0; q < N; ++q) sh.v[q][threadIdx.x] = v[q];
+  __syncthreads();
+  if (threadIdx.x < 16 * N) {
+    const int q = threadIdx.x / 16, seg = threadIdx.x % 16;
+    double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+    for (int k = 0; k < 16; k += 2) {
+      s0 += sh.v[q][seg + 16 * k];
+      s1 += sh.v[q][seg + 16 * (k + 1)];
+    }
+    sh.seg[seg][q] = s0 + s1;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (threadIdx.x < 32) {
+    double s = 0.0;
+    if (threadIdx.x < N) {
 #pragma unroll
-    for (int q = 0; q < N; ++q) {
-      double s = 0.0;
-      for (int k = 0; k < TB / 32; ++k) s += sh[q][k];
-      v[q] = s;
+      for (int k = 0; k < 16; ++k) s += sh.seg[k][threadIdx.x];
     }
+#pragma unroll
+    for (int q = 0; q < N; ++q) v[q] = __shfl_sync(0xffffffffu, s, q);
   }
   __syncthreads();
 }
@@ -77,6 +96,40 @@ __host__ __device__ inline double rtsafe(const double* a, double lo, double hi) 
     if (f < 0.0) lo = x; else hi = x;
   }
   return x;
+}
+// The same root, found in float32 first on p'(hi t) / |p'(0)| (coefficients of order one in the bracket) and
+// finished by Newton steps in float64: two or three evaluations with a division each on the GPU's float64
+// unit, whose dependent operations take some 40 clocks, instead of eight. Falls back to rtsafe when a step
+// leaves the bracket or does not settle.
+__host__ __device__ inline double bracketed_root(const double* a, double lo, double hi) {
+  const double s = 1.0 / fabs(a[1]), w = hi;
+  const float c1 = a[1] < 0.0 ? -1.0f : 1.0f, c2 = (float)(2.0 * a[2] * w * s), c3 = (float)(3.0 * a[3] * w * w * s),
+              c4 = (float)(4.0 * a[4] * w * w * w * s);
+  float tl = (float)(lo / hi), th = 1.0f, t = 0.5f * (tl + th);
+  for (int it = 0; it < 40; ++it) {
+    const float f = c1 + t * (c2 + t * (c3 + t * c4));
+    const float df = c2 + t * (2.0f * c3 + t * 3.0f * c4);
+    if (f < 0.0f) tl = t; else th = t;
+    float tn = t - f / df;
+    if (!(tn > tl && tn < th)) tn = 0.5f * (tl + th);
+    const float d = fabsf(tn - t);
+    t = tn;
+    if (d <= 1e-6f * fabsf(t)) break;
+  }
+  double x = w * (double)t;
+  for (int it = 0; it < 6; ++it) {
+    const double f = qd1(a, x), df = qd2(a, x), dx = f / df;
+    x -= dx;
+    if (!(x >= lo && x <= hi)) break;
+    if (fabs(dx) <= 8.9e-16 * fabs(x)) return x;
+    if (fabs(dx) <= 1e-9 * fabs(x)) {  // quadratic: the next step is below the last place's rounding
+      const double f2 = qd1(a, x) / qd2(a, x);
+      x -= f2;
+      if (x >= lo && x <= hi && fabs(f2) <= 1e-13 * fabs(x)) return x;
+      break;
+    }
+  }
+  return rtsafe(a, lo, hi);
 }
 // First local minimum of a0 + a1 x + ... + a4 x^4 along x > 0 (a1 < 0):
 // the positive axis is cut at the real roots of p'' (where p' turns), p' is
@@ -123,7 +176,7 @@ __host__ __device__ inline int quartic_first_minimum(const double a[5], double* 
         if (++guard > 2000 || !isfinite(hi)) return 3;
       }
     }
-    *x_out = rtsafe(a, lo, hi);
+    *x_out = bracketed_root(a, lo, hi);
     return 0;
   }
   return 3;
@@ -149,7 +202,7 @@ __device__ __forceinline__ void grad_reduce_body(long count, const double* __res
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, o));
-  __shared__ double sh[3][TB / 32];
+  __shared__ SumScratch<3> sh;
   __shared__ double shm[TB / 32];
   const double wm = __longlong_as_double((long long)mb);
   if ((threadIdx.x & 31) == 0) shm[threadIdx.x >> 5] = wm;
@@ -166,22 +219,24 @@ __device__ __forceinline__ void grad_reduce_body(long count, const double* __res
 __device__ __forceinline__ void control_direction_body(Scalars* sc, const double* part, int mixed, int nparts, int bx_, int nbx_) {
   if (stopped(sc)) return;
   double v[3] = {0.0, 0.0, 0.0};
-  double mx = 0.0;
+  // max|G| on the bit patterns (non-negative values or NaNs, which order above every number)
+  unsigned long long mb = 0;
   for (int b = threadIdx.x; b < nparts; b += TB) {
     v[0] += part[b * 4 + 0];
     v[1] += part[b * 4 + 1];
     v[2] += part[b * 4 + 2];
-    const double a = part[b * 4 + 3];
-    mx = (a > mx || a != a) ? a : mx;
+    mb = max(mb, (unsigned long long)__double_as_longlong(part[b * 4 + 3]) & 0x7FFFFFFFFFFFFFFFull);
   }
-  __shared__ double sh[3][TB / 32];
-  __shared__ double shm[TB / 32];
-  const double wm = warp_max(mx);
-  if ((threadIdx.x & 31) == 0) shm[threadIdx.x >> 5] = wm;
+  __shared__ SumScratch<3> sh;
+  __shared__ unsigned long long shm[TB / 32];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, o));
+  if ((threadIdx.x & 31) == 0) shm[threadIdx.x >> 5] = mb;
   block_sum<3>(v, sh);
   if (threadIdx.x != 0) return;
-  double gmax = 0.0;
-  for (int k = 0; k < TB / 32; ++k) gmax = (shm[k] > gmax || shm[k] != shm[k]) ? shm[k] : gmax;
+#pragma unroll
+  for (int k = 0; k < TB / 32; ++k) mb = max(mb, shm[k]);
+  const double gmax = __longlong_as_double((long long)mb);
   const double gpg = v[0], gopg = v[1], gdo = v[2];
   sc->gmax = gmax;
   sc->gpg = gpg;
@@ -257,9 +312,10 @@ __device__ __forceinline__ float f32_trunc(double x) {
 // pipe) and sum each thread's products (four per tile) in float32 before the float64 block sums:
 // about 2^-20 of each term, far below the error of the tensor-core projections they come from
 // (mixed path).
+// quarters = 4: a unit is eight rows of a tile (for small n, so that more SMs share the float64 work).
 template <bool F32>
 __device__ __forceinline__ void traces_body(int n, const double* __restrict__ SWHW, const double* __restrict__ Proj,
-              double* part, const Scalars* sc, int bx_, int nbx_) {
+              double* part, const Scalars* sc, int bx_, int nbx_, int quarters = 1) {
   if (stopped(sc)) return;
   const int tiles = (n + 31) / 32;
   __shared__ double tHW[32][33], tH1[32][33], tH2[32][33];
@@ -273,7 +329,8 @@ __device__ __forceinline__ void traces_body(int n, const double* __restrict__ SW
   for (int q = 0; q < kNumTraces; ++q) f[q] = 0.0f;
   // 32 x 32 tiles bx_, bx_ + nbx_, ... of the n x n blocks (one per block of the batched launch,
   // several per block of the single launch, whose partial sums then number fewer)
-  for (int tile = bx_; tile < tiles * tiles; tile += nbx_) {
+  for (int unit = bx_; unit < tiles * tiles * quarters; unit += nbx_) {
+    const int tile = unit / quarters, r_first = (unit % quarters) * 8, r_last = quarters == 1 ? 32 : r_first + 8;
     const int I = tile / tiles, J = tile % tiles;
     __syncthreads();  // the previous tile's staged transposes have been read
     // load Y^T tiles: element (i, j) of tile (I, J) needs Y[j][i] from tile (J, I)
@@ -285,7 +342,7 @@ __device__ __forceinline__ void traces_body(int n, const double* __restrict__ SW
       tH2[r][tx] = ok ? Proj[(long)gi * l4 + 2L * n + gj] : 0.0;
     }
     __syncthreads();
-    for (int r = ty; r < 32; r += 8) {
+    for (int r = r_first + ty; r < r_last; r += 8) {
       const int gi = I * 32 + r, gj = J * 32 + tx;
       if (gi >= n || gj >= n) continue;
       const double sw = SWHW[(long)gi * l2 + gj];
@@ -323,8 +380,8 @@ __device__ __forceinline__ void traces_body(int n, const double* __restrict__ SW
       }
     }
   }
-  __shared__ double sh[kNumTraces][TB / 32];
-  if (F32) {
+  if constexpr (F32) {
+    __shared__ double sh[kNumTraces][TB / 32];
     // warp sums in float32 (shuffles on the float32 units), one float64 value per warp; the
     // diagonal traces t0, t3 stay float64 throughout
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -346,12 +403,13 @@ __device__ __forceinline__ void traces_body(int n, const double* __restrict__ SW
       for (int k = 0; k < TB / 32; ++k) acc += sh[threadIdx.x][k];
       part[(long)bx_ * kNumTraces + threadIdx.x] = acc;
     }
-    return;
-  }
-  block_sum<kNumTraces>(t, sh);
-  if (threadIdx.x == 0) {
+  } else {
+    __shared__ SumScratch<kNumTraces> sh;
+    block_sum<kNumTraces>(t, sh);
+    if (threadIdx.x == 0) {
 #pragma unroll
-    for (int q = 0; q < kNumTraces; ++q) part[(long)bx_ * kNumTraces + q] = t[q];
+      for (int q = 0; q < kNumTraces; ++q) part[(long)bx_ * kNumTraces + q] = t[q];
+    }
   }
 }
 __device__ __forceinline__ void control_linesearch_body(Scalars* sc, const double* part, int nblocks, int bx_, int nbx_) {
@@ -418,11 +476,12 @@ __device__ __forceinline__ void control_linesearch_body(Scalars* sc, const doubl
   sc->iter_round += 1;
   sc->have_dir = 1;
 }
-__device__ __forceinline__ void update_subspace_body(int n, double* SWHW, const double* __restrict__ Proj, const Scalars* sc, int bx_, int nbx_) {
+__device__ __forceinline__ void update_subspace_body(int n, double* SWHW, const double* __restrict__ Proj, const Scalars* sc, int bx_, int nbx_, int quarters = 1) {
   if (stopped(sc)) return;
   const double x = sc->x, x2 = x * x;
   const int tiles = (n + 31) / 32;
-  const int I = bx_ / tiles, J = bx_ % tiles;
+  const int tile = bx_ / quarters, r_first = (bx_ % quarters) * 8, r_last = quarters == 1 ? 32 : r_first + 8;
+  const int I = tile / tiles, J = tile % tiles;
   __shared__ double tH1[32][33], tS1[32][33];
   const long l2 = 2L * n, l4 = 4L * n;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -433,7 +492,7 @@ __device__ __forceinline__ void update_subspace_body(int n, double* SWHW, const 
     tS1[r][tx] = ok ? Proj[(long)gi * l4 + n + gj] : 0.0;
   }
   __syncthreads();
-  for (int r = ty; r < 32; r += 8) {
+  for (int r = r_first + ty; r < r_last; r += 8) {
     const int gi = I * 32 + r, gj = J * 32 + tx;
     if (gi >= n || gj >= n) continue;
     const double* pr = Proj + (long)gi * l4;

@@ -6,6 +6,8 @@
 // Reductions use fixed grids and fixed summation orders: results are bitwise
 // reproducible from run to run.
 #include "omm_internal.cuh"
+
+#include <algorithm>
 #include "iter_device.cuh"
 #include "fused_device.cuh"
 
@@ -71,8 +73,8 @@ __global__ void direction_kernel(long count, const double* __restrict__ PG, doub
 template <bool F32>
 __global__ void __launch_bounds__(TB)
 traces_kernel(int n, const double* __restrict__ SWHW, const double* __restrict__ Proj,
-              double* part, const Scalars* sc) {
-  traces_body<F32>(n, SWHW, Proj, part, sc, blockIdx.x, gridDim.x);
+              double* part, const Scalars* sc, int quarters) {
+  traces_body<F32>(n, SWHW, Proj, part, sc, blockIdx.x, gridDim.x, quarters);
 }
 
 
@@ -122,8 +124,8 @@ __global__ void update_state_kernel(int n, long m, double* C, double* Y4, const 
 
 // H_W += x (H' + H'^T) + x^2 H''; S_W likewise (Eq. 16), on 32x32 tiles
 __global__ void __launch_bounds__(TB)
-update_subspace_kernel(int n, double* SWHW, const double* __restrict__ Proj, const Scalars* sc) {
-  update_subspace_body(n, SWHW, Proj, sc, blockIdx.x, gridDim.x);
+update_subspace_kernel(int n, double* SWHW, const double* __restrict__ Proj, const Scalars* sc, int quarters) {
+  update_subspace_body(n, SWHW, Proj, sc, blockIdx.x, gridDim.x, quarters);
 }
 
 
@@ -152,7 +154,7 @@ functional_kernel(int n, const double* __restrict__ SWHW, double* part) {
     if (gi == gj) v[0] += SWHW[(long)gi * l2 + n + gj];
     v[1] = fma(SWHW[(long)gi * l2 + gj], tHW[tx][r], v[1]);
   }
-  __shared__ double sh[2][TB / 32];
+  __shared__ SumScratch<2> sh;
   block_sum<2>(v, sh);
   if (threadIdx.x == 0) {
     part[blockIdx.x * 2 + 0] = v[0];
@@ -167,7 +169,7 @@ finish_functional_kernel(Scalars* sc, const double* part, int nblocks) {
     v[0] += part[b * 2 + 0];
     v[1] += part[b * 2 + 1];
   }
-  __shared__ double sh[2][TB / 32];
+  __shared__ SumScratch<2> sh;
   block_sum<2>(v, sh);
   if (threadIdx.x == 0) sc->E = 4.0 * v[0] - 2.0 * v[1];
 }
@@ -250,7 +252,7 @@ void launch_fill(cudaStream_t st, long count, double v, double* d) {
 }
 void launch_grad_reduce(cudaStream_t st, long count, const double* G, const double* PG, const double* Gold,
                         const double* Dir, double* part, const Scalars* sc) {
-  grad_reduce_kernel<<<kReduceBlocks, TB, 0, st>>>(count, G, PG, Gold, Dir, part, sc);
+  grad_reduce_kernel<<<reduce_blocks(count), TB, 0, st>>>(count, G, PG, Gold, Dir, part, sc);
   OMM_LAUNCH_CHECK();
 }
 void launch_control_direction(cudaStream_t st, Scalars* sc, const double* part, int mixed, int nparts) {
@@ -265,16 +267,21 @@ int traces_blocks(int n) {
   const int t = (n + 31) / 32;
   return t * t;
 }
-// a tile per CTA while two waves of CTAs hold them all (n <= 544: with four tiles per CTA an n = 128 solve
-// ran them on 4 SMs, 23 us); above, four tiles per CTA, so that fewer partial sums are left
+// The float64 work of a 32 x 32 tile (nine products per element at two lanes per clock, and the block sums)
+// keeps an SM busy for some 10 us, so a small n spreads each tile over four CTAs (n <= 256: up to two waves of
+// them; an n = 36 solve ran its four tiles on 4 SMs, 16 us). A tile per CTA up to two waves (n <= 544); above,
+// four tiles per CTA, so that fewer partial sums are left.
+static int tile_quarters(int n) { return traces_blocks(n) <= 76 ? 4 : 1; }
 int traces_partials(int n) {
   const int tiles = traces_blocks(n);
-  return tiles <= 2 * 152 ? tiles : (tiles + 3) / 4;
+  return tiles <= 76 ? 4 * tiles : (tiles <= 304 ? tiles : (tiles + 3) / 4);
 }
+// 1024 elements and more per CTA: the block sums cost each CTA as much float64 time as 2000 elements
+int reduce_blocks(long count) { return (int)std::min<long>(kReduceBlocks, (count + 1023) / 1024); }
 void launch_traces(cudaStream_t st, int n, const double* SWHW, const double* Proj, double* part,
                    const Scalars* sc, bool fp32_products) {
-  if (fp32_products) traces_kernel<true><<<traces_partials(n), TB, 0, st>>>(n, SWHW, Proj, part, sc);
-  else traces_kernel<false><<<traces_partials(n), TB, 0, st>>>(n, SWHW, Proj, part, sc);
+  if (fp32_products) traces_kernel<true><<<traces_partials(n), TB, 0, st>>>(n, SWHW, Proj, part, sc, tile_quarters(n));
+  else traces_kernel<false><<<traces_partials(n), TB, 0, st>>>(n, SWHW, Proj, part, sc, tile_quarters(n));
   OMM_LAUNCH_CHECK();
 }
 void launch_control_linesearch(cudaStream_t st, Scalars* sc, const double* part, int nblocks) {
@@ -299,8 +306,8 @@ update_state_split_kernel(long n, long m, double* C, double* Y4, const double* D
 }
 __global__ void __launch_bounds__(TB)
 update_subspace_split_kernel(int n, double* SWHW, const double* __restrict__ Proj, const double* __restrict__ Wref,
-                             __nv_bfloat16* Whi, __nv_bfloat16* Wlo, long ldw, const Scalars* sc) {
-  dev::update_subspace_split_body(n, SWHW, Proj, Wref, Whi, Wlo, ldw, sc, blockIdx.x, gridDim.x);
+                             __nv_bfloat16* Whi, __nv_bfloat16* Wlo, long ldw, const Scalars* sc, int quarters) {
+  dev::update_subspace_split_body(n, SWHW, Proj, Wref, Whi, Wlo, ldw, sc, blockIdx.x, gridDim.x, quarters);
 }
 }  // namespace
 
@@ -356,11 +363,12 @@ void launch_reduce_unpreconditioned(cudaStream_t st, long n, long m, const doubl
 }
 void launch_update_subspace_split(cudaStream_t st, int n, double* SWHW, const double* Proj, const double* Wref,
                                   __nv_bfloat16* Whi, __nv_bfloat16* Wlo, long ldw, const Scalars* sc) {
-  update_subspace_split_kernel<<<traces_blocks(n), TB, 0, st>>>(n, SWHW, Proj, Wref, Whi, Wlo, ldw, sc);
+  update_subspace_split_kernel<<<traces_blocks(n) * tile_quarters(n), TB, 0, st>>>(n, SWHW, Proj, Wref, Whi, Wlo, ldw, sc,
+                                                                                 tile_quarters(n));
   OMM_LAUNCH_CHECK();
 }
 void launch_update_subspace(cudaStream_t st, int n, double* SWHW, const double* Proj, const Scalars* sc) {
-  update_subspace_kernel<<<traces_blocks(n), TB, 0, st>>>(n, SWHW, Proj, sc);
+  update_subspace_kernel<<<traces_blocks(n) * tile_quarters(n), TB, 0, st>>>(n, SWHW, Proj, sc, tile_quarters(n));
   OMM_LAUNCH_CHECK();
 }
 void launch_scale_copy(cudaStream_t st, long count, const double* src, double a, double* dst, const Scalars* sc) {

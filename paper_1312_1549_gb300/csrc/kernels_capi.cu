@@ -163,7 +163,7 @@ omm_status omm_kernel_quartic_coefficients(int n, const double* SWHW, const doub
   omm_status rc = OMM_OK;
   try {
     OMM_CUDA_TRY(cudaMalloc((void**)&sc, sizeof(Scalars)));
-    OMM_CUDA_TRY(cudaMalloc((void**)&part, (size_t)traces_blocks(n) * kNumTraces * sizeof(double)));
+    OMM_CUDA_TRY(cudaMalloc((void**)&part, (size_t)traces_partials(n) * kNumTraces * sizeof(double)));
     Scalars h;
     std::memset(&h, 0, sizeof(h));
     h.E = E;

@@ -170,7 +170,7 @@ void iterate_fp64(omm_ctx* c) {
   } else
     launch_scale_copy(c->st, nm, c->G, 1.0, c->PG, c->sc);
   launch_grad_reduce(c->st, nm, c->G, c->PG, c->Gold, c->Dir, c->part, c->sc);
-  launch_control_direction(c->st, c->sc, c->part, 0, kReduceBlocks);
+  launch_control_direction(c->st, c->sc, c->part, 0, reduce_blocks(nm));
   launch_direction(c->st, nm, c->PG, c->Dir, c->sc);
   pf.begin(c->st);
   dgemm(c->st, 0, 1, n, m, m, 1.0, c->Dir, m, 0, c->HS, m, mm, 0.0, c->Y4 + 2 * nm, m, nm, 2, 0, skip);
@@ -385,7 +385,7 @@ omm_status omm_create(int m, int n, const double* H, const double* S, const doub
     dev_alloc(&c->Proj, 4L * n * n, c->st);
     dev_alloc(&c->nn, (size_t)n * n, c->st);
     dev_alloc(&c->part, (size_t)kReduceBlocks * 4, c->st);
-    dev_alloc(&c->part2, (size_t)traces_blocks(n) * kNumTraces, c->st);
+    dev_alloc(&c->part2, (size_t)std::max(traces_blocks(n), traces_partials(n)) * kNumTraces, c->st);
     if (o.precision == OMM_PREC_MIXED) {
       c->mixed = mixed_create(c->st, m, n, c->HS, c->P);
       if (o.debug_expire_wait) mixed_set_expire(c->mixed, 1);
