@@ -399,16 +399,35 @@ void emu_density(EmuState* es, cudaStream_t st, const double* C, const double* S
   emu::gemm(st, es->opXT, es->opCTb, n, s, tc::Epilogue{D, m, m, 0, 1.0, 0.0, m, m, nullptr, es->err}, es->slab);
 }
 
-// out = -(2 C^T H~_W C + eta D) given out = D (dE/dS at the minimum), float64-class:
-// V = C^T H_W from the sliced C^T and H_W (C^T, sliced, as left by emu_density), then one
-// sliced product out = -2 V (C^T)^T - eta out.
-void emu_minus_edm(EmuState* es, cudaStream_t st, const double* SWHW, double eta, double* out) {
+namespace {
+// W (n x n) = -2 H_W - eta (4I - 2 S_W) from SWHW = [S_W | H_W] (n x 2n)
+__global__ void edm_weights_kernel(int n, const double* __restrict__ SWHW, double eta, double* W) {
+  const long count = (long)n * n;
+  for (long idx = blockIdx.x * (long)blockDim.x + threadIdx.x; idx < count; idx += (long)gridDim.x * blockDim.x) {
+    const long i = idx / n, j = idx - i * n;
+    const double* row = SWHW + i * 2L * n;
+    W[idx] = -2.0 * row[n + j] - eta * ((i == j ? 4.0 : 0.0) - 2.0 * row[j]);
+  }
+}
+}  // namespace
+
+// out = -(2 C^T H~_W C + eta D) (dE/dS at the minimum), float64-class. With D = C^T (4I - 2 S_W) C both
+// terms share the outer coefficients: V = C^T W with W = -2 H~_W - eta (4I - 2 S_W), then one sliced
+// product out = V (C^T)^T (forming D first took a second m x m x n product: 5.4 ms at m = 6656, n = 1024).
+void emu_minus_edm(EmuState* es, cudaStream_t st, const double* C, const double* SWHW, double eta, double* out) {
   const int m = es->m, n = es->n, s = kDensitySlices;
-  double* VT = es->T64 + (long)m * n;  // m x n
-  emu::slice_rows(st, SWHW + n, n, n, 2L * n, s, es->SWs, es->ldn, nullptr);  // H_W is symmetric
+  const long mn = (long)m * n;
+  double* CT = es->T64;       // m x n
+  double* VT = es->T64 + mn;  // m x n; first the n x n weights
+  emu::transpose(st, C, n, m, m, CT, n);
+  emu::slice_rows(st, CT, m, n, n, s, es->CTs, es->ldn, nullptr);
+  const long nn = (long)n * n;
+  edm_weights_kernel<<<(unsigned)std::min<long>((nn + 255) / 256, 4096), 256, 0, st>>>(n, SWHW, eta, VT);
+  OMM_LAUNCH_CHECK();
+  emu::slice_rows(st, VT, n, n, n, s, es->SWs, es->ldn, nullptr);  // symmetric like H~_W and S_W
   emu::gemm(st, es->opCT, es->opSW, n, s, tc::Epilogue{VT, n, n, 0, 1.0, 0.0, m, n, nullptr, es->err}, es->slab);
   emu::slice_rows(st, VT, m, n, n, s, es->XTs, es->ldn, nullptr);
-  emu::gemm(st, es->opXT, es->opCTb, n, s, tc::Epilogue{out, m, m, 0, -2.0, -eta, m, m, nullptr, es->err}, es->slab);
+  emu::gemm(st, es->opXT, es->opCTb, n, s, tc::Epilogue{out, m, m, 0, 1.0, 0.0, m, m, nullptr, es->err}, es->slab);
 }
 
 }  // namespace omm

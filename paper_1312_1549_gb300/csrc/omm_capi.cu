@@ -696,8 +696,7 @@ omm_status omm_backward(omm_ctx* c, double* dEdH, double* dEdS) {
     if (dEdS) {
       if (!is_device_ptr(dEdS)) { ensure_mm(c); tS = c->mm; }
       if (c->emu && !c->opts.native_certificate) {  // float64-class, like the certificate
-        emu_density(c->emu, c->st, c->C, c->SWHW, tS);
-        emu_minus_edm(c->emu, c->st, c->SWHW, c->eta, tS);
+        emu_minus_edm(c->emu, c->st, c->C, c->SWHW, c->eta, tS);
       } else {
         density_into(c, tS);
         minus_edm_into(c, tS);
