@@ -138,8 +138,9 @@ struct omm_batch {
                                              // (width, + 1000 for 256-row tiles on SM pairs, + 2000 on
                                              // clusters of two pairs sharing A)
   double ms_autotune = 0.0;
-  // refreshes and certificates of different instances run concurrently on these
+  // the starts, refreshes and certificates of different instances run concurrently on these
   cudaStream_t pool[kRefreshStreams] = {};
+  cudaEvent_t forked = nullptr, joined[kRefreshStreams] = {};
   std::vector<double> gemm_flop[kGroupedGemms];  // issued flops of each instance's group
 };
 
@@ -155,6 +156,9 @@ void batch_destroy(omm_batch* b) {
       cudaStreamSynchronize(q);
       cudaStreamDestroy(q);
     }
+  if (b->forked) cudaEventDestroy(b->forked);
+  for (cudaEvent_t e : b->joined)
+    if (e) cudaEventDestroy(e);
   if (b->exec) cudaGraphExecDestroy(b->exec);
   if (b->graph) cudaGraphDestroy(b->graph);
   for (omm_ctx* c : b->ctx) {
@@ -218,9 +222,30 @@ void enqueue_line_search(omm_batch* b) {
   timed_gemm(b, b->gG, pl);  // G and its split
 }
 
-// start a mixed round of instance i from its current (just recomputed) state
-void begin_round(omm_batch* b, int i, double g_ref, int iter_total) {
+// the pool streams used by `used` instances start after what is queued on the batch stream, and the batch
+// stream goes on after them
+void fork_pool(omm_batch* b, int used) {
+  OMM_CUDA_TRY(cudaEventRecord(b->forked, b->st));
+  for (int k = 0; k < std::min(used, kRefreshStreams); ++k) OMM_CUDA_TRY(cudaStreamWaitEvent(b->pool[k], b->forked, 0));
+}
+void join_pool(omm_batch* b, int used) {
+  for (int k = 0; k < std::min(used, kRefreshStreams); ++k) {
+    OMM_CUDA_TRY(cudaEventRecord(b->joined[k], b->pool[k]));
+    OMM_CUDA_TRY(cudaStreamWaitEvent(b->st, b->joined[k], 0));
+  }
+}
+// instance c's launches go to stream q while this lives
+struct OnStream {
+  omm_ctx* c;
+  cudaStream_t saved;
+  OnStream(omm_ctx* c_, cudaStream_t q) : c(c_), saved(c_->st) { c->st = q; }
+  ~OnStream() { c->st = saved; }
+};
+
+// start a mixed round of instance i from its current (just recomputed) state, on stream q
+void begin_round(omm_batch* b, int i, cudaStream_t q, double g_ref, int iter_total) {
   omm_ctx* c = b->ctx[i];
+  OnStream on(c, q);
   Scalars& h = *c->sc_host;
   const double E_keep = h.E, g_keep = h.gmax;
   reset_loop_flags(c, false);
@@ -366,6 +391,8 @@ omm_status omm_create_batched(int count, const int* m, const int* n, const doubl
       }
     }
     for (cudaStream_t& q : b->pool) OMM_CUDA_TRY(cudaStreamCreateWithFlags(&q, cudaStreamNonBlocking));
+    OMM_CUDA_TRY(cudaEventCreateWithFlags(&b->forked, cudaEventDisableTiming));
+    for (cudaEvent_t& e : b->joined) OMM_CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     alloc(&b->args, count, b->st);
     alloc(&b->err, 1, b->st);
     OMM_CUDA_TRY(cudaMemsetAsync(b->err, 0, sizeof(int), b->st));
@@ -444,19 +471,24 @@ omm_status omm_solve_batched(omm_batch* b, const double* const* C0, double* cons
     OMM_CUDA_TRY(cudaEventCreate(&g1));
     b->prof.reset();
     OMM_CUDA_TRY(cudaEventRecord(e0, b->st));
+    // first states on the pool streams: each is a chain of some twenty small launches (48 k points of m = 104
+    // one after another took 7 ms)
+    fork_pool(b, cnt);
     for (int i = 0; i < cnt; ++i) {
       omm_ctx* c = b->ctx[i];
+      cudaStream_t q = b->pool[i % kRefreshStreams];
+      OnStream on(c, q);
       c->solved = false;
-      copy_in(c->C, C0[i], (size_t)c->n * c->m, b->st);
+      copy_in(c->C, C0[i], (size_t)c->n * c->m, q);
       if (c->red) {  // C_r = L^T C0 (Sec. 2.4)
-        reduce_coefficients(c->red, b->st, c->n, c->C, c->Dir);
-        OMM_CUDA_TRY(cudaMemcpyAsync(c->C, c->Dir, (size_t)c->n * c->m * sizeof(double), cudaMemcpyDeviceToDevice,
-                                     b->st));
+        reduce_coefficients(c->red, q, c->n, c->C, c->Dir);
+        OMM_CUDA_TRY(cudaMemcpyAsync(c->C, c->Dir, (size_t)c->n * c->m * sizeof(double), cudaMemcpyDeviceToDevice, q));
       }
       reset_loop_flags(c, true);
       write_scalars(c);
-      mixed_recompute_state(c->mixed, b->st, c->sc, c->C, c->Y4, c->SWHW, c->G, c->part, c->part2);
+      mixed_recompute_state(c->mixed, q, c->sc, c->C, c->Y4, c->SWHW, c->G, c->part, c->part2);
     }
+    join_pool(b, cnt);
     OMM_CUDA_TRY(cudaMemcpyAsync(b->sc_host_all, b->sc_all, cnt * sizeof(Scalars), cudaMemcpyDeviceToHost, b->st));
     OMM_CUDA_TRY(cudaStreamSynchronize(b->st));
     for (int i = 0; i < cnt; ++i) {
@@ -468,8 +500,9 @@ omm_status omm_solve_batched(omm_batch* b, const double* const* C0, double* cons
         write_scalars(b->ctx[i]);
         continue;
       }
-      begin_round(b, i, h.gmax, 0);
+      begin_round(b, i, b->pool[i % kRefreshStreams], h.gmax, 0);
     }
+    join_pool(b, cnt);
     // profiling reads the GEMM events after every replay
     const int check = profile ? 1 : b->ctx[0]->opts.check_every;
     for (int poll = 0;; ++poll) {
@@ -580,8 +613,9 @@ omm_status omm_solve_batched(omm_batch* b, const double* const* C0, double* cons
         }
         ++refinements[i];
         round_start[i] = h.iter;
-        begin_round(b, i, h.gmax, h.iter);
+        begin_round(b, i, b->pool[i % kRefreshStreams], h.gmax, h.iter);
       }
+      join_pool(b, kRefreshStreams);
       ms_refresh_wall += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t_pass).count();
     }
     OMM_CUDA_TRY(cudaEventRecord(e1, b->st));
