@@ -42,9 +42,9 @@ constexpr int NB = 64;
 // The factor, the inverse and the Gram block take 44 thousand FMAs each, 11 us
 // each at the two per clock of one SM, so the work is laid out for that pipe:
 // no FMA on zeros beyond 8-wide blocks, all eight warps busy, short dependent
-// chains. Right-looking in panels of eight columns: warp 0 factors a panel
-// with its rows in registers (pivots and column entries by shuffles, one
-// rsqrt per pivot), then all warps apply its rank-8 update on 8 x 8 blocks.
+// chains. Right-looking in panels of eight columns: a panel is factored with
+// its rows in registers (pivots and column entries by shuffles, one rsqrt per
+// pivot on the chain), then all warps apply its rank-8 update on 8 x 8 blocks.
 // The inverse joins inverted diagonal blocks of edge 8, 16 and 32:
 // X21 = -X22 (L21 X11), the contraction cut at the triangles.
 // (One column at a time with three barriers each, one thread per column of the
@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(kLeaf64Threads)
 leaf_f64_kernel(double* A, long lda, int b, double* Linv, int* info, int col_offset, double* Pblk, long ldp) {
   __shared__ double L[NB][NB + 1];
   __shared__ double X[NB][NB + 1];
-  __shared__ double rdiag[NB];
+  __shared__ double rdiag[NB], pivot[NB];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   constexpr int kWarps = kLeaf64Threads / 32;
   for (int idx = tid; idx < NB * NB; idx += kLeaf64Threads) {
@@ -67,48 +67,40 @@ leaf_f64_kernel(double* A, long lda, int b, double* Linv, int* info, int col_off
   __syncthreads();
   for (int p0 = 0; p0 < b; p0 += 8) {
     const int pw = min(8, b - p0);
-    if (warp == 0) {  // lane l holds rows p0 + l and p0 + l + 32
-      double r[2][8];
+    // lanes 0-7 of the first three warps hold the panel's diagonal rows (each warp factors its own copy,
+    // so that no warp waits for another's pivots), lanes 8-31 the rows below, 24 to a warp
+    const int i = lane < 8 ? p0 + lane : p0 + 8 + 24 * warp + lane - 8;
+    if (warp < 3 && (warp == 0 || p0 + 8 + 24 * warp < b)) {
+      double r[8];
 #pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        const int i = p0 + lane + 32 * t;
-#pragma unroll
-        for (int c = 0; c < 8; ++c) r[t][c] = (i < b && c < pw && p0 + c <= i) ? L[i][p0 + c] : 0.0;
-      }
+      for (int c = 0; c < 8; ++c) r[c] = (i < b && c < pw && p0 + c <= i) ? L[i][p0 + c] : 0.0;
+      __syncwarp();
 #pragma unroll
       for (int c = 0; c < 8; ++c) {
         if (c < pw) {
-          double d = __shfl_sync(0xffffffffu, r[0][c], c);  // the pivot, row p0 + c
+          double d = __shfl_sync(0xffffffffu, r[c], c);  // the pivot, row p0 + c
           if (!(d > 0.0)) {
-            if (lane == 0) atomicCAS(info, 0, col_offset + p0 + c + 1);
+            if (warp == 0 && lane == 0) atomicCAS(info, 0, col_offset + p0 + c + 1);
             d = 1.0;
           }
-          // 1 / sqrt(d) and sqrt(d) to the last place: one Newton step each on rsqrt's value
-          double rs = rsqrt(d), sq = sqrt(d);
+          // 1 / sqrt(d) to the last place: one Newton step on rsqrt's value
+          double rs = rsqrt(d);
           if (rs > 0.0) rs = fma(0.5 * rs, fma(-(d * rs), rs, 1.0), rs);  // (0 only for an infinite pivot)
-#pragma unroll
-          for (int t = 0; t < 2; ++t) {
-            const int i = p0 + lane + 32 * t;
-            if (i > p0 + c) r[t][c] *= rs;
-            else if (i == p0 + c) r[t][c] = sq;
+          if (warp == 0 && lane == 0) {
+            rdiag[p0 + c] = rs;
+            pivot[p0 + c] = d;
           }
-          if (lane == 0) rdiag[p0 + c] = rs;
+          r[c] *= rs;
 #pragma unroll
-          for (int l = 0; l < 8; ++l) {
-            if (l > c) {
-              const double lc = __shfl_sync(0xffffffffu, r[0][c], l);  // L[p0 + l][p0 + c]
-              if (lane >= l) r[0][l] = fma(-r[0][c], lc, r[0][l]);
-              if (p0 + 32 < b) r[1][l] = fma(-r[1][c], lc, r[1][l]);
-            }
-          }
+          for (int l = 0; l < 8; ++l)
+            if (l > c) r[l] = fma(-r[c], __shfl_sync(0xffffffffu, r[c], l), r[l]);  // L[p0 + l][p0 + c]
         }
       }
-#pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        const int i = p0 + lane + 32 * t;
+      // (entries above the diagonal, and the diagonal itself, are left to what follows)
+      if (warp == 0 || lane >= 8) {
 #pragma unroll
         for (int c = 0; c < 8; ++c)
-          if (i < b && c < pw && p0 + c <= i) L[i][p0 + c] = r[t][c];
+          if (i < b && c < pw && p0 + c < i) L[i][p0 + c] = r[c];
       }
     }
     __syncthreads();
@@ -130,6 +122,10 @@ leaf_f64_kernel(double* A, long lda, int b, double* Linv, int* info, int col_off
       q += kWarps;
     }
     __syncthreads();
+  }
+  if (tid < b) {  // the factor's diagonal, sqrt(d), off the panels' chain
+    const double d = pivot[tid], t = d * rdiag[tid];
+    L[tid][tid] = rdiag[tid] > 0.0 ? fma(0.5 * rdiag[tid], fma(-t, t, d), t) : d;
   }
   // inverses of the 8 x 8 diagonal blocks: warp w's lane c solves column c of block w
   if (8 * warp < b && lane < 8 && 8 * warp + lane < b) {

@@ -403,14 +403,15 @@ sliced_pair_kernel(const __grid_constant__ GroupDesc g, const __grid_constant__ 
 }
 
 // C += alpha x (the slabs of the workers whose share starts inside the tile, in order). One CTA per
-// 32 x 32 block of a left-over tile; bmt rows per tile, ctas CTAs per worker (rows 128 q .. of a tile belong to
-// its q-th CTA). A tile that no share starts in is left alone.
+// 8 x 32 block of a left-over tile (a small product's few tiles have up to a hundred slabs each, and every
+// slab costs a block of 32 x 32 some thousand clocks of float64 adds); bmt rows per tile, bmt / 128 CTAs per
+// worker (rows 128 q .. of a tile belong to its q-th CTA). A tile that no share starts in is left alone.
 __global__ void __launch_bounds__(256)
 slab_reduce_kernel(const __grid_constant__ GroupDesc g, int npairs, const __grid_constant__ SlicedWork w, int bmt) {
-  const int subs_n = g.bn / 32, subs = (bmt / 32) * subs_n;
+  const int subs_n = g.bn / 32, subs = (bmt / 8) * subs_n;
   const int tile = w.full * w.nw + blockIdx.x / subs, sub = blockIdx.x % subs;
   const int mb = tile % w.tiles_m, nb = tile / w.tiles_m;
-  const int r0 = (sub / subs_n) * 32, c0 = (sub % subs_n) * 32;
+  const int r0 = (sub / subs_n) * 8, c0 = (sub % subs_n) * 32;
   const int row0 = mb * bmt + r0, col0 = nb * g.bn + c0;
   if (row0 >= g.ep.M || col0 >= g.ep.N) return;
   long base, per;
@@ -426,26 +427,28 @@ slab_reduce_kernel(const __grid_constant__ GroupDesc g, int npairs, const __grid
   int first = (int)((base - line.base) * w.nr / line.len);
   while (first < w.nr && line.begin(w, first) <= base) ++first;
   if (first >= w.nr || line.begin(w, first) >= base + per) return;
+  int last = (int)((base + per - line.base) * w.nr / line.len) + 1;  // one past the last such worker
+  while (last > first && (last > w.nr || line.begin(w, last - 1) >= base + per)) --last;
   const int ctas = bmt / BM;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  double v[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int q = first; q < w.nr && line.begin(w, q) < base + per; ++q) {
-    const double* slab = w.slab + ((long)q * ctas + r0 / BM) * 2 * BM * g.bn + (r0 % BM) + tx;
+  const int rr = threadIdx.x & 7, cc = threadIdx.x >> 3;  // eight rows (64 bytes) of a column
+  const double* slab = w.slab + ((long)first * ctas + r0 / BM) * 2 * BM * g.bn + (r0 % BM) + rr + (long)(c0 + cc) * BM;
+  const long step = (long)ctas * 2 * BM * g.bn;
+  double v = 0.0;
+  int q = first;
+  for (; q + 8 <= last; q += 8, slab += 8 * step) {  // eight loads in flight
+    double x[8];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] += slab[(long)(c0 + ty + 8 * k) * BM];
+    for (int k = 0; k < 8; ++k) x[k] = slab[k * step];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v += x[k];
   }
-  __shared__ double t[32][33];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) t[ty + 8 * k][tx] = v[k];  // [column][row]
+  for (; q < last; ++q, slab += step) v += *slab;
+  __shared__ double t[32][9];
+  t[cc][rr] = v;
   __syncthreads();
-  const int col = col0 + tx;
-  if (col >= g.ep.N) return;
+  const int col = col0 + (threadIdx.x & 31), row = row0 + (threadIdx.x >> 5);
+  if (col >= g.ep.N || row >= g.ep.M) return;
   const long blk = col / g.ep.split_cols;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int row = row0 + ty + 8 * k;
-    if (row >= g.ep.M) continue;
-    double* p = g.ep.C + blk * g.ep.split_stride + (long)row * g.ep.ldc + (col - blk * g.ep.split_cols);
-    *p = fma(g.ep.alpha, t[tx][ty + 8 * k], *p);
-  }
+  double* p = g.ep.C + blk * g.ep.split_stride + (long)row * g.ep.ldc + (col - blk * g.ep.split_cols);
+  *p = fma(g.ep.alpha, t[threadIdx.x & 31][threadIdx.x >> 5], *p);
 }

@@ -1529,7 +1529,7 @@ void gemm_sliced(cudaStream_t st, const Operand& A, const Operand& B, int K, con
   if (!best_whole) {  // some share starts inside a tile
     const int bmt = best_shape.pair ? 2 * BM : BM;
     const int left = best.tiles - best.full * best.nw;
-    slab_reduce_kernel<<<(unsigned)(left * (bmt / 32) * (best_shape.bn / 32)), 256, 0, st>>>(g, pl.n, best, bmt);
+    slab_reduce_kernel<<<(unsigned)(left * (bmt / 8) * (best_shape.bn / 32)), 256, 0, st>>>(g, pl.n, best, bmt);
     OMM_LAUNCH_CHECK();
   }
 }
