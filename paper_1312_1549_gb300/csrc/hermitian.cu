@@ -273,25 +273,25 @@ omm_status omm_solve_hermitian(omm_ctx* c, const double* C0, double* C, double* 
 omm_status omm_backward_hermitian(omm_ctx* c, double* dEdH, double* dEdS) {
   omm_status rc = check_hermitian(c, "omm_backward_hermitian");
   if (rc != OMM_OK) return rc;
+  if ((dEdH || dEdS) && !c->solved) return fail(OMM_ERR_STATE, "omm_backward_hermitian: no converged solve");
   const int m = c->mc;
   double* tmp = nullptr;
   try {
     alloc(&tmp, 4 * (size_t)m * m, c->st);
-    c->hermitian = false;
-    for (int k = 0; k < 2 && rc == OMM_OK; ++k) {
-      double* out = k == 0 ? dEdH : dEdS;
-      if (!out) continue;
-      rc = k == 0 ? omm_backward(c, tmp, nullptr) : omm_backward(c, nullptr, tmp);
-      if (rc == OMM_OK) extract_matrix(c->st, m, tmp, c->hz_stage, out);
+    // the density stays in tmp for dE/dS, and the host waits once
+    if (dEdH) {
+      form_density(c, tmp);
+      extract_matrix(c->st, m, tmp, c->hz_stage, dEdH);
     }
-    c->hermitian = true;
+    if (dEdS) {
+      form_minus_edm(c, tmp, dEdH != nullptr);
+      extract_matrix(c->st, m, tmp, c->hz_stage, dEdS);
+    }
     OMM_CUDA_TRY(cudaStreamSynchronize(c->st));
     mem::release(tmp, c->st);
   } catch (const std::bad_alloc&) {
-    c->hermitian = true;
     return fail(OMM_ERR_OOM, "omm_backward_hermitian: device allocation failed");
   } catch (const CudaError& err) {
-    c->hermitian = true;
     cudaStreamSynchronize(c->st);
     mem::release(tmp, c->st);
     return fail(OMM_ERR_CUDA, std::string("omm_backward_hermitian: ") + err.what + ": " + cudaGetErrorString(err.err));

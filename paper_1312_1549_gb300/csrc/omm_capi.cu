@@ -235,6 +235,20 @@ void minus_edm_into(omm_ctx* c, double* out) {
   launch_symmetrize_lower(c->st, m, out);
 }
 
+void form_density(omm_ctx* c, double* out) {
+  if (c->emu && !c->opts.native_certificate) emu_density(c->emu, c->st, c->C, c->SWHW, out);
+  else density_into(c, out);
+}
+
+void form_minus_edm(omm_ctx* c, double* out, bool holds_density) {
+  if (c->emu && !c->opts.native_certificate) {  // float64-class, like the certificate
+    emu_minus_edm(c->emu, c->st, c->C, c->SWHW, c->eta, out);
+  } else {
+    if (!holds_density) density_into(c, out);
+    minus_edm_into(c, out);
+  }
+}
+
 void ensure_mm(omm_ctx* c) {
   if (!c->mm) dev_alloc(&c->mm, (size_t)c->m * c->m, c->st);
 }
@@ -636,8 +650,7 @@ omm_status omm_solve(omm_ctx* c, const double* C0, double* Cout, double* E, doub
           ensure_mm(c);
           tgt = c->mm;
         }
-        if (c->emu && !c->opts.native_certificate) emu_density(c->emu, c->st, c->C, c->SWHW, tgt);
-        else density_into(c, tgt);
+        form_density(c, tgt);
         if (tgt != D)
           OMM_CUDA_TRY(cudaMemcpyAsync(D, tgt, (size_t)m * m * sizeof(double), cudaMemcpyDefault, c->st));
         flop += 2.0 * n * (double)n * m + 2.0 * m * (double)m * n;
@@ -688,19 +701,14 @@ omm_status omm_backward(omm_ctx* c, double* dEdH, double* dEdS) {
     double* tS = dEdS;
     if (dEdH && !is_device_ptr(dEdH)) { ensure_mm(c); tH = c->mm; }
     if (dEdH) {
-      // the same density matrix omm_solve returns
-      if (c->emu && !c->opts.native_certificate) emu_density(c->emu, c->st, c->C, c->SWHW, tH);
-      else density_into(c, tH);
+      form_density(c, tH);  // the same density matrix omm_solve returns
       if (tH != dEdH) OMM_CUDA_TRY(cudaMemcpyAsync(dEdH, tH, bytes, cudaMemcpyDefault, c->st));
     }
     if (dEdS) {
       if (!is_device_ptr(dEdS)) { ensure_mm(c); tS = c->mm; }
-      if (c->emu && !c->opts.native_certificate) {  // float64-class, like the certificate
-        emu_minus_edm(c->emu, c->st, c->C, c->SWHW, c->eta, tS);
-      } else {
-        density_into(c, tS);
-        minus_edm_into(c, tS);
-      }
+      const bool native = !c->emu || c->opts.native_certificate;
+      if (dEdH && native && tS != tH) OMM_CUDA_TRY(cudaMemcpyAsync(tS, tH, bytes, cudaMemcpyDeviceToDevice, c->st));
+      form_minus_edm(c, tS, dEdH != nullptr && native);
       if (tS != dEdS) OMM_CUDA_TRY(cudaMemcpyAsync(dEdS, tS, bytes, cudaMemcpyDefault, c->st));
     }
     OMM_CUDA_TRY(cudaStreamSynchronize(c->st));

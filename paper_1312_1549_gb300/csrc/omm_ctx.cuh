@@ -64,6 +64,10 @@ void reset_loop_flags(omm_ctx* c, bool full);
 void read_scalars(omm_ctx* c);
 void write_scalars(omm_ctx* c);
 void density_into(omm_ctx* c, double* out);
+// dE/dH = D and dE/dS = -EDM of the converged point (m x m, device, on c->st); holds_density: out already
+// holds D (which only the native form uses)
+void form_density(omm_ctx* c, double* out);
+void form_minus_edm(omm_ctx* c, double* out, bool holds_density);
 void destroy(omm_ctx* c);
 int batch_count(const omm_batch* b);
 // real form of a Hermitian problem: C <- the nearest real form of a complex C (each pair of rows
