@@ -94,6 +94,93 @@ __global__ void __launch_bounds__(dev::TB) b_update_subspace_kernel(const IterAr
                                   a.ld4, a.sc, blockIdx.x, a.tiles);
 }
 
+// ---- native float64 recompute of many small instances at once (k points): each step of
+// recompute_state_fp64 is one launch over the stopped instances (blockIdx.z) instead of one per instance, whose
+// ten launches each kept the host busy for most of a pass (48 k points of m = 208, n = 32: 2 ms per pass)
+struct StateArgs {
+  int n, m;
+  int nc, mc;  // real form of an nc x mc complex problem (0: none)
+  double *C, *G, *Y4, *SWHW, *part, *part2;
+  const double* HS;
+  Scalars* sc;
+};
+
+constexpr int kST = 16;          // output tile of the products: one element per thread
+constexpr int kSK = 32;          // contracted elements per stage
+constexpr int kStateGmax = 8;    // max|G| partials per instance
+
+// C (M x N) = A (M x K) op(B): op(B) = B^T for B N x K (transB) or B K x N; finish(row, col, sum) stores
+template <typename F>
+__device__ __forceinline__ void state_product(const double* A, long lda, const double* B, long ldb, bool transB, int M,
+                                              int N, int K, int row0, int col0, F finish) {
+  __shared__ double As[kSK][kST + 1], Bs[kSK][kST + 1];
+  const int tid = threadIdx.x, tx = tid % kST, ty = tid / kST;
+  double acc = 0.0;
+  for (int k0 = 0; k0 < K; k0 += kSK) {
+    __syncthreads();
+#pragma unroll
+    for (int idx = tid; idx < kST * kSK; idx += 256) {
+      const int i = idx / kSK, k = idx % kSK;
+      As[k][i] = (row0 + i < M && k0 + k < K) ? A[(long)(row0 + i) * lda + k0 + k] : 0.0;
+      const int j = transB ? idx / kSK : idx % kST, kb = transB ? idx % kSK : idx / kST;
+      Bs[kb][j] = (col0 + j < N && k0 + kb < K) ? (transB ? B[(long)(col0 + j) * ldb + k0 + kb]
+                                                          : B[(long)(k0 + kb) * ldb + col0 + j])
+                                                : 0.0;
+    }
+    __syncthreads();
+#pragma unroll 8
+    for (int k = 0; k < kSK; ++k) acc = fma(As[k][ty], Bs[k][tx], acc);
+  }
+  if (row0 + ty < M && col0 + tx < N) finish(row0 + ty, col0 + tx, acc);
+}
+
+__global__ void __launch_bounds__(256) s_project_kernel(const StateArgs* __restrict__ A, const int* list) {
+  const StateArgs a = A[list[blockIdx.z]];
+  if (a.nc > 0) project_rows(a.nc, a.mc, a.C, blockIdx.x, gridDim.x);
+}
+// HC, SC = C [H~; S]^T (blockIdx.y: tile row and operator)
+__global__ void __launch_bounds__(256) s_operators_kernel(const StateArgs* __restrict__ A, const int* list) {
+  const StateArgs a = A[list[blockIdx.z]];
+  const int op = blockIdx.y & 1, row0 = (blockIdx.y >> 1) * kST, col0 = blockIdx.x * kST;
+  if (row0 >= a.n || col0 >= a.m) return;
+  double* out = a.Y4 + (long)op * a.n * a.m;
+  state_product(a.C, a.m, a.HS + (long)op * a.m * a.m, a.m, true, a.n, a.m, a.m, row0, col0,
+                [&](int i, int j, double v) { out[(long)i * a.m + j] = v; });
+}
+// S_W, H_W = C [SC; HC]^T
+__global__ void __launch_bounds__(256) s_subspace_kernel(const StateArgs* __restrict__ A, const int* list) {
+  const StateArgs a = A[list[blockIdx.z]];
+  const int op = blockIdx.y & 1, row0 = (blockIdx.y >> 1) * kST, col0 = blockIdx.x * kST;  // op 0: S_W, 1: H_W
+  if (row0 >= a.n || col0 >= a.n) return;
+  state_product(a.C, a.m, a.Y4 + (op ? 0L : (long)a.n * a.m), a.m, true, a.n, a.n, a.m, row0, col0,
+                [&](int i, int j, double v) { a.SWHW[(long)i * 2 * a.n + op * a.n + j] = v; });
+}
+// G = 8 HC - 4 [S_W | H_W] [HC; SC]; the first CTAs also take the functional's partial sums
+__global__ void __launch_bounds__(256) s_gradient_kernel(const StateArgs* __restrict__ A, const int* list) {
+  const StateArgs a = A[list[blockIdx.z]];
+  const int row0 = blockIdx.y * kST, col0 = blockIdx.x * kST;
+  if (row0 >= a.n || col0 >= a.m) return;
+  state_product(a.SWHW, 2L * a.n, a.Y4, a.m, false, a.n, a.m, 2 * a.n, row0, col0, [&](int i, int j, double v) {
+    const long at = (long)i * a.m + j;
+    a.G[at] = fma(1.0, 8.0 * a.Y4[at], -4.0 * v);
+  });
+}
+__global__ void __launch_bounds__(dev::TB) s_functional_kernel(const StateArgs* __restrict__ A, const int* list) {
+  const StateArgs a = A[list[blockIdx.z]];
+  const int t = (a.n + 31) / 32;
+  if ((int)blockIdx.x < t * t) dev::functional_body(a.n, a.SWHW, a.part2, blockIdx.x);
+}
+__global__ void __launch_bounds__(dev::TB) s_gmax_kernel(const StateArgs* __restrict__ A, const int* list) {
+  const StateArgs a = A[list[blockIdx.z]];
+  dev::gmax_body((long)a.n * a.m, a.G, a.part, blockIdx.x, gridDim.x);
+}
+__global__ void __launch_bounds__(dev::TB) s_finish_kernel(const StateArgs* __restrict__ A, const int* list) {
+  const StateArgs a = A[list[blockIdx.z]];
+  const int t = (a.n + 31) / 32;
+  if (blockIdx.x == 0) dev::finish_functional_body(a.sc, a.part2, t * t);
+  else dev::finish_gmax_body(a.sc, a.part, kStateGmax);
+}
+
 struct Grouped {
   tc::GroupDesc* dev = nullptr;
   int ngroups = 0, tiles = 0;
@@ -123,6 +210,10 @@ struct omm_batch {
   Scalars* sc_all = nullptr;       // device, count entries (each context's sc points here)
   Scalars* sc_host_all = nullptr;  // pinned
   IterArgs* args = nullptr;        // device
+  StateArgs* state_args = nullptr;  // device: the instances whose recompute is native float64
+  int* state_list = nullptr;        // device, count entries: those of a pass
+  int* state_list_host = nullptr;   // pinned
+  int state_n = 0, state_m = 0;     // largest sizes among them
   Grouped gPG, gHD, gPr, gG;
   int max_rows = 0;        // largest 2n (vector-kernel grid)
   int max_tiles = 0;       // largest n x n tile count
@@ -170,6 +261,9 @@ void batch_destroy(omm_batch* b) {
   }
   for (Grouped* g : {&b->gPG, &b->gHD, &b->gPr, &b->gG}) mem::release(g->dev, b->st);
   mem::release(b->args, b->st);
+  mem::release(b->state_args, b->st);
+  mem::release(b->state_list, b->st);
+  if (b->state_list_host) cudaFreeHost(b->state_list_host);
   mem::release(b->err, b->st);
   mem::release(b->sc_all, b->st);
   if (b->sc_host_all) cudaFreeHost(b->sc_host_all);
@@ -191,6 +285,28 @@ void timed_gemm(omm_batch* b, const Grouped& g, const tc::PairList& pl) {
   b->prof.begin(b->st);
   tc::gemm_persistent(b->st, g.dev, g.ngroups, g.tiles, pl, b->err, g.bn, g.pair, g.quad);
   b->prof.end(b->st, 0.0);
+}
+
+// float64 recompute of the states of the instances in state_list_host[0, cnt), on stream q
+void recompute_states(omm_batch* b, int cnt, cudaStream_t q) {
+  const unsigned tn = (unsigned)((b->state_n + kST - 1) / kST), tm = (unsigned)((b->state_m + kST - 1) / kST), z = (unsigned)cnt;
+  const StateArgs* A = b->state_args;
+  const int* list = b->state_list;
+  OMM_CUDA_TRY(cudaMemcpyAsync(b->state_list, b->state_list_host, cnt * sizeof(int), cudaMemcpyHostToDevice, q));
+  s_project_kernel<<<dim3(8, 1, z), 256, 0, q>>>(A, list);
+  OMM_LAUNCH_CHECK();
+  s_operators_kernel<<<dim3(tm, 2 * tn, z), 256, 0, q>>>(A, list);
+  OMM_LAUNCH_CHECK();
+  s_subspace_kernel<<<dim3(tn, 2 * tn, z), 256, 0, q>>>(A, list);
+  OMM_LAUNCH_CHECK();
+  s_functional_kernel<<<dim3((unsigned)traces_blocks(b->state_n), 1, z), dev::TB, 0, q>>>(A, list);
+  OMM_LAUNCH_CHECK();
+  s_gradient_kernel<<<dim3(tm, tn, z), 256, 0, q>>>(A, list);
+  OMM_LAUNCH_CHECK();
+  s_gmax_kernel<<<dim3(kStateGmax, 1, z), dev::TB, 0, q>>>(A, list);
+  OMM_LAUNCH_CHECK();
+  s_finish_kernel<<<dim3(2, 1, z), dev::TB, 0, q>>>(A, list);
+  OMM_LAUNCH_CHECK();
 }
 
 // one line search of every instance (captured into the graph)
@@ -394,6 +510,9 @@ omm_status omm_create_batched(int count, const int* m, const int* n, const doubl
     OMM_CUDA_TRY(cudaEventCreateWithFlags(&b->forked, cudaEventDisableTiming));
     for (cudaEvent_t& e : b->joined) OMM_CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     alloc(&b->args, count, b->st);
+    alloc(&b->state_args, count, b->st);
+    alloc(&b->state_list, count, b->st);
+    OMM_CUDA_TRY(cudaMallocHost((void**)&b->state_list_host, count * sizeof(int)));
     alloc(&b->err, 1, b->st);
     OMM_CUDA_TRY(cudaMemsetAsync(b->err, 0, sizeof(int), b->st));
     OMM_CUDA_TRY(cudaMemcpyAsync(b->args, args.data(), count * sizeof(IterArgs), cudaMemcpyHostToDevice, b->st));
@@ -470,6 +589,18 @@ omm_status omm_solve_batched(omm_batch* b, const double* const* C0, double* cons
     OMM_CUDA_TRY(cudaEventCreate(&g0));
     OMM_CUDA_TRY(cudaEventCreate(&g1));
     b->prof.reset();
+    std::vector<StateArgs> state(cnt);  // (a Hermitian batch's contexts learn of their real form after the create)
+    for (int i = 0; i < cnt; ++i) {
+      const omm_ctx* c = b->ctx[i];
+      const bool real_form = c->real_form && !c->red;
+      state[i] = StateArgs{c->n, c->m, real_form ? c->nc : 0, real_form ? c->mc : 0, c->C, c->G, c->Y4, c->SWHW, c->part,
+                           c->part2, c->HS, c->sc};
+      if (c->emu == nullptr) {
+        b->state_n = std::max(b->state_n, c->n);
+        b->state_m = std::max(b->state_m, c->m);
+      }
+    }
+    OMM_CUDA_TRY(cudaMemcpyAsync(b->state_args, state.data(), cnt * sizeof(StateArgs), cudaMemcpyHostToDevice, b->st));
     OMM_CUDA_TRY(cudaEventRecord(e0, b->st));
     // first states on the pool streams: each is a chain of some twenty small launches (48 k points of m = 104
     // one after another took 7 ms)
@@ -542,7 +673,7 @@ omm_status omm_solve_batched(omm_batch* b, const double* const* C0, double* cons
       // (float64-class, or native float64 on request) enqueued, spread over the pool
       // streams so that the small instances' products overlap on the GPU
       const auto t_pass = std::chrono::steady_clock::now();
-      std::vector<int> todo;
+      std::vector<int> todo, grouped;  // grouped: small instances, whose native recomputes run as one
       for (int i = 0; i < cnt; ++i) {
         if (finished[i]) continue;
         omm_ctx* c = b->ctx[i];
@@ -566,6 +697,11 @@ omm_status omm_solve_batched(omm_batch* b, const double* const* C0, double* cons
         }
         if (h.done && h.stop_reason == 2) energy_stop[i] = 1;
         last_done[i] = h.done != 0;
+        if (c->emu == nullptr) {  // taken together below
+          grouped.push_back(i);
+          todo.push_back(i);
+          continue;
+        }
         const bool native = (last_done[i] && c->opts.native_certificate != 0) || c->emu == nullptr;
         cudaStream_t q = b->pool[todo.size() % kRefreshStreams];
         c->st = q;
@@ -578,6 +714,12 @@ omm_status omm_solve_batched(omm_batch* b, const double* const* C0, double* cons
         todo.push_back(i);
       }
       if (todo.empty()) continue;
+      if (!grouped.empty()) {
+        std::copy(grouped.begin(), grouped.end(), b->state_list_host);
+        OMM_CUDA_TRY(cudaEventRecord(g0, b->pool[0]));
+        recompute_states(b, (int)grouped.size(), b->pool[0]);
+        OMM_CUDA_TRY(cudaEventRecord(g1, b->pool[0]));
+      }
       for (cudaStream_t q : b->pool) OMM_CUDA_TRY(cudaStreamSynchronize(q));
       OMM_CUDA_TRY(cudaMemcpyAsync(b->sc_host_all, b->sc_all, cnt * sizeof(Scalars), cudaMemcpyDeviceToHost, b->st));
       OMM_CUDA_TRY(cudaStreamSynchronize(b->st));
@@ -594,7 +736,7 @@ omm_status omm_solve_batched(omm_batch* b, const double* const* C0, double* cons
           write_scalars(c);
           continue;
         }
-        (certify ? ms_cert : ms_ref)[i] += elapsed(c->ev[0], c->ev[1]);
+        (certify ? ms_cert : ms_ref)[i] += c->emu == nullptr ? elapsed(g0, g1) : elapsed(c->ev[0], c->ev[1]);
         ++rounds[i];
         if (!std::isfinite(h.gmax) || !std::isfinite(h.E)) {
           result[i] = OMM_ERR_NONFINITE;

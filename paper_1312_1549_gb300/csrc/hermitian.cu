@@ -65,19 +65,7 @@ __global__ void extract_matrix_kernel(int m, const double* __restrict__ src, dou
 
 // the nearest real form: rows j and n + j of C_e (2n x 2m) averaged onto one complex row
 __global__ void project_rows_kernel(int n, int m, double* __restrict__ Ce) {
-  const long count = (long)n * m;
-  const long ld = 2L * m;
-  for (long idx = blockIdx.x * (long)blockDim.x + threadIdx.x; idx < count; idx += (long)gridDim.x * blockDim.x) {
-    const long j = idx / m, k = idx % m;
-    double* top = Ce + j * ld;
-    double* bot = Ce + (n + j) * ld;
-    const double re = 0.5 * (top[k] + bot[m + k]);
-    const double im = 0.5 * (top[m + k] - bot[k]);
-    top[k] = re;
-    top[m + k] = im;
-    bot[k] = -im;
-    bot[m + k] = re;
-  }
+  project_rows(n, m, Ce, blockIdx.x, gridDim.x);
 }
 
 unsigned grid_for(long count) { return (unsigned)std::min<long>((count + 255) / 256, 4096); }

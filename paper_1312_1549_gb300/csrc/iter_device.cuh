@@ -510,5 +510,78 @@ __device__ __forceinline__ void scale_copy_body(long count, const double* src, d
     dst[i] = a * src[i];
 }
 
+// ---- the parts of a state recompute that are not products
+__device__ __forceinline__ void functional_body(int n, const double* __restrict__ SWHW, double* part, int bx_) {
+  const int tiles = (n + 31) / 32;
+  const int I = bx_ / tiles, J = bx_ % tiles;
+  __shared__ double tHW[32][33];
+  const long l2 = 2L * n;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  for (int r = ty; r < 32; r += 8) {
+    const int gi = J * 32 + r, gj = I * 32 + tx;
+    tHW[r][tx] = (gi < n && gj < n) ? SWHW[(long)gi * l2 + n + gj] : 0.0;
+  }
+  __syncthreads();
+  double v[2] = {0.0, 0.0};
+  for (int r = ty; r < 32; r += 8) {
+    const int gi = I * 32 + r, gj = J * 32 + tx;
+    if (gi >= n || gj >= n) continue;
+    if (gi == gj) v[0] += SWHW[(long)gi * l2 + n + gj];
+    v[1] = fma(SWHW[(long)gi * l2 + gj], tHW[tx][r], v[1]);
+  }
+  __shared__ SumScratch<2> sh;
+  block_sum<2>(v, sh);
+  if (threadIdx.x == 0) {
+    part[bx_ * 2 + 0] = v[0];
+    part[bx_ * 2 + 1] = v[1];
+  }
+}
+
+__device__ __forceinline__ void finish_functional_body(Scalars* sc, const double* part, int nblocks) {
+  double v[2] = {0.0, 0.0};
+  for (int b = threadIdx.x; b < nblocks; b += TB) {
+    v[0] += part[b * 2 + 0];
+    v[1] += part[b * 2 + 1];
+  }
+  __shared__ SumScratch<2> sh;
+  block_sum<2>(v, sh);
+  if (threadIdx.x == 0) sc->E = 4.0 * v[0] - 2.0 * v[1];
+}
+
+__device__ __forceinline__ void gmax_body(long count, const double* G, double* part, int bx_, int nbx_) {
+  double mx = 0.0;
+  for (long i = bx_ * (long)TB + threadIdx.x; i < count; i += (long)nbx_ * TB) {
+    const double a = fabs(G[i]);
+    mx = (a > mx || a != a) ? a : mx;
+  }
+  __shared__ double shm[TB / 32];
+  const double wm = warp_max(mx);
+  if ((threadIdx.x & 31) == 0) shm[threadIdx.x >> 5] = wm;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double m = 0.0;
+    for (int k = 0; k < TB / 32; ++k) m = (shm[k] > m || shm[k] != shm[k]) ? shm[k] : m;
+    part[bx_] = m;
+  }
+}
+
+__device__ __forceinline__ void finish_gmax_body(Scalars* sc, const double* part, int nblocks) {
+  double mx = 0.0;
+  for (int b = threadIdx.x; b < nblocks; b += TB) {
+    const double a = part[b];
+    mx = (a > mx || a != a) ? a : mx;
+  }
+  __shared__ double shm[TB / 32];
+  const double wm = warp_max(mx);
+  if ((threadIdx.x & 31) == 0) shm[threadIdx.x >> 5] = wm;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double m = 0.0;
+    for (int k = 0; k < TB / 32; ++k) m = (shm[k] > m || shm[k] != shm[k]) ? shm[k] : m;
+    sc->gmax = m;
+  }
+}
+
+
 }  // namespace dev
 }  // namespace omm

@@ -137,76 +137,21 @@ __global__ void scale_copy_kernel(long count, const double* src, double a, doubl
 // partial sums of Tr H_W and Tr(S_W H_W) = sum_ij S_W,ij H_W,ji
 __global__ void __launch_bounds__(TB)
 functional_kernel(int n, const double* __restrict__ SWHW, double* part) {
-  const int tiles = (n + 31) / 32;
-  const int I = blockIdx.x / tiles, J = blockIdx.x % tiles;
-  __shared__ double tHW[32][33];
-  const long l2 = 2L * n;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  for (int r = ty; r < 32; r += 8) {
-    const int gi = J * 32 + r, gj = I * 32 + tx;
-    tHW[r][tx] = (gi < n && gj < n) ? SWHW[(long)gi * l2 + n + gj] : 0.0;
-  }
-  __syncthreads();
-  double v[2] = {0.0, 0.0};
-  for (int r = ty; r < 32; r += 8) {
-    const int gi = I * 32 + r, gj = J * 32 + tx;
-    if (gi >= n || gj >= n) continue;
-    if (gi == gj) v[0] += SWHW[(long)gi * l2 + n + gj];
-    v[1] = fma(SWHW[(long)gi * l2 + gj], tHW[tx][r], v[1]);
-  }
-  __shared__ SumScratch<2> sh;
-  block_sum<2>(v, sh);
-  if (threadIdx.x == 0) {
-    part[blockIdx.x * 2 + 0] = v[0];
-    part[blockIdx.x * 2 + 1] = v[1];
-  }
+  functional_body(n, SWHW, part, blockIdx.x);
 }
 
 __global__ void __launch_bounds__(TB)
 finish_functional_kernel(Scalars* sc, const double* part, int nblocks) {
-  double v[2] = {0.0, 0.0};
-  for (int b = threadIdx.x; b < nblocks; b += TB) {
-    v[0] += part[b * 2 + 0];
-    v[1] += part[b * 2 + 1];
-  }
-  __shared__ SumScratch<2> sh;
-  block_sum<2>(v, sh);
-  if (threadIdx.x == 0) sc->E = 4.0 * v[0] - 2.0 * v[1];
+  finish_functional_body(sc, part, nblocks);
 }
 
 __global__ void __launch_bounds__(TB)
-gmax_kernel(long count, const double* __restrict__ G, double* part) {
-  double mx = 0.0;
-  for (long i = blockIdx.x * (long)TB + threadIdx.x; i < count; i += (long)gridDim.x * TB) {
-    const double a = fabs(G[i]);
-    mx = (a > mx || a != a) ? a : mx;
-  }
-  __shared__ double shm[TB / 32];
-  const double wm = warp_max(mx);
-  if ((threadIdx.x & 31) == 0) shm[threadIdx.x >> 5] = wm;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double m = 0.0;
-    for (int k = 0; k < TB / 32; ++k) m = (shm[k] > m || shm[k] != shm[k]) ? shm[k] : m;
-    part[blockIdx.x] = m;
-  }
+gmax_kernel(long count, const double* G, double* part) {
+  gmax_body(count, G, part, blockIdx.x, gridDim.x);
 }
 
 __global__ void __launch_bounds__(TB) finish_gmax_kernel(Scalars* sc, const double* part) {
-  double mx = 0.0;
-  for (int b = threadIdx.x; b < kReduceBlocks; b += TB) {
-    const double a = part[b];
-    mx = (a > mx || a != a) ? a : mx;
-  }
-  __shared__ double shm[TB / 32];
-  const double wm = warp_max(mx);
-  if ((threadIdx.x & 31) == 0) shm[threadIdx.x >> 5] = wm;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double m = 0.0;
-    for (int k = 0; k < TB / 32; ++k) m = (shm[k] > m || shm[k] != shm[k]) ? shm[k] : m;
-    sc->gmax = m;
-  }
+  finish_gmax_body(sc, part, kReduceBlocks);
 }
 
 __global__ void two_i_minus_kernel(int n, const double* SW, long ldsw, double* out) {

@@ -76,4 +76,23 @@ int batch_count(const omm_batch* b);
 // directions that leave the real forms (they are flat: the functional does not see them).
 void project_real_form(omm_ctx* c, cudaStream_t st);
 
+#ifdef __CUDACC__
+// rows j and n + j of a real form C_e (2n x 2m) averaged onto one complex row, block bx of nbx
+__device__ __forceinline__ void project_rows(int n, int m, double* __restrict__ Ce, int bx, int nbx) {
+  const long count = (long)n * m;
+  const long ld = 2L * m;
+  for (long idx = bx * (long)blockDim.x + threadIdx.x; idx < count; idx += (long)nbx * blockDim.x) {
+    const long j = idx / m, k = idx % m;
+    double* top = Ce + j * ld;
+    double* bot = Ce + (n + j) * ld;
+    const double re = 0.5 * (top[k] + bot[m + k]);
+    const double im = 0.5 * (top[m + k] - bot[k]);
+    top[k] = re;
+    top[m + k] = im;
+    bot[k] = -im;
+    bot[m + k] = re;
+  }
+}
+#endif
+
 }  // namespace omm
