@@ -15,6 +15,7 @@
 #include "fused_device.cuh"
 #include "iter_device.cuh"
 #include "omm_ctx.cuh"
+#include "pdl.cuh"
 #include "split_device.cuh"
 #include "tc_gemm.cuh"
 
@@ -48,6 +49,7 @@ struct IterArgs {
 
 // without a preconditioner: the Polak-Ribiere sums with PG = G (also writes PG and G_old)
 __global__ void __launch_bounds__(dev::TB) b_reduce_unpreconditioned_kernel(const IterArgs* __restrict__ A) {
+  dev::pdl_begin();
   const IterArgs& a = A[blockIdx.y];
   dev::reduce_unpreconditioned_body(a.n, a.m, a.G, a.Gold, a.Dir32, a.PG32, a.ldm, a.part, a.sc, blockIdx.x,
                                     gridDim.x);
@@ -56,6 +58,7 @@ __global__ void __launch_bounds__(dev::TB) b_reduce_unpreconditioned_kernel(cons
 // Polak-Ribiere coefficient and stopping tests: from the P G epilogue's partial sums, or (without a
 // preconditioner) from the reduction kernel's
 __global__ void __launch_bounds__(dev::TB) b_control_direction_kernel(const IterArgs* __restrict__ A) {
+  dev::pdl_begin();
   const IterArgs& a = A[blockIdx.y];
   if (a.precond) dev::control_direction_body(a.sc, a.red, 1, a.nparts, 0, 1);
   else dev::control_direction_body(a.sc, a.part, 1, kBatchReduceBlocks, 0, 1);
@@ -63,24 +66,28 @@ __global__ void __launch_bounds__(dev::TB) b_control_direction_kernel(const Iter
 
 // Delta and its split (the operand of the next two products)
 __global__ void __launch_bounds__(256) b_direction_kernel(const IterArgs* __restrict__ A) {
+  dev::pdl_begin();
   const IterArgs& a = A[blockIdx.y];
   dev::direction_split32_body(a.n, a.m, a.PG32, a.Dir32, a.D_hi, a.D_hi + (long)a.n * a.ldm, a.ldm, a.sc, blockIdx.x,
                               gridDim.x);
 }
 
 __global__ void __launch_bounds__(dev::TB) b_traces_kernel(const IterArgs* __restrict__ A) {
+  dev::pdl_begin();
   const IterArgs& a = A[blockIdx.y];
   if ((int)blockIdx.x >= a.tiles) return;
   dev::traces_body<true>(a.n, a.SWHW, a.Proj, a.part2, a.sc, blockIdx.x, a.tiles);
 }
 
 __global__ void __launch_bounds__(dev::TB) b_control_linesearch_kernel(const IterArgs* __restrict__ A) {
+  dev::pdl_begin();
   const IterArgs& a = A[blockIdx.y];
   dev::control_linesearch_body(a.sc, a.part2, a.tiles, 0, 1);
 }
 
 // the state update and the splits of the new dHC, dSC, HC, SC
 __global__ void __launch_bounds__(256) b_update_state_kernel(const IterArgs* __restrict__ A) {
+  dev::pdl_begin();
   const IterArgs& a = A[blockIdx.y];
   dev::update_state_split32_body(a.n, a.m, a.C, a.Y4, a.Dir32, a.HD32, a.dY32, a.Y_hi, a.Y_hi + 6L * a.n * a.ldm,
                                  a.ldm, a.sc, blockIdx.x, gridDim.x);
@@ -88,6 +95,7 @@ __global__ void __launch_bounds__(256) b_update_state_kernel(const IterArgs* __r
 
 // H_W, S_W and the split of [dS_W | dH_W]
 __global__ void __launch_bounds__(dev::TB) b_update_subspace_kernel(const IterArgs* __restrict__ A) {
+  dev::pdl_begin();
   const IterArgs& a = A[blockIdx.y];
   if ((int)blockIdx.x >= a.tiles) return;
   dev::update_subspace_split_body(a.n, a.SWHW, a.Proj, a.Wref, a.W_hi + 2L * a.n, a.W_hi + (long)a.n * a.ld4 + 2L * a.n,
@@ -318,22 +326,22 @@ void enqueue_line_search(omm_batch* b) {
   if (b->precond) {
     timed_gemm(b, b->gPG, tc::pairs_single());  // P G (one bf16 pass), the Polak-Ribiere products and max|G|, G_old <- G
   } else {
-    b_reduce_unpreconditioned_kernel<<<dim3(kBatchReduceBlocks, cnt), dev::TB, 0, st>>>(b->args);
+    launch_pdl(st, dim3(kBatchReduceBlocks, cnt), dim3(dev::TB), 0, b_reduce_unpreconditioned_kernel, b->args);
     OMM_LAUNCH_CHECK();
   }
-  b_control_direction_kernel<<<dim3(1, cnt), dev::TB, 0, st>>>(b->args);
+  launch_pdl(st, dim3(1, cnt), dim3(dev::TB), 0, b_control_direction_kernel, b->args);
   OMM_LAUNCH_CHECK();
-  b_direction_kernel<<<rows_grid, 256, 0, st>>>(b->args);
+  launch_pdl(st, rows_grid, dim3(256), 0, b_direction_kernel, b->args);
   OMM_LAUNCH_CHECK();
   timed_gemm(b, b->gHD, pl);  // [H D; S D] and its split
   timed_gemm(b, b->gPr, pl);
-  b_traces_kernel<<<dim3(b->max_tiles, cnt), dev::TB, 0, st>>>(b->args);
+  launch_pdl(st, dim3(b->max_tiles, cnt), dim3(dev::TB), 0, b_traces_kernel, b->args);
   OMM_LAUNCH_CHECK();
-  b_control_linesearch_kernel<<<dim3(1, cnt), dev::TB, 0, st>>>(b->args);
+  launch_pdl(st, dim3(1, cnt), dim3(dev::TB), 0, b_control_linesearch_kernel, b->args);
   OMM_LAUNCH_CHECK();
-  b_update_state_kernel<<<rows_grid, 256, 0, st>>>(b->args);
+  launch_pdl(st, rows_grid, dim3(256), 0, b_update_state_kernel, b->args);
   OMM_LAUNCH_CHECK();
-  b_update_subspace_kernel<<<dim3(b->max_tiles, cnt), dev::TB, 0, st>>>(b->args);
+  launch_pdl(st, dim3(b->max_tiles, cnt), dim3(dev::TB), 0, b_update_subspace_kernel, b->args);
   OMM_LAUNCH_CHECK();
   timed_gemm(b, b->gG, pl);  // G and its split
 }

@@ -7,6 +7,7 @@
 // It serves the float64 OMM path, the float64 refinement and certificate of
 // the mixed path, and the Cholesky inverse of the preconditioner.
 #include "omm_internal.cuh"
+#include "pdl.cuh"
 
 #include <cooperative_groups.h>
 
@@ -23,6 +24,7 @@ dgemm_kernel(int transA, int transB, int M, int N, int K, double alpha,
              const double* __restrict__ A, long lda, long sA,
              const double* __restrict__ B, long ldb, long sB,
              double beta, double* C, long ldc, long sC, int tri, const int* skip) {
+  dev::pdl_begin();
   if (skip != nullptr && (skip[0] | skip[1])) return;
   const int row0 = blockIdx.y * BM;
   const int col0 = blockIdx.x * BN;
@@ -124,6 +126,7 @@ __global__ void __launch_bounds__(NT)
 dgemm_small_kernel(int transA, int transB, int M, int N, int K, double alpha, const double* __restrict__ A, long lda,
                    long sA, const double* __restrict__ B, long ldb, long sB, double beta, double* C, long ldc,
                    long sC, int tri, const int* skip, int ks) {
+  dev::pdl_begin();
   if (skip != nullptr && (skip[0] | skip[1])) return;
   constexpr int R = T / 16;                // outputs per thread and dimension
   constexpr int LD = T * SK / NT;          // elements of each operand a thread stages
@@ -270,28 +273,30 @@ void dgemm(cudaStream_t st, int transA, int transB, int M, int N, int K, double 
            double beta, double* C, long ldc, long strideC, int batch, int tri, const int* skip) {
   if (M <= 0 || N <= 0 || batch <= 0) return;
   const Split sp = choose_split(M, N, std::max(K, 1), batch);
-  if (sp.tile == 64) {
-    dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, batch);
-    dgemm_kernel<<<grid, NT, 0, st>>>(transA, transB, M, N, K, alpha, A, lda, strideA, B, ldb,
-                                       strideB, beta, C, ldc, strideC, tri, skip);
-    OMM_LAUNCH_CHECK();
-    return;
-  }
+  // the products of a line search (those with stop flags) start early, see pdl.cuh
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(((N + sp.tile - 1) / sp.tile) * sp.ks), (unsigned)((M + sp.tile - 1) / sp.tile),
                      (unsigned)batch);
   cfg.blockDim = dim3(NT);
   cfg.stream = st;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = (unsigned)sp.ks;
-  attr.val.clusterDim.y = 1;
-  attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  auto kernel = sp.tile == 32 ? dgemm_small_kernel<32> : dgemm_small_kernel<16>;
-  OMM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, transA, transB, M, N, K, alpha, A, lda, strideA, B, ldb, strideB,
-                                  beta, C, ldc, strideC, tri, skip, sp.ks));
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = skip != nullptr ? 1 : 0;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)sp.ks;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  if (sp.tile == 64) {
+    cfg.numAttrs = 1;
+    OMM_CUDA_TRY(cudaLaunchKernelEx(&cfg, dgemm_kernel, transA, transB, M, N, K, alpha, A, lda, strideA, B, ldb, strideB,
+                                    beta, C, ldc, strideC, tri, skip));
+  } else {
+    cfg.numAttrs = 2;
+    auto kernel = sp.tile == 32 ? dgemm_small_kernel<32> : dgemm_small_kernel<16>;
+    OMM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, transA, transB, M, N, K, alpha, A, lda, strideA, B, ldb, strideB, beta,
+                                    C, ldc, strideC, tri, skip, sp.ks));
+  }
   OMM_LAUNCH_CHECK();
 }
 

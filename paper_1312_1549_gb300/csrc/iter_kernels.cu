@@ -10,6 +10,7 @@
 #include <algorithm>
 #include "iter_device.cuh"
 #include "fused_device.cuh"
+#include "pdl.cuh"
 
 namespace omm {
 namespace {
@@ -45,6 +46,7 @@ __global__ void __launch_bounds__(TB)
 grad_reduce_kernel(long count, const double* __restrict__ G, const double* __restrict__ PG,
                    const double* __restrict__ Gold, const double* __restrict__ Dir,
                    double* part, const Scalars* sc) {
+  dev::pdl_begin();
   grad_reduce_body(count, G, PG, Gold, Dir, part, sc, blockIdx.x, gridDim.x);
 }
 
@@ -54,12 +56,14 @@ grad_reduce_kernel(long count, const double* __restrict__ G, const double* __res
 // Polak-Ribiere coefficient and the stopping tests (one block).
 __global__ void __launch_bounds__(TB)
 control_direction_kernel(Scalars* sc, const double* part, int mixed, int nparts) {
+  dev::pdl_begin();
   control_direction_body(sc, part, mixed, nparts, blockIdx.x, gridDim.x);
 }
 
 
 __global__ void direction_kernel(long count, const double* __restrict__ PG, double* Dir,
                                  const Scalars* sc) {
+  dev::pdl_begin();
   direction_body(count, PG, Dir, sc, blockIdx.x, gridDim.x);
 }
 
@@ -74,6 +78,7 @@ template <bool F32>
 __global__ void __launch_bounds__(TB)
 traces_kernel(int n, const double* __restrict__ SWHW, const double* __restrict__ Proj,
               double* part, const Scalars* sc, int quarters) {
+  dev::pdl_begin();
   traces_body<F32>(n, SWHW, Proj, part, sc, blockIdx.x, gridDim.x, quarters);
 }
 
@@ -95,6 +100,7 @@ using namespace dev;
 // quartic coefficients (Eq. 13), line minimum and bookkeeping (one block)
 __global__ void __launch_bounds__(TB)
 control_linesearch_kernel(Scalars* sc, const double* part, int nblocks) {
+  dev::pdl_begin();
   control_linesearch_body(sc, part, nblocks, blockIdx.x, gridDim.x);
 }
 
@@ -102,6 +108,7 @@ control_linesearch_kernel(Scalars* sc, const double* part, int nblocks) {
 // C += x Delta; HC += x HDelta; SC += x SDelta; G_old = G; G = 8 HC (the GEMM adds -4 [..])
 __global__ void update_state_kernel(int n, long m, double* C, double* Y4, const double* Dir,
                                     double* G, double* Gold, const Scalars* sc) {
+  dev::pdl_begin();
   if (stopped(sc)) return;
   const double x = sc->x;
   const long count = (long)n * m;
@@ -125,6 +132,7 @@ __global__ void update_state_kernel(int n, long m, double* C, double* Y4, const 
 // H_W += x (H' + H'^T) + x^2 H''; S_W likewise (Eq. 16), on 32x32 tiles
 __global__ void __launch_bounds__(TB)
 update_subspace_kernel(int n, double* SWHW, const double* __restrict__ Proj, const Scalars* sc, int quarters) {
+  dev::pdl_begin();
   update_subspace_body(n, SWHW, Proj, sc, blockIdx.x, gridDim.x, quarters);
 }
 
@@ -197,15 +205,15 @@ void launch_fill(cudaStream_t st, long count, double v, double* d) {
 }
 void launch_grad_reduce(cudaStream_t st, long count, const double* G, const double* PG, const double* Gold,
                         const double* Dir, double* part, const Scalars* sc) {
-  grad_reduce_kernel<<<reduce_blocks(count), TB, 0, st>>>(count, G, PG, Gold, Dir, part, sc);
+  launch_pdl(st, dim3(reduce_blocks(count)), dim3(TB), 0, grad_reduce_kernel, count, G, PG, Gold, Dir, part, sc);
   OMM_LAUNCH_CHECK();
 }
 void launch_control_direction(cudaStream_t st, Scalars* sc, const double* part, int mixed, int nparts) {
-  control_direction_kernel<<<1, TB, 0, st>>>(sc, part, mixed, nparts);
+  launch_pdl(st, dim3(1), dim3(TB), 0, control_direction_kernel, sc, part, mixed, nparts);
   OMM_LAUNCH_CHECK();
 }
 void launch_direction(cudaStream_t st, long count, const double* PG, double* Dir, const Scalars* sc) {
-  direction_kernel<<<grid_for(count), TB, 0, st>>>(count, PG, Dir, sc);
+  launch_pdl(st, dim3(grid_for(count)), dim3(TB), 0, direction_kernel, count, PG, Dir, sc);
   OMM_LAUNCH_CHECK();
 }
 int traces_blocks(int n) {
@@ -225,17 +233,17 @@ int traces_partials(int n) {
 int reduce_blocks(long count) { return (int)std::min<long>(kReduceBlocks, (count + 1023) / 1024); }
 void launch_traces(cudaStream_t st, int n, const double* SWHW, const double* Proj, double* part,
                    const Scalars* sc, bool fp32_products) {
-  if (fp32_products) traces_kernel<true><<<traces_partials(n), TB, 0, st>>>(n, SWHW, Proj, part, sc, tile_quarters(n));
-  else traces_kernel<false><<<traces_partials(n), TB, 0, st>>>(n, SWHW, Proj, part, sc, tile_quarters(n));
+  if (fp32_products) launch_pdl(st, dim3(traces_partials(n)), dim3(TB), 0, traces_kernel<true>, n, SWHW, Proj, part, sc, tile_quarters(n));
+  else launch_pdl(st, dim3(traces_partials(n)), dim3(TB), 0, traces_kernel<false>, n, SWHW, Proj, part, sc, tile_quarters(n));
   OMM_LAUNCH_CHECK();
 }
 void launch_control_linesearch(cudaStream_t st, Scalars* sc, const double* part, int nblocks) {
-  control_linesearch_kernel<<<1, TB, 0, st>>>(sc, part, nblocks);
+  launch_pdl(st, dim3(1), dim3(TB), 0, control_linesearch_kernel, sc, part, nblocks);
   OMM_LAUNCH_CHECK();
 }
 void launch_update_state(cudaStream_t st, int n, long m, double* C, double* Y4, const double* Dir,
                          double* G, double* Gold, const Scalars* sc) {
-  update_state_kernel<<<grid_for((long)n * m), TB, 0, st>>>(n, m, C, Y4, Dir, G, Gold, sc);
+  launch_pdl(st, dim3(grid_for((long)n * m)), dim3(TB), 0, update_state_kernel, n, m, C, Y4, Dir, G, Gold, sc);
   OMM_LAUNCH_CHECK();
 }
 namespace {
@@ -252,6 +260,7 @@ update_state_split_kernel(long n, long m, double* C, double* Y4, const double* D
 __global__ void __launch_bounds__(TB)
 update_subspace_split_kernel(int n, double* SWHW, const double* __restrict__ Proj, const double* __restrict__ Wref,
                              __nv_bfloat16* Whi, __nv_bfloat16* Wlo, long ldw, const Scalars* sc, int quarters) {
+  dev::pdl_begin();
   dev::update_subspace_split_body(n, SWHW, Proj, Wref, Whi, Wlo, ldw, sc, blockIdx.x, gridDim.x, quarters);
 }
 }  // namespace
@@ -276,44 +285,47 @@ namespace {
 __global__ void __launch_bounds__(256)
 direction_split32_kernel(long n, long m, const float* PG, float* Dir, __nv_bfloat16* hi, __nv_bfloat16* lo, long ldm,
                          const Scalars* sc) {
+  dev::pdl_begin();
   dev::direction_split32_body(n, m, PG, Dir, hi, lo, ldm, sc, blockIdx.x, gridDim.x);
 }
 __global__ void __launch_bounds__(256)
 update_state_split32_kernel(long n, long m, double* C, double* Y4, const float* Dir, const float* HD32, float* dY32,
                             __nv_bfloat16* Yhi, __nv_bfloat16* Ylo, long ldm, const Scalars* sc) {
+  dev::pdl_begin();
   dev::update_state_split32_body(n, m, C, Y4, Dir, HD32, dY32, Yhi, Ylo, ldm, sc, blockIdx.x, gridDim.x);
 }
 __global__ void __launch_bounds__(TB)
 reduce_unpreconditioned_kernel(long n, long m, const double* G, double* Gold, const float* Dir, float* PG, long ldm,
                                double* part, const Scalars* sc) {
+  dev::pdl_begin();
   dev::reduce_unpreconditioned_body(n, m, G, Gold, Dir, PG, ldm, part, sc, blockIdx.x, gridDim.x);
 }
 }  // namespace
 
 void launch_direction_split32(cudaStream_t st, long n, long m, const float* PG, float* Dir, __nv_bfloat16* hi,
                               __nv_bfloat16* lo, long ldm, const Scalars* sc) {
-  direction_split32_kernel<<<pair_grid(n, m), 256, 0, st>>>(n, m, PG, Dir, hi, lo, ldm, sc);
+  launch_pdl(st, dim3(pair_grid(n, m)), dim3(256), 0, direction_split32_kernel, n, m, PG, Dir, hi, lo, ldm, sc);
   OMM_LAUNCH_CHECK();
 }
 void launch_update_state_split32(cudaStream_t st, long n, long m, double* C, double* Y4, const float* Dir,
                                  const float* HD32, float* dY32, __nv_bfloat16* Yhi, __nv_bfloat16* Ylo, long ldm,
                                  const Scalars* sc) {
-  update_state_split32_kernel<<<pair_grid(n, m), 256, 0, st>>>(n, m, C, Y4, Dir, HD32, dY32, Yhi, Ylo, ldm, sc);
+  launch_pdl(st, dim3(pair_grid(n, m)), dim3(256), 0, update_state_split32_kernel, n, m, C, Y4, Dir, HD32, dY32, Yhi, Ylo, ldm, sc);
   OMM_LAUNCH_CHECK();
 }
 void launch_reduce_unpreconditioned(cudaStream_t st, long n, long m, const double* G, double* Gold, const float* Dir,
                                     float* PG, long ldm, double* part, const Scalars* sc) {
-  reduce_unpreconditioned_kernel<<<kReduceBlocks, TB, 0, st>>>(n, m, G, Gold, Dir, PG, ldm, part, sc);
+  launch_pdl(st, dim3(kReduceBlocks), dim3(TB), 0, reduce_unpreconditioned_kernel, n, m, G, Gold, Dir, PG, ldm, part, sc);
   OMM_LAUNCH_CHECK();
 }
 void launch_update_subspace_split(cudaStream_t st, int n, double* SWHW, const double* Proj, const double* Wref,
                                   __nv_bfloat16* Whi, __nv_bfloat16* Wlo, long ldw, const Scalars* sc) {
-  update_subspace_split_kernel<<<traces_blocks(n) * tile_quarters(n), TB, 0, st>>>(n, SWHW, Proj, Wref, Whi, Wlo, ldw, sc,
+  launch_pdl(st, dim3(traces_blocks(n) * tile_quarters(n)), dim3(TB), 0, update_subspace_split_kernel, n, SWHW, Proj, Wref, Whi, Wlo, ldw, sc,
                                                                                  tile_quarters(n));
   OMM_LAUNCH_CHECK();
 }
 void launch_update_subspace(cudaStream_t st, int n, double* SWHW, const double* Proj, const Scalars* sc) {
-  update_subspace_kernel<<<traces_blocks(n) * tile_quarters(n), TB, 0, st>>>(n, SWHW, Proj, sc, tile_quarters(n));
+  launch_pdl(st, dim3(traces_blocks(n) * tile_quarters(n)), dim3(TB), 0, update_subspace_kernel, n, SWHW, Proj, sc, tile_quarters(n));
   OMM_LAUNCH_CHECK();
 }
 void launch_scale_copy(cudaStream_t st, long count, const double* src, double a, double* dst, const Scalars* sc) {

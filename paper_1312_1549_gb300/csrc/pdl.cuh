@@ -1,0 +1,37 @@
+// Programmatic dependent launch for the kernels of a line search: a kernel's launch and prologue (barriers,
+// tensor memory) lie beside the last CTAs of the kernel before it instead of after it. Every kernel launched
+// this way calls dev::pdl_begin() before it touches memory that earlier kernels write or read: it waits until
+// they are complete and their writes are visible. No kernel lets the next one start before its CTAs exit: an
+// early start fills SMs that happen to have room, and the float64-bound products then ran up to 15 % slower. A
+// line search is a chain of eleven kernels; float64 solve of m = 207, n = 36 with gradients 8.8 -> 7.0 ms, of
+// m = 416, n = 64 9.0 -> 7.8 ms.
+#pragma once
+#include <cuda_runtime.h>
+
+#include <utility>
+
+#include "omm_internal.cuh"
+
+namespace omm {
+namespace dev {
+__device__ __forceinline__ void pdl_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+}  // namespace dev
+
+template <typename... P, typename... A>
+void launch_pdl(cudaStream_t st, dim3 grid, dim3 block, size_t smem, void (*kernel)(P...), A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  OMM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...));
+}
+
+}  // namespace omm

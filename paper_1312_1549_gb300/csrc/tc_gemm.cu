@@ -22,6 +22,7 @@
 #include <cuda_bf16.h>
 
 #include "omm_internal.cuh"
+#include "pdl.cuh"
 #include "split_device.cuh"
 #include "tc_gemm.cuh"
 
@@ -610,6 +611,7 @@ __device__ __forceinline__ void persistent_body(const GroupDesc* __restrict__ gr
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
+  dev::pdl_begin();
   if (groups[0].ep.expire) {
     // tests of the timeout status: a bounded wait on a barrier nothing arrives at, before any
     // copy or MMA is issued; the CTA then only frees its tensor memory
@@ -927,6 +929,7 @@ __device__ __forceinline__ void pair_body(const GroupDesc* __restrict__ groups, 
   cluster_sync_all();  // the barriers of both CTAs are initialised before any copy, commit or arrival
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
+  dev::pdl_begin();
   if (groups[0].ep.expire) {
     // tests of the timeout status (as in the single-CTA kernel): nothing is issued
     if (threadIdx.x == 0) {
@@ -1396,7 +1399,7 @@ void gemm_persistent(cudaStream_t st, const GroupDesc* groups_dev, int ngroups, 
       throw CudaError{cudaErrorInvalidValue, "tc::gemm_persistent: SM-pair tiles are 128, 192 or 256 wide"};
     const unsigned grid = 4u * (unsigned)std::min(total_tiles, quad_clusters());
     auto go = [&](auto kernel) {
-      kernel<<<grid, NTHREADS, SMEM_BYTES, st>>>(groups_dev, ngroups, total_tiles, pl, err);
+      launch_pdl(st, dim3(grid), dim3(NTHREADS), SMEM_BYTES, kernel, groups_dev, ngroups, total_tiles, pl, err);
     };
     if (bn == 256) fused ? go(gemm_quad_kernel<256, true>) : go(gemm_quad_kernel<256, false>);
     else if (bn == 192) fused ? go(gemm_quad_kernel<192, true>) : go(gemm_quad_kernel<192, false>);
@@ -1409,7 +1412,7 @@ void gemm_persistent(cudaStream_t st, const GroupDesc* groups_dev, int ngroups, 
       throw CudaError{cudaErrorInvalidValue, "tc::gemm_persistent: SM-pair tiles are 128, 192 or 256 wide"};
     const unsigned grid = 2u * (unsigned)std::min(total_tiles, pair_clusters());
     auto go = [&](auto kernel) {
-      kernel<<<grid, NTHREADS, SMEM_BYTES, st>>>(groups_dev, ngroups, total_tiles, pl, err);
+      launch_pdl(st, dim3(grid), dim3(NTHREADS), SMEM_BYTES, kernel, groups_dev, ngroups, total_tiles, pl, err);
     };
     if (bn == 256) fused ? go(gemm_pair_kernel<256, true>) : go(gemm_pair_kernel<256, false>);
     else if (bn == 192) fused ? go(gemm_pair_kernel<192, true>) : go(gemm_pair_kernel<192, false>);
@@ -1419,7 +1422,7 @@ void gemm_persistent(cudaStream_t st, const GroupDesc* groups_dev, int ngroups, 
   }
   const unsigned grid = (unsigned)std::min(total_tiles, sm_count());
   auto go = [&](auto kernel) {
-    kernel<<<grid, NTHREADS, SMEM_BYTES, st>>>(groups_dev, ngroups, total_tiles, pl, err);
+    launch_pdl(st, dim3(grid), dim3(NTHREADS), SMEM_BYTES, kernel, groups_dev, ngroups, total_tiles, pl, err);
   };
   if (bn == 256) fused ? go(gemm_persistent_kernel<true, 256>) : go(gemm_persistent_kernel<false, 256>);
   else if (bn == 128) fused ? go(gemm_persistent_kernel<true, 128>) : go(gemm_persistent_kernel<false, 128>);
