@@ -57,6 +57,7 @@ struct MixedState {
   // one line search as a CUDA graph, with the buffers it was captured for
   cudaGraphExec_t ls_exec = nullptr;
   const void* ls_key[3] = {nullptr, nullptr, nullptr};
+  long ls_kernels = 0;
   bool ls_failed = false;
 };
 
@@ -413,6 +414,7 @@ void mixed_iterate_replay(MixedState* ms, cudaStream_t st, Scalars* sc, double* 
   const void* key[3] = {C, G, sc};
   if (ms->ls_exec && std::equal(key, key + 3, ms->ls_key)) {
     OMM_CUDA_TRY(cudaGraphLaunch(ms->ls_exec, st));
+    count_launches(ms->ls_kernels);
     return;
   }
   drop_graph(ms);
@@ -423,11 +425,14 @@ void mixed_iterate_replay(MixedState* ms, cudaStream_t st, Scalars* sc, double* 
   cudaGraph_t graph = nullptr;
   bool ok = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) == cudaSuccess;
   if (ok && cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+    const unsigned long long before = launches_counted();
     try {
       mixed_iterate(ms, cap, sc, C, Dir, G, Gold, PG, Y4, SWHW, Proj, part, part2, HS, P, precond, pf);
     } catch (...) {
       ok = false;
     }
+    ms->ls_kernels = (long)(launches_counted() - before);
+    count_launches(-ms->ls_kernels);
     ok = (cudaStreamEndCapture(cap, &graph) == cudaSuccess) && ok && graph != nullptr;
     ok = ok && cudaGraphInstantiate(&ms->ls_exec, graph, 0) == cudaSuccess;
   } else {
@@ -444,6 +449,7 @@ void mixed_iterate_replay(MixedState* ms, cudaStream_t st, Scalars* sc, double* 
   }
   std::copy(key, key + 3, ms->ls_key);
   OMM_CUDA_TRY(cudaGraphLaunch(ms->ls_exec, st));
+  count_launches(ms->ls_kernels);
 }
 
 }  // namespace omm

@@ -30,6 +30,8 @@ const char* last_error_cstr() { return g_last_error.c_str(); }
 
 std::atomic<unsigned long long> g_launches{0};
 void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
+void count_launches(long n) { g_launches.fetch_add((unsigned long long)n, std::memory_order_relaxed); }
+unsigned long long launches_counted() { return g_launches.load(); }
 
 void Profiler::begin(cudaStream_t st) {
   if (!on) return;

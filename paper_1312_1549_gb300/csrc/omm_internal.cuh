@@ -57,8 +57,11 @@ struct CudaError {
 void set_last_error(const std::string& msg);
 const char* last_error_cstr();
 
-// every kernel launch of the library is counted (omm_launch_count)
+// every kernel launch of the library is counted (omm_launch_count); a graph's kernels with each replay
+// (counted while it is captured, they are taken off again)
 void count_launch();
+void count_launches(long n);
+unsigned long long launches_counted();
 #define OMM_LAUNCH_CHECK()                   \
   do {                                       \
     ::omm::count_launch();                   \
