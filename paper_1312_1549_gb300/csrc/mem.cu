@@ -16,17 +16,19 @@ namespace mem {
 namespace {
 
 std::mutex g_mu;
-std::map<int, cudaMemPool_t> g_pools;
+std::map<int, cudaMemPool_t> g_pools;          // contexts: freed memory is kept for the next one
+std::map<int, cudaMemPool_t> g_scratch_pools;  // scratch of single calls: at most kScratchKeep stays reserved
+constexpr uint64_t kScratchKeep = 2ull << 30;
 
-cudaMemPool_t pool_of_current_device() {
+cudaMemPool_t pool_of_current_device(std::map<int, cudaMemPool_t>& pools, uint64_t keep) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) {
     cudaGetLastError();
     throw std::bad_alloc();
   }
   std::lock_guard<std::mutex> lock(g_mu);
-  auto it = g_pools.find(dev);
-  if (it != g_pools.end()) return it->second;
+  auto it = pools.find(dev);
+  if (it != pools.end()) return it->second;
   cudaMemPoolProps props{};
   props.allocType = cudaMemAllocationTypePinned;
   props.location.type = cudaMemLocationTypeDevice;
@@ -36,22 +38,29 @@ cudaMemPool_t pool_of_current_device() {
     cudaGetLastError();
     throw std::bad_alloc();
   }
-  uint64_t keep = UINT64_MAX;  // keep freed memory for reuse (no release at synchronisation points)
+  // what is reserved beyond `keep` goes back to the driver at the next synchronisation point
   cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
-  g_pools[dev] = pool;
+  pools[dev] = pool;
   return pool;
 }
 
-}  // namespace
-
-void* alloc(size_t bytes, cudaStream_t st) {
-  cudaMemPool_t pool = pool_of_current_device();
+void* alloc_from(cudaMemPool_t pool, size_t bytes, cudaStream_t st) {
   void* p = nullptr;
   if (cudaMallocFromPoolAsync(&p, bytes ? bytes : 1, pool, st) != cudaSuccess) {
     cudaGetLastError();
     throw std::bad_alloc();
   }
   return p;
+}
+
+}  // namespace
+
+void* alloc(size_t bytes, cudaStream_t st) {
+  return alloc_from(pool_of_current_device(g_pools, UINT64_MAX), bytes, st);
+}
+
+void* alloc_scratch(size_t bytes, cudaStream_t st) {
+  return alloc_from(pool_of_current_device(g_scratch_pools, kScratchKeep), bytes, st);
 }
 
 void release(void* p, cudaStream_t st) {

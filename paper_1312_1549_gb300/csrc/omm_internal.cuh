@@ -80,6 +80,8 @@ unsigned long long launches_counted();
 // streams after a synchronisation with st. release(nullptr) is ignored.
 namespace mem {
 void* alloc(size_t bytes, cudaStream_t st);
+// the same from a second pool that keeps at most 2 GiB reserved (scratch of the step-level entry points)
+void* alloc_scratch(size_t bytes, cudaStream_t st);
 void release(void* p, cudaStream_t st);
 template <typename T>
 void alloc(T** p, size_t count, cudaStream_t st) {
