@@ -352,6 +352,7 @@ omm_status omm_create(int m, int n, const double* H, const double* S, const doub
     OMM_CUDA_TRY(cudaMallocHost((void**)&c->sc_host, sizeof(Scalars)));
     dev_alloc(&c->sc, 1, c->st);
     dev_alloc(&c->info_dev, 1, c->st);
+    OMM_CUDA_TRY(cudaMemsetAsync(c->info_dev, 0, sizeof(int), c->st));  // read below also where nothing is factored
     dev_alloc(&c->HS, 2 * mm, c->st);
     OMM_CUDA_TRY(cudaEventRecord(c->ev[0], c->st));
     copy_in(c->HS, H, mm, c->st);
