@@ -41,9 +41,10 @@ omm_status omm_kernel_spd_inverse(int m, const double* A, double* P, int* info, 
  * scheme; about 2^-50 of each row-scaled operand), with the 64 x 64 diagonal
  * blocks factored and inverted in float64. Arguments, ownership and *info as
  * for omm_kernel_spd_inverse; OMM_ERR_TIMEOUT if a bounded wait of a tensor-core
- * GEMM expired. Workspace (allocated inside the call): about 2.3 m^2 float64 plus
- * 20 m^2 bytes of slices and up to 430 MB of chunk sums; a second stream runs the
- * Y^T Y updates beside the factorisation and is joined before the call returns. */
+ * GEMM expired. Workspace (from the library's scratch pool, given back by the call):
+ * about 2.8 m^2 float64 plus 33 m^2 bytes of slices and 240 MB of float64 sums; two more
+ * streams run the products that the factorisation does not wait for and are joined
+ * before the call returns. */
 omm_status omm_kernel_spd_inverse_sliced(int m, const double* A, double* P, int* info, void* stream);
 
 /* The preconditioner-grade variant the mixed solver uses (omm_opts.precond_slices): the same

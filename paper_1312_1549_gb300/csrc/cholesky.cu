@@ -16,13 +16,19 @@
 // halves so that every product has a long contraction:
 //   chol_inv([A11 A21^T; A21 A22]):  L11, Y11 = chol_inv(A11);
 //     L21 = A21 Y11^T;  A22 -= L21 L21^T;  L22, Y22 = chol_inv(A22);
-//     Y21 = -(Y22 L21) Y11                         (Y = L^-1)
+//     Y21 = -Y22 (L21 Y11)                         (Y = L^-1)
 //   lauum(Y) = Y^T Y:  P22 = lauum(Y22);  P21 = Y22^T Y21;
 //     P11 = lauum(Y11) + Y21^T Y21
 // with leaves factored and inverted by one CTA (which also writes the leaf's block of Y^T Y):
 // 64 x 64 in float64 for float64-class results, 128 x 128 in float32 for the preconditioner. The
 // P updates of a node run on a second stream as soon as its Y is final, beside the factorisation
-// of the blocks that follow.
+// of the blocks that follow. W = L21 Y11 does not need the right half, so it runs on a third stream
+// beside that half's factorisation: the chain of a node is three products instead of the four that
+// -(Y22 L21) Y11 makes, and neither transposes nor copies. The chain is what bounds the inverse (51 nodes one
+// after another at m = 3328): float64-class inverse 17.9 -> 15.7 ms, Cholesky-flavour solve of m = 2944
+// 46.4 -> 44.3 ms. W and Y21 take one slice more than the other products: sliced by columns W loses more than
+// Y22 L21 by rows, and the error of P would be up to 30 % larger than in that order; with the extra slice it is
+// 5 to 25 % smaller (against a refined inverse, m = 160 to 3328), for 3 % of the time.
 #include "emu.cuh"
 #include "omm_internal.cuh"
 #include "split_device.cuh"
@@ -511,7 +517,39 @@ void spd_factor_inverse(cudaStream_t st, int m, double* A, double* Y, double* wo
 // ------------------------------------------------------------------ float64-class (sliced) variant
 namespace {
 
-constexpr int kInvSlices = 10;  // the most slices a product of this file takes (workspace sizing)
+// Streams beside the caller's and the events between them. They may be released with work pending: the driver
+// frees them once it is done.
+struct Streams {
+  std::vector<cudaEvent_t> events;
+  std::vector<cudaStream_t> streams;
+
+  Streams() = default;
+  Streams(const Streams&) = delete;
+  Streams& operator=(const Streams&) = delete;
+  ~Streams() {
+    for (cudaStream_t s : streams) cudaStreamDestroy(s);
+    for (cudaEvent_t e : events) cudaEventDestroy(e);
+  }
+  // a stream that starts after what `from` holds so far
+  cudaStream_t fork(cudaStream_t from) {
+    cudaStream_t s = nullptr;
+    OMM_CUDA_TRY(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+    streams.push_back(s);
+    wait(s, from);
+    return s;
+  }
+  cudaEvent_t record(cudaStream_t st) {
+    cudaEvent_t e = nullptr;
+    OMM_CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    events.push_back(e);
+    OMM_CUDA_TRY(cudaEventRecord(e, st));
+    return e;
+  }
+  // `st` goes on after what `other` holds so far
+  void wait(cudaStream_t st, cudaStream_t other) { OMM_CUDA_TRY(cudaStreamWaitEvent(st, record(other), 0)); }
+};
+
+constexpr int kInvSlices = 10;  // the most slices of a lane's products; W and Y21 take one more (workspace sizing)
 
 long round8(long x) { return (x + 7) / 8 * 8; }
 
@@ -526,26 +564,25 @@ struct Lane {
   double* slab = nullptr;     // float64 sums of the sliced products
 };
 
-struct SlicedWork {
+struct SlicedWork : Streams {
   int m = 0;
   int nb = NB;               // leaf edge: 64 (float64 leaves) or 128 (float32 leaves)
-  double* A = nullptr;       // the matrix, factor L in its lower triangle
+  double* A = nullptr;       // the matrix, factor L in its lower triangle; blocks above the diagonal take W^T
   double* Y = nullptr;       // L^-1 (lower triangle, zero above)
   double* P = nullptr;
-  double* prod = nullptr;    // one product of the factorisation
   double* leaf = nullptr;    // nb x nb inverse of a diagonal block
   int* info = nullptr;
   int* err = nullptr;
-  Lane main, side;           // factorisation and inverse on `main`; the P = Y^T Y updates on `side`
-  std::vector<cudaEvent_t> events;
+  // factorisation and inverse on `main`; the P = Y^T Y updates on `side`; the products W on `ahead`
+  Lane main, side, ahead;
 };
 
 // C (M x N, ldc) = alpha A B^T + beta C with A (M x K, lda) and B (N x K, ldb) row-major;
-// the slices of A go to sl0, those of B to sl1 (or B = A: one slicing, both maps)
+// the slices of A go to sl0, those of B to sl1 (or B = A: one slicing, both maps); `more` slices than the lane's
 void sliced_nt(Lane& L, int* err, int M, int N, int K, double alpha, const double* A, long lda, const double* B,
-               long ldb, double beta, double* C, long ldc) {
+               long ldb, double beta, double* C, long ldc, int more = 0) {
   const long ld = round8(K);
-  const int s = L.slices;
+  const int s = L.slices + more;
   emu::slice_rows(L.st, A, M, K, lda, s, L.sl0, ld, nullptr);
   const tc::Operand oa = tc::make_operand(L.sl0, M, K, ld, s, true);
   tc::Operand ob;
@@ -604,29 +641,26 @@ void chol_inv(SlicedWork& w, int r0, int b) {
   chol_inv(w, r0, b1);
   double* A21 = w.A + (long)r1 * m + r0;
   double* A22 = w.A + (long)r1 * m + r1;
+  double* A12 = w.A + (long)r0 * m + r1;
   const double* Y11 = w.Y + (long)r0 * m + r0;
   const double* Y22 = w.Y + (long)r1 * m + r1;
   double* Y21 = w.Y + (long)r1 * m + r0;
-  // L21 = A21 Y11^T (to scratch, then over A21)
-  sliced_nt(L, w.err, b2, b1, b1, 1.0, A21, m, Y11, m, 0.0, w.prod, b1);
-  OMM_CUDA_TRY(cudaMemcpy2DAsync(A21, sizeof(double) * m, w.prod, sizeof(double) * b1, sizeof(double) * b1, b2,
-                                 cudaMemcpyDeviceToDevice, L.st));
+  // L21 = A21 Y11^T, over A21 (the product reads slices)
+  sliced_nt(L, w.err, b2, b1, b1, 1.0, A21, m, Y11, m, 0.0, A21, m);
+  w.wait(w.ahead.st, L.st);
+  // W^T = Y11^T L21^T, over A12, which nothing reads (Y11^T: b1 x b1)
+  emu::transpose(w.ahead.st, Y11, b1, b1, m, w.ahead.tr0, b1);
+  sliced_nt(w.ahead, w.err, b1, b2, b1, 1.0, w.ahead.tr0, b1, A21, m, 0.0, A12, m, 1);
+  cudaEvent_t done = w.record(w.ahead.st);
   // A22 -= L21 L21^T
   sliced_nt(L, w.err, b2, b2, b1, -1.0, A21, m, A21, m, 1.0, A22, m);
   chol_inv(w, r1, b2);
-  // Z = Y22 L21 (b2 x b1): B operand L21^T (b1 x b2)
-  emu::transpose(L.st, A21, b2, b1, m, L.tr0, b2);
-  sliced_nt(L, w.err, b2, b1, b2, 1.0, Y22, m, L.tr0, b2, 0.0, w.prod, b1);
-  // Y21 = -Z Y11: B operand Y11^T (b1 x b1)
-  emu::transpose(L.st, Y11, b1, b1, m, L.tr1, b1);
-  sliced_nt(L, w.err, b2, b1, b1, -1.0, w.prod, b1, L.tr1, b1, 0.0, Y21, m);
+  // Y21 = -Y22 W
+  OMM_CUDA_TRY(cudaStreamWaitEvent(L.st, done, 0));
+  sliced_nt(L, w.err, b2, b1, b2, -1.0, Y22, m, A12, m, 0.0, Y21, m, 1);
   if (w.P == nullptr) return;  // the factor and its inverse only
   // this node's Y is final: its P updates may start
-  cudaEvent_t ev = nullptr;
-  OMM_CUDA_TRY(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
-  w.events.push_back(ev);
-  OMM_CUDA_TRY(cudaEventRecord(ev, L.st));
-  OMM_CUDA_TRY(cudaStreamWaitEvent(w.side.st, ev, 0));
+  w.wait(w.side.st, L.st);
   p_update(w, r0, b1, b2);
 }
 
@@ -634,11 +668,11 @@ void chol_inv(SlicedWork& w, int r0, int b) {
 // The same recursion with every operand kept as a bf16 pair in an m x m matrix of its own: A (the part still
 // to be factored), L and Y = L^-1. The products read blocks of these matrices where they stand -- transposed
 // factors as MN-major operands -- and their epilogues write the split of the result beside or instead of
-// the float64 one, so a node of the recursion is four products on the main stream and two on the side
-// stream, with no operand to split, transpose or copy (that was fourteen launches on the main stream, on a
+// the float64 one, so a node of the recursion is four products on the main stream and two beside it,
+// with no operand to split, transpose or copy (that was fourteen launches on the main stream, on a
 // chain that runs node after node). Only A and P exist in float64: the leaves and the updates of A read A,
 // P is the result.
-struct SplitInverse {
+struct SplitInverse : Streams {
   int m = 0;
   long ld = 0;
   double* A = nullptr;
@@ -647,7 +681,6 @@ struct SplitInverse {
   int* info = nullptr;
   int* err = nullptr;
   cudaStream_t st = nullptr, side = nullptr;
-  std::vector<cudaEvent_t> events;
 
   enum Role { kA, kB };
   // block (r0, c0) as an operand: rows x cols with cols contracted, or (mn) rows contracted
@@ -692,11 +725,7 @@ struct SplitInverse {
     emu::gemm_split(st, view(As, r1, r0, b2, b1, kA, false), view(Ys, r0, r0, b1, b1, kB, true), b1,
                     into(Ys, r1, r0, b2, b1, -1.0));
     // this node's Y is final: its part of P = Y^T Y, beside the factorisation of the blocks that follow
-    cudaEvent_t ev = nullptr;
-    OMM_CUDA_TRY(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
-    events.push_back(ev);
-    OMM_CUDA_TRY(cudaEventRecord(ev, st));
-    OMM_CUDA_TRY(cudaStreamWaitEvent(side, ev, 0));
+    wait(side, st);
     const tc::Operand y21 = view(Ys, r1, r0, b2, b1, kB, true);
     // P21 = Y22^T Y21; P11 += Y21^T Y21
     emu::gemm_split(side, view(Ys, r1, r1, b2, b2, kA, true), y21, b2,
@@ -710,11 +739,10 @@ struct SplitInverse {
 
 size_t spd_inverse_sliced_workspace_bytes(int m) {
   const long h = (m + 1) / 2 + NL;  // the largest off-diagonal block edge (either leaf size)
-  // Y, prod, leaf; per lane: tr0, tr1, slab
-  const size_t f64 = (size_t)m * m + (size_t)h * h + (size_t)NL * NL +
-                     2 * (2 * (size_t)h * h + (size_t)tc::sliced_workspace_doubles());
-  const size_t bf = 2 * 2 * (size_t)kInvSlices * (size_t)h * round8(h);  // per lane: sl0, sl1
-  // (the split form's three pairs of m x m need less: 12 m round8(m) bytes of these 38 m^2 and more)
+  // Y, leaf; tr0, tr1 of one lane, tr0 of another; a slab per lane
+  const size_t f64 = (size_t)m * m + (size_t)NL * NL + 3 * ((size_t)h * h + (size_t)tc::sliced_workspace_doubles());
+  const size_t bf = 3 * 2 * (size_t)(kInvSlices + 1) * (size_t)h * round8(h);  // per lane: sl0, sl1
+  // (the split form's three pairs of m x m need less: 12 m round8(m) bytes of these 47 m^2 and more)
   return f64 * sizeof(double) + bf * sizeof(__nv_bfloat16) + 4 * 256;
 }
 
@@ -740,36 +768,16 @@ void split_impl(cudaStream_t st, int m, double* A, double* P, void* work, int* i
   w.Ls = w.Ys + pair;
   w.As = w.Ls + pair;
   prepare_leaf();
-  OMM_CUDA_TRY(cudaStreamCreateWithFlags(&w.side, cudaStreamNonBlocking));
-  // streams and events may be released with work pending: the driver frees them once it is done
-  auto cleanup = [&]() {
-    cudaStreamDestroy(w.side);
-    for (cudaEvent_t e : w.events) cudaEventDestroy(e);
-  };
-  try {
-    OMM_CUDA_TRY(cudaMemsetAsync(info_dev, 0, sizeof(int), st));
-    // zeros above the diagonal of Y; and every element a copy may touch past the end of a block (it meets
-    // zeros of the other operand) has to be a number
-    OMM_CUDA_TRY(cudaMemsetAsync(w.Ys, 0, 2 * pair * sizeof(__nv_bfloat16), st));
-    OMM_CUDA_TRY(cudaMemsetAsync(P, 0, sizeof(double) * m * (size_t)m, st));
-    tc::split(st, A, m, m, m, w.As, w.As + m * w.ld, w.ld, nullptr);
-    cudaEvent_t ready = nullptr;  // the side stream starts after the memsets
-    OMM_CUDA_TRY(cudaEventCreateWithFlags(&ready, cudaEventDisableTiming));
-    w.events.push_back(ready);
-    OMM_CUDA_TRY(cudaEventRecord(ready, st));
-    OMM_CUDA_TRY(cudaStreamWaitEvent(w.side, ready, 0));
-    w.node(0, m);
-    cudaEvent_t done = nullptr;  // join: the main stream waits for the last P update
-    OMM_CUDA_TRY(cudaEventCreateWithFlags(&done, cudaEventDisableTiming));
-    w.events.push_back(done);
-    OMM_CUDA_TRY(cudaEventRecord(done, w.side));
-    OMM_CUDA_TRY(cudaStreamWaitEvent(st, done, 0));
-    launch_symmetrize_lower(st, m, P);
-  } catch (...) {
-    cleanup();
-    throw;
-  }
-  cleanup();
+  OMM_CUDA_TRY(cudaMemsetAsync(info_dev, 0, sizeof(int), st));
+  // zeros above the diagonal of Y; and every element a copy may touch past the end of a block (it meets
+  // zeros of the other operand) has to be a number
+  OMM_CUDA_TRY(cudaMemsetAsync(w.Ys, 0, 2 * pair * sizeof(__nv_bfloat16), st));
+  OMM_CUDA_TRY(cudaMemsetAsync(P, 0, sizeof(double) * m * (size_t)m, st));
+  tc::split(st, A, m, m, m, w.As, w.As + m * w.ld, w.ld, nullptr);
+  w.side = w.fork(st);
+  w.node(0, m);
+  w.wait(st, w.side);
+  launch_symmetrize_lower(st, m, P);
 }
 
 // P = A^-1 (P != nullptr) and/or L, Y = L^-1 (Y_out != nullptr: A keeps L, zero above the diagonal)
@@ -787,62 +795,44 @@ void sliced_impl(cudaStream_t st, int m, double* A, double* P, double* Y_out, vo
   double* f = static_cast<double*>(work);
   w.Y = Y_out ? Y_out : f;
   f += (long)m * m;
-  w.prod = f;
-  f += h * h;
   w.leaf = f;
   f += NL * NL;
-  for (Lane* L : {&w.main, &w.side}) {
-    L->tr0 = f;
+  for (double** t : {&w.side.tr0, &w.side.tr1, &w.ahead.tr0}) {
+    *t = f;
     f += h * h;
-    L->tr1 = f;
-    f += h * h;
+  }
+  for (Lane* L : {&w.main, &w.side, &w.ahead}) {
     L->slab = f;
     f += tc::sliced_workspace_doubles();
   }
   uintptr_t p = (reinterpret_cast<uintptr_t>(f) + 255) & ~uintptr_t(255);
-  const size_t sl = (size_t)kInvSlices * h * round8(h);
-  w.main.sl0 = reinterpret_cast<__nv_bfloat16*>(p);
-  w.main.sl1 = w.main.sl0 + sl;
-  w.side.sl0 = w.main.sl1 + sl;
-  w.side.sl1 = w.side.sl0 + sl;
-  w.main.st = st;
-  w.main.slices = w.side.slices = std::min(std::max(slices, 2), kInvSlices);
-  if (w.nb == NL) prepare_leaf();
-  if (P) OMM_CUDA_TRY(cudaStreamCreateWithFlags(&w.side.st, cudaStreamNonBlocking));
-  // streams and events may be released with work pending: the driver frees them once it is done
-  auto cleanup = [&]() {
-    if (w.side.st) cudaStreamDestroy(w.side.st);
-    for (cudaEvent_t e : w.events) cudaEventDestroy(e);
-  };
-  try {
-    OMM_CUDA_TRY(cudaMemsetAsync(info_dev, 0, sizeof(int), st));
-    OMM_CUDA_TRY(cudaMemsetAsync(w.Y, 0, sizeof(double) * m * (size_t)m, st));
-    if (P) {
-      OMM_CUDA_TRY(cudaMemsetAsync(P, 0, sizeof(double) * m * (size_t)m, st));
-      cudaEvent_t ready = nullptr;  // the side lane starts after the memsets
-      OMM_CUDA_TRY(cudaEventCreateWithFlags(&ready, cudaEventDisableTiming));
-      w.events.push_back(ready);
-      OMM_CUDA_TRY(cudaEventRecord(ready, st));
-      OMM_CUDA_TRY(cudaStreamWaitEvent(w.side.st, ready, 0));
-    }
-    chol_inv(w, 0, m);
-    if (P) {
-      cudaEvent_t done = nullptr;  // join: the main lane waits for the last P update
-      OMM_CUDA_TRY(cudaEventCreateWithFlags(&done, cudaEventDisableTiming));
-      w.events.push_back(done);
-      OMM_CUDA_TRY(cudaEventRecord(done, w.side.st));
-      OMM_CUDA_TRY(cudaStreamWaitEvent(st, done, 0));
-      launch_symmetrize_lower(st, m, P);
-    }
-    if (Y_out) {
-      zero_upper_kernel<<<1024, 256, 0, st>>>(m, A);
-      OMM_LAUNCH_CHECK();
-    }
-  } catch (...) {
-    cleanup();
-    throw;
+  const size_t sl = (size_t)(kInvSlices + 1) * h * round8(h);
+  __nv_bfloat16* q = reinterpret_cast<__nv_bfloat16*>(p);
+  for (Lane* L : {&w.main, &w.side, &w.ahead}) {
+    L->sl0 = q;
+    L->sl1 = q + sl;
+    L->slices = std::min(std::max(slices, 2), kInvSlices);
+    q += 2 * sl;
   }
-  cleanup();
+  w.main.st = st;
+  if (w.nb == NL) prepare_leaf();
+  OMM_CUDA_TRY(cudaMemsetAsync(info_dev, 0, sizeof(int), st));
+  OMM_CUDA_TRY(cudaMemsetAsync(w.Y, 0, sizeof(double) * m * (size_t)m, st));
+  if (P) {
+    OMM_CUDA_TRY(cudaMemsetAsync(P, 0, sizeof(double) * m * (size_t)m, st));
+    w.side.st = w.fork(st);
+  }
+  w.ahead.st = w.fork(st);
+  chol_inv(w, 0, m);
+  w.wait(st, w.ahead.st);
+  if (P) {
+    w.wait(st, w.side.st);
+    launch_symmetrize_lower(st, m, P);
+  }
+  if (Y_out) {
+    zero_upper_kernel<<<1024, 256, 0, st>>>(m, A);
+    OMM_LAUNCH_CHECK();
+  }
 }
 
 }  // namespace

@@ -41,8 +41,8 @@ struct Operand {
 // whose products are summed in FP32 accumulators of their own (one, or several
 // over parts of the contraction) and added in float64. nchunk = 0: all pairs
 // form one chunk. Chunks are honoured by gemm_sliced only.
-constexpr int kMaxPairs = 64;
-constexpr int kMaxChunks = 32;
+constexpr int kMaxPairs = 72;
+constexpr int kMaxChunks = 36;
 struct PairList {
   int n;
   unsigned char a[kMaxPairs];
