@@ -31,6 +31,7 @@
 // 5 to 25 % smaller (against a refined inverse, m = 160 to 3328), for 3 % of the time.
 #include "emu.cuh"
 #include "omm_internal.cuh"
+#include "pdl.cuh"
 #include "split_device.cuh"
 #include "tc_gemm.cuh"
 
@@ -60,6 +61,7 @@ constexpr int kLeaf64Threads = 256;
 
 __global__ void __launch_bounds__(kLeaf64Threads)
 leaf_f64_kernel(double* A, long lda, int b, double* Linv, int* info, int col_offset, double* Pblk, long ldp) {
+  dev::pdl_begin();
   __shared__ double L[NB][NB + 1];
   __shared__ double X[NB][NB + 1];
   __shared__ double rdiag[NB], pivot[NB];
@@ -239,6 +241,7 @@ __device__ __forceinline__ double to_f64(float v) { return dev::f64_of_f32(v); }
 __global__ void __launch_bounds__(kLeafThreads)
 leaf_f32_kernel(const double* A, long lda, int b, double* Linv, __nv_bfloat16* Xhi, __nv_bfloat16* Xlo, long ldx,
                 int* info, int col_offset, double* Pblk, long ldp) {
+  dev::pdl_begin();
   extern __shared__ float smf[];
   float (*L)[NL + 1] = reinterpret_cast<float (*)[NL + 1]>(smf);
   float (*X)[NL + 1] = reinterpret_cast<float (*)[NL + 1]>(smf + NL * (NL + 1));
@@ -423,11 +426,17 @@ __global__ void zero_upper_kernel(int m, double* A) {
   }
 }
 
-__global__ void copy_block_kernel(int b, const double* src, long lds, double* dst, long ldd) {
-  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < b * b; idx += gridDim.x * blockDim.x) {
-    const int i = idx / b, j = idx % b;
+__global__ void copy_block_kernel(int rows, int cols, const double* src, long lds, double* dst, long ldd) {
+  dev::pdl_begin();
+  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < rows * cols; idx += gridDim.x * blockDim.x) {
+    const int i = idx / cols, j = idx % cols;
     dst[(long)i * ldd + j] = src[(long)i * lds + j];
   }
+}
+void copy_block(cudaStream_t st, int rows, int cols, const double* src, long lds, double* dst, long ldd) {
+  const int blocks = std::max(1, std::min((rows * cols + 255) / 256, 608));
+  launch_pdl(st, dim3(blocks), dim3(256), 0, copy_block_kernel, rows, cols, src, lds, dst, ldd);
+  OMM_LAUNCH_CHECK();
 }
 
 struct Work {
@@ -440,9 +449,7 @@ void trtri_rec(cudaStream_t st, int m, double* Y, const Work& w, int r0, int r1)
   const int nb_blocks = (r1 - r0 + NB - 1) / NB;
   if (nb_blocks <= 1) {
     const int b = r1 - r0;
-    copy_block_kernel<<<16, 256, 0, st>>>(b, w.Dinv + (long)(r0 / NB) * NB * NB, NB,
-                                          Y + (long)r0 * m + r0, m);
-    OMM_LAUNCH_CHECK();
+    copy_block(st, b, b, w.Dinv + (long)(r0 / NB) * NB * NB, NB, Y + (long)r0 * m + r0, m);
     return;
   }
   const int mid = r0 + (nb_blocks / 2) * NB;
@@ -475,15 +482,15 @@ void factor_blocked(cudaStream_t st, int m, double* A, const Work& w, int* info_
     const int k = kb * NB;
     const int b = (m - k < NB) ? (m - k) : NB;
     double* Akk = A + (long)k * m + k;
-    leaf_f64_kernel<<<1, kLeaf64Threads, 0, st>>>(Akk, m, b, w.Dinv + (long)kb * NB * NB, info_dev, k, nullptr, 0);
+    launch_pdl(st, dim3(1), dim3(kLeaf64Threads), 0, leaf_f64_kernel, Akk, m, b, w.Dinv + (long)kb * NB * NB, info_dev, k,
+               nullptr, 0);
     OMM_LAUNCH_CHECK();
     const int r = m - k - b;
     if (r > 0) {
       double* A21 = A + (long)(k + b) * m + k;
       // L21 = A21 * Linv^T (to scratch, then back)
       dgemm(st, 0, 1, r, b, b, 1.0, A21, m, 0, w.Dinv + (long)kb * NB * NB, NB, 0, 0.0, w.tmp, b, 0);
-      OMM_CUDA_TRY(cudaMemcpy2DAsync(A21, sizeof(double) * m, w.tmp, sizeof(double) * b,
-                                     sizeof(double) * b, r, cudaMemcpyDeviceToDevice, st));
+      copy_block(st, r, b, w.tmp, b, A21, m);
       // A22 -= L21 L21^T (lower tiles)
       double* A22 = A + (long)(k + b) * m + (k + b);
       dgemm(st, 0, 1, r, r, b, -1.0, A21, m, 0, A21, m, 0, 1.0, A22, m, 0, 1, kTriLower);
@@ -600,13 +607,13 @@ void leaf(SlicedWork& w, int r0, int b) {
   const long m = w.m;
   double* pb = w.P ? w.P + r0 * m + r0 : nullptr;
   if (w.nb == NL)  // a preconditioner: 128-wide float32 leaves (see leaf_f32_kernel)
-    leaf_f32_kernel<<<1, kLeafThreads, kLeafSmem, w.main.st>>>(w.A + r0 * m + r0, m, b, w.leaf, nullptr, nullptr, 0,
-                                                               w.info, r0, pb, m);
+    launch_pdl(w.main.st, dim3(1), dim3(kLeafThreads), kLeafSmem, leaf_f32_kernel, w.A + r0 * m + r0, m, b, w.leaf,
+               nullptr, nullptr, 0, w.info, r0, pb, m);
   else
-    leaf_f64_kernel<<<1, kLeaf64Threads, 0, w.main.st>>>(w.A + r0 * m + r0, m, b, w.leaf, w.info, r0, pb, m);
+    launch_pdl(w.main.st, dim3(1), dim3(kLeaf64Threads), 0, leaf_f64_kernel, w.A + r0 * m + r0, m, b, w.leaf, w.info, r0,
+               pb, m);
   OMM_LAUNCH_CHECK();
-  copy_block_kernel<<<16, 256, 0, w.main.st>>>(b, w.leaf, w.nb, w.Y + r0 * m + r0, m);
-  OMM_LAUNCH_CHECK();
+  copy_block(w.main.st, b, b, w.leaf, w.nb, w.Y + r0 * m + r0, m);
 }
 
 int half_of(int b, int nb) { return ((b / nb + 1) / 2) * nb; }  // a multiple of nb, about b / 2
@@ -701,7 +708,8 @@ struct SplitInverse : Streams {
     if (b <= NL) {
       __nv_bfloat16* y = Ys + r0 * ld + r0;
       const long at = (long)r0 * m + r0;
-      leaf_f32_kernel<<<1, kLeafThreads, kLeafSmem, st>>>(A + at, m, b, nullptr, y, y + m * ld, ld, info, r0, P + at, m);
+      launch_pdl(st, dim3(1), dim3(kLeafThreads), kLeafSmem, leaf_f32_kernel, A + at, m, b, nullptr, y, y + m * ld, ld, info,
+                 r0, P + at, m);
       OMM_LAUNCH_CHECK();
       return;
     }

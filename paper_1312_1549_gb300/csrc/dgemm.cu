@@ -273,7 +273,6 @@ void dgemm(cudaStream_t st, int transA, int transB, int M, int N, int K, double 
            double beta, double* C, long ldc, long strideC, int batch, int tri, const int* skip) {
   if (M <= 0 || N <= 0 || batch <= 0) return;
   const Split sp = choose_split(M, N, std::max(K, 1), batch);
-  // the products of a line search (those with stop flags) start early, see pdl.cuh
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(((N + sp.tile - 1) / sp.tile) * sp.ks), (unsigned)((M + sp.tile - 1) / sp.tile),
                      (unsigned)batch);
@@ -281,7 +280,7 @@ void dgemm(cudaStream_t st, int transA, int transB, int M, int N, int K, double 
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = skip != nullptr ? 1 : 0;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;  // see pdl.cuh
   attr[1].id = cudaLaunchAttributeClusterDimension;
   attr[1].val.clusterDim.x = (unsigned)sp.ks;
   attr[1].val.clusterDim.y = 1;

@@ -19,6 +19,7 @@
 // 1e-10 of |A||B| at K = 1000.) With s = 10 slices the result carries about
 // 50 bits of each row-scaled operand.
 #include "emu.cuh"
+#include "pdl.cuh"
 #include "tc_gemm.cuh"
 
 #include <algorithm>
@@ -47,6 +48,7 @@ template <int TPR, int CH>
 __global__ void __launch_bounds__(TPR < 256 ? 256 : TPR)
 slice_rows_kernel(const double* __restrict__ src, long rows, long cols, long ld_src, int s,
                   __nv_bfloat16* __restrict__ dst, long ld_dst, long slice_stride, const Scalars* sc) {
+  dev::pdl_begin();
   constexpr int THREADS = TPR < 256 ? 256 : TPR, RPB = THREADS / TPR, WPR = TPR / 32;
   if (stopped(sc)) return;
   const int sub = threadIdx.x / TPR, t = threadIdx.x % TPR;
@@ -155,6 +157,7 @@ slice_rows_kernel(const double* __restrict__ src, long rows, long cols, long ld_
 // dst (cols x rows) = src^T, 32 x 32 shared-memory tiles
 __global__ void transpose_kernel(const double* __restrict__ src, long rows, long cols, long ld_src,
                                  double* __restrict__ dst, long ld_dst) {
+  dev::pdl_begin();
   __shared__ double tile[32][33];
   const long tiles_c = (cols + 31) / 32;
   const long r0 = (blockIdx.x / tiles_c) * 32, c0 = (blockIdx.x % tiles_c) * 32;
@@ -185,8 +188,8 @@ void slice_rows(cudaStream_t st, const double* src, long rows, long cols, long l
                 __nv_bfloat16* dst, long ld_dst, const Scalars* sc) {
   if (rows <= 0) return;
   auto go = [&](auto kernel, int threads, int rows_per_block) {
-    kernel<<<(unsigned)((rows + rows_per_block - 1) / rows_per_block), threads, 0, st>>>(
-        src, rows, cols, ld_src, s, dst, ld_dst, rows * ld_dst, sc);
+    launch_pdl(st, dim3((unsigned)((rows + rows_per_block - 1) / rows_per_block)), dim3(threads), 0, kernel, src, rows,
+               cols, ld_src, s, dst, ld_dst, rows * ld_dst, sc);
     OMM_LAUNCH_CHECK();
   };
   // a row's threads: as few as hold it in registers (4 CH TPR columns), so that short rows fill whole warps
@@ -198,7 +201,7 @@ void slice_rows(cudaStream_t st, const double* src, long rows, long cols, long l
 
 void transpose(cudaStream_t st, const double* src, long rows, long cols, long ld_src, double* dst, long ld_dst) {
   const long blocks = ((rows + 31) / 32) * ((cols + 31) / 32);
-  transpose_kernel<<<(unsigned)blocks, 256, 0, st>>>(src, rows, cols, ld_src, dst, ld_dst);
+  launch_pdl(st, dim3((unsigned)blocks), dim3(256), 0, transpose_kernel, src, rows, cols, ld_src, dst, ld_dst);
   OMM_LAUNCH_CHECK();
 }
 

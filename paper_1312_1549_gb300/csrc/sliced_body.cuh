@@ -213,6 +213,7 @@ __device__ __forceinline__ void sliced_body(const GroupDesc& g, const PairList& 
   else __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
+  dev::pdl_begin();
 
   if (warp == 0 && lane == 0) {
     // ---------------- TMA producer (with PAIR both CTAs)
@@ -408,6 +409,7 @@ sliced_pair_kernel(const __grid_constant__ GroupDesc g, const __grid_constant__ 
 // worker (rows 128 q .. of a tile belong to its q-th CTA). A tile that no share starts in is left alone.
 __global__ void __launch_bounds__(256)
 slab_reduce_kernel(const __grid_constant__ GroupDesc g, int npairs, const __grid_constant__ SlicedWork w, int bmt) {
+  dev::pdl_begin();
   const int subs_n = g.bn / 32, subs = (bmt / 8) * subs_n;
   const int tile = w.full * w.nw + blockIdx.x / subs, sub = blockIdx.x % subs;
   const int mb = tile % w.tiles_m, nb = tile / w.tiles_m;

@@ -1442,7 +1442,7 @@ void gemm_split(cudaStream_t st, const Operand& A, const Operand& B, int K, cons
   if (ep.M >= 2 * BM && pair_units >= pair_clusters()) {
     const GroupDesc gp = make_group(A, B, K, ep, 0, BN, nullptr, true);
     const unsigned pgrid = 2u * (unsigned)std::min(pair_units, pair_clusters());
-    gemm_pair_one_kernel<<<pgrid, NTHREADS, SMEM_BYTES, st>>>(gp, pair_units, pl, ep.err);
+    launch_pdl(st, dim3(pgrid), dim3(NTHREADS), SMEM_BYTES, gemm_pair_one_kernel, gp, pair_units, pl, ep.err);
     OMM_LAUNCH_CHECK();
     return;
   }
@@ -1463,7 +1463,7 @@ void gemm_split(cudaStream_t st, const Operand& A, const Operand& B, int K, cons
   const GroupDesc g = make_group(A, B, K, ep, 0, bn);
   const int tiles = tiles_of(ep, bn);
   auto go = [&](auto kernel) {
-    kernel<<<(unsigned)std::min(tiles, sm_count()), NTHREADS, SMEM_BYTES, st>>>(g, tiles, pl, ep.err);
+    launch_pdl(st, dim3((unsigned)std::min(tiles, sm_count())), dim3(NTHREADS), SMEM_BYTES, kernel, g, tiles, pl, ep.err);
   };
   if (bn == 256) go(gemm_persistent_one_kernel<256>);
   else if (bn == 128) go(gemm_persistent_one_kernel<128>);
@@ -1522,17 +1522,18 @@ void gemm_sliced(cudaStream_t st, const Operand& A, const Operand& B, int K, con
     }
   }
   const GroupDesc g = make_group(A, B, K, ep, 0, best_shape.bn, sparse, best_shape.pair);
-  if (best_shape.pair)
-    sliced_pair_kernel<<<2u * (unsigned)best.nw, NTHREADS, SMEM_BYTES, st>>>(g, pl, best, ep.err);
-  else if (best_shape.bn == 256)
-    sliced_kernel<256><<<(unsigned)best.nw, NTHREADS, SMEM_BYTES, st>>>(g, pl, best, ep.err);
-  else
-    sliced_kernel<128><<<(unsigned)best.nw, NTHREADS, SMEM_BYTES, st>>>(g, pl, best, ep.err);
+  auto go = [&](auto kernel, unsigned ctas) {
+    launch_pdl(st, dim3(ctas), dim3(NTHREADS), SMEM_BYTES, kernel, g, pl, best, ep.err);
+  };
+  if (best_shape.pair) go(sliced_pair_kernel, 2u * (unsigned)best.nw);
+  else if (best_shape.bn == 256) go(sliced_kernel<256>, (unsigned)best.nw);
+  else go(sliced_kernel<128>, (unsigned)best.nw);
   OMM_LAUNCH_CHECK();
   if (!best_whole) {  // some share starts inside a tile
     const int bmt = best_shape.pair ? 2 * BM : BM;
     const int left = best.tiles - best.full * best.nw;
-    slab_reduce_kernel<<<(unsigned)(left * (bmt / 8) * (best_shape.bn / 32)), 256, 0, st>>>(g, pl.n, best, bmt);
+    launch_pdl(st, dim3((unsigned)(left * (bmt / 8) * (best_shape.bn / 32))), dim3(256), 0, slab_reduce_kernel, g, pl.n, best,
+               bmt);
     OMM_LAUNCH_CHECK();
   }
 }
