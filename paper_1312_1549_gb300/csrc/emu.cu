@@ -10,14 +10,14 @@
 // (i, j) every product a b <= 256 units of 2^(e_r + f_c - 5(i+j+2)), so all
 // products of one level d = i + j share one unit per output element and a
 // level of (d+1) pairs summed over K stays an integer below (d+1) K 256
-// units: exact in the FP32 accumulator while that is <= 2^24. Each launch
-// therefore takes at most 2^24 / (256 K) pairs of one level (all pairs of a
-// level for K <= 1638, nine for the Si512 contraction K = 6656), so every
-// launch is exact and the float64 epilogue sums the launches. (Lumping
-// several levels into one FP32 accumulator is not exact: the tensor cores'
-// FP32 adder truncates, and those errors grow linearly with K — measured
-// 1e-10 of |A||B| at K = 1000.) With s = 10 slices the result carries about
-// 50 bits of each row-scaled operand.
+// units: exact in the FP32 accumulator while that is <= 2^24. The pairs are
+// therefore summed in chunks that keep this bound in units of the chunk's
+// smallest level (level_chunks: 11 chunks for the Si512 contraction K = 6656,
+// 5 for K = 64), so every chunk is exact, and the float64 epilogue adds the
+// chunks. (Levels lumped beyond that bound are not exact: the tensor cores'
+// FP32 adder truncates, and those errors grow linearly with K -- measured
+// 1e-10 of |A||B| at K = 1000 with all levels in one accumulator.) With s = 10
+// slices the result carries about 50 bits of each row-scaled operand.
 #include "emu.cuh"
 #include "pdl.cuh"
 #include "tc_gemm.cuh"

@@ -6,14 +6,14 @@
 //   warp 1      TMEM allocation and the MMA issuer (one lane)
 //   warps 2-5   epilogue: tcgen05.ld of the 128 x 256 FP32 accumulator,
 //               C = alpha * acc + beta * C written in float64
-// Each CTA computes one 128 x 256 (or 128 x 128) tile of C = A B^T with A (M x K)
+// A CTA computes 128 x 256 (or narrower, down to 32 columns) tiles of C = A B^T with A (M x K)
 // and B (N x K) both K-major bf16 (or B MN-major); the split form also runs on
 // pairs of SMs (a cluster of two CTAs, tcgen05 cta_group::2, 256-row tiles; see
 // pair_body). Operands are stacks of slices; a pair list
 // says which slice products are accumulated (passes over K into the same
 // accumulator). "Split" operands x = x_hi + x_lo use the three pairs
 // A_hi B_hi + A_hi B_lo + A_lo B_hi, which keep about 16 significant bits;
-// the float64 emulation (emu_gemm.cu) uses fixed-point slices.
+// the float64 emulation (emu.cu) uses fixed-point slices.
 //
 // Every wait on an mbarrier is bounded (globaltimer, 2 s): on expiry the
 // kernel records an error code, stops issuing work and frees its TMEM.
