@@ -37,7 +37,7 @@ omm_status omm_kernel_spd_inverse(int m, const double* A, double* P, int* info, 
 /* The same P = A^-1 (Sec. 2.4, Eq. 17) with float64-class products on the BF16
  * tensor cores, as the mixed-precision solver computes its preconditioner: a
  * recursive Cholesky factorisation, inverse and product L^-T L^-1 on halves,
- * whose off-diagonal products use 10 fixed-point slices per operand (the Ozaki
+ * whose off-diagonal products use 10 or 11 fixed-point slices per operand (the Ozaki
  * scheme; about 2^-50 of each row-scaled operand), with the 64 x 64 diagonal
  * blocks factored and inverted in float64. Arguments, ownership and *info as
  * for omm_kernel_spd_inverse; OMM_ERR_TIMEOUT if a bounded wait of a tensor-core
