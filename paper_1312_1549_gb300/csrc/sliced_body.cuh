@@ -1,17 +1,6 @@
 // The sliced (float64-class) product: a pair list of slice products cut into chunks, every chunk an
-// exact integer sum in the FP32 accumulator, the chunks added in float64. Included by tc_gemm.cu.
-//
-// Work: a stage is one 64-wide K block of one slice pair of one output tile; a tile has npairs x
-// (its K blocks) of them. A worker (a CTA, or with PAIR the two CTAs of a cluster) takes `full` whole
-// tiles, tile index worker + k nw, and the stages of the tiles that are left over form one line that
-// is shared evenly among nr workers, cutting tiles and even chunks where a share begins and ends: a part
-// of an exact integer sum is exact too, so nothing is lost. (Whole tiles only left SMs idle: 104 tiles of
-// 256 x 256 on 76 pairs take two rounds for 1.37 rounds of work, 36 tiles of 128 x 256 use 36 of 152
-// SMs.) Workers on whole tiles, and on the same fraction of a tile, walk the slice pairs in step and
-// share the slices through L2; shares at arbitrary places of the line do not (the slices of a
-// 1024 x 6656 x 6656 product are 1 GB), which costs more than it balances once they outgrow L2 (that
-// product with its slicing: 5.3 ms in whole tiles, 5.5 with one even line, 3.9 with this; a 1495 x 260
-// state's products 0.9-1.4 ms each before, 0.13-0.22 now).
+// exact integer sum in the FP32 accumulator, the chunks added in float64. How its work is shared is in
+// sliced_plan.cuh. Included by tc_gemm.cu.
 //
 // Sums: each CTA adds the pieces of a tile in a private 128 x TBN float64 slab laid out column by
 // column, so that the 32 lanes of a warp (32 rows) touch 256 contiguous bytes, and a batch of columns
@@ -20,104 +9,6 @@
 // segment that holds a tile's first stage writes alpha x sum + beta C to C at its end; a worker whose
 // share starts inside a tile leaves that segment's sum in its slab for slab_reduce_kernel.
 #pragma once
-
-struct SlicedWork {
-  double* slab;  // 2 x 128 x TBN per CTA: [0] a share's first, headless segment, [1] scratch
-  int nw;        // workers
-  int full;      // whole tiles of each
-  int nr;        // workers that share the left-over tiles' stages (0: none left)
-  int tiles_m;   // tiles along M (the fast index)
-  int tiles;     // all tiles
-};
-
-// the line of the stages of the left-over tiles, positions counted from the first stage of tile 0
-struct Line {
-  long base, len;
-  __device__ __forceinline__ long begin(const SlicedWork& w, int worker) const { return base + len * worker / w.nr; }
-};
-__device__ __forceinline__ Line line_of(const GroupDesc& g, const SlicedWork& w, int npairs) {
-  const int t0 = w.full * w.nw;
-  Line l;
-  if (g.kb_off != nullptr) {
-    const int nb = t0 / w.tiles_m, mb = t0 - nb * w.tiles_m;
-    const long unit = (long)npairs * w.tiles_m;
-    l.base = t0 < w.tiles ? unit * g.kb_off[nb] + (long)npairs * mb * (g.kb_off[nb + 1] - g.kb_off[nb]) : 0;
-    l.len = unit * g.kb_off[w.tiles / w.tiles_m] - l.base;
-  } else {
-    const long per = (long)npairs * ((g.K + BK - 1) / BK);
-    l.base = per * t0;
-    l.len = per * (w.tiles - t0);
-  }
-  return l;
-}
-
-// one tile's run of stages [s0, s1) inside a worker's work
-struct Segment {
-  int mb, nb;
-  KBlocks kbs;
-  int s0, s1;
-};
-
-// walks the segments of one worker; every role of its CTAs walks the same ones
-struct Walk {
-  int worker, k;
-  long pos, end;
-  __device__ __forceinline__ Walk(const GroupDesc& g, const SlicedWork& w, int npairs, int worker_) : worker(worker_), k(0) {
-    pos = end = 0;
-    if (worker < w.nr) {
-      const Line l = line_of(g, w, npairs);
-      pos = l.begin(w, worker);
-      end = l.begin(w, worker + 1);
-    }
-  }
-  __device__ __forceinline__ void kblocks(const GroupDesc& g, int nb, KBlocks& kbs) const {
-    if (g.kb_off != nullptr) {
-      const int o0 = g.kb_off[nb];
-      kbs.list = g.kb_idx + o0;
-      kbs.count = g.kb_off[nb + 1] - o0;
-    } else {
-      kbs.list = nullptr;
-      kbs.count = (g.K + BK - 1) / BK;
-    }
-  }
-  __device__ __forceinline__ bool next(const GroupDesc& g, const SlicedWork& w, int npairs, Segment& s) {
-    if (k < w.full) {
-      const int tile = worker + k * w.nw;
-      ++k;
-      s.mb = tile % w.tiles_m;
-      s.nb = tile / w.tiles_m;
-      kblocks(g, s.nb, s.kbs);
-      s.s0 = 0;
-      s.s1 = npairs * s.kbs.count;
-      return true;
-    }
-    if (pos >= end) return false;
-    if (g.kb_off != nullptr) {  // the column block whose tiles hold this position
-      const long unit = (long)npairs * w.tiles_m;
-      int lo = 0, hi = w.tiles / w.tiles_m - 1;
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (unit * g.kb_off[mid] <= pos) lo = mid; else hi = mid - 1;
-      }
-      kblocks(g, lo, s.kbs);
-      const int per = npairs * s.kbs.count;
-      const long rem = pos - unit * g.kb_off[lo];
-      s.nb = lo;
-      s.mb = (int)(rem / per);
-      s.s0 = (int)(rem - (long)s.mb * per);
-    } else {
-      kblocks(g, 0, s.kbs);
-      const int per = npairs * s.kbs.count;
-      const long tile = pos / per;
-      s.s0 = (int)(pos - tile * per);
-      s.mb = (int)(tile % w.tiles_m);
-      s.nb = (int)(tile / w.tiles_m);
-    }
-    s.s1 = (int)min((long)npairs * s.kbs.count, s.s0 + (end - pos));
-    pos += s.s1 - s.s0;
-    return true;
-  }
-};
 
 // alpha v + beta C for 16 columns of one row (all loads of C before its stores)
 __device__ __forceinline__ void store_row16(const Epilogue& ep, int row, int col0, const double (&v)[16]) {
@@ -416,21 +307,9 @@ slab_reduce_kernel(const __grid_constant__ GroupDesc g, int npairs, const __grid
   const int r0 = (sub / subs_n) * 8, c0 = (sub % subs_n) * 32;
   const int row0 = mb * bmt + r0, col0 = nb * g.bn + c0;
   if (row0 >= g.ep.M || col0 >= g.ep.N) return;
-  long base, per;
-  if (g.kb_off != nullptr) {
-    const int o0 = g.kb_off[nb];
-    per = (long)npairs * (g.kb_off[nb + 1] - o0);
-    base = (long)npairs * w.tiles_m * o0 + mb * per;
-  } else {
-    per = (long)npairs * ((g.K + BK - 1) / BK);
-    base = tile * per;
-  }
-  const Line line = line_of(g, w, npairs);
-  int first = (int)((base - line.base) * w.nr / line.len);
-  while (first < w.nr && line.begin(w, first) <= base) ++first;
-  if (first >= w.nr || line.begin(w, first) >= base + per) return;
-  int last = (int)((base + per - line.base) * w.nr / line.len) + 1;  // one past the last such worker
-  while (last > first && (last > w.nr || line.begin(w, last - 1) >= base + per)) --last;
+  const Slabs slabs = slabs_of(g, w, npairs, tile);
+  const int first = slabs.first, last = slabs.last;
+  if (first >= last) return;
   const int ctas = bmt / BM;
   const int rr = threadIdx.x & 7, cc = threadIdx.x >> 3;  // eight rows (64 bytes) of a column
   const double* slab = w.slab + ((long)first * ctas + r0 / BM) * 2 * BM * g.bn + (r0 % BM) + rr + (long)(c0 + cc) * BM;

@@ -23,6 +23,7 @@
 
 #include "omm_internal.cuh"
 #include "pdl.cuh"
+#include "sliced_plan.cuh"
 #include "split_device.cuh"
 #include "tc_gemm.cuh"
 
@@ -39,10 +40,6 @@ namespace omm {
 namespace tc {
 namespace {
 
-// K is consumed in stages of BK = 64 contracted columns (one 128-byte swizzle atom of bf16 per
-// row). Stages of 32 columns (64-byte swizzle) were measured slower: twice the barrier and commit
-// round trips per contracted column, for no gain in the bytes kept in flight.
-constexpr int BM = 128, BN = 256, BK = 64;
 constexpr int A_BYTES = BM * BK * 2;
 constexpr int B_BYTES = BN * BK * 2;
 // the stage ring; 224 KB (seven or eight single-pass stages) was measured slower than 192 KB:
@@ -546,12 +543,6 @@ __device__ __forceinline__ int find_group(const GroupDesc* __restrict__ groups, 
 // b, b + gridDim.x, ... of all groups. The accumulator is double-buffered in
 // TMEM (2 x 256 columns) so the epilogue of one tile overlaps the main loop
 // of the next; the producer's stage ring continues across tiles.
-// The K blocks of one output tile: all of them, or the listed ones where B is block-sparse.
-struct KBlocks {
-  const int* list;  // null: 0 .. count-1
-  int count;
-  __device__ __forceinline__ int at(int i) const { return list ? list[i] : i; }
-};
 __device__ __forceinline__ KBlocks tile_kblocks(const GroupDesc* g, int local, int tiles_m) {
   KBlocks kb;
   if (g->kb_off != nullptr) {
@@ -1480,59 +1471,21 @@ void gemm_sliced(cudaStream_t st, const Operand& A, const Operand& B, int K, con
   if (ep.skip != nullptr || ep.mode != kEpPlain || ep.c_f32 || ep.bf_hi != nullptr || slab == nullptr)
     throw CudaError{cudaErrorInvalidValue, "tc::gemm_sliced: plain float64 epilogue and a workspace"};
   if (ep.M <= 0 || ep.N <= 0 || K <= 0) return;
-  const long nkb = (K + BK - 1) / BK;
-  const int nchunk = pl.nchunk > 0 ? pl.nchunk : 1;
-  // Tile shape and number of workers with the shortest estimated time, in SM clocks. A stage takes as
-  // long as its copies: about 55 bytes per clock land in an SM's shared memory, 32 KB for a pair's 256 x
-  // 256 or one SM's 128 x 128 tile, 48 KB for 128 x 256. Adding a piece to a running sum costs a float64
-  // add per element, about one per clock and SM, beside the stages that follow; the last piece's add and
-  // about 5000 clocks of start-up are exposed, and where shares do not end with tiles the slab pass too.
-  struct Shape { int bn; bool pair; double cycles; };
-  const Shape shapes[3] = {{256, true, 600.0}, {256, false, 900.0}, {128, false, 600.0}};
-  // shares at arbitrary places only while the slices stay in L2 (see sliced_body.cuh)
-  int slices = 0;
-  for (int p = 0; p < pl.n; ++p) slices = std::max(slices, std::max((int)pl.a[p], (int)pl.b[p]) + 1);
-  const bool resident = 2.0 * slices * ((double)ep.M + ep.N) * K <= 100e6;
-  SlicedWork best{};
-  Shape best_shape = shapes[1];
-  double best_t = 0.0;
-  bool best_whole = false;
-  for (const Shape& sh : shapes) {
-    if (sparse != nullptr && sh.bn != 256) continue;  // block lists are made for 256 rows
-    const int bmt = sh.pair ? 2 * BM : BM, workers = sh.pair ? pair_clusters() : sm_count();
-    const int tm = (ep.M + bmt - 1) / bmt, tn = (ep.N + sh.bn - 1) / sh.bn, tiles = tm * tn;
-    const double per_tile = sparse ? (double)pl.n * sparse->nnz / tn : (double)pl.n * nkb;
-    const int full = tiles / workers, left = tiles - full * workers;
-    const int most = std::min<int>(workers, std::max<int>(left, (int)(left * per_tile / 8)));  // 8 stages each or more
-    const double add = (double)std::min(ep.M, BM) * std::min(ep.N, sh.bn);  // elements of one CTA's piece
-    for (int k = 0; k < 2; ++k) {
-      // left-over tiles in equal parts (one or more workers each), or evenly over all workers
-      const int nr = left == 0 ? 0 : (k == 0 ? left * (most / left) : most);
-      if (k == 1 && (left == 0 || !resident)) continue;
-      const bool whole = nr == 0 || (sparse == nullptr && nr == left);
-      const double stages = full * per_tile + (nr ? left * per_tile / nr : 0.0);
-      const double t = std::max(stages * sh.cycles, nchunk * stages / per_tile * add) + add + 5000.0 +
-                       (whole ? 0.0 : 9000.0 + add / 8.0);
-      if (best_t == 0.0 || t < best_t) {
-        best = SlicedWork{slab, full > 0 ? workers : nr, full, nr, tm, tiles};
-        best_shape = sh;
-        best_whole = whole;
-        best_t = t;
-      }
-    }
-  }
-  const GroupDesc g = make_group(A, B, K, ep, 0, best_shape.bn, sparse, best_shape.pair);
+  SlicedPlan plan = plan_sliced(ep.M, ep.N, K, pl, sparse, pair_clusters(), sm_count());
+  SlicedWork& w = plan.work;
+  w.slab = slab;
+  const GroupDesc g = make_group(A, B, K, ep, 0, plan.bn, sparse, plan.pair);
   auto go = [&](auto kernel, unsigned ctas) {
-    launch_pdl(st, dim3(ctas), dim3(NTHREADS), SMEM_BYTES, kernel, g, pl, best, ep.err);
+    launch_pdl(st, dim3(ctas), dim3(NTHREADS), SMEM_BYTES, kernel, g, pl, w, ep.err);
   };
-  if (best_shape.pair) go(sliced_pair_kernel, 2u * (unsigned)best.nw);
-  else if (best_shape.bn == 256) go(sliced_kernel<256>, (unsigned)best.nw);
-  else go(sliced_kernel<128>, (unsigned)best.nw);
+  if (plan.pair) go(sliced_pair_kernel, 2u * (unsigned)w.nw);
+  else if (plan.bn == 256) go(sliced_kernel<256>, (unsigned)w.nw);
+  else go(sliced_kernel<128>, (unsigned)w.nw);
   OMM_LAUNCH_CHECK();
-  if (!best_whole) {  // some share starts inside a tile
-    const int bmt = best_shape.pair ? 2 * BM : BM;
-    const int left = best.tiles - best.full * best.nw;
-    launch_pdl(st, dim3((unsigned)(left * (bmt / 8) * (best_shape.bn / 32))), dim3(256), 0, slab_reduce_kernel, g, pl.n, best,
+  if (!plan.whole) {  // some share starts inside a tile
+    const int bmt = plan.pair ? 2 * BM : BM;
+    const int left = w.tiles - w.full * w.nw;
+    launch_pdl(st, dim3((unsigned)(left * (bmt / 8) * (plan.bn / 32))), dim3(256), 0, slab_reduce_kernel, g, pl.n, w,
                bmt);
     OMM_LAUNCH_CHECK();
   }
@@ -1610,6 +1563,7 @@ void block_lists(cudaStream_t st, const double* B, long rows, long cols, long ld
       }
     }
     bl.nnz = (long)idx[w].size();
+    bl.off_host = off[w];
     // the stream was synchronised above, so no earlier launch still reads the old lists; the host
     // vectors live until the copies are done
     OMM_CUDA_TRY(cudaMemcpyAsync(bl.off, off[w].data(), off[w].size() * sizeof(int), cudaMemcpyHostToDevice, st));

@@ -149,6 +149,7 @@ struct BlockLists {
   int nblocks = 0;
   long nnz = 0;
   long dense = 0;  // nblocks x K blocks
+  std::vector<int> off_host;  // off, for the plan of a sliced product
 };
 // (re)computes lists[k] for B (rows x cols float64, leading dimension ld, device) and row blocks of
 // widths[k] (64, 128, 192 or 256), k < count, from one pass over B; the first call allocates room for a
