@@ -33,11 +33,11 @@
 #include "leaf_f64.cuh"
 #include "omm_internal.cuh"
 #include "pdl.cuh"
+#include "side_streams.cuh"
 #include "split_device.cuh"
 #include "tc_gemm.cuh"
 
 #include <algorithm>
-#include <vector>
 
 namespace omm {
 namespace {
@@ -392,38 +392,6 @@ void spd_factor_inverse(cudaStream_t st, int m, double* A, double* Y, double* wo
 // ------------------------------------------------------------------ float64-class (sliced) variant
 namespace {
 
-// Streams beside the caller's and the events between them. They may be released with work pending: the driver
-// frees them once it is done.
-struct Streams {
-  std::vector<cudaEvent_t> events;
-  std::vector<cudaStream_t> streams;
-
-  Streams() = default;
-  Streams(const Streams&) = delete;
-  Streams& operator=(const Streams&) = delete;
-  ~Streams() {
-    for (cudaStream_t s : streams) cudaStreamDestroy(s);
-    for (cudaEvent_t e : events) cudaEventDestroy(e);
-  }
-  // a stream that starts after what `from` holds so far
-  cudaStream_t fork(cudaStream_t from) {
-    cudaStream_t s = nullptr;
-    OMM_CUDA_TRY(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
-    streams.push_back(s);
-    wait(s, from);
-    return s;
-  }
-  cudaEvent_t record(cudaStream_t st) {
-    cudaEvent_t e = nullptr;
-    OMM_CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-    events.push_back(e);
-    OMM_CUDA_TRY(cudaEventRecord(e, st));
-    return e;
-  }
-  // `st` goes on after what `other` holds so far
-  void wait(cudaStream_t st, cudaStream_t other) { OMM_CUDA_TRY(cudaStreamWaitEvent(st, record(other), 0)); }
-};
-
 constexpr int kInvSlices = 10;  // the most slices of a lane's products; W and Y21 take one more (workspace sizing)
 
 long round8(long x) { return (x + 7) / 8 * 8; }
@@ -658,7 +626,7 @@ void split_impl(cudaStream_t st, int m, double* A, double* P, void* work, int* i
   tc::split(st, A, m, m, m, w.As, w.As + m * w.ld, w.ld, nullptr);
   w.side = w.fork(st);
   w.node(0, m);
-  w.wait(st, w.side);
+  w.join(st);
   launch_symmetrize_lower(st, m, P);
 }
 
@@ -706,9 +674,8 @@ void sliced_impl(cudaStream_t st, int m, double* A, double* P, double* Y_out, vo
   }
   w.ahead.st = w.fork(st);
   chol_inv(w, 0, m);
-  w.wait(st, w.ahead.st);
+  w.join(st);
   if (P) {
-    w.wait(st, w.side.st);
     launch_symmetrize_lower(st, m, P);
   }
   if (Y_out) {
