@@ -394,7 +394,8 @@ namespace {
 
 constexpr int kInvSlices = 10;  // the most slices of a lane's products; W and Y21 take one more (workspace sizing)
 
-long round8(long x) { return (x + 7) / 8 * 8; }
+long round_up(long x, long unit) { return (x + unit - 1) / unit * unit; }
+long round8(long x) { return round_up(x, 8); }
 
 // scratch of one stream's products
 struct Lane {
@@ -524,9 +525,12 @@ void chol_inv(SlicedWork& w, int r0, int b) {
 struct SplitInverse : Streams {
   int m = 0;
   long ld = 0;
+  // rows between the hi and the lo half of a pair: a product that contracts over rows of both operands (Y^T Y)
+  // runs on to the end of a 64-row block, where zero rows have to follow row m
+  long half = 0;
   double* A = nullptr;
   double* P = nullptr;
-  __nv_bfloat16 *As = nullptr, *Ls = nullptr, *Ys = nullptr;  // [hi; lo], 2m x ld each
+  __nv_bfloat16 *As = nullptr, *Ls = nullptr, *Ys = nullptr;  // [hi; lo], 2 half x ld each
   int* info = nullptr;
   int* err = nullptr;
   cudaStream_t st = nullptr, side = nullptr;
@@ -534,7 +538,7 @@ struct SplitInverse : Streams {
   enum Role { kA, kB };
   // block (r0, c0) as an operand: rows x cols with cols contracted, or (mn) rows contracted
   tc::Operand view(const __nv_bfloat16* x, int r0, int c0, int rows, int cols, Role role, bool mn) const {
-    return tc::make_operand_view(x + r0 * ld + c0, m, cols, ld, 2, role == kA, 0, rows, mn, 2L * m - r0);
+    return tc::make_operand_view(x + r0 * ld + c0, half, cols, ld, 2, role == kA, 0, rows, mn, 2L * half - r0);
   }
   // the split of an M x N product into block (r0, c0) of x, alpha times it
   tc::Epilogue into(__nv_bfloat16* x, int r0, int c0, int M, int N, double alpha) const {
@@ -542,7 +546,7 @@ struct SplitInverse : Streams {
     ep.c_f32 = 1;
     ep.bf_hi = x + r0 * ld + c0;
     ep.bf_ld = ld;
-    ep.bf_lo = m * ld;
+    ep.bf_lo = half * ld;
     return ep;
   }
 
@@ -550,7 +554,7 @@ struct SplitInverse : Streams {
     if (b <= NL) {
       __nv_bfloat16* y = Ys + r0 * ld + r0;
       const long at = (long)r0 * m + r0;
-      launch_pdl(st, dim3(1), dim3(kLeafThreads), kLeafSmem, leaf_f32_kernel, A + at, m, b, nullptr, y, y + m * ld, ld, info,
+      launch_pdl(st, dim3(1), dim3(kLeafThreads), kLeafSmem, leaf_f32_kernel, A + at, m, b, nullptr, y, y + half * ld, ld, info,
                  r0, P + at, m);
       OMM_LAUNCH_CHECK();
       return;
@@ -592,7 +596,7 @@ size_t spd_inverse_sliced_workspace_bytes(int m) {
   // Y, leaf; tr0, tr1 of one lane, tr0 of another; a slab per lane
   const size_t f64 = (size_t)m * m + (size_t)NL * NL + 3 * ((size_t)h * h + (size_t)tc::sliced_workspace_doubles());
   const size_t bf = 3 * 2 * (size_t)(kInvSlices + 1) * (size_t)h * round8(h);  // per lane: sl0, sl1
-  // (the split form's three pairs of m x m need less: 12 m round8(m) bytes of these 47 m^2 and more)
+  // (the split form's three pairs of m x m need less: 12 bytes per element of the padded matrix of these 47 and more)
   return f64 * sizeof(double) + bf * sizeof(__nv_bfloat16) + 4 * 256;
 }
 
@@ -613,17 +617,18 @@ void split_impl(cudaStream_t st, int m, double* A, double* P, void* work, int* i
   w.info = info_dev;
   w.err = err_dev;
   w.st = st;
-  const size_t pair = 2 * (size_t)m * w.ld;
+  w.half = round_up(m, 64);
+  const size_t pair = 2 * (size_t)w.half * w.ld;
   w.Ys = reinterpret_cast<__nv_bfloat16*>((reinterpret_cast<uintptr_t>(work) + 255) & ~uintptr_t(255));
   w.Ls = w.Ys + pair;
   w.As = w.Ls + pair;
   prepare_leaf();
   OMM_CUDA_TRY(cudaMemsetAsync(info_dev, 0, sizeof(int), st));
-  // zeros above the diagonal of Y; and every element a copy may touch past the end of a block (it meets
-  // zeros of the other operand) has to be a number
+  // zeros above the diagonal of Y and past row m; and every element that a contraction over rows of Y or L may
+  // touch past the end of a block has to be a number (it meets zeros of the other operand)
   OMM_CUDA_TRY(cudaMemsetAsync(w.Ys, 0, 2 * pair * sizeof(__nv_bfloat16), st));
   OMM_CUDA_TRY(cudaMemsetAsync(P, 0, sizeof(double) * m * (size_t)m, st));
-  tc::split(st, A, m, m, m, w.As, w.As + m * w.ld, w.ld, nullptr);
+  tc::split(st, A, m, m, m, w.As, w.As + w.half * w.ld, w.ld, nullptr);
   w.side = w.fork(st);
   w.node(0, m);
   w.join(st);
