@@ -65,9 +65,8 @@ namespace {
 
 long round8(long x) { return (x + 7) / 8 * 8; }
 // partial-sum slots of the P G product's epilogue (n x m): one per epilogue warp and tile, four warps on
-// 128 rows, at the narrowest tile (32 columns); 256-row tiles and the odd column tile of a two-pair
-// cluster are rounded up into it
-long red_slots(long n, long m) { return 4 * 2 * ((n + 255) / 256) * ((m + 31) / 32 + 8); }
+// 128 rows, at the narrowest tile (32 columns), the rows rounded up to 256-row tiles
+long red_slots(long n, long m) { return 4 * 2 * ((n + 255) / 256) * ((m + 31) / 32); }
 
 template <typename T>
 void alloc(T** p, size_t count, cudaStream_t st) {
@@ -338,9 +337,8 @@ void build_plans(MixedState* ms, cudaStream_t st, Scalars* sc, double* G, double
     const tc::TileShape ts = tc::choose_tile_shape(st, {spec}, plan_pairs(k), &ms_tune);
     ms->plan_shape[k] = ts;
     ms->ms_autotune += ms_tune;
-    h[k] = tc::make_group(*opA[k], *opB[k], K[k], ep[k], 0, ts.bn, ts.quad ? nullptr : spec.sparse[tc::sparse_slot(ts.bn)],
-                          ts.pair, ts.quad);
-    ms->plan_tiles[k] = tc::tiles_of(ep[k], ts.bn, ts.pair, ts.quad);
+    h[k] = tc::make_group(*opA[k], *opB[k], K[k], ep[k], 0, ts.bn, spec.sparse[tc::sparse_slot(ts.bn)], ts.pair);
+    ms->plan_tiles[k] = tc::tiles_of(ep[k], ts.bn, ts.pair);
   }
   if (!ms->plans) alloc(&ms->plans, 4, st);
   OMM_CUDA_TRY(cudaMemcpyAsync(ms->plans, h, sizeof(h), cudaMemcpyHostToDevice, st));
@@ -350,7 +348,7 @@ void build_plans(MixedState* ms, cudaStream_t st, Scalars* sc, double* G, double
 
 void run_plan(MixedState* ms, cudaStream_t st, int k) {
   tc::gemm_persistent(st, ms->plans + k, 1, ms->plan_tiles[k], plan_pairs(k), ms->err, ms->plan_shape[k].bn,
-                      ms->plan_shape[k].pair, ms->plan_shape[k].quad);
+                      ms->plan_shape[k].pair);
 }
 
 }  // namespace
@@ -358,7 +356,7 @@ void run_plan(MixedState* ms, cudaStream_t st, int k) {
 int mixed_reduce_parts(const MixedState* ms) {
   // one slot of partial sums per epilogue warp of every P G output tile (eight on an SM pair's tile)
   const tc::TileShape& ts = ms->plan_shape[kPlanPG];
-  return 4 * ms->plan_tiles[kPlanPG] * (ts.quad ? 4 : (ts.pair ? 2 : 1));
+  return 4 * ms->plan_tiles[kPlanPG] * (ts.pair ? 2 : 1);
 }
 
 void mixed_iterate(MixedState* ms, cudaStream_t st, Scalars* sc, double* C, double* Dir, double* G,

@@ -124,18 +124,15 @@ inline void gemm(cudaStream_t st, const Operand& A, const Operand& B, int K, int
 // only), or, with pair,
 // 256 x bn on a cluster of two SMs that share the MMA (tcgen05 cta_group::2; bn = 128, 192 or 256;
 // the split form or a single pass).
-// With quad (pair set too), a cluster of two SM pairs side by side along N shares the A operand
-// through TMA multicast: a work unit is 256 x 2 bn (dense B only).
 struct TileShape {
   int bn = 256;
   bool pair = false;
-  bool quad = false;
-  int code() const { return bn + (quad ? 2000 : (pair ? 1000 : 0)); }  // as reported in omm_info
+  int code() const { return bn + (pair ? 1000 : 0); }  // as reported in omm_info
 };
-int tiles_of(const Epilogue& ep, int bn = 256, bool pair = false, bool quad = false);  // work units of one GEMM
+int tiles_of(const Epilogue& ep, int bn = 256, bool pair = false);  // work units of one GEMM
 // the partial-sum slots (one per epilogue warp and 128 x bn quarter) a kEpReduce GEMM writes
 inline int reduce_slots(const Epilogue& ep, const TileShape& ts) {
-  return 4 * tiles_of(ep, ts.bn, ts.pair, ts.quad) * (ts.quad ? 4 : (ts.pair ? 2 : 1));
+  return 4 * tiles_of(ep, ts.bn, ts.pair) * (ts.pair ? 2 : 1);
 }
 
 // One GEMM of a grouped launch (device array element; tensor maps in global memory).
@@ -170,20 +167,19 @@ struct alignas(64) GroupDesc {
   int K, rowsA, rowsB, tile_begin;  // rowsA, rowsB: rows between the slices of A and B
   int offA, offB;                   // first row of A and B inside each slice
   int a_mn, b_mn;                   // A, B is MN-major (its rows are the contracted index)
-  int bn;    // output tile width (all groups of one launch share it, pair and quad)
+  int bn;    // output tile width (all groups of one launch share it and pair)
   int pair;  // 256-row tiles on a cluster of two SMs
-  int quad;  // two such pairs per cluster, sharing A
   const int* kb_off;  // block sparsity of B for row blocks of bn (null: dense)
   const int* kb_idx;
 };
 GroupDesc make_group(const Operand& A, const Operand& B, int K, const Epilogue& ep, int tile_begin, int bn = 256,
-                     const BlockLists* sparse = nullptr, bool pair = false, bool quad = false);
+                     const BlockLists* sparse = nullptr, bool pair = false);
 // groups_dev: ngroups descriptors in device memory, sorted by tile_begin; all share the pair list
 void prepare_persistent();  // kernel attributes (call before a stream capture)
 // persistent grouped launch: one CTA per SM, double-buffered TMEM accumulators; err receives a
 // nonzero code if a bounded wait expired
 void gemm_persistent(cudaStream_t st, const GroupDesc* groups_dev, int ngroups, int total_tiles, const PairList& pl,
-                     int* err, int bn = 256, bool pair = false, bool quad = false);
+                     int* err, int bn = 256, bool pair = false);
 // one split-form GEMM (pairs_split3) whose descriptor travels as a kernel parameter; either operand may
 // be MN-major
 void gemm_split(cudaStream_t st, const Operand& A, const Operand& B, int K, const Epilogue& ep);
@@ -196,7 +192,7 @@ long sliced_workspace_doubles();
 // Tile-shape autotuner: times one persistent launch over these GEMMs (the operands as given,
 // their epilogues with the outputs redirected to scratch) with each candidate shape -- 128 x 256, 128
 // x 128, 128 x 64 and (dense K-major B) 128 x 32 on one SM, and (split form or single pass, allow_pair)
-// 256 x 128, 256 x 192 and 256 x 256 on SM pairs, and (dense B) the same on clusters of two pairs sharing A
+// 256 x 128, 256 x 192 and 256 x 256 on SM pairs
 // -- returns the fastest, and remembers it per shape signature for the life of the process.
 // ms_spent receives the time spent timing (0 when the answer came from the cache).
 struct GemmSpec {

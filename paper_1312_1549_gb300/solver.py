@@ -202,7 +202,7 @@ def gemm_tc_pair(A, B, C, alpha=1.0, beta=0.0, tile_n=256, b_kn=False, block_spa
     """The tensor-core contraction on pairs of SMs (256-row tiles, tcgen05 cta_group::2): C = alpha A B^T
     + beta C (B N x K), or with b_kn C = alpha A B + beta C (B K x N, read MN-major); npass 3 (split
     form) or 1 (single bf16 pass); tile_n 128, 192 (K-major B only) or 256; block_sparse skips the K
-    blocks where B is zero; cluster_pairs 2 runs two pairs per cluster that share A (dense B)."""
+    blocks where B is zero; cluster_pairs 2 (dense B) runs the same kernels as 1."""
     M, K = A.shape
     Nn = B.shape[1] if b_kn else B.shape[0]
     N.check(N.lib().omm_kernel_gemm_tc_pair(M, Nn, K, _ptr(A), _ptr(B), float(alpha), float(beta), _ptr(C),
