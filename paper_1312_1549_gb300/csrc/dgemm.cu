@@ -242,6 +242,8 @@ struct Split {
   int tile, ks;
 };
 
+constexpr long kMaxGridY = 65535;
+
 // The tile and the split with the shortest estimated time. An SM works off its CTAs' FMAs at two
 // per clock (their loads overlap each other's FMAs); a CTA alone needs about 700 clocks per stage
 // for its loads; meeting over a cluster costs about 2500 clocks and storing a partial tile.
@@ -250,6 +252,7 @@ Split choose_split(long M, long N, long K, long batch) {
   double best_t = 0.0;
   const double nsm = sms();
   for (int tile : {64, 32, 16}) {
+    if (tile < 64 && (M + tile - 1) / tile > kMaxGridY) continue;  // tile rows are grid rows
     const double tiles = (double)((M + tile - 1) / tile) * (double)((N + tile - 1) / tile) * (double)batch;
     for (int ks = 1; ks <= (tile == 64 ? 1 : 8); ks *= 2) {
       if (ks > 1 && K < (long)SK * ks) break;
