@@ -68,10 +68,15 @@ unsigned long long launches_counted();
     OMM_CUDA_TRY(cudaGetLastError());        \
   } while (0)
 
+// (a failing call also leaves its error for cudaGetLastError: it is taken off, or the check of the next launch,
+// the library's or another's, would find it)
 #define OMM_CUDA_TRY(call)                                                   \
   do {                                                                       \
     cudaError_t e__ = (call);                                                \
-    if (e__ != cudaSuccess) throw ::omm::CudaError{e__, #call};              \
+    if (e__ != cudaSuccess) {                                                \
+      cudaGetLastError();                                                    \
+      throw ::omm::CudaError{e__, #call};                                    \
+    }                                                                        \
   } while (0)
 
 // ------------------------------------------------------------------ device memory
