@@ -29,9 +29,13 @@ void set_last_error(const std::string& msg) { g_last_error = msg; }
 const char* last_error_cstr() { return g_last_error.c_str(); }
 
 std::atomic<unsigned long long> g_launches{0};
-void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
-void count_launches(long n) { g_launches.fetch_add((unsigned long long)n, std::memory_order_relaxed); }
-unsigned long long launches_counted() { return g_launches.load(); }
+thread_local unsigned long long t_launches = 0;
+void count_launch() { count_launches(1); }
+void count_launches(long n) {
+  g_launches.fetch_add((unsigned long long)n, std::memory_order_relaxed);
+  t_launches += (unsigned long long)n;
+}
+unsigned long long launches_counted() { return t_launches; }
 
 void Profiler::begin(cudaStream_t st) {
   if (!on) return;

@@ -61,7 +61,7 @@ const char* last_error_cstr();
 // (counted while it is captured, they are taken off again)
 void count_launch();
 void count_launches(long n);
-unsigned long long launches_counted();
+unsigned long long launches_counted();  // by the calling thread
 #define OMM_LAUNCH_CHECK()                   \
   do {                                       \
     ::omm::count_launch();                   \
