@@ -191,7 +191,7 @@ omm_status omm_create(int m, int n, const double* H, const double* S, const doub
  * Stops when max|G| < tol_grad (G of Eq. 12, certified in float64), or by the
  * relative energy change of Eq. 18 when e_tol > 0.
  * Errors: OMM_ERR_ARG, OMM_ERR_UNBOUNDED, OMM_ERR_NO_CONVERGENCE,
- * OMM_ERR_NONFINITE, OMM_ERR_CUDA. */
+ * OMM_ERR_NONFINITE, OMM_ERR_TIMEOUT, OMM_ERR_OOM, OMM_ERR_CUDA. */
 omm_status omm_solve(omm_ctx* ctx, const double* C0, double* C, double* E, double* D,
                      omm_info* info);
 
@@ -200,11 +200,12 @@ omm_status omm_solve(omm_ctx* ctx, const double* C0, double* C, double* E, doubl
  *   dEdH = D = 2 C (2I - S_W) C^T,
  *   dEdS = -EDM = -(2 C H~_W C^T + eta D).
  * By the envelope theorem these are exact at the minimum (derived from Eq. 8
- * with H~ = H - eta S). Errors: OMM_ERR_STATE (no converged solve), OMM_ERR_CUDA. */
+ * with H~ = H - eta S). Errors: OMM_ERR_STATE (no converged solve), OMM_ERR_OOM,
+ * OMM_ERR_CUDA. */
 omm_status omm_backward(omm_ctx* ctx, double* dEdH, double* dEdS);
 
 /* Replace H (SCF warm start: S, T and P are kept; Sec. 2.5.2). With opts.cholesky the new
- * H is reduced with the kept factor: H_r = L^-1 H L^-T. */
+ * H is reduced with the kept factor: H_r = L^-1 H L^-T. Errors: OMM_ERR_ARG, OMM_ERR_OOM, OMM_ERR_TIMEOUT, OMM_ERR_CUDA. */
 omm_status omm_update_H(omm_ctx* ctx, const double* H);
 
 /* Release every resource of the context (NULL is ignored). */

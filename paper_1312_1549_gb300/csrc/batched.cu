@@ -588,6 +588,12 @@ omm_status omm_solve_batched(omm_batch* b, const double* const* C0, double* cons
   float ms_total = 0.f;
   double ms_graph = 0.0, gemm_flop = 0.0, ms_refresh_wall = 0.0;
   const bool profile = b->opts.profile != 0;
+  auto give_up = [&]() {  // after a failing call: nothing goes on that reads the caller's arrays
+    for (cudaStream_t q : b->pool) cudaStreamSynchronize(q);
+    cudaStreamSynchronize(b->st);
+    for (cudaEvent_t ev : {e0, e1, g0, g1})
+      if (ev) cudaEventDestroy(ev);
+  };
   try {
     OMM_CUDA_TRY(cudaEventCreate(&e0));
     OMM_CUDA_TRY(cudaEventCreate(&e1));
@@ -709,13 +715,12 @@ omm_status omm_solve_batched(omm_batch* b, const double* const* C0, double* cons
         }
         const bool native = (last_done[i] && c->opts.native_certificate != 0) || c->emu == nullptr;
         cudaStream_t q = b->pool[todo.size() % kRefreshStreams];
-        c->st = q;
+        OnStream on(c, q);
         OMM_CUDA_TRY(cudaEventRecord(c->ev[0], q));
         project_real_form(c, q);
         if (native) recompute_state_fp64(c);
         else emu_recompute_state(c->emu, q, c->sc, c->C, c->Y4, c->SWHW, c->G, c->part, c->part2);
         OMM_CUDA_TRY(cudaEventRecord(c->ev[1], q));
-        c->st = b->st;
         todo.push_back(i);
       }
       if (todo.empty()) continue;
@@ -816,9 +821,11 @@ omm_status omm_solve_batched(omm_batch* b, const double* const* C0, double* cons
       if (result[i] != OMM_OK && worst == OMM_OK) worst = result[i];
     }
     OMM_CUDA_TRY(cudaStreamSynchronize(b->st));
+  } catch (const std::bad_alloc&) {
+    give_up();
+    return fail(OMM_ERR_OOM, "omm_solve_batched: allocation failed");
   } catch (const CudaError& e) {
-    for (cudaEvent_t ev : {e0, e1, g0, g1})
-      if (ev) cudaEventDestroy(ev);
+    give_up();
     return fail(OMM_ERR_CUDA, std::string("omm_solve_batched: ") + e.what + ": " + cudaGetErrorString(e.err));
   }
   for (cudaEvent_t ev : {e0, e1, g0, g1}) cudaEventDestroy(ev);

@@ -278,13 +278,18 @@ struct EmuState {
   long ldn = 0;
   tc::Operand opHS, opC, opY, opW, opYT, opCT, opXT, opSW, opCTb;  // opCTb: C^T as a B operand
   int* err = nullptr;
-  double* slab = nullptr;     // float64 sums of the sliced products (tc::sliced_workspace_doubles)
   const tc::BlockLists* hs_blocks = nullptr;  // block sparsity of [H~; S] (256-row blocks), the mixed state's
 };
 
 namespace {
 // D needs |dD| <= 1e-7 at O(1) entries: 8 slices (40 bits) leave a wide margin
 constexpr int kDensitySlices = 8;
+
+// float64 sums of the sliced products of one call: 80 MB, which only the streams that have such products
+// running need, not every context (64 contexts of one batch held 5 GB between them)
+struct Slab : mem::Lease<double> {
+  explicit Slab(cudaStream_t st) : Lease((size_t)tc::sliced_workspace_doubles(), st) {}
+};
 }
 
 EmuState* emu_create(cudaStream_t st, int m, int n, int slices, const double* HS, const tc::BlockLists* hs_blocks) {
@@ -307,7 +312,6 @@ EmuState* emu_create(cudaStream_t st, int m, int n, int slices, const double* HS
     alloc(&es->XTs, (size_t)kDensitySlices * m * es->ldn, st);
     alloc(&es->SWs, (size_t)kDensitySlices * n * es->ldn, st);
     alloc(&es->err, 1, st);
-    alloc(&es->slab, (size_t)tc::sliced_workspace_doubles(), st);
     OMM_CUDA_TRY(cudaMemsetAsync(es->err, 0, sizeof(int), st));
     emu::slice_rows(st, HS, 2L * m, m, m, slices, es->HSs, ldm, nullptr);
     es->hs_blocks = hs_blocks;
@@ -333,7 +337,7 @@ void emu_update_H(EmuState* es, cudaStream_t st, const double* HS) {
 
 void emu_destroy(EmuState* es, cudaStream_t st) {
   if (!es) return;
-  void* bufs[] = {es->HSs, es->Cs, es->Ys, es->Ws, es->YTs, es->T64, es->CTs, es->XTs, es->SWs, es->err, es->slab};
+  void* bufs[] = {es->HSs, es->Cs, es->Ys, es->Ws, es->YTs, es->T64, es->CTs, es->XTs, es->SWs, es->err};
   for (void* b : bufs) mem::release(b, st);
   delete es;
 }
@@ -350,14 +354,15 @@ void emu_recompute_state(EmuState* es, cudaStream_t st, Scalars* sc, const doubl
                          double* SWHW, double* G, double* part, double* part2) {
   const int m = es->m, n = es->n, s = es->s;
   const long nm = (long)n * m;
+  const Slab slab(st);
   emu::slice_rows(st, C, n, m, m, s, es->Cs, es->ldm, nullptr);
   // [HC; SC] (n x m layout) = C [H~; S]^T
   emu::gemm(st, es->opC, es->opHS, m, s, tc::Epilogue{Y4, m, m, nm, 1.0, 0.0, n, 2 * m, nullptr, es->err},
-            es->slab, es->hs_blocks);
+            slab, es->hs_blocks);
   emu::slice_rows(st, Y4, 2L * n, m, m, s, es->Ys, es->ldm, nullptr);
   // [S_W | H_W] = C [SC; HC]^T
   emu::gemm(st, es->opC, es->opY, m, s,
-            tc::Epilogue{SWHW + n, 2L * n, n, -(long)n, 1.0, 0.0, n, 2 * n, nullptr, es->err}, es->slab);
+            tc::Epilogue{SWHW + n, 2L * n, n, -(long)n, 1.0, 0.0, n, 2 * n, nullptr, es->err}, slab);
   launch_functional(st, n, SWHW, part2);
   launch_finish_functional(st, sc, part2, traces_blocks(n));
   // G = 8 HC - 4 [S_W | H_W] [HC; SC]
@@ -366,7 +371,7 @@ void emu_recompute_state(EmuState* es, cudaStream_t st, Scalars* sc, const doubl
   emu::slice_rows(st, es->T64, m, 2L * n, 2L * n, s, es->YTs, es->ld2n, nullptr);
   launch_scale_copy(st, nm, Y4, 8.0, G, nullptr);
   emu::gemm(st, es->opW, es->opYT, 2 * n, s, tc::Epilogue{G, m, m, 0, -4.0, 1.0, n, m, nullptr, es->err},
-            es->slab);
+            slab);
   launch_gmax(st, nm, G, part);
   launch_finish_gmax(st, sc, part);
 }
@@ -390,16 +395,17 @@ __global__ void combine_kernel(long count, double a, const double* __restrict__ 
 void emu_density(EmuState* es, cudaStream_t st, const double* C, const double* SWHW, double* D) {
   const int m = es->m, n = es->n, s = kDensitySlices;
   const long mn = (long)m * n;
+  const Slab slab(st);
   double* CT = es->T64;       // m x n
   double* XT = es->T64 + mn;  // m x n
   emu::transpose(st, C, n, m, m, CT, n);
   emu::slice_rows(st, CT, m, n, n, s, es->CTs, es->ldn, nullptr);
   emu::slice_rows(st, SWHW, n, n, 2L * n, s, es->SWs, es->ldn, nullptr);   // S_W is symmetric
-  emu::gemm(st, es->opCT, es->opSW, n, s, tc::Epilogue{XT, n, n, 0, 1.0, 0.0, m, n, nullptr, es->err}, es->slab);
+  emu::gemm(st, es->opCT, es->opSW, n, s, tc::Epilogue{XT, n, n, 0, 1.0, 0.0, m, n, nullptr, es->err}, slab);
   combine_kernel<<<(unsigned)std::min<long>((mn + 255) / 256, 4096), 256, 0, st>>>(mn, 4.0, CT, -2.0, XT, XT);
   OMM_LAUNCH_CHECK();
   emu::slice_rows(st, XT, m, n, n, s, es->XTs, es->ldn, nullptr);
-  emu::gemm(st, es->opXT, es->opCTb, n, s, tc::Epilogue{D, m, m, 0, 1.0, 0.0, m, m, nullptr, es->err}, es->slab);
+  emu::gemm(st, es->opXT, es->opCTb, n, s, tc::Epilogue{D, m, m, 0, 1.0, 0.0, m, m, nullptr, es->err}, slab);
 }
 
 namespace {
@@ -420,6 +426,7 @@ __global__ void edm_weights_kernel(int n, const double* __restrict__ SWHW, doubl
 void emu_minus_edm(EmuState* es, cudaStream_t st, const double* C, const double* SWHW, double eta, double* out) {
   const int m = es->m, n = es->n, s = kDensitySlices;
   const long mn = (long)m * n;
+  const Slab slab(st);
   double* CT = es->T64;       // m x n
   double* VT = es->T64 + mn;  // m x n; first the n x n weights
   emu::transpose(st, C, n, m, m, CT, n);
@@ -428,9 +435,9 @@ void emu_minus_edm(EmuState* es, cudaStream_t st, const double* C, const double*
   edm_weights_kernel<<<(unsigned)std::min<long>((nn + 255) / 256, 4096), 256, 0, st>>>(n, SWHW, eta, VT);
   OMM_LAUNCH_CHECK();
   emu::slice_rows(st, VT, n, n, n, s, es->SWs, es->ldn, nullptr);  // symmetric like H~_W and S_W
-  emu::gemm(st, es->opCT, es->opSW, n, s, tc::Epilogue{VT, n, n, 0, 1.0, 0.0, m, n, nullptr, es->err}, es->slab);
+  emu::gemm(st, es->opCT, es->opSW, n, s, tc::Epilogue{VT, n, n, 0, 1.0, 0.0, m, n, nullptr, es->err}, slab);
   emu::slice_rows(st, VT, m, n, n, s, es->XTs, es->ldn, nullptr);
-  emu::gemm(st, es->opXT, es->opCTb, n, s, tc::Epilogue{out, m, m, 0, 1.0, 0.0, m, m, nullptr, es->err}, es->slab);
+  emu::gemm(st, es->opXT, es->opCTb, n, s, tc::Epilogue{out, m, m, 0, 1.0, 0.0, m, m, nullptr, es->err}, slab);
 }
 
 }  // namespace omm

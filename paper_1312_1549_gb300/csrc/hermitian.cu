@@ -263,9 +263,8 @@ omm_status omm_backward_hermitian(omm_ctx* c, double* dEdH, double* dEdS) {
   if (rc != OMM_OK) return rc;
   if ((dEdH || dEdS) && !c->solved) return fail(OMM_ERR_STATE, "omm_backward_hermitian: no converged solve");
   const int m = c->mc;
-  double* tmp = nullptr;
   try {
-    alloc(&tmp, 4 * (size_t)m * m, c->st);
+    const mem::Lease<double> tmp(4 * (size_t)m * m, c->st);
     // the density stays in tmp for dE/dS, and the host waits once
     if (dEdH) {
       form_density(c, tmp);
@@ -276,12 +275,10 @@ omm_status omm_backward_hermitian(omm_ctx* c, double* dEdH, double* dEdS) {
       extract_matrix(c->st, m, tmp, c->hz_stage, dEdS);
     }
     OMM_CUDA_TRY(cudaStreamSynchronize(c->st));
-    mem::release(tmp, c->st);
   } catch (const std::bad_alloc&) {
     return fail(OMM_ERR_OOM, "omm_backward_hermitian: device allocation failed");
   } catch (const CudaError& err) {
     cudaStreamSynchronize(c->st);
-    mem::release(tmp, c->st);
     return fail(OMM_ERR_CUDA, std::string("omm_backward_hermitian: ") + err.what + ": " + cudaGetErrorString(err.err));
   }
   return rc;

@@ -476,6 +476,8 @@ omm_status omm_update_H(omm_ctx* c, const double* H) {
     c->solved = false;
     if (c->red && reduction_error(c->red, c->st) != 0)
       return fail(OMM_ERR_TIMEOUT, "omm_update_H: a bounded device wait expired in the reduction");
+  } catch (const std::bad_alloc&) {
+    return fail(OMM_ERR_OOM, "omm_update_H: device allocation failed");
   } catch (const CudaError& e) {
     return fail(OMM_ERR_CUDA, std::string("omm_update_H: ") + e.what + ": " + cudaGetErrorString(e.err));
   }

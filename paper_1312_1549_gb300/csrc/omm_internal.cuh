@@ -93,6 +93,20 @@ void alloc(T** p, size_t count, cudaStream_t st) {
   *p = nullptr;
   *p = static_cast<T*>(alloc(count * sizeof(T), st));
 }
+// memory for the work that is queued on st while this lives, given back in the order of st
+template <typename T>
+class Lease {
+ public:
+  Lease(size_t count, cudaStream_t st) : st_(st) { alloc(&p_, count, st); }
+  ~Lease() { release(p_, st_); }
+  Lease(const Lease&) = delete;
+  Lease& operator=(const Lease&) = delete;
+  operator T*() const { return p_; }
+
+ private:
+  T* p_ = nullptr;
+  cudaStream_t st_;
+};
 }  // namespace mem
 
 // ------------------------------------------------------------------ kernel timing

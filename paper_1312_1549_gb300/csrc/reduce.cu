@@ -36,7 +36,6 @@ struct Reduction {
   __nv_bfloat16* slA = nullptr;  // slices of the A operand (up to m x m)
   __nv_bfloat16* slB = nullptr;  // slices of the B operand (m x m)
   long ldm = 0;
-  double* slab = nullptr;  // float64 sums of the sliced products
   int* err = nullptr;
   tc::BlockLists blY, blYT, blLT;  // nonzero K blocks of Y, L^-T, L^T as B operands
 };
@@ -52,12 +51,13 @@ void alloc(T** p, size_t count, cudaStream_t st) {
 void sliced_product(Reduction* r, cudaStream_t st, const double* A, long M, const double* B,
                     const tc::BlockLists* lists, double* out) {
   const int m = r->m;
+  const mem::Lease<double> slab((size_t)tc::sliced_workspace_doubles(), st);  // float64 sums
   emu::slice_rows(st, A, M, m, m, kRedSlices, r->slA, r->ldm, nullptr);
   emu::slice_rows(st, B, m, m, m, kRedSlices, r->slB, r->ldm, nullptr);
   const tc::Operand oa = tc::make_operand(r->slA, M, m, r->ldm, kRedSlices, true);
   const tc::Operand ob = tc::make_operand(r->slB, m, m, r->ldm, kRedSlices, false);
   emu::gemm(st, oa, ob, m, kRedSlices, tc::Epilogue{out, m, m, 0, 1.0, 0.0, (int)M, m, nullptr, r->err},
-            r->slab, lists);
+            slab, lists);
 }
 
 }  // namespace
@@ -85,7 +85,6 @@ Reduction* reduction_create(cudaStream_t st, int m, bool sliced, double* S, int*
       alloc(&r->YT, mm, st);
       alloc(&r->slA, (size_t)kRedSlices * m * r->ldm, st);
       alloc(&r->slB, (size_t)kRedSlices * m * r->ldm, st);
-      alloc(&r->slab, (size_t)tc::sliced_workspace_doubles(), st);
       alloc(reinterpret_cast<char**>(&work), spd_inverse_sliced_workspace_bytes(m), st);
       spd_factor_inverse_sliced(st, m, S, r->Y, work, info_dev, r->err);
       emu::transpose(st, S, m, m, m, r->L, m);     // L^T
@@ -111,7 +110,7 @@ Reduction* reduction_create(cudaStream_t st, int m, bool sliced, double* S, int*
 
 void reduction_destroy(Reduction* r, cudaStream_t st) {
   if (!r) return;
-  void* bufs[] = {r->L, r->Y, r->YT, r->W, r->slA, r->slB, r->slab, r->err};
+  void* bufs[] = {r->L, r->Y, r->YT, r->W, r->slA, r->slB, r->err};
   for (void* b : bufs) mem::release(b, st);
   tc::free_block_lists(r->blY, st);
   tc::free_block_lists(r->blYT, st);
