@@ -211,6 +211,11 @@ omm_status omm_update_H(omm_ctx* ctx, const double* H);
 /* Release every resource of the context (NULL is ignored). */
 void omm_free(omm_ctx* ctx);
 
+/* The library keeps device memory reserved for reuse: that of freed contexts and batches, and up to
+ * 2 GiB of the scratch of the entry points of omm_kernels.h. This call gives what the current device
+ * has of it unused back to the driver, after waiting for the device. Errors: OMM_ERR_CUDA. */
+omm_status omm_release_unused(void);
+
 /* ---- batches of independent problems (k-points, spins, snapshots) ---- */
 typedef struct omm_batch omm_batch; /* opaque; owned by the library */
 

@@ -7,7 +7,9 @@
  * "host"; all work is ordered on `stream` (cudaStream_t as void*, NULL = legacy
  * default stream) and the call returns after it completes. Errors are
  * returned as omm_status (see omm.h), never raised; the library never
- * traps or aborts.
+ * traps or aborts. Where a call takes scratch from the library's scratch pool,
+ * up to 2 GiB of it stay reserved for the next call (omm_release_unused of
+ * omm.h gives that back too); the rest is given back when the call ends.
  */
 #ifndef OMM_GB300_OMM_KERNELS_H
 #define OMM_GB300_OMM_KERNELS_H

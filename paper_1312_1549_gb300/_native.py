@@ -69,6 +69,7 @@ _SIGNATURES = {
     "omm_backward": (_I, [_P, _P, _P]),
     "omm_update_H": (_I, [_P, _P]),
     "omm_free": (None, [_P]),
+    "omm_release_unused": (_I, []),
     "omm_status_str": (ct.c_char_p, [_I]),
     "omm_last_error": (ct.c_char_p, []),
     "omm_launch_count": (ct.c_ulonglong, []),

@@ -38,7 +38,8 @@ cudaMemPool_t pool_of_current_device(std::map<int, cudaMemPool_t>& pools, uint64
     cudaGetLastError();
     throw std::bad_alloc();
   }
-  // what is reserved beyond `keep` goes back to the driver at the next synchronisation point
+  // what is reserved beyond `keep` goes back to the driver at a synchronisation after its release (trim_scratch
+  // does not leave that to the caller, whose next one may be far away)
   cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
   pools[dev] = pool;
   return pool;
@@ -66,6 +67,29 @@ void* alloc_scratch(size_t bytes, cudaStream_t st) {
 void release(void* p, cudaStream_t st) {
   if (p == nullptr) return;
   if (cudaFreeAsync(p, st) != cudaSuccess) cudaGetLastError();
+}
+
+void trim_scratch(cudaStream_t st) noexcept {
+  cudaMemPool_t pool = nullptr;
+  try {
+    pool = pool_of_current_device(g_scratch_pools, kScratchKeep);
+  } catch (const std::bad_alloc&) {
+    return;
+  }
+  uint64_t reserved = 0;
+  if (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  if (reserved <= kScratchKeep) return;
+  if (cudaStreamSynchronize(st) != cudaSuccess || cudaMemPoolTrimTo(pool, kScratchKeep) != cudaSuccess)
+    cudaGetLastError();
+}
+
+void release_unused() {
+  OMM_CUDA_TRY(cudaDeviceSynchronize());  // pending releases are complete
+  OMM_CUDA_TRY(cudaMemPoolTrimTo(pool_of_current_device(g_pools, UINT64_MAX), 0));
+  OMM_CUDA_TRY(cudaMemPoolTrimTo(pool_of_current_device(g_scratch_pools, kScratchKeep), 0));
 }
 
 }  // namespace mem

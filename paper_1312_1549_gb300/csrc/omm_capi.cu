@@ -731,4 +731,15 @@ omm_status omm_backward(omm_ctx* c, double* dEdH, double* dEdS) {
 
 void omm_free(omm_ctx* c) { destroy(c); }
 
+omm_status omm_release_unused(void) {
+  try {
+    mem::release_unused();
+  } catch (const std::bad_alloc&) {  // no pool can be made
+    return fail(OMM_ERR_CUDA, "omm_release_unused: no memory pool");
+  } catch (const CudaError& e) {
+    return fail(OMM_ERR_CUDA, std::string("omm_release_unused: ") + e.what + ": " + cudaGetErrorString(e.err));
+  }
+  return OMM_OK;
+}
+
 }  // extern "C"

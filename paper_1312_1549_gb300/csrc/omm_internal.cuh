@@ -88,6 +88,10 @@ void* alloc(size_t bytes, cudaStream_t st);
 // the same from a second pool that keeps at most 2 GiB reserved (scratch of the step-level entry points)
 void* alloc_scratch(size_t bytes, cudaStream_t st);
 void release(void* p, cudaStream_t st);
+// once a call's scratch is released on st: what the second pool has beyond 2 GiB goes back to the driver
+void trim_scratch(cudaStream_t st) noexcept;
+// what both pools of the current device hold unused goes back to the driver
+void release_unused();
 template <typename T>
 void alloc(T** p, size_t count, cudaStream_t st) {
   *p = nullptr;

@@ -220,6 +220,11 @@ def gemm_emu(A, B, C, alpha=1.0, beta=0.0, slices=10, stream=None):
     return C
 
 
+def release_unused():
+    """Give the device memory that the library keeps reserved but does not use back to the driver."""
+    N.check(N.lib().omm_release_unused(), "omm_release_unused")
+
+
 def launch_count():
     """Kernels launched by the library in this process."""
     return int(N.lib().omm_launch_count())

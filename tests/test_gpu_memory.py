@@ -53,3 +53,23 @@ for s in solvers[::8]:
     ref = D if ref is None else ref
     assert torch.equal(D, ref)
 """)
+
+
+def test_scratch_of_a_call_is_given_back():
+    """The float64-class inverse of m = 9472 takes more than 4 GB of scratch; at most 2 GiB of it stay reserved after
+    the call (allowing for the driver's 64 MiB), and nothing after release_unused."""
+    run("""
+m = 9472
+A = torch.eye(m, device="cuda", dtype=torch.float64)
+P = torch.empty_like(A)
+small = torch.eye(64, device="cuda", dtype=torch.float64)
+steps.spd_inverse(small, sliced=True)
+steps.release_unused()
+torch.cuda.synchronize()
+taken()
+steps.spd_inverse(A, P, sliced=True)
+assert taken() <= (2 << 30) + (64 << 20), taken()
+steps.release_unused()
+assert taken() <= 64 << 20, taken()
+assert torch.equal(P, A)
+""")
