@@ -44,9 +44,10 @@ omm_status omm_kernel_spd_inverse(int m, const double* A, double* P, int* info, 
  * blocks factored and inverted in float64. Arguments, ownership and *info as
  * for omm_kernel_spd_inverse; OMM_ERR_TIMEOUT if a bounded wait of a tensor-core
  * GEMM expired. Workspace (from the library's scratch pool, given back by the call):
- * about 2.8 m^2 float64 plus 33 m^2 bytes of slices and 240 MB of float64 sums; two more
+ * about 2.75 m^2 float64 plus 32 m^2 bytes of slices and 240 MB of float64 sums; two more
  * streams run the products that the factorisation does not wait for and are joined
- * before the call returns. */
+ * before the call returns. Where that much is not to be had, one more stream, 21 m^2 bytes
+ * of slices and 160 MB of sums, with the same result. */
 omm_status omm_kernel_spd_inverse_sliced(int m, const double* A, double* P, int* info, void* stream);
 
 /* The preconditioner-grade variant the mixed solver uses (omm_opts.precond_slices): the same

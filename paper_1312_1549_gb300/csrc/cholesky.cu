@@ -392,7 +392,7 @@ void spd_factor_inverse(cudaStream_t st, int m, double* A, double* Y, double* wo
 // ------------------------------------------------------------------ float64-class (sliced) variant
 namespace {
 
-constexpr int kInvSlices = 10;  // the most slices of a lane's products; W and Y21 take one more (workspace sizing)
+constexpr int kInvSlices = 10;  // the most slices of a lane's products; W and Y21 take one more
 
 long round_up(long x, long unit) { return (x + unit - 1) / unit * unit; }
 long round8(long x) { return round_up(x, 8); }
@@ -497,16 +497,16 @@ void chol_inv(SlicedWork& w, int r0, int b) {
   double* Y21 = w.Y + (long)r1 * m + r0;
   // L21 = A21 Y11^T, over A21 (the product reads slices)
   sliced_nt(L, w.err, b2, b1, b1, 1.0, A21, m, Y11, m, 0.0, A21, m);
-  w.wait(w.ahead.st, L.st);
+  if (w.ahead.st != L.st) w.wait(w.ahead.st, L.st);
   // W^T = Y11^T L21^T, over A12, which nothing reads (Y11^T: b1 x b1)
   emu::transpose(w.ahead.st, Y11, b1, b1, m, w.ahead.tr0, b1);
   sliced_nt(w.ahead, w.err, b1, b2, b1, 1.0, w.ahead.tr0, b1, A21, m, 0.0, A12, m, 1);
-  cudaEvent_t done = w.record(w.ahead.st);
+  const cudaEvent_t done = w.ahead.st != L.st ? w.record(w.ahead.st) : nullptr;
   // A22 -= L21 L21^T
   sliced_nt(L, w.err, b2, b2, b1, -1.0, A21, m, A21, m, 1.0, A22, m);
   chol_inv(w, r1, b2);
   // Y21 = -Y22 W
-  OMM_CUDA_TRY(cudaStreamWaitEvent(L.st, done, 0));
+  if (done != nullptr) OMM_CUDA_TRY(cudaStreamWaitEvent(L.st, done, 0));
   sliced_nt(L, w.err, b2, b1, b2, -1.0, Y22, m, A12, m, 0.0, Y21, m, 1);
   if (w.P == nullptr) return;  // the factor and its inverse only
   // this node's Y is final: its P updates may start
@@ -589,44 +589,72 @@ struct SplitInverse : Streams {
   }
 };
 
-}  // namespace
-
-size_t spd_inverse_sliced_workspace_bytes(int m) {
-  const long h = (m + 1) / 2 + NL;  // the largest off-diagonal block edge (either leaf size)
-  // Y, leaf; tr0, tr1 of one lane, tr0 of another; a slab per lane
-  const size_t f64 = (size_t)m * m + (size_t)NL * NL + 3 * ((size_t)h * h + (size_t)tc::sliced_workspace_doubles());
-  const size_t bf = 3 * 2 * (size_t)(kInvSlices + 1) * (size_t)h * round8(h);  // per lane: sl0, sl1
-  // (the split form's three pairs of m x m need less: 12 bytes per element of the padded matrix of these 47 and more)
-  return f64 * sizeof(double) + bf * sizeof(__nv_bfloat16) + 4 * 256;
-}
-
-namespace {
 void prepare_leaf() {
   static const cudaError_t e =  // thread-safe, once
       cudaFuncSetAttribute(leaf_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kLeafSmem);
   OMM_CUDA_TRY(e);
 }
 
+// Scratch of the split form from `base`, or its size alone.
+size_t carve(SplitInverse& w, int m, void* base) {
+  w.m = m;
+  w.ld = round8(m);
+  w.half = round_up(m, 64);
+  const size_t pair = 2 * (size_t)w.half * w.ld;
+  w.Ys = reinterpret_cast<__nv_bfloat16*>(round_up((long)reinterpret_cast<uintptr_t>(base), 256));
+  w.Ls = w.Ys + pair;
+  w.As = w.Ls + pair;
+  return 3 * pair * sizeof(__nv_bfloat16) + 256;
+}
+
+// Scratch of the sliced form from `base`, or its size alone. `Y`: L^-1 is not the caller's; `side`: P is wanted;
+// `ahead`: a lane of its own for the products W, which otherwise take the main lane's room and stream.
+size_t carve(SlicedWork& w, int m, int slices, bool Y, bool side, bool ahead, void* base) {
+  const long h = (m + 1) / 2 + NL;  // the largest off-diagonal block edge (either leaf size)
+  uintptr_t p = reinterpret_cast<uintptr_t>(base);
+  auto take = [&](size_t bytes) {
+    void* at = reinterpret_cast<void*>(p = (p + 255) & ~uintptr_t(255));
+    p += bytes;
+    return at;
+  };
+  auto f64 = [&](size_t count) { return static_cast<double*>(take(count * sizeof(double))); };
+  auto lane = [&](Lane& L, int most) {
+    L.slices = slices;
+    L.slab = f64(tc::sliced_workspace_doubles());
+    for (__nv_bfloat16** sl : {&L.sl0, &L.sl1})
+      *sl = static_cast<__nv_bfloat16*>(take((size_t)most * h * round8(h) * sizeof(__nv_bfloat16)));
+  };
+  w.m = m;
+  if (Y) w.Y = f64((size_t)m * m);
+  w.leaf = f64(NL * NL);
+  lane(w.main, slices + 1);  // W and Y21 take one slice more
+  if (side) {
+    lane(w.side, slices);
+    w.side.tr0 = f64((size_t)h * h);
+    w.side.tr1 = f64((size_t)h * h);
+  }
+  if (ahead) lane(w.ahead, slices + 1);
+  else w.ahead = w.main;
+  w.ahead.tr0 = f64((size_t)h * h);
+  return p - reinterpret_cast<uintptr_t>(base) + 256;
+}
+
+int slices_of(int slices) { return std::min(std::max(slices, 2), kInvSlices); }
+
 // P = A^-1 in the 3-term split form
 void split_impl(cudaStream_t st, int m, double* A, double* P, void* work, int* info_dev, int* err_dev) {
   SplitInverse w;
-  w.m = m;
-  w.ld = round8(m);
+  carve(w, m, work);
   w.A = A;
   w.P = P;
   w.info = info_dev;
   w.err = err_dev;
   w.st = st;
-  w.half = round_up(m, 64);
-  const size_t pair = 2 * (size_t)w.half * w.ld;
-  w.Ys = reinterpret_cast<__nv_bfloat16*>((reinterpret_cast<uintptr_t>(work) + 255) & ~uintptr_t(255));
-  w.Ls = w.Ys + pair;
-  w.As = w.Ls + pair;
   prepare_leaf();
   OMM_CUDA_TRY(cudaMemsetAsync(info_dev, 0, sizeof(int), st));
   // zeros above the diagonal of Y and past row m; and every element that a contraction over rows of Y or L may
   // touch past the end of a block has to be a number (it meets zeros of the other operand)
-  OMM_CUDA_TRY(cudaMemsetAsync(w.Ys, 0, 2 * pair * sizeof(__nv_bfloat16), st));
+  OMM_CUDA_TRY(cudaMemsetAsync(w.Ys, 0, (w.As - w.Ys) * sizeof(__nv_bfloat16), st));
   OMM_CUDA_TRY(cudaMemsetAsync(P, 0, sizeof(double) * m * (size_t)m, st));
   tc::split(st, A, m, m, m, w.As, w.As + w.half * w.ld, w.ld, nullptr);
   w.side = w.fork(st);
@@ -637,38 +665,16 @@ void split_impl(cudaStream_t st, int m, double* A, double* P, void* work, int* i
 
 // P = A^-1 (P != nullptr) and/or L, Y = L^-1 (Y_out != nullptr: A keeps L, zero above the diagonal)
 void sliced_impl(cudaStream_t st, int m, double* A, double* P, double* Y_out, void* work, int* info_dev,
-                 int* err_dev, int slices) {
-  const long h = (m + 1) / 2 + NL;
+                 int* err_dev, int slices, bool ahead) {
   SlicedWork w;
-  w.m = m;
   // preconditioner grade: 128-wide float32 leaves; float64-class: 64-wide float64 leaves
   w.nb = slices < kInvSlices ? NL : NB;
+  carve(w, m, slices_of(slices), Y_out == nullptr, P != nullptr, ahead, work);
+  if (Y_out) w.Y = Y_out;
   w.A = A;
   w.P = P;
   w.info = info_dev;
   w.err = err_dev;
-  double* f = static_cast<double*>(work);
-  w.Y = Y_out ? Y_out : f;
-  f += (long)m * m;
-  w.leaf = f;
-  f += NL * NL;
-  for (double** t : {&w.side.tr0, &w.side.tr1, &w.ahead.tr0}) {
-    *t = f;
-    f += h * h;
-  }
-  for (Lane* L : {&w.main, &w.side, &w.ahead}) {
-    L->slab = f;
-    f += tc::sliced_workspace_doubles();
-  }
-  uintptr_t p = (reinterpret_cast<uintptr_t>(f) + 255) & ~uintptr_t(255);
-  const size_t sl = (size_t)(kInvSlices + 1) * h * round8(h);
-  __nv_bfloat16* q = reinterpret_cast<__nv_bfloat16*>(p);
-  for (Lane* L : {&w.main, &w.side, &w.ahead}) {
-    L->sl0 = q;
-    L->sl1 = q + sl;
-    L->slices = std::min(std::max(slices, 2), kInvSlices);
-    q += 2 * sl;
-  }
   w.main.st = st;
   if (w.nb == NL) prepare_leaf();
   OMM_CUDA_TRY(cudaMemsetAsync(info_dev, 0, sizeof(int), st));
@@ -677,12 +683,10 @@ void sliced_impl(cudaStream_t st, int m, double* A, double* P, double* Y_out, vo
     OMM_CUDA_TRY(cudaMemsetAsync(P, 0, sizeof(double) * m * (size_t)m, st));
     w.side.st = w.fork(st);
   }
-  w.ahead.st = w.fork(st);
+  w.ahead.st = ahead ? w.fork(st) : st;
   chol_inv(w, 0, m);
   w.join(st);
-  if (P) {
-    launch_symmetrize_lower(st, m, P);
-  }
+  if (P) launch_symmetrize_lower(st, m, P);
   if (Y_out) {
     zero_upper_kernel<<<1024, 256, 0, st>>>(m, A);
     OMM_LAUNCH_CHECK();
@@ -691,15 +695,29 @@ void sliced_impl(cudaStream_t st, int m, double* A, double* P, double* Y_out, vo
 
 }  // namespace
 
+size_t spd_inverse_sliced_workspace_bytes(int m, int slices, bool ahead) {
+  if (slices == 1) {
+    SplitInverse w;
+    return carve(w, m, nullptr);
+  }
+  SlicedWork w;
+  return carve(w, m, slices_of(slices), true, true, ahead, nullptr);
+}
+
+size_t spd_factor_inverse_sliced_workspace_bytes(int m) {
+  SlicedWork w;
+  return carve(w, m, kInvSlices, false, false, true, nullptr);
+}
+
 void spd_inverse_sliced(cudaStream_t st, int m, double* A, double* P, void* work, int* info_dev, int* err_dev,
-                        int slices) {
+                        int slices, bool ahead) {
   if (slices == 1) split_impl(st, m, A, P, work, info_dev, err_dev);
-  else sliced_impl(st, m, A, P, nullptr, work, info_dev, err_dev, slices);
+  else sliced_impl(st, m, A, P, nullptr, work, info_dev, err_dev, slices, ahead);
 }
 
 void spd_factor_inverse_sliced(cudaStream_t st, int m, double* A, double* Y, void* work, int* info_dev,
                                int* err_dev) {
-  sliced_impl(st, m, A, nullptr, Y, work, info_dev, err_dev, kInvSlices);
+  sliced_impl(st, m, A, nullptr, Y, work, info_dev, err_dev, kInvSlices, true);
 }
 
 }  // namespace omm

@@ -115,11 +115,18 @@ omm_status spd_inverse_sliced_impl(const char* who, int m, const double* A, doub
   try {
     const size_t mm = (size_t)m * m;
     double* W = scratch.get<double>(mm);
-    void* work = scratch.get<char>(spd_inverse_sliced_workspace_bytes(m));
+    void* work = nullptr;
+    bool ahead = true;
+    try {
+      work = scratch.get<char>(spd_inverse_sliced_workspace_bytes(m, slices, ahead));
+    } catch (const std::bad_alloc&) {  // a third less, without the products that run ahead
+      ahead = false;
+      work = scratch.get<char>(spd_inverse_sliced_workspace_bytes(m, slices, ahead));
+    }
     int* flags = scratch.get<int>(2);  // [0] pivot info, [1] bounded-wait failures
     OMM_CUDA_TRY(cudaMemsetAsync(flags, 0, 2 * sizeof(int), st));
     OMM_CUDA_TRY(cudaMemcpyAsync(W, A, mm * sizeof(double), cudaMemcpyDefault, st));
-    spd_inverse_sliced(st, m, W, P, work, flags, flags + 1, slices);
+    spd_inverse_sliced(st, m, W, P, work, flags, flags + 1, slices, ahead);
     int h[2] = {0, 0};
     OMM_CUDA_TRY(cudaMemcpyAsync(h, flags, sizeof(h), cudaMemcpyDeviceToHost, st));
     OMM_CUDA_TRY(cudaStreamSynchronize(st));

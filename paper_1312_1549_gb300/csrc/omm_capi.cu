@@ -348,6 +348,7 @@ omm_status omm_create(int m, int n, const double* H, const double* S, const doub
   double* A = nullptr;
   double* work = nullptr;
   int* inv_err = nullptr;
+  bool ahead = true;  // of the sliced inverse
   try {
     const long mm = (long)m * m, nm = (long)n * m;
     for (auto& e : c->ev) OMM_CUDA_TRY(cudaEventCreate(&e));
@@ -379,7 +380,15 @@ omm_status omm_create(int m, int n, const double* H, const double* S, const doub
       dev_alloc(&c->P, mm, c->st);
       tmp_alloc(&A, mm, c->st);
       if (sliced_inverse) {
-        tmp_alloc(&work, (spd_inverse_sliced_workspace_bytes(m) + sizeof(double) - 1) / sizeof(double), c->st);
+        auto doubles = [&]() {
+          return (spd_inverse_sliced_workspace_bytes(m, o.precond_slices, ahead) + sizeof(double) - 1) / sizeof(double);
+        };
+        try {
+          tmp_alloc(&work, doubles(), c->st);
+        } catch (const std::bad_alloc&) {  // a third less, without the products that run ahead
+          ahead = false;
+          tmp_alloc(&work, doubles(), c->st);
+        }
         tmp_alloc(&inv_err, 1, c->st);
         OMM_CUDA_TRY(cudaMemsetAsync(inv_err, 0, sizeof(int), c->st));
       } else {
@@ -392,7 +401,7 @@ omm_status omm_create(int m, int n, const double* H, const double* S, const doub
         OMM_CUDA_TRY(cudaMemcpyAsync(A, c->HS + mm, mm * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
       }
       OMM_CUDA_TRY(cudaEventRecord(c->ev[2], c->st));
-      if (sliced_inverse) spd_inverse_sliced(c->st, m, A, c->P, work, c->info_dev, inv_err, o.precond_slices);
+      if (sliced_inverse) spd_inverse_sliced(c->st, m, A, c->P, work, c->info_dev, inv_err, o.precond_slices, ahead);
       else spd_inverse(c->st, m, A, c->P, work, c->info_dev);
       OMM_CUDA_TRY(cudaEventRecord(c->ev[3], c->st));
     }

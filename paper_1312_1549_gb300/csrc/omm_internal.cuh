@@ -167,12 +167,15 @@ void spd_inverse(cudaStream_t st, int m, double* A, double* P, double* work, int
 // The same inverse with sliced tensor-core products (`slices` fixed-point slices of 5 bits,
 // 2..10; 10 is float64-class); A is overwritten. err_dev receives a nonzero code if a bounded
 // wait of a tensor-core GEMM expired.
-size_t spd_inverse_sliced_workspace_bytes(int m);
+// ahead: with room for a third stream, on which products run ahead of the factorisation (see cholesky.cu); without
+// it the results are the same, later. Callers fall back to that where the larger workspace is not to be had.
+size_t spd_inverse_sliced_workspace_bytes(int m, int slices, bool ahead);
 void spd_inverse_sliced(cudaStream_t st, int m, double* A, double* P, void* work, int* info_dev, int* err_dev,
-                        int slices = 10);
+                        int slices, bool ahead);
 // The factor alone, for the reduction to standard form: A = L L^T with L left in A (lower
-// triangle, zero above) and Y = L^-1 (lower, zero above); same workspaces as the inverses.
+// triangle, zero above) and Y = L^-1 (lower, zero above); the float64 form has the inverse's workspace.
 void spd_factor_inverse(cudaStream_t st, int m, double* A, double* Y, double* work, int* info_dev);
+size_t spd_factor_inverse_sliced_workspace_bytes(int m);
 void spd_factor_inverse_sliced(cudaStream_t st, int m, double* A, double* Y, void* work, int* info_dev,
                                int* err_dev);
 

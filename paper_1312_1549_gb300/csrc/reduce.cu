@@ -85,7 +85,7 @@ Reduction* reduction_create(cudaStream_t st, int m, bool sliced, double* S, int*
       alloc(&r->YT, mm, st);
       alloc(&r->slA, (size_t)kRedSlices * m * r->ldm, st);
       alloc(&r->slB, (size_t)kRedSlices * m * r->ldm, st);
-      alloc(reinterpret_cast<char**>(&work), spd_inverse_sliced_workspace_bytes(m), st);
+      alloc(reinterpret_cast<char**>(&work), spd_factor_inverse_sliced_workspace_bytes(m), st);
       spd_factor_inverse_sliced(st, m, S, r->Y, work, info_dev, r->err);
       emu::transpose(st, S, m, m, m, r->L, m);     // L^T
       emu::transpose(st, r->Y, m, m, m, r->YT, m);  // L^-T
