@@ -10,121 +10,6 @@
 namespace omm {
 namespace dev {
 
-// n x m arrays, by (row, column pair) units: Delta = -PG + beta Delta (Sec. 2.3, Polak-Ribiere
-// direction; beta = 0 restarts) and its split into hi/lo (leading dimension ldm)
-__device__ __forceinline__ void direction_split_body(long n, long m, const double* __restrict__ PG,
-                                                     double* __restrict__ Dir, __nv_bfloat16* __restrict__ hi,
-                                                     __nv_bfloat16* __restrict__ lo, long ldm, const Scalars* sc,
-                                                     int bx, int nbx) {
-  if (stopped(sc)) return;
-  const double beta = sc->beta;
-  const bool restart = sc->restart_dir != 0;  // beta = 0: the direction is -PG
-  const long units = pair_units(n, m);
-  for (long u = bx; u < units; u += nbx) {
-    long r, c;
-    unit_pos(u, m, r, c);
-    if (c >= m) continue;
-    const double* p = PG + r * m + c;
-    double* d = Dir + r * m + c;
-    const long off = r * ldm + c;
-    const bool vec = c + 1 < m && ((reinterpret_cast<uintptr_t>(p) | reinterpret_cast<uintptr_t>(d)) & 15) == 0 &&
-                     ((reinterpret_cast<uintptr_t>(hi + off) | reinterpret_cast<uintptr_t>(lo + off)) & 3) == 0;
-    if (vec) {
-      const double2 a = *reinterpret_cast<const double2*>(p);
-      double2 x;
-      if (restart) {  // -PG: a sign flip on the integer pipe
-        x = make_double2(__longlong_as_double(__double_as_longlong(a.x) ^ (long long)0x8000000000000000ull),
-                         __longlong_as_double(__double_as_longlong(a.y) ^ (long long)0x8000000000000000ull));
-      } else {        // one float64 FMA per element (the negation folds into it)
-        const double2 b = *reinterpret_cast<const double2*>(d);
-        x = make_double2(fma(beta, b.x, -a.x), fma(beta, b.y, -a.y));
-      }
-      *reinterpret_cast<double2*>(d) = x;
-      split_store2_fast(x.x, x.y, hi, lo, off);
-    } else {
-      for (int k = 0; k < 2 && c + k < m; ++k) {
-        const double x = restart ? __longlong_as_double(__double_as_longlong(p[k]) ^ (long long)0x8000000000000000ull)
-                                 : fma(beta, d[k], -p[k]);
-        d[k] = x;
-        split_store_fast(x, hi, lo, off + k);
-      }
-    }
-  }
-}
-
-// one element of the state update of Eq. 16 (mixed path: dHC, dSC are the changes since the last
-// float64-class refresh, the corrections of the incremental gradient): five float64 FMAs
-__device__ __forceinline__ void update_element(double x, double& C, double dir, double& HC, double& SC, double HD,
-                                               double SD, double& dHC, double& dSC) {
-  C = fma(x, dir, C);
-  HC = fma(x, HD, HC);
-  SC = fma(x, SD, SC);
-  dHC = fma(x, HD, dHC);
-  dSC = fma(x, SD, dSC);
-}
-
-// (row, column pair) units of n x m arrays: C, HC, SC += x (Delta, H Delta, S Delta) and dHC, dSC
-// += x (H Delta, S Delta) (Eq. 16 and the footnote of Sec. 2.3), and the bf16 splits of the new
-// values into the operand stack [dHC; dSC; HC; SC; ...] (6n rows of leading dimension ldm; Ylo is
-// its lo half). G is not touched: the gradient GEMM's epilogue forms it.
-__device__ __forceinline__ void update_state_split_body(long n, long m, double* __restrict__ C,
-                                                        double* __restrict__ Y4, const double* __restrict__ Dir,
-                                                        double* __restrict__ dY, __nv_bfloat16* __restrict__ Yhi,
-                                                        __nv_bfloat16* __restrict__ Ylo, long ldm,
-                                                        const Scalars* sc, int bx, int nbx) {
-  if (stopped(sc)) return;
-  const double x = sc->x;
-  const long nm = n * m;
-  const bool base_ok = ((m & 1) == 0) &&
-                       ((reinterpret_cast<uintptr_t>(C) | reinterpret_cast<uintptr_t>(Y4) |
-                         reinterpret_cast<uintptr_t>(dY) | reinterpret_cast<uintptr_t>(Dir)) & 15) == 0 &&
-                       ((reinterpret_cast<uintptr_t>(Yhi) | reinterpret_cast<uintptr_t>(Ylo)) & 3) == 0 &&
-                       (ldm & 1) == 0;
-  const long units = pair_units(n, m);
-  for (long u = bx; u < units; u += nbx) {
-    long r, k;
-    unit_pos(u, m, r, k);
-    if (k >= m) continue;
-    const long o = r * m + k;
-    // stack rows of dHC, dSC, HC, SC for Wannier function r
-    const long odh = r * ldm + k, ods = (n + r) * ldm + k, oh = (2 * n + r) * ldm + k, os = (3 * n + r) * ldm + k;
-    if (base_ok) {  // k even, m even: the pair is complete and 16-byte aligned
-      double2 C2 = *reinterpret_cast<double2*>(C + o), H2 = *reinterpret_cast<double2*>(Y4 + o);
-      double2 S2 = *reinterpret_cast<double2*>(Y4 + nm + o), DH2 = *reinterpret_cast<double2*>(dY + o);
-      double2 DS2 = *reinterpret_cast<double2*>(dY + nm + o);
-      const double2 D2 = *reinterpret_cast<const double2*>(Dir + o);
-      const double2 HD2 = *reinterpret_cast<const double2*>(Y4 + 2 * nm + o);
-      const double2 SD2 = *reinterpret_cast<const double2*>(Y4 + 3 * nm + o);
-      update_element(x, C2.x, D2.x, H2.x, S2.x, HD2.x, SD2.x, DH2.x, DS2.x);
-      update_element(x, C2.y, D2.y, H2.y, S2.y, HD2.y, SD2.y, DH2.y, DS2.y);
-      *reinterpret_cast<double2*>(C + o) = C2;
-      *reinterpret_cast<double2*>(Y4 + o) = H2;
-      *reinterpret_cast<double2*>(Y4 + nm + o) = S2;
-      *reinterpret_cast<double2*>(dY + o) = DH2;
-      *reinterpret_cast<double2*>(dY + nm + o) = DS2;
-      split_store2_fast(DH2.x, DH2.y, Yhi, Ylo, odh);
-      split_store2_fast(DS2.x, DS2.y, Yhi, Ylo, ods);
-      split_store2_fast(H2.x, H2.y, Yhi, Ylo, oh);
-      split_store2_fast(S2.x, S2.y, Yhi, Ylo, os);
-    } else {
-      for (int t = 0; t < 2 && k + t < m; ++t) {
-        const long e = o + t;
-        double Cv = C[e], Hv = Y4[e], Sv = Y4[nm + e], DHv = dY[e], DSv = dY[nm + e];
-        update_element(x, Cv, Dir[e], Hv, Sv, Y4[2 * nm + e], Y4[3 * nm + e], DHv, DSv);
-        C[e] = Cv;
-        Y4[e] = Hv;
-        Y4[nm + e] = Sv;
-        dY[e] = DHv;
-        dY[nm + e] = DSv;
-        split_store_fast(DHv, Yhi, Ylo, odh + t);
-        split_store_fast(DSv, Yhi, Ylo, ods + t);
-        split_store_fast(Hv, Yhi, Ylo, oh + t);
-        split_store_fast(Sv, Yhi, Ylo, os + t);
-      }
-    }
-  }
-}
-
 // ---- the mixed path's float32 side quantities (Delta, P G, [H Delta; S Delta], [dHC; dSC]:
 // leading dimension ldm; the float64 state C, HC, SC, G has leading dimension m)
 

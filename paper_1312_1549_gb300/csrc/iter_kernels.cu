@@ -36,11 +36,6 @@ __global__ void add_scaled_kernel(long count, const double* S, const double* T, 
     A[i] = S[i] + (T ? T[i] * s : 0.0);
 }
 
-__global__ void fill_kernel(long count, double v, double* d) {
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < count; i += (long)gridDim.x * blockDim.x)
-    d[i] = v;
-}
-
 // partials of <G,PG>, <G_old,PG>, <G,Delta_old>, max|G| per block
 __global__ void __launch_bounds__(TB)
 grad_reduce_kernel(long count, const double* __restrict__ G, const double* __restrict__ PG,
@@ -199,10 +194,6 @@ void launch_add_scaled(cudaStream_t st, long count, const double* S, const doubl
   add_scaled_kernel<<<grid_for(count), TB, 0, st>>>(count, S, T, s, A);
   OMM_LAUNCH_CHECK();
 }
-void launch_fill(cudaStream_t st, long count, double v, double* d) {
-  fill_kernel<<<grid_for(count), TB, 0, st>>>(count, v, d);
-  OMM_LAUNCH_CHECK();
-}
 void launch_grad_reduce(cudaStream_t st, long count, const double* G, const double* PG, const double* Gold,
                         const double* Dir, double* part, const Scalars* sc) {
   launch_pdl(st, dim3(reduce_blocks(count)), dim3(TB), 0, grad_reduce_kernel, count, G, PG, Gold, Dir, part, sc);
@@ -247,16 +238,6 @@ void launch_update_state(cudaStream_t st, int n, long m, double* C, double* Y4, 
   OMM_LAUNCH_CHECK();
 }
 namespace {
-__global__ void __launch_bounds__(256)
-direction_split_kernel(long n, long m, const double* __restrict__ PG, double* __restrict__ Dir,
-                       __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo, long ldm, const Scalars* sc) {
-  dev::direction_split_body(n, m, PG, Dir, hi, lo, ldm, sc, blockIdx.x, gridDim.x);
-}
-__global__ void __launch_bounds__(256)
-update_state_split_kernel(long n, long m, double* C, double* Y4, const double* Dir, double* dY, __nv_bfloat16* Yhi,
-                          __nv_bfloat16* Ylo, long ldm, const Scalars* sc) {
-  dev::update_state_split_body(n, m, C, Y4, Dir, dY, Yhi, Ylo, ldm, sc, blockIdx.x, gridDim.x);
-}
 __global__ void __launch_bounds__(TB)
 update_subspace_split_kernel(int n, double* SWHW, const double* __restrict__ Proj, const double* __restrict__ Wref,
                              __nv_bfloat16* Whi, __nv_bfloat16* Wlo, long ldw, const Scalars* sc, int quarters) {
@@ -271,16 +252,6 @@ static unsigned pair_grid(long rows, long cols) {
   return (unsigned)(units < 1 ? 1 : (units > 16384 ? 16384 : units));
 }
 
-void launch_direction_split(cudaStream_t st, long n, long m, const double* PG, double* Dir, __nv_bfloat16* hi,
-                            __nv_bfloat16* lo, long ldm, const Scalars* sc) {
-  direction_split_kernel<<<pair_grid(n, m), 256, 0, st>>>(n, m, PG, Dir, hi, lo, ldm, sc);
-  OMM_LAUNCH_CHECK();
-}
-void launch_update_state_split(cudaStream_t st, long n, long m, double* C, double* Y4, const double* Dir, double* dY,
-                               __nv_bfloat16* Yhi, __nv_bfloat16* Ylo, long ldm, const Scalars* sc) {
-  update_state_split_kernel<<<pair_grid(n, m), 256, 0, st>>>(n, m, C, Y4, Dir, dY, Yhi, Ylo, ldm, sc);
-  OMM_LAUNCH_CHECK();
-}
 namespace {
 __global__ void __launch_bounds__(256)
 direction_split32_kernel(long n, long m, const float* PG, float* Dir, __nv_bfloat16* hi, __nv_bfloat16* lo, long ldm,

@@ -190,25 +190,18 @@ void launch_grad_reduce(cudaStream_t st, long count, const double* G, const doub
 // <G_old,PG>, <G,Delta_old>, max|G|)
 void launch_control_direction(cudaStream_t st, Scalars* sc, const double* part, int mixed, int nparts);
 void launch_direction(cudaStream_t st, long count, const double* PG, double* Dir, const Scalars* sc);
-// the mixed path's fused forms: the direction (n x m) and its bf16 split (leading dimension ldm);
-// the state update of C, HC, SC, dHC, dSC with the splits of the new dHC, dSC, HC, SC into the
-// operand stack rows [0, 4n) (Yhi, Ylo: the stack's hi and lo halves); the update of H_W, S_W
-// with the split of [dS_W | dH_W] into W (Whi, Wlo: its columns 2n..4n, leading dimension ldw)
-void launch_direction_split(cudaStream_t st, long n, long m, const double* PG, double* Dir, __nv_bfloat16* hi,
-                            __nv_bfloat16* lo, long ldm, const Scalars* sc);
-void launch_update_state_split(cudaStream_t st, long n, long m, double* C, double* Y4, const double* Dir, double* dY,
-                               __nv_bfloat16* Yhi, __nv_bfloat16* Ylo, long ldm, const Scalars* sc);
-void launch_update_subspace_split(cudaStream_t st, int n, double* SWHW, const double* Proj, const double* Wref,
-                                  __nv_bfloat16* Whi, __nv_bfloat16* Wlo, long ldw, const Scalars* sc);
-// the same steps on the mixed path's float32 side quantities (Delta, P G, [H Delta; S Delta],
-// [dHC; dSC], leading dimension ldm): the direction and its split; the state update with three
-// float64 FMAs per element; without a preconditioner, the reductions with PG = G (PG and G_old
-// written)
+// the mixed path's fused forms, on its float32 side quantities (Delta, P G, [H Delta; S Delta], [dHC; dSC], leading
+// dimension ldm): the direction (n x m) and its bf16 split; the state update of C, HC, SC, dHC, dSC with three float64
+// FMAs per element and the splits of the new dHC, dSC, HC, SC into the operand stack rows [0, 4n) (Yhi, Ylo: the
+// stack's hi and lo halves); the update of H_W, S_W with the split of [dS_W | dH_W] into W (Whi, Wlo: its columns
+// 2n..4n, leading dimension ldw); without a preconditioner, the reductions with PG = G (PG and G_old written)
 void launch_direction_split32(cudaStream_t st, long n, long m, const float* PG, float* Dir, __nv_bfloat16* hi,
                               __nv_bfloat16* lo, long ldm, const Scalars* sc);
 void launch_update_state_split32(cudaStream_t st, long n, long m, double* C, double* Y4, const float* Dir,
                                  const float* HD32, float* dY32, __nv_bfloat16* Yhi, __nv_bfloat16* Ylo, long ldm,
                                  const Scalars* sc);
+void launch_update_subspace_split(cudaStream_t st, int n, double* SWHW, const double* Proj, const double* Wref,
+                                  __nv_bfloat16* Whi, __nv_bfloat16* Wlo, long ldw, const Scalars* sc);
 void launch_reduce_unpreconditioned(cudaStream_t st, long n, long m, const double* G, double* Gold, const float* Dir,
                                     float* PG, long ldm, double* part, const Scalars* sc);
 // fp32_products: the mixed path's traces (float32 products of the tensor-core projections)
@@ -230,7 +223,6 @@ void launch_gmax(cudaStream_t st, long count, const double* G, double* part);
 void launch_finish_gmax(cudaStream_t st, Scalars* sc, const double* part);
 void launch_two_i_minus(cudaStream_t st, int n, const double* SW, long ldsw, double* out);  // 2I - S_W
 void launch_symmetrize_lower(cudaStream_t st, int m, double* A);  // A[j,i] = A[i,j], i > j
-void launch_fill(cudaStream_t st, long count, double v, double* dst);
 
 // Device-side line minimum (first local minimum of the quartic along x > 0).
 
