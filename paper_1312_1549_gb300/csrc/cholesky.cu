@@ -25,8 +25,8 @@
 // of the blocks that follow. W = L21 Y11 does not need the right half, so it runs on a third stream
 // beside that half's factorisation: the chain of a node is three products instead of the four that
 // -(Y22 L21) Y11 makes, and neither transposes nor copies. The chain is what bounds the inverse (51 nodes one
-// after another at m = 3328): float64-class inverse 17.9 -> 15.7 ms, Cholesky-flavour solve of m = 2944
-// 46.4 -> 44.3 ms. W and Y21 take one slice more than the other products: sliced by columns W loses more than
+// after another at m = 3328): by this alone the float64-class inverse went from 17.9 to 15.7 ms (13.5 with what
+// followed), a Cholesky-flavour solve of m = 2944 from 46.4 to 44.3 (43.3). W and Y21 take one slice more than the other products: sliced by columns W loses more than
 // Y22 L21 by rows, and the error of P would be up to 30 % larger than in that order; with the extra slice it is
 // 5 to 25 % smaller (against a refined inverse, m = 160 to 3328), for 3 % of the time.
 #include "emu.cuh"
@@ -53,7 +53,7 @@ leaf_f64_kernel(double* A, long lda, int b, double* Linv, long ldi, int* info, i
 
 // The Gram block Y^T Y (both triangles) of a leaf's inverse Y (b x b, zero above the diagonal) into Pblk: another
 // 44 thousand FMAs, beside the factorisation instead of at the end of each leaf of its chain (20 of a leaf's 100 us;
-// float64-class inverse of m = 3328, 52 leaves: 14.5 -> 13.6 ms).
+// by this alone the float64-class inverse of m = 3328, 52 leaves, went from 14.5 to 13.6 ms).
 __global__ void __launch_bounds__(kLeaf64Threads)
 gram_f64_kernel(int b, const double* Y, long ldy, double* Pblk, long ldp) {
   dev::pdl_begin();

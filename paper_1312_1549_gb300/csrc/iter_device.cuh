@@ -27,7 +27,7 @@ __device__ __forceinline__ double warp_max(double v) {
 }
 // Sums of N values over the TB threads; the results are in thread 0 (in v). A float64 add takes its warp
 // about 30 clocks of the SM's float64 unit however many lanes are active, so the N sums lie side by side in
-// the lanes: thread (seg, q) adds the q-th values of TB / kSegs threads, then thread q the kSegs partial sums
+// the lanes: thread (q, seg) adds the q-th values of sixteen threads, then thread q the sixteen partial sums
 // (N (TB / 32 + 2) / 2 adds or so; a shuffle tree per value and warp took 5 N per warp, 13 thousand clocks
 // for the eleven traces). sh: N x (TB + 1) doubles. Fixed order.
 template <int N>

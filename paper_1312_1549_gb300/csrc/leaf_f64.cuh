@@ -17,8 +17,8 @@ namespace dev {
 // The inverse joins inverted diagonal blocks of edge 8, 16 and 32:
 // X21 = -X22 (L21 X11), the contraction cut at the triangles.
 // (One column at a time with three barriers each, one thread per column of the
-// inverse and two divisions per pivot it took 150-215 us per block; the float64-class inverse at
-// m = 3328, 52 blocks one after another, went from 30.1 to 25.9 ms.)
+// inverse and two divisions per pivot it took 150-215 us per block, 67 to 83 now; by this alone the float64-class
+// inverse at m = 3328, 52 blocks one after another, went from 30.1 to 25.9 ms.)
 constexpr int NB = 64;
 constexpr int kLeaf64Threads = 256;
 

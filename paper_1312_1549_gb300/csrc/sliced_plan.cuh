@@ -10,8 +10,8 @@
 // SMs.) Workers on whole tiles, and on the same fraction of a tile, walk the slice pairs in step and
 // share the slices through L2; shares at arbitrary places of the line do not (the slices of a
 // 1024 x 6656 x 6656 product are 1 GB), which costs more than it balances once they outgrow L2 (that
-// product with its slicing: 5.3 ms in whole tiles, 5.5 with one even line, 3.9 with this; a 1495 x 260
-// state's products 0.9-1.4 ms each before, 0.13-0.22 now).
+// product with its slicing and its scratch: 5.3 ms in whole tiles, 5.5 with one even line, 3.9 with this, 3.0
+// since the scratch comes from a pool; a 1495 x 260 state's products 0.9-1.4 ms each before, 0.14 now).
 #pragma once
 
 #include <algorithm>
