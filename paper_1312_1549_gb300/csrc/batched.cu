@@ -397,6 +397,14 @@ omm_status omm_create_batched(int count, const int* m, const int* n, const doubl
   b->opts = o;
   b->precond = o.no_precondition == 0 && o.cholesky == 0;
   b->ctx.assign(count, nullptr);
+  // the instances' streams start after what is queued on the batch stream, which may still be writing the inputs
+  cudaError_t ready = cudaEventCreateWithFlags(&b->forked, cudaEventDisableTiming);
+  if (ready == cudaSuccess) ready = cudaEventRecord(b->forked, b->st);
+  if (ready != cudaSuccess) {
+    cudaGetLastError();
+    batch_destroy(b);
+    return fail(OMM_ERR_CUDA, std::string("omm_create_batched: ") + cudaGetErrorString(ready));
+  }
   // per-instance setup (float64 Cholesky inverse etc.) from several host threads, each on its
   // own stream, so that the small factorisations of different instances overlap on the GPU
   {
@@ -410,6 +418,8 @@ omm_status omm_create_batched(int count, const int* m, const int* n, const doubl
       cudaSetDevice(device);
       cudaStream_t s = nullptr;
       if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) s = nullptr;
+      if (cudaStreamWaitEvent(s, b->forked, 0) != cudaSuccess) cudaEventSynchronize(b->forked);
+      cudaGetLastError();  // (either may fail: then the instances share the default stream, or the host waits)
       for (int i = next++; i < count; i = next++) {
         rcs[i] = omm_create(m[i], n[i], H[i], S[i], T ? T[i] : nullptr, eta[i], tau[i], &o, s, &b->ctx[i]);
         if (rcs[i] != OMM_OK) msgs[i] = omm_last_error();
@@ -512,7 +522,6 @@ omm_status omm_create_batched(int count, const int* m, const int* n, const doubl
       }
     }
     for (cudaStream_t& q : b->pool) OMM_CUDA_TRY(cudaStreamCreateWithFlags(&q, cudaStreamNonBlocking));
-    OMM_CUDA_TRY(cudaEventCreateWithFlags(&b->forked, cudaEventDisableTiming));
     for (cudaEvent_t& e : b->joined) OMM_CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     alloc(&b->args, count, b->st);
     alloc(&b->state_args, count, b->st);
