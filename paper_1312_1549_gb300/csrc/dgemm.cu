@@ -115,7 +115,7 @@ dgemm_kernel(int transA, int transB, int M, int N, int K, double alpha,
 // every SM without one idles while the others work through 64 x 64 x K FMAs at two per clock: the
 // products of an m = 207, n = 36 solve took 176 us each on 4 to 16 SMs, 12 now. (By this alone the energy
 // and gradients of that system went from 65.6 to 11.1 ms, a solve of m = 416, n = 64 from 76.1 to 11.4; they
-// take 7.1 and 7.8 with what followed.) Here a tile is 16 x 16 or 32 x 32 and CTA q of a
+// take 7 to 8 with what followed.) Here a tile is 16 x 16 or 32 x 32 and CTA q of a
 // cluster of KS sums the q-th part of the contraction; the partial tiles meet in shared memory over
 // the cluster (fixed order, so results stay reproducible) and every CTA stores its share of the rows.
 // The float64 pipe takes a warp's FMA every 16 clocks, so one output per thread and two

@@ -165,6 +165,8 @@ struct SlicedPlan {
 };
 // pairs: clusters of two CTAs that the device holds at once; sms: its SMs
 inline SlicedPlan plan_sliced(int M, int N, int K, const PairList& pl, const BlockLists* sparse, int pairs, int sms) {
+  if (sparse != nullptr && (long)sparse->off_host.size() != (N + 255) / 256 + 1)
+    throw CudaError{cudaErrorInvalidValue, "tc::plan_sliced: block lists do not match the tiles"};
   const long nkb = (K + BK - 1) / BK;
   const int nchunk = pl.nchunk > 0 ? pl.nchunk : 1;
   // Tile shape and number of workers with the shortest estimated time, in SM clocks. A stage takes as
